@@ -37,7 +37,7 @@ REFERENCE_SAMPLE = 64      # images per step of the --impl reference arm: the wh
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from an ncu capture (profiles/), by kernel
 # (kernels changed since their capture, or never captured, have no entry and report null)
 NCU_TRAFFIC_BYTES = {"stage1": 66078208, "gather": 10355200, "scores": 87525888, "sinkhorn_reg": 4935424,
-                     "merge": 118104064, "density_tile": 318402048}
+                     "merge": 118104064, "density_tile": None}
 
 
 def cpu_threads() -> int:
@@ -202,7 +202,7 @@ def density_line(args) -> dict:
                          "traffic": NCU_TRAFFIC_BYTES["density_tile"]},
             "e2e": {"value": batch / e2e_ms * 1e3, "unit": "images/s", "h2d_bytes_per_step": nbytes,
                     "d2h_bytes_per_step": 4 * batch, "ms_per_step": e2e_ms},
-            "gpu_launches": 2 * args.steps, "clocks": clocks}
+            "gpu_launches": 3 * args.steps, "clocks": clocks}
     if not args.no_cpu_baseline:
         from oracle import density as od
         sample = host[:4].numpy()

@@ -1,201 +1,279 @@
 // Textual density rho of page images (Eq. 9; Appendix B): BT.601 grayscale, 3 x 3 Sobel gradient
 // magnitude, threshold tau, fraction of edge pixels per token patch, mean over the patches.
 //
-// The arithmetic is exact.  With 8-bit channels, 1000 * 255 * I = 299 R + 587 G + 114 B is an integer
-// below 2^18, the Sobel sums are integers below 2^21 in magnitude, and
+// The counts are exact.  With 8-bit channels, 1000 * 255 * I = 299 R + 587 G + 114 B is an integer
+// below 2^18, the Sobel sums are integers below 2^21 in magnitude, so all of them are exact in fp32, and
 //     G >= tau   <=>   Gx_int^2 + Gy_int^2 >= (255000 tau)^2,
-// a comparison of a 64-bit integer with a constant the host rounds up once.  Every pixel's decision is
-// therefore the one exact arithmetic takes, and the counts do not depend on the order of anything.
+// the right side rounded up once by the host.  The difference of the two sides is formed in fp32 by two
+// fused multiply-adds (error below 2^-22 of the threshold where it is small); a pixel that comes within 2^-21 of the
+// threshold is decided again in 64-bit integers.
 // Pixels outside the image take the value of the nearest pixel inside.
 //
-// One CTA of 288 threads per 64 x 64 tile of pixels (one token patch of 64 x 64, or 4 / 16 patches of
-// 32 x 32 / 16 x 16):
-//   1. a tile row is up to 192 contiguous bytes, 16-byte aligned (the image width is a multiple of
-//      16): a thread fetches 48 bytes = 16 pixels with three 16-byte loads, and the one-pixel ring left
-//      and right of the tile pixel by pixel; every load of the CTA is issued before the first use (one
-//      trip to memory); the pixels become integer gray values in a 66-row tile in shared memory.  The
-//      gray value of a pixel is two dp2a instructions on the words as loaded (16-bit weights against
-//      the bytes of a word, whichever of the four alignments the 3-byte pixel has), no byte is
-//      extracted;
-//   2. 256 threads each walk down 8 rows of two adjacent columns with the horizontal sums of three
-//      rows in registers: 1.5 shared-memory loads and about a dozen integer operations per pixel; the
-//      rows and columns of a thread lie in one patch, so the counts are reduced over the lanes that
-//      share a patch and added to the patch's counter in shared memory.
-// The kernel is bound by instruction issue, not by memory, which is why the instruction count per
-// pixel is what the layout above is about.
-// The CTA writes its patches' counts and adds their sum to the image's count (integer atomics: the
-// result does not depend on the order); a second small kernel turns the image counts into rho.
+// A CTA owns a tile of up to 256 x 64 pixels.  It fetches the tile's rows and the one above and below (3 bytes per
+// pixel, plus 16 bytes on either side for the ring) as one tiled TMA box (pages seen as 32-bit words); four such
+// CTAs share an SM, so that one loads while the others compute.  A thread owns 16 adjacent columns of 8 rows (16 x 8
+// threads: four warps, one for each scheduler of the SM) and walks down the rows:
+//   * 16 pixels are 12 words of shared memory, read as three 16-byte vectors (48 bytes from lane to lane:
+//     no bank conflicts); a pixel's gray value is two dp2a on the words as loaded, added to the bits of
+//     1.5 x 2^23 (even rows) or subtracted from those of -1.5 x 2^23 (odd rows), so that the integer comes out as
+//     a float, off by a bias that cancels in every sum below: rows u, m, d give d - u and (2 m + u) + d;
+//   * from there two pixels per instruction (f32x2; pixel i is paired with pixel i + 8, so that a pixel's
+//     left and right neighbours are whole register pairs too): vertical sums a = u + 2 m + d, b = d - u from
+//     the two rows kept in registers, then gx, gy across, squares, comparison by the sign of the difference.
+// What bounds it: 3 bytes per pixel from DRAM, 48 us for 64 pages of 1280 x 1280 at 6.55 TB/s, against 12 warp
+// instructions per 32 pixels (2.8 of them dp2a, 4.4 packed fp32, which take the FMA pipes two cycles each).  Those
+// pages: 141 us with integer gray values passed through shared memory and 64-bit comparisons (36 instructions per
+// pixel), 70 us = 4.5 TB/s now.
 #include <cstdint>
 #include <algorithm>
+#include <atomic>
 #include <cmath>
+#include <type_traits>
 
 #include <cuda_runtime.h>
 
 #include "../../include/rtprune.h"
+#include "ptx.cuh"
 
 namespace rtp {
 
-constexpr int kDnTile = 64;                        // tile side in pixels
-constexpr int kDnThreads = 288;                    // 66 rows x 4 groups of 16 pixels = 264 fetch tasks
-constexpr int kDnRows = 8;                         // rows a thread of the Sobel walk covers (8 warps x 8 rows)
-constexpr int kDnPitch = 72;                       // gray tile row: ring at [3], pixels at [4 .. 67], ring at [68]
+constexpr int kDnBand = 64;                        // rows per CTA, at most
+constexpr int kDnSeg = 256;                        // columns per CTA, at most: 16 threads of 16 columns
+constexpr int kDnWalk = 8;                         // rows per thread
+constexpr int kDnThreads = (kDnSeg / 16) * (kDnBand / kDnWalk);
+constexpr int kDnRowPitch = kDnSeg * 3 + 32;       // bytes: 16 in front of the segment's first pixel, 16 behind
+constexpr int kDnSmemBytes = (kDnBand + 2) * kDnRowPitch;         // 52 KB: four CTAs per SM
 
-__device__ inline int gray_of(uint32_t r, uint32_t g, uint32_t b) { return (int)(299u * r + 587u * g + 114u * b); }
+// 16-bit weight pairs (low half | high half << 16) for dp2a: low half times the lower byte of the selected byte pair
+// of the data word, high half times the upper one.  SIGN = -1: the negative weights.
+template <int SIGN> __host__ __device__ constexpr int weights(int lo, int hi) { return (SIGN * lo & 0xffff) | (int)((uint32_t)(SIGN * hi) << 16); }
+// Bits of SIGN x 1.5 x 2^23: an integer n below 2^22 added to (subtracted from) them adds n to the value.
+template <int SIGN> __host__ __device__ constexpr int magic() { return SIGN > 0 ? 0x4B400000 : (int)0xCB400000; }
 
-// 16-bit weight pairs (low half | high half << 16) for dp2a: low half times the lower byte of the
-// selected byte pair of the data word, high half times the upper one.
-constexpr uint32_t kW_RG = 299u | (587u << 16);
-constexpr uint32_t kW_B0 = 114u;
-constexpr uint32_t kW_0R = 299u << 16;
-constexpr uint32_t kW_GB = 587u | (114u << 16);
+typedef unsigned long long f32x2;                  // two floats in a register pair
 
-// Gray values of the 4 pixels whose 12 bytes are the words a, b, c (R G B R | G B R G | B R G B).
-__device__ inline int4 gray4(uint32_t a, uint32_t b, uint32_t c)
+__device__ inline f32x2 pack2(uint32_t lo, uint32_t hi)
 {
-    int4 o;
-    o.x = (int)__dp2a_lo(kW_RG, a, __dp2a_hi(kW_B0, a, 0u));     // R, G = a[0], a[1]; B = a[2]
-    o.y = (int)__dp2a_hi(kW_0R, a, __dp2a_lo(kW_GB, b, 0u));     // R = a[3]; G, B = b[0], b[1]
-    o.z = (int)__dp2a_hi(kW_RG, b, __dp2a_lo(kW_B0, c, 0u));     // R, G = b[2], b[3]; B = c[0]
-    o.w = (int)__dp2a_lo(kW_0R, c, __dp2a_hi(kW_GB, c, 0u));     // R = c[1]; G, B = c[2], c[3]
-    return o;
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+__device__ inline void unpack2(f32x2 v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ inline f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ inline f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ inline float min3_abs(float a, float b, float c)
+{
+    float r;
+    asm("min.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ inline f32x2 both(float x) { return pack2(__float_as_uint(x), __float_as_uint(x)); }
+
+__device__ inline int dp2a_lo(int w, uint32_t bytes, int c)
+{
+    int r;
+    asm("dp2a.lo.s32.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(w), "r"(bytes), "r"(c));
+    return r;
+}
+__device__ inline int dp2a_hi(int w, uint32_t bytes, int c)
+{
+    int r;
+    asm("dp2a.hi.s32.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(w), "r"(bytes), "r"(c));
+    return r;
+}
+// Bits of the (biased) gray value of the pixel whose three bytes are: the lower three of a word; the upper three;
+// the top byte of a and the lower two of b; the upper two of a and the lowest of b.
+template <int S> __device__ inline uint32_t gray_low3(uint32_t v)
+{
+    return (uint32_t)dp2a_lo(weights<S>(299, 587), v, dp2a_hi(weights<S>(114, 0), v, magic<S>()));
+}
+template <int S> __device__ inline uint32_t gray_high3(uint32_t v)
+{
+    return (uint32_t)dp2a_lo(weights<S>(0, 299), v, dp2a_hi(weights<S>(587, 114), v, magic<S>()));
+}
+template <int S> __device__ inline uint32_t gray_1_2(uint32_t a, uint32_t b)
+{
+    return (uint32_t)dp2a_hi(weights<S>(0, 299), a, dp2a_lo(weights<S>(587, 114), b, magic<S>()));
+}
+template <int S> __device__ inline uint32_t gray_2_1(uint32_t a, uint32_t b)
+{
+    return (uint32_t)dp2a_hi(weights<S>(299, 587), a, dp2a_lo(weights<S>(114, 0), b, magic<S>()));
 }
 
-// What a thread fetches for one tile: 16 pixels of a tile row (12 words) and, for the first 132
-// threads, the word that holds one pixel of the ring left or right of the tile.
-struct DnFetch {
+// The gray values of one row at a thread's 16 pixels as floats: pair i + 1 holds pixels i and i + 8, pairs 0 and 9
+// their neighbours at both ends.  `row` = shared memory of the thread's 48 bytes (16-byte aligned, a word of the
+// ring before and after it).
+template <int S> __device__ inline void dn_gray_row(const uint8_t *row, bool first_col, bool last_col, f32x2 (&p)[10])
+{
     uint32_t w[12];
-    uint32_t ring;
-};
-
-// A tile: image, origin, extent (the last tile of a row or column may be narrower).
-struct DnTile {
-    int img, x0, y0, tw, th;
-};
-
-// Issues the loads of a tile.  Task = (tile row ty = tid / 4, group of 16 pixels gx = tid % 4); the ring
-// pixel of a row is the upper three bytes of the word that ends where the tile starts, or the lower
-// three of the word that starts where it ends (3 x0 and 3 (x0 + tw) are multiples of 4); at the
-// image's left and right border the nearest pixel inside sits at the other end of its word.
-__device__ inline void dn_fetch(const uint8_t *__restrict__ images, int H, int W, const DnTile &q, int tid, DnFetch &f)
-{
-    const uint8_t *im = images + (size_t)q.img * H * W * 3;
-    const int ty = tid >> 2, gx = tid & 3;
-    if (ty < q.th + 2 && 16 * gx < q.tw) {
-        const int y = min(max(q.y0 + ty - 1, 0), H - 1);
-        const uint4 *src = reinterpret_cast<const uint4 *>(im + ((size_t)y * W + q.x0 + 16 * gx) * 3);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const uint4 v = __ldg(src + k);
-            f.w[4 * k] = v.x;
-            f.w[4 * k + 1] = v.y;
-            f.w[4 * k + 2] = v.z;
-            f.w[4 * k + 3] = v.w;
-        }
+    for (int k = 0; k < 3; ++k) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(row + 16 * k);
+        w[4 * k] = v.x;
+        w[4 * k + 1] = v.y;
+        w[4 * k + 2] = v.z;
+        w[4 * k + 3] = v.w;
     }
-    if (tid < 2 * (q.th + 2)) {
-        const int ry = tid >> 1, right = tid & 1;
-        const int y = min(max(q.y0 + ry - 1, 0), H - 1);
-        const uint8_t *row = im + (size_t)y * W * 3;
-        int off;                                     // byte offset of the word within the row
-        if (right) off = (q.x0 + q.tw < W) ? 3 * (q.x0 + q.tw) : 3 * W - 4;
-        else off = (q.x0 > 0) ? 3 * q.x0 - 4 : 0;
-        f.ring = __ldg(reinterpret_cast<const uint32_t *>(row + off));
+    uint32_t left = gray_high3<S>(*reinterpret_cast<const uint32_t *>(row - 4));
+    uint32_t right = gray_low3<S>(*reinterpret_cast<const uint32_t *>(row + 48));
+    uint32_t g[16];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {                  // four pixels in three words: R G B R | G B R G | B R G B
+        g[4 * k] = gray_low3<S>(w[3 * k]);
+        g[4 * k + 1] = gray_1_2<S>(w[3 * k], w[3 * k + 1]);
+        g[4 * k + 2] = gray_2_1<S>(w[3 * k + 1], w[3 * k + 2]);
+        g[4 * k + 3] = gray_high3<S>(w[3 * k + 2]);
     }
+    if (first_col) left = g[0];                    // beyond the image's border: the nearest pixel inside
+    if (last_col) right = g[15];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) p[i + 1] = pack2(g[i], g[i + 8]);
+    p[0] = pack2(left, g[7]);
+    p[9] = pack2(g[8], right);
 }
 
-// Gray values of what dn_fetch loaded, into the tile in shared memory.
-__device__ inline void dn_store(int *s_gray, int W, const DnTile &q, int tid, const DnFetch &f)
+// Edge pixels of the decision in exact arithmetic minus those of the fp32 decision, over pairs whose sum of
+// squares came close to the threshold.
+__device__ __noinline__ int dn_exact_pair(f32x2 gx, f32x2 gy, float T, unsigned long long thr2)
 {
-    const int ty = tid >> 2, gx = tid & 3;
-    if (ty < q.th + 2 && 16 * gx < q.tw) {
-        int4 *dst = reinterpret_cast<int4 *>(s_gray + ty * kDnPitch + 4 + 16 * gx);
+    float x[2], y[2];
+    unpack2(gx, x[0], x[1]);
+    unpack2(gy, y[0], y[1]);
+    int corr = 0;
 #pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4) dst[k4] = gray4(f.w[3 * k4], f.w[3 * k4 + 1], f.w[3 * k4 + 2]);
+    for (int e = 0; e < 2; ++e) {
+        const long long ix = (long long)x[e], iy = (long long)y[e];
+        const bool exact = (unsigned long long)(ix * ix + iy * iy) >= thr2;
+        const bool fast = fmaf(x[e], x[e], fmaf(y[e], y[e], -T)) >= 0.f;
+        corr += (exact ? 1 : 0) - (fast ? 1 : 0);
     }
-    if (tid < 2 * (q.th + 2)) {
-        const int right = tid & 1;
-        // pixel in bytes 0-2 of the word: right ring inside the image, or left ring clamped to pixel 0
-        const bool low = right ? (q.x0 + q.tw < W) : (q.x0 == 0);
-        const uint32_t v = f.ring;
-        const int g = low ? (int)__dp2a_lo(kW_RG, v, __dp2a_hi(kW_B0, v, 0u))
-                          : (int)__dp2a_lo(kW_0R, v, __dp2a_hi(kW_GB, v, 0u));
-        s_gray[(tid >> 1) * kDnPitch + (right ? 4 + q.tw : 3)] = g;
-    }
+    return corr;
 }
 
-// One CTA per tile.  grid = (tiles across, tiles down, batch).
-__global__ void __launch_bounds__(kDnThreads, 7)
-density_tile_kernel(const uint8_t *__restrict__ images, int H, int W, int p, unsigned long long thr2,
-                    int32_t *__restrict__ edge_counts, uint32_t *__restrict__ image_counts)
+// Zeroes the counters the tile kernel adds to (its grid dependency).
+__global__ void density_clear_kernel(uint32_t *__restrict__ image_counts, int batch, int32_t *__restrict__ edge_counts,
+                                     int patches)
 {
-    __shared__ __align__(16) int s_gray[(kDnTile + 2) * kDnPitch];
-    __shared__ int s_cnt[16];                        // up to 4 x 4 patches in a tile
-    const int tid = threadIdx.x;
-    DnTile q;
-    q.img = blockIdx.z;
-    q.x0 = blockIdx.x * kDnTile;
-    q.y0 = blockIdx.y * kDnTile;
-    q.tw = min(kDnTile, W - q.x0);                   // multiples of the patch (and of 16)
-    q.th = min(kDnTile, H - q.y0);
-    const int npt = kDnTile / p;                     // patches per tile side
-    DnFetch f;
-    dn_fetch(images, H, W, q, tid, f);
-    if (tid < 16) s_cnt[tid] = 0;
-    dn_store(s_gray, W, q, tid, f);
+    ptx::grid_dep_launch();
+    const int n = blockDim.x * gridDim.x, i0 = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int i = i0; i < batch; i += n) image_counts[i] = 0;
+    for (int i = i0; i < patches; i += n) edge_counts[i] = 0;
+}
+
+// grid = (segments of seg_w columns, bands of band_h rows, batch).  Launched as a programmatic dependent of
+// density_clear_kernel.
+__global__ void __launch_bounds__(kDnThreads, 4)
+density_tile_kernel(const __grid_constant__ CUtensorMap map, int H, int W, int p, int seg_w, int band_h,
+                    unsigned long long thr2, int32_t *__restrict__ edge_counts, uint32_t *__restrict__ image_counts)
+{
+    extern __shared__ __align__(128) uint8_t tile[];
+    __shared__ uint64_t s_full;
+    __shared__ int s_cnt[(kDnBand / 16) * (kDnSeg / 16)], s_total;     // of each (partial) patch: [row][16 columns]
+    const int walk = threadIdx.y, xt = 16 * threadIdx.x;       // rows kDnWalk * walk .., columns xt .. of the tile
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x, nth = blockDim.x * blockDim.y;
+    const int img = blockIdx.z, x0 = blockIdx.x * seg_w, y0 = blockIdx.y * band_h;
+    const int sw = min(seg_w, W - x0), bh = min(band_h, H - y0);        // multiples of 16
+    const int pr = min(p, band_h);                   // rows of a patch within the band
+    const int shift = 31 - __clz(p), pshift = 31 - __clz(pr);           // (powers of two)
+    ptx::grid_dep_launch();
+    if (tid == 0) {
+        ptx::mbar_init(&s_full, 1);
+        ptx::fence_mbar_init();
+        s_total = 0;
+    }
+    for (int i = tid; i < (kDnBand / 16) * (kDnSeg / 16); i += nth) s_cnt[i] = 0;
     __syncthreads();
 
-    // ---- Sobel, threshold, count: thread = (columns 2 cp and 2 cp + 1, block of kDnRows rows) ----------
-    const int cp = tid & 31, r0 = (tid >> 5) * kDnRows;
-    const bool active = tid < 256 && 2 * cp < q.tw && r0 < q.th;
-    int cnt = 0;
-    if (active) {
-        // horizontal sums of a tile row at the two columns: smooth s = l + 2 m + r, difference d = r - l
-        auto hrow = [&](int trow, int &s0, int &d0, int &s1, int &d1) {
-            const int *g = s_gray + trow * kDnPitch + 3 + 2 * cp;    // image columns x-1 .. x+2, x = 2 cp
-            const int g0 = g[0];
-            const int2 g12 = *reinterpret_cast<const int2 *>(g + 1);
-            const int g3 = g[3];
-            s0 = g0 + 2 * g12.x + g12.y;
-            d0 = g12.y - g0;
-            s1 = g12.x + 2 * g12.y + g3;
-            d1 = g3 - g12.x;
-        };
-        auto edge = [&](int gx, int gy) {
-            const unsigned long long g2 =
-                (unsigned long long)((long long)gx * gx) + (unsigned long long)((long long)gy * gy);
-            return g2 >= thr2 ? 1 : 0;
-        };
-        int su0, du0, su1, du1, sm0, dm0, sm1, dm1, sd0, dd0, sd1, dd1;
-        hrow(r0, su0, du0, su1, du1);                // tile row r0 = image row y0 + r0 - 1
-        hrow(r0 + 1, sm0, dm0, sm1, dm1);
-#pragma unroll
-        for (int r = 0; r < kDnRows; ++r) {          // th is a multiple of 16: the block is whole
-            hrow(r0 + r + 2, sd0, dd0, sd1, dd1);
-            cnt += edge(du0 + 2 * dm0 + dd0, su0 - sd0);
-            cnt += edge(du1 + 2 * dm1 + dd1, su1 - sd1);
-            su0 = sm0; du0 = dm0; su1 = sm1; du1 = dm1;
-            sm0 = sd0; dm0 = dd0; sm1 = sd1; dm1 = dd1;
-        }
+    // rows y0 - 1 .. y0 + band_h, 16 bytes in front of the first pixel (what lies outside the pages arrives as zeros
+    // and is replaced below)
+    if (tid == 0) {
+        ptx::mbar_arrive_expect_tx(&s_full, (uint32_t)((band_h + 2) * kDnRowPitch));
+        ptx::tma_load_3d(ptx::smem_u32(tile), &map, &s_full, (3 * x0 - 16) / 4, y0 - 1, img);
     }
-    // the lanes that share a patch: p / 2 of them (a warp holds the 64 columns of one block of rows)
-    if (tid < 256) {
-        const int width = p >> 1;
-        for (int o = width >> 1; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        if ((cp & (width - 1)) == 0 && active) atomicAdd(&s_cnt[(r0 / p) * npt + (2 * cp) / p], cnt);
+    const bool landed = ptx::mbar_wait(&s_full, 0);
+    if (landed && kDnWalk * walk < bh && xt < sw) {
+        const bool first_col = x0 + xt == 0, last_col = x0 + xt + 16 == W;
+        const uint8_t *base = tile + kDnWalk * walk * kDnRowPitch + 16 + 3 * xt;
+        const float T = (float)thr2, tol = T * 4.7683716e-7f;            // 2^-21
+        const f32x2 minus_T = both(-T), two = both(2.f), minus = both(-1.f);
+        f32x2 r0[10], r1[10];                         // the row above and the row of the sums taken next, in turn
+        int below = 0, corr = 0;                      // pixels under the threshold; exact decisions that differ
+        dn_gray_row<1>(y0 + kDnWalk * walk == 0 ? base + kDnRowPitch : base, first_col, last_col, r0);
+        dn_gray_row<-1>(base + kDnRowPitch, first_col, last_col, r1);
+        const uint8_t *last = base + (y0 + kDnWalk * (walk + 1) == H ? kDnWalk : kDnWalk + 1) * kDnRowPitch;
+        // one row of sums: u the row above, m the row itself; the row below takes u's place
+        auto row_of_sums = [&](auto sign, f32x2 (&u)[10], f32x2 (&m)[10], const uint8_t *row) {
+            f32x2 g[10];
+            dn_gray_row<decltype(sign)::value>(row, first_col, last_col, g);
+            f32x2 a0 = add2(fma2(m[0], two, u[0]), g[0]), b0 = fma2(u[0], minus, g[0]);
+            f32x2 a1 = add2(fma2(m[1], two, u[1]), g[1]), b1 = fma2(u[1], minus, g[1]);
+            u[0] = g[0];
+            u[1] = g[1];
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {             // four pairs at a time: gx and gy stay in registers
+                float near = 3.0e38f;
+                f32x2 gx[4], gy[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int i = 4 * part + e + 2;
+                    const f32x2 a2 = add2(fma2(m[i], two, u[i]), g[i]), b2 = fma2(u[i], minus, g[i]);
+                    u[i] = g[i];
+                    gx[e] = fma2(a0, minus, a2);
+                    gy[e] = fma2(b1, two, add2(b0, b2));
+                    a0 = a1;
+                    a1 = a2;
+                    b0 = b1;
+                    b1 = b2;
+                    const f32x2 v = fma2(gx[e], gx[e], fma2(gy[e], gy[e], minus_T));
+                    float x, y;
+                    unpack2(v, x, y);
+                    below += (int)(__float_as_uint(x) >> 31);
+                    below += (int)(__float_as_uint(y) >> 31);
+                    near = min3_abs(near, x, y);
+                }
+                if (near < tol) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) corr += dn_exact_pair(gx[e], gy[e], T, thr2);
+                }
+            }
+        };
+#pragma unroll                                        // (whole: no registers are moved from row to row)
+        for (int r = 0; r < kDnWalk; r += 2) {
+            row_of_sums(std::integral_constant<int, 1>(), r0, r1, base + (r + 2) * kDnRowPitch);
+            row_of_sums(std::integral_constant<int, -1>(), r1, r0, r + 3 > kDnWalk ? last : base + (r + 3) * kDnRowPitch);
+        }
+        // eight rows of one patch row (patches are 16 rows at least)
+        const int count = 16 * kDnWalk - below + corr;
+        atomicAdd(&s_cnt[((kDnWalk * walk) >> pshift) * (kDnSeg / 16) + (xt >> shift)], count);
+        atomicAdd(&s_total, count);
     }
     __syncthreads();
-    if (tid < npt * npt) {
-        const int pi = tid / npt, pj = tid - pi * npt;
-        if (pi * p < q.th && pj * p < q.tw && edge_counts) {
-            const int gy = q.y0 / p + pi, gx = q.x0 / p + pj;
-            edge_counts[((size_t)q.img * (H / p) + gy) * (W / p) + gx] = s_cnt[tid];
+    // the band's patches are whole (stored) or shared with the bands below and above (added)
+    ptx::grid_dep_wait();                             // the counters have been cleared
+    if (edge_counts) {
+        const int ncol = (sw + p - 1) >> shift, ncell = (bh >> pshift) * (kDnSeg / 16);
+        for (int i = tid; i < ncell; i += nth) {
+            const int pi = i / (kDnSeg / 16), pj = i % (kDnSeg / 16);
+            if (pj >= ncol) continue;
+            int32_t *e = edge_counts + ((size_t)img * (H >> shift) + ((y0 + pi * pr) >> shift)) * (W >> shift) + (x0 >> shift) + pj;
+            if (pr == p) *e = s_cnt[i];
+            else atomicAdd(e, s_cnt[i]);
         }
     }
-    if (tid == 32) {
-        int total = 0;
-        for (int k = 0; k < npt * npt; ++k) total += s_cnt[k];
-        atomicAdd(image_counts + q.img, (uint32_t)total);
-    }
+    if (tid == 0) atomicAdd(image_counts + img, (uint32_t)s_total);
 }
 
 // rho = average over the patches of (edge pixels / patch pixels); the patches are equal, so this is the
@@ -203,8 +281,49 @@ density_tile_kernel(const uint8_t *__restrict__ images, int H, int W, int p, uns
 __global__ void density_finish_kernel(const uint32_t *__restrict__ image_counts, int batch, float inv_pixels,
                                       float *__restrict__ rho)
 {
+    ptx::grid_dep_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < batch) rho[i] = (float)image_counts[i] * inv_pixels;
+}
+
+// Launch that may begin while the kernel ahead of it in the stream drains (it waits for it itself).
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// The pages as a 3-D tensor of 32-bit words (x, row, page); boxes of one tile.
+static bool pages_map(CUtensorMap *map, const uint8_t *images, int batch, int H, int W, int band_h)
+{
+    typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                      const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                                      CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static std::atomic<void *> encode{nullptr};       // the driver's entry point, looked up once
+    void *fn = encode.load(std::memory_order_relaxed);
+    if (!fn) {
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess)
+            return false;
+        encode.store(fn, std::memory_order_relaxed);
+    }
+    const cuuint64_t dims[3] = {(cuuint64_t)W * 3 / 4, (cuuint64_t)H, (cuuint64_t)batch};
+    const cuuint64_t strides[2] = {(cuuint64_t)W * 3, (cuuint64_t)W * 3 * (cuuint64_t)H};
+    const cuuint32_t box[3] = {kDnRowPitch / 4, (cuuint32_t)band_h + 2, 1}, unit[3] = {1, 1, 1};
+    return ((EncodeTiledFn)fn)(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<uint8_t *>(images), dims, strides, box,
+                               unit, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace rtp
@@ -225,11 +344,29 @@ extern "C" rtprune_status_t rtprune_density(void *cuda_stream, const uint8_t *im
     const double t = (double)tau * 255000.0;
     const double t2 = std::ceil(t * t);
     const unsigned long long thr2 = t2 >= 1.8e19 ? ~0ull : (unsigned long long)t2;
-    if (cudaMemsetAsync(image_counts, 0, sizeof(uint32_t) * (size_t)batch, st) != cudaSuccess) return RTPRUNE_ERR_CUDA;
-    if (batch > 65535 || (height + kDnTile - 1) / kDnTile > 65535) return RTPRUNE_ERR_UNSUPPORTED;
-    dim3 grid((unsigned)((width + kDnTile - 1) / kDnTile), (unsigned)((height + kDnTile - 1) / kDnTile), (unsigned)batch);
-    density_tile_kernel<<<grid, kDnThreads, 0, st>>>(images, height, width, patch, thr2, edge_counts, image_counts);
-    density_finish_kernel<<<(batch + 255) / 256, 256, 0, st>>>(image_counts, batch,
-                                                             1.f / ((float)height * (float)width), rho);
+    if (batch > 65535 || (height + kDnBand - 1) / kDnBand > 65535) return RTPRUNE_ERR_UNSUPPORTED;
+    // columns: equal segments, multiples of 64 (whole patches)
+    const int nseg = (width + kDnSeg - 1) / kDnSeg;
+    const int seg_w = std::min(kDnSeg, ((width + nseg - 1) / nseg + 63) / 64 * 64);
+    const int nx = (width + seg_w - 1) / seg_w;
+    // rows: bands of 64; of 16 when those would leave half the device idle (the two extra rows of a band then cost
+    // an eighth instead of a thirty-second)
+    int band_h = kDnBand;
+    while (band_h > 16 && (long long)batch * nx * ((height + band_h - 1) / band_h) < 2 * 148) band_h >>= 1;
+    const int patches = (edge_counts && band_h < patch) ? batch * (height / patch) * (width / patch) : 0;
+    const int n_clear = std::max((int)batch, patches);
+    density_clear_kernel<<<std::min((n_clear + 255) / 256, 148), 256, 0, st>>>(image_counts, batch, edge_counts, patches);
+    CUtensorMap map;
+    if (!pages_map(&map, images, batch, height, width, band_h)) return RTPRUNE_ERR_CUDA;
+    if (cudaFuncSetAttribute(density_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDnSmemBytes) != cudaSuccess)
+        return RTPRUNE_ERR_CUDA;
+    const dim3 threads((unsigned)(std::min(seg_w, (int)width) / 16), (unsigned)(band_h / kDnWalk));
+    const dim3 grid((unsigned)nx, (unsigned)((height + band_h - 1) / band_h), (unsigned)batch);
+    if (launch_dependent(density_tile_kernel, grid, threads, (size_t)kDnSmemBytes, st, map, height, width, patch,
+                         seg_w, band_h, thr2, edge_counts, image_counts) != cudaSuccess)
+        return RTPRUNE_ERR_CUDA;
+    if (launch_dependent(density_finish_kernel, dim3((unsigned)(batch + 255) / 256), dim3(256), (size_t)0, st,
+                         (const uint32_t *)image_counts, batch, 1.f / ((float)height * (float)width), rho) != cudaSuccess)
+        return RTPRUNE_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? RTPRUNE_OK : RTPRUNE_ERR_CUDA;
 }

@@ -129,6 +129,14 @@ __device__ inline void tma_load_2d(uint32_t dst_smem, const CUtensorMap *map, ui
         ::"r"(dst_smem), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
         : "memory");
 }
+// 3-D tiled load: box at (x, y, z), as above.
+__device__ inline void tma_load_3d(uint32_t dst_smem, const CUtensorMap *map, uint64_t *bar, int x, int y, int z)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(dst_smem), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
+        : "memory");
+}
 // 1-D bulk load global -> shared (both 16-byte aligned, size a multiple of 16); completion is counted
 // in bytes on the mbarrier.
 __device__ inline void bulk_load(uint32_t dst_smem, const void *src_global, uint32_t bytes, uint64_t *bar)
