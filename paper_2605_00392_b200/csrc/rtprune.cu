@@ -13,7 +13,7 @@
 #include "common.cuh"
 #include "exact.cuh"
 #include "fused.cuh"
-#include "gemm_simt.cuh"
+#include "gemm_fp32_umma.cuh"
 #include "merge_umma.cuh"
 #include "scores_umma.cuh"
 #include "sinkhorn.cuh"
@@ -418,7 +418,6 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
     float *kmat = (float *)(ws + L.kmat);
     const int maxN = plan->max_tokens;
     const int maxB = max_pruned(params, maxN);
-    const int mtiles = (maxN + kSimtTile - 1) / kSimtTile;
     constexpr bool kTensor = std::is_same<T, __nv_bfloat16>::value;
     __nv_bfloat16 *pbuf = kTensor ? (__nv_bfloat16 *)(ws + L.pbuf) : nullptr;
     const int pbuf_pitch = (std::max(maxB, 1) + 63) / 64 * 64;   // <= L.pbuf_pitch_max
@@ -472,11 +471,12 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                                  L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done)))
                 return RTPRUNE_ERR_CUDA;
         } else {
-            const int btiles = (maxB + kSimtTile - 1) / kSimtTile;
-            dim3 grid(mtiles * btiles, batch);
-            scores_simt_kernel<T><<<grid, 256, 0, st>>>((const T *)X, offsets, plan->d, btiles,
-                                                       o.counts, order, norms, kmat,
-                                                       L.kmat_stride, maxN, total);
+            const int btiles = (maxB + kF3Tile - 1) / kF3Tile, mtiles = (maxN + kF3Tile - 1) / kF3Tile;
+            if (!c.ok(launch_pdl(scores_fp32_umma_kernel, dim3((unsigned)(mtiles * btiles), (unsigned)batch), dim3(kF3Prod + 32),
+                                 (size_t)kF3SmemBytes, st, 1u, (const float *)X, offsets, plan->d, btiles,
+                                 (const int32_t *)o.counts, (const int32_t *)order, (const float *)norms, kmat,
+                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header))))
+                return RTPRUNE_ERR_CUDA;
         }
         if (!c.ok(cudaGetLastError())) return RTPRUNE_ERR_CUDA;
         launched(plan, st, "scores");
@@ -620,11 +620,17 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                              (WsHeader *)(ws + L.header), (const int32_t *)ready_list)))
             return RTPRUNE_ERR_CUDA;
     } else {
-        const int dtiles = (plan->d + kSimtTile - 1) / kSimtTile;
-        dim3 grid(mtiles * dtiles, batch);
-        merge_simt_kernel<T><<<grid, 256, 0, st>>>((const T *)X, offsets, plan->d, dtiles, o.counts,
-                                                  o.out_offsets, order, kmat, L.kmat_stride, maxN,
-                                                  total, params->alpha, (T *)o.Y, o.kept_idx);
+        const int mtiles = (maxN + kF3Tile - 1) / kF3Tile, nct = (plan->d + kM3N - 1) / kM3N;
+        // output tiles per task: a quarter of a row of tiles, fewer when the device would not have two tasks per SM
+        int ct_run = (nct + 3) / 4;
+        while (ct_run > 1 && (long long)batch * mtiles * ((nct + ct_run - 1) / ct_run) < 2LL * plan->sm_count) ct_run = (ct_run + 1) / 2;
+        const long long ntasks = (long long)batch * mtiles * ((nct + ct_run - 1) / ct_run);
+        if (!c.ok(launch_pdl(merge_fp32_umma_kernel, dim3((unsigned)std::min<long long>(ntasks, plan->sm_count)),
+                             dim3(kM3Threads), (size_t)kM3SmemBytes, st, 1u, (const float *)X, offsets, plan->d, batch,
+                             mtiles, ct_run, (const int32_t *)o.counts, (const int32_t *)o.out_offsets, (const int32_t *)order,
+                             (const float *)kmat, L.kmat_stride, maxN, total, params->alpha, (float *)o.Y, o.kept_idx,
+                             (WsHeader *)(ws + L.header))))
+            return RTPRUNE_ERR_CUDA;
     }
     if (!c.ok(cudaGetLastError())) return RTPRUNE_ERR_CUDA;
     launched(plan, st, "merge");
@@ -824,6 +830,12 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
             delete p;
             return RTPRUNE_ERR_CUDA;
         }
+    }
+    if (dtype == RTPRUNE_FP32 &&
+        (!c.ok(cudaFuncSetAttribute(scores_fp32_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kF3SmemBytes)) ||
+         !c.ok(cudaFuncSetAttribute(merge_fp32_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kM3SmemBytes)))) {
+        delete p;
+        return RTPRUNE_ERR_CUDA;
     }
     // The fused stage-2 kernel: clusters of 2 CTAs with all of an SM's shared memory each; how many the
     // device runs at once is what a run's grid is capped at (its clusters then loop over the images).

@@ -344,6 +344,7 @@ stage1_kernel(const T *__restrict__ X, const int32_t *__restrict__ offsets, int 
         if (tid == 0) {
             int seq = hdr->launch_seq + 1;
             if (seq == 0) seq = 1;         // 0 is what a fresh workspace holds
+            hdr->merge_next = 0;           // (fp32 storage: the kernel that copies pruned rows does not run)
             ptx::st_release_gpu(&hdr->launch_seq, seq);
             __threadfence();
         }
