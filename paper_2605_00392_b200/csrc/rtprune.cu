@@ -26,6 +26,14 @@ using namespace rtp;
 
 static_assert(sizeof(rtprune_params_t) == 64, "rtprune_params_t layout is part of the ABI");
 
+// Streams and events of rtprune_run_host's pipeline.
+struct HostPipe {
+    static constexpr int kGroups = 8;
+    int device;
+    cudaStream_t in, out;
+    cudaEvent_t begin, end, copied[kGroups], solved[kGroups];
+};
+
 struct rtprune_plan_s {
     int d;
     rtprune_dtype_t dtype;
@@ -61,6 +69,7 @@ struct rtprune_plan_s {
     MapSet maps[kMapSets];
     int map_next;           // entry the next miss replaces
     int64_t last_host_ns;   // host time the most recent rtprune_run call spent inside the library
+    HostPipe *host_pipe;    // rtprune_run_host's, from its first pipelined call on
     uint32_t poll_limit;    // polls after which stage 1's waits on its copies give up (ptx::kSpinLimit; tests lower it)
 };
 
@@ -170,6 +179,13 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     cfg.attrs = attr;
     cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// out_offsets of a batch that was run in groups.
+__global__ void __launch_bounds__(256) scan_counts_kernel(const int32_t *counts, int32_t *out_offsets, int batch)
+{
+    __shared__ int scratch[32];
+    scan_counts<256>(counts, out_offsets, batch, scratch);
 }
 
 // Test aid (rtprune_test_expire_waits): two waits that nothing ends, with a short poll limit.
@@ -660,7 +676,7 @@ rtprune_status_t run_device(rtprune_plan_t *plan, cudaStream_t st, const void *X
 
 // Device arena of rtprune_run_host: device copies of the inputs and outputs, then the workspace.
 struct Arena {
-    size_t X, offsets, rho, Y, out_offsets, counts, kept_idx, merged_idx, partner, weight, stats,
+    size_t X, offsets, rho, Y, out_offsets, group_offsets, counts, kept_idx, merged_idx, partner, weight, stats,
         ws, total;
 };
 
@@ -680,6 +696,7 @@ Arena make_arena(const rtprune_plan_t *p)
     a.rho = take(nb * 4);
     a.Y = take(tot * p->d * esz);
     a.out_offsets = take((nb + 1) * 4);
+    a.group_offsets = take((nb + 1 + HostPipe::kGroups) * 4);
     a.counts = take(nb * 4);
     a.kept_idx = take(tot * 4);
     a.merged_idx = take(tot * 4);
@@ -689,6 +706,76 @@ Arena make_arena(const rtprune_plan_t *p)
     a.ws = take(p->ws.total);
     a.total = off;
     return a;
+}
+
+// Pipelines of plans that are gone, for the next ones (creating one takes about a millisecond): at most kMaxIdle.  A
+// pipeline's streams may still be draining; what its next owner enqueues is ordered behind that.
+constexpr int kMaxIdle = 4;
+std::mutex g_pipe_mutex;
+HostPipe *g_idle_pipes[kMaxIdle] = {};
+
+void destroy_pipe(HostPipe *h)
+{
+    if (h->in) cudaStreamDestroy(h->in);
+    if (h->out) cudaStreamDestroy(h->out);
+    if (h->begin) cudaEventDestroy(h->begin);
+    if (h->end) cudaEventDestroy(h->end);
+    for (int g = 0; g < HostPipe::kGroups; ++g) {
+        if (h->copied[g]) cudaEventDestroy(h->copied[g]);
+        if (h->solved[g]) cudaEventDestroy(h->solved[g]);
+    }
+    delete h;
+}
+
+bool host_pipeline(rtprune_plan_t *plan)
+{
+    if (plan->host_pipe) return true;
+    {
+        std::lock_guard<std::mutex> lock(g_pipe_mutex);
+        for (HostPipe *&h : g_idle_pipes)
+            if (h && h->device == plan->device) {
+                plan->host_pipe = h;
+                h = nullptr;
+                return true;
+            }
+    }
+    HostPipe *h = new (std::nothrow) HostPipe();       // (all zero)
+    if (!h) return false;
+    h->device = plan->device;
+    Checked c{plan};
+    bool ok = c.ok(cudaStreamCreateWithFlags(&h->in, cudaStreamNonBlocking)) &&
+              c.ok(cudaStreamCreateWithFlags(&h->out, cudaStreamNonBlocking)) &&
+              c.ok(cudaEventCreateWithFlags(&h->begin, cudaEventDisableTiming)) &&
+              c.ok(cudaEventCreateWithFlags(&h->end, cudaEventDisableTiming));
+    for (int g = 0; g < HostPipe::kGroups && ok; ++g)
+        ok = c.ok(cudaEventCreateWithFlags(&h->copied[g], cudaEventDisableTiming)) &&
+             c.ok(cudaEventCreateWithFlags(&h->solved[g], cudaEventDisableTiming));
+    if (!ok) {
+        destroy_pipe(h);
+        return false;
+    }
+    plan->host_pipe = h;
+    return true;
+}
+
+void release_pipe(HostPipe *h)
+{
+    {
+        std::lock_guard<std::mutex> lock(g_pipe_mutex);
+        for (HostPipe *&slot : g_idle_pipes)
+            if (!slot) {
+                slot = h;
+                return;
+            }
+    }
+    destroy_pipe(h);
+}
+
+// Kept tokens of an image of n tokens at a fixed ratio: the expression stage 1 evaluates, in the same arithmetic.
+int fixed_kept(float r_fixed, int n)
+{
+    const int b = (int)std::floor(std::fmaf(std::fmax(r_fixed, 0.f), (float)n, 0.5f));
+    return n - std::max(0, std::min(b, n - 1));
 }
 
 }  // namespace
@@ -746,6 +833,7 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
     for (int i = 0; i < rtprune_plan_s::kMapSets; ++i) p->maps[i].valid = false;
     p->map_next = 0;
     p->last_host_ns = 0;
+    p->host_pipe = nullptr;
     p->poll_limit = ptx::kSpinLimit;
     p->profiling = false;
     p->ev_count = 0;
@@ -1104,47 +1192,79 @@ rtprune_status_t rtprune_run_host(rtprune_plan_t *plan, void *cuda_stream, const
     }
     rtprune_params_t p = *params;
     p.rho = rho_host ? (const float *)(base + a.rho) : nullptr;
-    if (!c.ok(cudaMemcpyAsync(base + a.X, X_host, (size_t)total_tokens * row, cudaMemcpyHostToDevice, st)) ||
-        !c.ok(cudaMemcpyAsync(base + a.offsets, offsets_host, ((size_t)batch + 1) * 4, cudaMemcpyHostToDevice, st)))
+    int32_t *d_offsets = (int32_t *)(base + a.offsets), *d_out = (int32_t *)(base + a.out_offsets);
+    int32_t *d_counts = (int32_t *)(base + a.counts), *d_kept = (int32_t *)(base + a.kept_idx);
+    int32_t *d_merged = (int32_t *)(base + a.merged_idx), *d_partner = (int32_t *)(base + a.partner);
+    float *d_weight = (float *)(base + a.weight), *d_stats = (float *)(base + a.stats);
+
+    // The batch goes through in groups of images: the copy of the next group's tokens runs under the kernels of this
+    // one and the copy of the last one's output (the link carries both directions at once).  Groups of 4 MB at least
+    // (a copy of that size takes about what the launches and kernels of a group take).  With a dynamic ratio the place
+    // of a group's output rows is only known on the device: one group.
+    int groups = 1;
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    (void)cudaStreamIsCapturing(st, &capturing);
+    if (!p.dynamic && !plan->profiling && capturing == cudaStreamCaptureStatusNone) {
+        groups = (int)std::min<long long>(std::min<int>(batch, HostPipe::kGroups),
+                                          std::max<long long>(1, (long long)((size_t)total_tokens * row >> 22)));
+        if (groups > 1 && !host_pipeline(plan)) groups = 1;
+    }
+    HostPipe *pipe = plan->host_pipe;
+    cudaStream_t in = groups > 1 ? pipe->in : st, out = groups > 1 ? pipe->out : st;
+    if (groups > 1 && (!c.ok(cudaEventRecord(pipe->begin, st)) || !c.ok(cudaStreamWaitEvent(in, pipe->begin, 0)) ||
+                       !c.ok(cudaStreamWaitEvent(out, pipe->begin, 0))))
         return RTPRUNE_ERR_CUDA;
-    if (rho_host && !c.ok(cudaMemcpyAsync(base + a.rho, rho_host, (size_t)batch * 4, cudaMemcpyHostToDevice, st)))
+    if (!c.ok(cudaMemcpyAsync(d_offsets, offsets_host, ((size_t)batch + 1) * 4, cudaMemcpyHostToDevice, in)) ||
+        (rho_host && !c.ok(cudaMemcpyAsync(base + a.rho, rho_host, (size_t)batch * 4, cudaMemcpyHostToDevice, in))) ||
+        !c.ok(cudaMemsetAsync(base + a.ws + plan->ws.header, 0, plan->ws.clear_bytes, st)))
         return RTPRUNE_ERR_CUDA;
-    if (!c.ok(cudaMemsetAsync(base + a.ws + plan->ws.header, 0, plan->ws.clear_bytes, st)))
-        return RTPRUNE_ERR_CUDA;
-    DevOut o{base + a.Y,
-             (int32_t *)(base + a.out_offsets),
-             (int32_t *)(base + a.counts),
-             (int32_t *)(base + a.kept_idx),
-             (int32_t *)(base + a.merged_idx),
-             (int32_t *)(base + a.partner),
-             (float *)(base + a.weight),
-             (float *)(base + a.stats)};
-    s = run_device(plan, st, base + a.X, (const int32_t *)(base + a.offsets), batch,
-                   (int)total_tokens, &p,
-                   base + a.ws, o);
-    if (s != RTPRUNE_OK) return s;
-    // Rows of Y to bring back: with a fixed ratio every image's kept count is known here (the expression stage 1
-    // evaluates, in the same arithmetic); a dynamic ratio is decided on the device, so all rows are copied.
-    size_t y_rows = (size_t)total_tokens;
-    if (!p.dynamic) {
-        y_rows = 0;
-        const float r = std::fmax(p.r_fixed, 0.f);
-        for (int i = 0; i < batch; ++i) {
-            const int n = offsets_host[i + 1] - offsets_host[i];
-            int b = (int)std::floor(std::fmaf(r, (float)n, 0.5f));
-            b = std::max(0, std::min(b, n - 1));
-            y_rows += (size_t)(n - b);
+    int i0 = 0;
+    size_t kept0 = 0;                      // output rows of the groups before (fixed ratio)
+    for (int g = 0; g < groups; ++g) {
+        // images [i0, i1): the cut nearest to equal shares of the tokens, at least one image each
+        int i1 = g == groups - 1 ? batch : i0 + 1;
+        while (i1 < batch - (groups - 1 - g) && (long long)offsets_host[i1] * groups < (g + 1LL) * total_tokens) ++i1;
+        const size_t t0 = (size_t)offsets_host[i0], t1 = (size_t)offsets_host[i1];
+        if (!c.ok(cudaMemcpyAsync(base + a.X + t0 * row, (const char *)X_host + t0 * row, (t1 - t0) * row, cudaMemcpyHostToDevice, in)))
+            return RTPRUNE_ERR_CUDA;
+        if (groups > 1 && (!c.ok(cudaEventRecord(pipe->copied[g], in)) || !c.ok(cudaStreamWaitEvent(st, pipe->copied[g], 0))))
+            return RTPRUNE_ERR_CUDA;
+        // the group's images keep their places in X and in the workspace; its outputs are packed behind the groups' before
+        rtprune_params_t pg = p;
+        if (pg.rho) pg.rho += i0;
+        DevOut o{base + a.Y + kept0 * row, groups > 1 ? (int32_t *)(base + a.group_offsets) + i0 + g : d_out, d_counts + i0,
+                 d_kept + kept0, d_merged - kept0, d_partner - kept0, d_weight - kept0, d_stats + (size_t)i0 * kStats};
+        const rtprune_status_t rs = run_device(plan, st, base + a.X, d_offsets + i0, i1 - i0, (int)total_tokens, &pg, base + a.ws, o);
+        if (rs != RTPRUNE_OK) return rs;
+        // Rows of Y to bring back: with a fixed ratio every image's kept count is known here; a dynamic ratio is
+        // decided on the device, so all rows are copied.
+        size_t rows = (size_t)total_tokens;
+        if (!p.dynamic) {
+            rows = 0;
+            for (int i = i0; i < i1; ++i) rows += (size_t)fixed_kept(p.r_fixed, offsets_host[i + 1] - offsets_host[i]);
         }
+        if (groups > 1 && (!c.ok(cudaEventRecord(pipe->solved[g], st)) || !c.ok(cudaStreamWaitEvent(out, pipe->solved[g], 0))))
+            return RTPRUNE_ERR_CUDA;
+        if (rows && !c.ok(cudaMemcpyAsync((char *)Y_host + kept0 * row, base + a.Y + kept0 * row, rows * row, cudaMemcpyDeviceToHost, out)))
+            return RTPRUNE_ERR_CUDA;
+        kept0 += rows;
+        i0 = i1;
+    }
+    if (groups > 1) {
+        scan_counts_kernel<<<1, 256, 0, st>>>(d_counts, d_out, batch);
+        ++plan->last_launches;
     }
     const size_t tot4 = (size_t)total_tokens * 4;
-    if (!c.ok(cudaMemcpyAsync(out_offsets_host, o.out_offsets, ((size_t)batch + 1) * 4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(counts_host, o.counts, (size_t)batch * 4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(kept_idx_host, o.kept_idx, tot4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(merged_idx_host, o.merged_idx, tot4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(merge_partner_host, o.merge_partner, tot4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(merge_weight_host, o.merge_weight, tot4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(stats_host, o.stats, (size_t)batch * kStats * 4, cudaMemcpyDeviceToHost, st)) ||
-        (y_rows && !c.ok(cudaMemcpyAsync(Y_host, o.Y, y_rows * row, cudaMemcpyDeviceToHost, st))))
+    if (!c.ok(cudaGetLastError()) ||
+        !c.ok(cudaMemcpyAsync(out_offsets_host, d_out, ((size_t)batch + 1) * 4, cudaMemcpyDeviceToHost, st)) ||
+        !c.ok(cudaMemcpyAsync(counts_host, d_counts, (size_t)batch * 4, cudaMemcpyDeviceToHost, st)) ||
+        !c.ok(cudaMemcpyAsync(kept_idx_host, d_kept, tot4, cudaMemcpyDeviceToHost, st)) ||
+        !c.ok(cudaMemcpyAsync(merged_idx_host, d_merged, tot4, cudaMemcpyDeviceToHost, st)) ||
+        !c.ok(cudaMemcpyAsync(merge_partner_host, d_partner, tot4, cudaMemcpyDeviceToHost, st)) ||
+        !c.ok(cudaMemcpyAsync(merge_weight_host, d_weight, tot4, cudaMemcpyDeviceToHost, st)) ||
+        !c.ok(cudaMemcpyAsync(stats_host, d_stats, (size_t)batch * kStats * 4, cudaMemcpyDeviceToHost, st)))
+        return RTPRUNE_ERR_CUDA;
+    if (groups > 1 && (!c.ok(cudaEventRecord(pipe->end, out)) || !c.ok(cudaStreamWaitEvent(st, pipe->end, 0))))
         return RTPRUNE_ERR_CUDA;
     return RTPRUNE_OK;
 }
@@ -1214,6 +1334,7 @@ void rtprune_destroy(rtprune_plan_t *plan)
 {
     if (!plan) return;
     if (plan->profiling) rtprune_profile_enable(plan, 0);
+    if (plan->host_pipe) release_pipe(plan->host_pipe);
     delete plan;
 }
 
