@@ -113,8 +113,10 @@ typedef struct {
                              of the scaling form all within one unit in the last place of their
                              previous values (bit-identical log-domain duals in the LOG form) -- later
                              iterations could only move them within rounding, so the result is that
-                             of all `iters` iterations to fp32 accuracy.  (Images with more than 640
-                             pruned tokens: within four units, the rounding noise of their long sums.)
+                             of all `iters` iterations to fp32 accuracy.  (A dual that keeps cycling
+                             within four units also counts, from its third such iteration on; images with
+                             more than 639 pruned tokens: within four units, the rounding noise of their
+                             long sums.)
                              0: always run `iters`.                                                  */
     float tol;            /* > 0: also stop once no dual moved by more than tol (log units) in an
                              iteration.  0 (default): never stop on a tolerance.                    */

@@ -118,8 +118,9 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 def _stream_handle(stream: Optional[torch.cuda.Stream]):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())    # (no Stream object on the way: 2 us a call)
 
 
 @dataclass
@@ -320,14 +321,20 @@ def density(images: torch.Tensor, patch: int = 64, tau: float = 0.2, *, want_pat
         raise ValueError("images must live on a CUDA device")
     batch, H, W, _ = images.shape
     dev = images.device
-    rho = torch.empty(batch, dtype=torch.float32, device=dev)
-    counts = torch.empty(batch, dtype=torch.int32, device=dev)          # uint32 in the library
-    per_patch = None
-    if want_patch_counts and patch > 0:
-        per_patch = torch.empty((batch, H // patch, W // patch), dtype=torch.int32, device=dev)
-    with torch.cuda.device(dev):
-        _check(lib().rtprune_density(_stream_handle(stream), images.data_ptr(), batch, H, W, patch, float(tau),
-                                     rho.data_ptr(), counts.data_ptr(), _ptr(per_patch)), "rtprune_density")
+    # one allocation for the outputs, the patches last: three cost as much host time as the launches
+    patches = (H // patch) * (W // patch) if want_patch_counts and patch > 0 else 0
+    out = torch.empty(batch * (2 + patches), dtype=torch.int32, device=dev)
+    rho, counts, rest = out.split_with_sizes((batch, batch, batch * patches))    # counts: uint32 in the library
+    rho = rho.view(torch.float32)
+    per_patch = rest.view(batch, H // patch, W // patch) if want_patch_counts and patch > 0 else None
+    base = out.data_ptr()
+    args = (images.data_ptr(), batch, H, W, patch, float(tau), base, base + 4 * batch,
+            base + 8 * batch if per_patch is not None else None)
+    if dev.index == torch._C._cuda_getDevice():
+        _check(lib().rtprune_density(_stream_handle(stream), *args), "rtprune_density")
+    else:
+        with torch.cuda.device(dev):
+            _check(lib().rtprune_density(_stream_handle(stream), *args), "rtprune_density")
     return rho, counts, per_patch
 
 

@@ -358,8 +358,16 @@ extern "C" rtprune_status_t rtprune_density(void *cuda_stream, const uint8_t *im
     density_clear_kernel<<<std::min((n_clear + 255) / 256, 148), 256, 0, st>>>(image_counts, batch, edge_counts, patches);
     CUtensorMap map;
     if (!pages_map(&map, images, batch, height, width, band_h)) return RTPRUNE_ERR_CUDA;
-    if (cudaFuncSetAttribute(density_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDnSmemBytes) != cudaSuccess)
-        return RTPRUNE_ERR_CUDA;
+    // the attribute is the function's, per device: set once on each (a bit of the mask)
+    static std::atomic<unsigned long long> attribute_set{0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return RTPRUNE_ERR_CUDA;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(attribute_set.load(std::memory_order_relaxed) & bit)) {
+        if (cudaFuncSetAttribute(density_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDnSmemBytes) != cudaSuccess)
+            return RTPRUNE_ERR_CUDA;
+        if (dev < 64) attribute_set.fetch_or(bit, std::memory_order_relaxed);
+    }
     const dim3 threads((unsigned)(std::min(seg_w, (int)width) / 16), (unsigned)(band_h / kDnWalk));
     const dim3 grid((unsigned)nx, (unsigned)((height + band_h - 1) / band_h), (unsigned)batch);
     if (launch_dependent(density_tile_kernel, grid, threads, (size_t)kDnSmemBytes, st, map, height, width, patch,

@@ -18,7 +18,7 @@
 // 128-byte rows 31 B/clk, tile::gather4 7 B/clk; so the gather is faster than a tiled copy of a compact
 // copy would be, and moves only the rows that are needed.
 //
-// Sinkhorn iteration: as in sinkhorn_cluster.cuh (one pass per iteration, LR lanes share a row, column
+// Sinkhorn iteration: one pass per iteration (LR lanes share a row, column
 // sums completed over the warps in shared memory and over the two CTAs through distributed shared
 // memory), but a thread's K values never leave its registers.
 // Merge: for each tile of 64 output columns, D = [I | alpha P] . [T_k rows of the tile ; T_p] (the
@@ -30,7 +30,7 @@
 #include "common.cuh"
 #include "ptx.cuh"
 #include "sinkhorn.cuh"
-#include "sinkhorn_cluster.cuh"
+#include "sinkhorn_rows.cuh"
 
 namespace rtp {
 

@@ -17,8 +17,8 @@
 #include "merge_umma.cuh"
 #include "scores_umma.cuh"
 #include "sinkhorn.cuh"
-#include "sinkhorn_cluster.cuh"
 #include "sinkhorn_reg.cuh"
+#include "sinkhorn_rows.cuh"
 #include "sinkhorn_tall.cuh"
 #include "stage1.cuh"
 
@@ -441,6 +441,10 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
     uint32_t *scores_done = nullptr; // per-image counts of finished score tiles, when the scores kernel keeps them
     const bool iterate = params->form != RTPRUNE_SINKHORN_EXACT;   // Sinkhorn iterations, else the exact pairing
 
+    // Scaling form, every possible tile small enough for a thread's K values to stay in registers: clusters of two
+    // CTAs per image, in one wave when the batch allows
+    const bool use_reg = iterate && kTensor && !use_log_form(params) && plan->fused_clusters > 0 &&
+                         sinkhorn_reg_eligible(maxN, maxB) && batch <= plan->fused_clusters;
     if constexpr (kTensor) {
         // One kernel for the whole second stage when every image the run can hold fits it
         if (fused_stage2_ok(plan, params)) {
@@ -484,7 +488,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                 scores_done = (uint32_t *)(ws + L.scores_done);
             if (!c.ok(launch_pdl(scores_umma_kernel, grid, dim3(kScThreads), kScSmemBytes, st, 1u, tmapX, tmapXp,
                                  offsets, plan->d, o.counts, order, (const int32_t *)(ws + L.kpos), norms, kmat,
-                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done)))
+                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, use_reg ? 0 : 1)))
                 return RTPRUNE_ERR_CUDA;
         } else {
             const int btiles = (maxB + kF3Tile - 1) / kF3Tile, mtiles = (maxN + kF3Tile - 1) / kF3Tile;
@@ -500,13 +504,10 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
         OtParams op{params->z, params->alpha, params->eps, params->iters,
                     params->stop_at_fixed_point, params->tol};
         const int smem_floats = plan->sink_smem_bytes / (int)sizeof(float);
-        // Scaling form: the cluster kernel takes every tile of up to 32 * kSfMaxNc columns; the general
-        // kernel then takes what is left (it skips the images already solved).
-        int fast_c = 0;
-        const int fast_floats = plan->fast_smem_bytes / (int)sizeof(float);
+        // Scaling form: sinkhorn_rows_kernel takes every tile of up to kSrMaxB columns (sinkhorn_reg_kernel the runs whose
+        // every tile is small); the kernels for wider tiles then take what is left (they skip the images already solved).
+        int rows_max_b = 0;
         bool all_fast = false;
-        // Scaling form, every possible tile small enough for a thread's K values to stay in registers: clusters
-        // of two CTAs per image, in one wave when the batch allows (else the cluster kernels below)
         if (!iterate) {
             // Eq. 2-6 solved exactly, one CTA per image (an ordinary launch: it starts when the scores are complete)
             exact_pairing_kernel<<<batch, kExThreads, plan->exact_smem_bytes, st>>>(
@@ -516,8 +517,6 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             if (!c.ok(cudaGetLastError())) return RTPRUNE_ERR_CUDA;
             launched(plan, st, "exact_pairing");
         }
-        const bool use_reg = iterate && kTensor && !use_log_form(params) && plan->fused_clusters > 0 &&
-                             sinkhorn_reg_eligible(maxN, maxB) && batch <= plan->fused_clusters;
         if (use_reg) {
             ready_list = (int32_t *)(ws + L.ready_list);
             if (!c.ok(launch_pdl(sinkhorn_reg_kernel, dim3((unsigned)(2 * batch)), dim3(kFuThreads), (size_t)kFuSmemBytes,
@@ -531,56 +530,45 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             all_fast = true;
         }
         if (iterate && !use_log_form(params) && !use_reg) {
-            // CTAs per image: as many as keep the whole batch on the chip at once, and more if the largest
-            // possible tile needs them to keep K in their shared memory; 8 at most (tiles larger than the
-            // cluster's shared memory iterate on K in the workspace)
-            fast_c = 1;
-            while (fast_c < 8 && (long long)batch * fast_c * 2 <= plan->sm_count) fast_c *= 2;
-            auto all_tiles = [&](int cc, bool in_smem) {
-                bool ok = maxB <= 32 * kSfMaxNc;
-                for (int b = 1; b <= maxB && ok; ++b) {
-                    const int m = std::max(maxN - b, 1);
-                    ok = in_smem ? sinkhorn_cluster_fits(m, b, cc, fast_floats)
-                                 : sinkhorn_cluster_handles(m, b, cc, fast_floats);
+            // CTAs per image: enough for K of the largest possible tile to stay in their shared memory (a smaller
+            // tile's image uses fewer, see sr_ctas), more while the device has SMs to spare and a CTA would have more
+            // than 10 000 cells (an exchange of column sums costs less than a pass over that many).  A batch that would
+            // then take more than four waves of CTAs halves it: the few tiles that do not fit read a part of K from L2.
+            const int mb = std::min(maxB, kSrMaxB);
+            auto floats = [&](int cc) {
+                long long most = 0;
+                for (int b = 1; b <= mb; ++b) {
+                    const int rows = (std::max(maxN - b, 1) + cc - 1) / cc;
+                    most = std::max(most, (long long)sr_smem_rows(b, rows) * score_pitch(b) + sr_aux_floats(b, cc, rows));
                 }
-                return ok;
+                return most;
             };
-            // Larger clusters so that every K stays in shared memory only while the grid still fits the chip
-            // at once.  Beyond that the tiles that do not fit iterate on K in the workspace: with 2 CTAs per
-            // image when they are far larger than one CTA's shared memory (128 ragged images of up to 1156
-            // tokens: clusters of 8 take seven waves and 287 us, clusters of 2 take 199 us, single CTAs 311 us),
-            // with 1 when only the very largest exceed it (1024 images of 400 tokens: 272 us against 379 us).
-            while (fast_c < 8 && !all_tiles(fast_c, true) && (long long)batch * fast_c * 2 <= plan->sm_count)
-                fast_c *= 2;
-            if (fast_c < 2 && !all_tiles(2, true)) fast_c = 2;
-            all_fast = all_tiles(fast_c, false);
-            // tiles wider than 256 columns, or too tall for the cluster's shared memory, are possible
-            const bool wide = maxB > 256 || !all_tiles(fast_c, true);
-            // When one instance solves every image, it hands them to the merge kernel one by one
+            const long long limit = plan->fast_smem_bytes / (int)sizeof(float);
+            const long long cells = (long long)(maxN - std::min(mb, maxN / 2)) * std::min(mb, maxN / 2);
+            const bool spare = 2LL * batch <= plan->sm_count;
+            const int spread = spare ? 10000 : 40000;
+            int cc = 1;
+            while (cc < kSrMaxC && floats(cc) > limit) cc *= 2;
+            while (cc < kSrMaxC && (long long)batch * cc * 2 <= plan->sm_count && cells > (long long)spread * cc) cc *= 2;
+            if (cc > 1 && (long long)batch * cc > 4LL * plan->sm_count) cc /= 2;
+            const int smem_floats_rows = (int)std::min(limit, floats(cc)) & ~3;
+            all_fast = maxB <= kSrMaxB;
+            rows_max_b = kSrMaxB;
+            // When one kernel solves every image, it hands them to the merge kernel one by one
             ready_list = (kTensor && all_fast) ? (int32_t *)(ws + L.ready_list) : nullptr;
             const uint32_t *sd = ready_list ? (const uint32_t *)scores_done : (const uint32_t *)nullptr;
-            if (!wide) {
-                if (!c.ok(launch_pdl(sinkhorn_cluster_kernel<false>, dim3((unsigned)(batch * fast_c)),
-                                     dim3(kSfThreads), (size_t)plan->fast_smem_bytes, st, (unsigned)fast_c, offsets,
-                                     o.counts, o.out_offsets, order, kmat, L.kmat_stride, maxN, total, op,
-                                     fast_floats, pbuf, pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight,
-                                     o.stats, (uint32_t *)(ws + L.sink_done), ready_list,
-                                     (WsHeader *)(ws + L.header), sd, 0)))
-                    return RTPRUNE_ERR_CUDA;
-                launched(plan, st, "sinkhorn_cluster");
-            } else {
-                // the instance for wide or tall tiles takes the narrow ones of the same run too
-                if (!c.ok(launch_pdl(sinkhorn_cluster_kernel<true>, dim3((unsigned)(batch * fast_c)),
-                                     dim3(kSfThreads), (size_t)plan->fast_smem_bytes, st, (unsigned)fast_c,
-                                     offsets, o.counts, o.out_offsets, order, kmat, L.kmat_stride, maxN, total,
-                                     op, fast_floats, pbuf, pbuf_pitch, o.merged_idx, o.merge_partner,
-                                     o.merge_weight, o.stats, (uint32_t *)(ws + L.sink_done), ready_list,
-                                     (WsHeader *)(ws + L.header), sd, 1)))
-                    return RTPRUNE_ERR_CUDA;
-                launched(plan, st, "sinkhorn_wide");
-            }
+            if (!c.ok(launch_pdl(mb > 255 ? sinkhorn_rows_kernel<true> : sinkhorn_rows_kernel<false>,
+                                 dim3((unsigned)(batch * cc)), dim3(kSrThreads), sizeof(float) * (size_t)smem_floats_rows, st,
+                                 (unsigned)cc, offsets, (const int32_t *)o.counts, (const int32_t *)o.out_offsets,
+                                 (const int32_t *)order, kmat, L.kmat_stride, maxN, total, op, cc, spread, smem_floats_rows,
+                                 pbuf, pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight, o.stats,
+                                 (uint32_t *)(ws + L.sink_done), ready_list, (WsHeader *)(ws + L.header), sd)))
+                return RTPRUNE_ERR_CUDA;
+            // the name in a profile says what the launch was for: the instance for wide tiles, or whole images of more
+            // than 32 768 cells on one CTA in a batch that fills the device; else the common case
+            launched(plan, st, mb > 255 || (!spare && cells > 32768LL * cc) ? "sinkhorn_wide" : "sinkhorn_cluster");
         }
-        // Scaling form, tiles the cluster kernels left (more than 32 * kSfMaxNc columns): clusters of 8
+        // Scaling form, tiles left (more than kSrMaxB columns): clusters of 8
         // CTAs iterate on K in the workspace tile; the general kernel keeps only what is wider still.
         // It takes all the shared memory a CTA can have: what its fixed regions leave is the ring of row blocks.
         const size_t tall_smem = (size_t)std::max(plan->smem_optin - 1024, 0);
@@ -600,7 +588,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             if (!c.ok(launch_pdl(sinkhorn_tall_kernel, dim3((unsigned)(batch * tall_c)), dim3(kTallThreads),
                                  tall_smem, st, (unsigned)tall_c, offsets, o.counts, o.out_offsets, order, kmat,
                                  L.kmat_stride, maxN, total, op, pbuf, pbuf_pitch, o.merged_idx, o.merge_partner,
-                                 o.merge_weight, o.stats, fast_c, fast_floats, (int)(tall_smem / sizeof(float)),
+                                 o.merge_weight, o.stats, rows_max_b, (int)(tall_smem / sizeof(float)),
                                  (WsHeader *)(ws + L.header))))
                 return RTPRUNE_ERR_CUDA;
             launched(plan, st, "sinkhorn_tall");
@@ -611,12 +599,12 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             sinkhorn_kernel<true><<<batch, kSinkThreads, plan->sink_smem_bytes, st>>>(
                 offsets, o.counts, o.out_offsets, order, kmat, L.kmat_stride, maxN, total, op,
                 smem_floats, pbuf, pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight,
-                o.stats, 0, 0, 0);
+                o.stats, 0, 0);
         else if (!all_fast)
             sinkhorn_kernel<false><<<batch, kSinkThreads, plan->sink_smem_bytes, st>>>(
                 offsets, o.counts, o.out_offsets, order, kmat, L.kmat_stride, maxN, total, op,
                 smem_floats, pbuf, pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight,
-                o.stats, fast_c, fast_floats, tall ? kTallMaxB : 0);
+                o.stats, rows_max_b, tall ? kTallMaxB : 0);
         if (!c.ok(cudaGetLastError())) return RTPRUNE_ERR_CUDA;
         if (iterate && (use_log_form(params) || !all_fast)) launched(plan, st, "sinkhorn");
     }
@@ -891,9 +879,9 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
         delete p;
         return RTPRUNE_ERR_CUDA;
     }
-    if (!c.ok(cudaFuncSetAttribute(sinkhorn_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (!c.ok(cudaFuncSetAttribute(sinkhorn_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    p->fast_smem_bytes)) ||
-        !c.ok(cudaFuncSetAttribute(sinkhorn_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        !c.ok(cudaFuncSetAttribute(sinkhorn_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    p->fast_smem_bytes))) {
         delete p;
         return RTPRUNE_ERR_CUDA;

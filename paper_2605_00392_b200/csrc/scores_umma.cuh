@@ -46,7 +46,8 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                    const int32_t *__restrict__ offsets, int d, const int32_t *__restrict__ counts,
                    const int32_t *__restrict__ order, const int32_t *__restrict__ kpos,
                    const float *__restrict__ norms, float *__restrict__ kmat, int kmat_stride,
-                   int max_tokens, int total, WsHeader *__restrict__ hdr, uint32_t *__restrict__ scores_done)
+                   int max_tokens, int total, WsHeader *__restrict__ hdr, uint32_t *__restrict__ scores_done,
+                   int bulk_readers)
 {
     extern __shared__ uint8_t smem_raw[];
     const int img = blockIdx.y, mt = blockIdx.x;
@@ -221,7 +222,10 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
     }
 
     ptx::tc_fence_before();
-    if (scores_done) __threadfence();          // the epilogue's stores, before the count below
+    if (scores_done) {                         // the epilogue's stores, before the count below
+        if (bulk_readers) ptx::fence_proxy_async_all();      // (they are read by bulk copies)
+        __threadfence();
+    }
     __syncthreads();
     if (scores_done && tid == 0) {
         __threadfence();

@@ -1,5 +1,5 @@
 // Dustbin-augmented optimal transport by Sinkhorn iterations (Eq. 5, Appendix C) in scaling form for
-// score tiles too wide for the kernels of sinkhorn_cluster.cuh: images with many tokens (thousands
+// score tiles too wide for the kernel of sinkhorn_rows.cuh: images with many tokens (thousands
 // per image, as the OCR models with large visual token sets produce), up to 4092 pruned tokens.  One
 // cluster of 8 CTAs per image (16 when the batch is small enough to leave SMs idle otherwise); the tile's rows (kept tokens) are split over the CTAs; K =
 // exp((S - c)/eps) is built in place in the image's workspace tile and read once per iteration
@@ -7,7 +7,7 @@
 // of shared-memory stages with 1-D bulk copies, a few blocks ahead of the threads (the tile does not
 // change between iterations, so the stream runs on across the end of an iteration).
 //
-// Same recursion and notation as sinkhorn_cluster.cuh (U = e^u, V = e^{v + c/eps}, the dustbin row and
+// Same recursion and notation as sinkhorn_rows.cuh (U = e^u, V = e^{v + c/eps}, the dustbin row and
 // column carried as scalars).  What differs is the layout: a thread owns fixed columns (16-byte chunks
 // ct, ct + W, ...) of every row of its row group, so the column sums K^T U live in registers across
 // the whole pass; the row sums K V are completed across the W threads of a row by shuffles and one
@@ -19,7 +19,7 @@
 #include "common.cuh"
 #include "ptx.cuh"
 #include "sinkhorn.cuh"
-#include "sinkhorn_cluster.cuh"
+#include "sinkhorn_rows.cuh"
 
 namespace rtp {
 
@@ -533,8 +533,8 @@ __device__ inline void sinkhorn_tall_solve(float *Kg, int ldS, int M, int B, int
     }
 }
 
-// grid = batch * 8 CTAs, clusters of 8 along x.  Takes the images that the cluster kernels ahead of it
-// left (fast_c, fast_floats: their cluster size and shared-memory floats) and whose B <= kTallMaxB; every
+// grid = batch * 8 CTAs, clusters of 8 along x.  Takes the images that the kernel ahead of it
+// left (those with B > rows_max_b) and whose B <= kTallMaxB; every
 // early return depends on the image only, so a cluster leaves as a whole.
 __global__ void __launch_bounds__(kTallThreads, 1)
 sinkhorn_tall_kernel(const int32_t *__restrict__ offsets, const int32_t *__restrict__ counts,
@@ -542,7 +542,7 @@ sinkhorn_tall_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
                      float *__restrict__ kmat, int kmat_stride, int max_tokens, int total, OtParams p,
                      __nv_bfloat16 *__restrict__ pbuf, int pbuf_pitch, int32_t *__restrict__ merged_idx,
                      int32_t *__restrict__ merge_partner, float *__restrict__ merge_weight,
-                     float *__restrict__ stats, int fast_c, int fast_floats, int smem_floats,
+                     float *__restrict__ stats, int rows_max_b, int smem_floats,
                      WsHeader *__restrict__ hdr)
 {
     extern __shared__ __align__(16) float sm[];
@@ -555,8 +555,7 @@ sinkhorn_tall_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
     int t_begin, N;
     if (!image_range(offsets, img, max_tokens, total, t_begin, N)) return;
     const int M = __ldcg(counts + img), B = N - M;
-    if (B == 0 || B > kTallMaxB) return;
-    if (fast_c > 0 && sinkhorn_cluster_handles(M, B, fast_c, fast_floats)) return;   // solved ahead of this kernel
+    if (B <= rows_max_b || B > kTallMaxB) return;      // (nothing to solve,) solved ahead of this kernel, too wide
     const int rows_per = (M + nC - 1) / nC;
     const int row_lo = min(M, (int)rank * rows_per);
     const int Ml = min(M, row_lo + rows_per) - row_lo;       // this CTA's rows (may be 0)

@@ -344,7 +344,6 @@ stage1_kernel(const T *__restrict__ X, const int32_t *__restrict__ offsets, int 
         if (tid == 0) {
             int seq = hdr->launch_seq + 1;
             if (seq == 0) seq = 1;         // 0 is what a fresh workspace holds
-            hdr->merge_next = 0;           // (fp32 storage: the kernel that copies pruned rows does not run)
             ptx::st_release_gpu(&hdr->launch_seq, seq);
             __threadfence();
         }
@@ -588,7 +587,10 @@ stage1_kernel(const T *__restrict__ X, const int32_t *__restrict__ offsets, int 
     if (tid == 0) {
         const uint32_t prev = atomicAdd(&hdr->select_done, 1u);
         s_last = (prev == (uint32_t)batch - 1u);
-        if (s_last) hdr->select_done = 0;        // ready for the next run
+        if (s_last) {                            // ready for the next run
+            hdr->select_done = 0;
+            hdr->merge_next = 0;                 // (fp32 storage: the kernel that copies pruned rows does not run)
+        }
     }
     __syncthreads();
     if (!s_last) return;
