@@ -19,6 +19,7 @@
 #include "sinkhorn.cuh"
 #include "sinkhorn_reg.cuh"
 #include "sinkhorn_rows.cuh"
+#include "sinkhorn_stream.cuh"
 #include "sinkhorn_tall.cuh"
 #include "stage1.cuh"
 
@@ -53,6 +54,7 @@ struct rtprune_plan_s {
     cudaEvent_t ev[RTPRUNE_PROFILE_MAX + 1];
     const char *ev_name[RTPRUNE_PROFILE_MAX];
     int ev_count;  // kernels recorded by the most recent run
+    int stream_clusters[kStMaxC + 1];   // clusters of c CTAs of sinkhorn_stream_kernel the device runs at once
     int tall_c16_clusters;  // clusters of 16 CTAs of the wide-tile Sinkhorn kernel the device runs at once (0: none)
     int fused_clusters;     // clusters of 2 CTAs of the fused stage-2 kernel the device runs at once (0: none)
     int exact_smem_bytes;   // dynamic shared memory of the exact-pairing kernel
@@ -568,10 +570,39 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             // than 32 768 cells on one CTA in a batch that fills the device; else the common case
             launched(plan, st, mb > 255 || (!spare && cells > 32768LL * cc) ? "sinkhorn_wide" : "sinkhorn_cluster");
         }
-        // Scaling form, tiles left (more than kSrMaxB columns): clusters of 8
-        // CTAs iterate on K in the workspace tile; the general kernel keeps only what is wider still.
-        // It takes all the shared memory a CTA can have: what its fixed regions leave is the ring of row blocks.
+        // Scaling form, tiles left (more than kSrMaxB columns)
         const size_t tall_smem = (size_t)std::max(plan->smem_optin - 1024, 0);
+        // Up to kStMaxB columns: clusters that stream K from the workspace, of the size (2 to 16) that needs the least
+        // time when a wave of images takes work / CTAs and a little for the exchanges
+        const bool stream = iterate && !use_log_form(params) && !all_fast && maxB <= kStMaxB;
+        if (stream) {
+            const int threads = st_threads(st_width(maxB));
+            int best = -1;
+            double least = 0.0;
+            for (int cc = kStMaxC; cc >= 2; --cc) {
+                const int nc = plan->stream_clusters[cc];
+                const int rows = (maxN - kSrMaxB - 1 + cc - 1) / cc + 1;
+                if (nc < 1 || sizeof(float) * (size_t)st_min_floats(st_width(maxB), cc, rows, threads / 32) > tall_smem) continue;
+                const double t = ((batch + nc - 1) / nc) * (1.0 / cc + 0.01);
+                if (best < 0 || t < least) {
+                    best = cc;
+                    least = t;
+                }
+            }
+            if (best < 0) return RTPRUNE_ERR_CUDA;
+            if (!c.ok(launch_pdl(threads == 512 ? sinkhorn_stream_kernel<512> : sinkhorn_stream_kernel<256>,
+                                 dim3((unsigned)(batch * best)), dim3((unsigned)threads), tall_smem, st,
+                                 (unsigned)best, offsets, (const int32_t *)o.counts, (const int32_t *)o.out_offsets,
+                                 (const int32_t *)order, kmat, L.kmat_stride, maxN, total, op,
+                                 (int)(tall_smem / sizeof(float)), pbuf, pbuf_pitch, o.merged_idx, o.merge_partner,
+                                 o.merge_weight, o.stats, rows_max_b, (WsHeader *)(ws + L.header))))
+                return RTPRUNE_ERR_CUDA;
+            launched(plan, st, "sinkhorn_tall");
+            all_fast = true;
+        }
+        // Wider tiles: clusters of 8 CTAs iterate on K in the workspace tile with a block barrier per block of rows; the
+        // general kernel keeps only what is wider still.  It takes all the shared memory a CTA can have: what its
+        // fixed regions leave is the ring of row blocks.
         const bool tall = iterate && !use_log_form(params) && !all_fast &&
                           sizeof(float) * (sinkhorn_tall_smem_floats(std::min(maxB, kTallMaxB), maxN) +
                                            kTallStageFloatsMax) <= tall_smem;
@@ -694,6 +725,48 @@ Arena make_arena(const rtprune_plan_t *p)
     a.ws = take(p->ws.total);
     a.total = off;
     return a;
+}
+
+// Clusters of 2 to kStMaxC CTAs of the kernel that streams wide tiles (more than 8 are beyond the portable size): how many
+// of each size the device runs at once.  Asked once per device.
+void stream_cluster_counts(int dev, int smem, int (&counts)[kStMaxC + 1])
+{
+    static std::mutex mutex;
+    static int known[kMaxDevices][kStMaxC + 1];
+    static bool asked[kMaxDevices] = {};
+    std::lock_guard<std::mutex> lock(mutex);
+    const bool keep = dev >= 0 && dev < kMaxDevices;
+    if (keep && asked[dev]) {
+        std::copy(known[dev], known[dev] + kStMaxC + 1, counts);
+        return;
+    }
+    std::fill(counts, counts + kStMaxC + 1, 0);
+    bool ok = true, large = true;
+    for (auto k : {sinkhorn_stream_kernel<256>, sinkhorn_stream_kernel<512>}) {
+        ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+        large = large && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    }
+    for (int cc = 2; ok && cc <= (large ? kStMaxC : 8); ++cc) {
+        // (one CTA per SM either way: its shared memory)
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)cc);
+        cfg.blockDim = dim3(256);
+        cfg.dynamicSmemBytes = (size_t)smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)cc;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, sinkhorn_stream_kernel<256>, &cfg) == cudaSuccess) counts[cc] = n;
+    }
+    (void)cudaGetLastError();
+    if (keep) {
+        std::copy(counts, counts + kStMaxC + 1, known[dev]);
+        asked[dev] = true;
+    }
 }
 
 // Pipelines of plans that are gone, for the next ones (creating one takes about a millisecond): at most kMaxIdle.  A
@@ -938,6 +1011,7 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
     if (dtype == RTPRUNE_BF16)
         (void)cudaFuncSetAttribute(sinkhorn_reg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFuSmemBytes);
     (void)cudaGetLastError();
+    stream_cluster_counts(dev, std::max(p->smem_optin - 1024, 0), p->stream_clusters);
     // Clusters of 16 CTAs (beyond the portable size) for the wide-tile Sinkhorn kernel: ask the device how
     // many it can run at once; a run uses them only if all its images fit that number.
     p->tall_c16_clusters = 0;

@@ -1,0 +1,27 @@
+"""The Sinkhorn kernel that streams score tiles of 640 to 2047 pruned tokens, where its widths change (a multiple of 256
+columns with the dustbin's), with few rows (warps and CTAs without any) and many, clusters of 2 to 16 CTAs.  fp32 storage
+and a small width keep the oracle short.  Marked gpu."""
+import pytest
+import torch
+
+from paper_2605_00392_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("lengths,r,iters", [([1278, 1280, 1282], 0.5, 12), ([1534, 1536], 0.5, 12), ([2048, 2046], 0.5, 8),
+                                             ([2100, 2600, 3070], 0.4999, 6), ([4094], 0.5, 5), ([700, 641, 642], 0.9985, 30),
+                                             ([2000], 0.99, 10), ([1300] * 40, 0.5, 6), ([1300] * 80, 0.5, 3), ([1500, 20], 0.5, 0),
+                                             ([1500], 0.5, 1)])
+def test_edges(lengths, r, iters):
+    import parity
+    w = synth.ragged(lengths, d=64, dtype=torch.float32, params=dict(r_fixed=r, iters=iters))
+    parity.check_workload(w, images=list(range(min(len(lengths), 3))))
+
+
+def test_all_iterations_and_tolerance():
+    import parity
+    w = synth.ragged([1600], d=64, dtype=torch.float32, params=dict(r_fixed=0.45))
+    a = parity.run_gpu(w, overrides=dict(stop_at_fixed_point=0)).out
+    b = parity.run_gpu(w, overrides=dict(tol=1e-3)).out
+    assert float(a.stats[0, 5]) == 100.0 and 1.0 <= float(b.stats[0, 5]) <= 5.0 and float(b.stats[0, 6]) <= 1e-3
