@@ -80,7 +80,7 @@ struct MergeQueue {
 // Bounded wait for the n-th unit of the queue.  false = gave up, or the kernel is being abandoned.
 __device__ inline bool merge_pop(MergeQueue *mq, const MergeBarriers *bars, uint32_t n, MergeUnit &q)
 {
-    for (uint32_t i = 0; i < ptx::kSpinLimit && !bars->abort_flag; ++i) {
+    for (uint32_t i = 0; i < ptx::kPollLimit && !bars->abort_flag; ++i) {
         if (mq->head > n) {
             __threadfence_block();
             q = mq->e[n % kMgQueue];
@@ -94,10 +94,10 @@ __device__ inline bool merge_pop(MergeQueue *mq, const MergeBarriers *bars, uint
 // Image in slot `slot` of the list of finished plans (bounded wait), -1 if it never shows up.
 __device__ inline int merge_wait_image(const int32_t *ready_list, int slot)
 {
-    for (uint32_t i = 0; i < ptx::kSpinLimit; ++i) {
+    for (uint32_t i = 0; i < ptx::kPollLimit; ++i) {
         const int v = ptx::ld_acquire_gpu(ready_list + slot);
         if (v != 0) return v - 1;
-        __nanosleep(200);
+        __nanosleep(40);
     }
     return -1;
 }
@@ -275,7 +275,7 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
                 // can take.  (The queue itself cannot fill up: fewer units are in flight than it holds.)
                 for (uint32_t i = 0; pushed - mq->prod >= (uint32_t)kMgLookahead ||
                                      pushed - mq->tail >= (uint32_t)kMgQueue; ++i) {
-                    if (i >= ptx::kSpinLimit || bars->abort_flag) return false;
+                    if (i >= ptx::kPollLimit || bars->abort_flag) return false;
                     __nanosleep(100);
                 }
                 mq->e[pushed % kMgQueue] = q;

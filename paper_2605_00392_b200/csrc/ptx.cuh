@@ -10,6 +10,7 @@ namespace rtp {
 namespace ptx {
 
 constexpr uint32_t kSpinLimit = 1u << 20;  // polls before a wait reports a timeout
+constexpr uint32_t kPollLimit = 8u * kSpinLimit;   // of the waits on words in memory, which sleep 40 ns or more between polls
 
 __device__ inline uint32_t smem_u32(const void *p)
 {
@@ -95,11 +96,11 @@ __device__ inline void st_release_gpu(int *p, int v)
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 // Bounded wait until *p == want (acquire).  false = gave up after `limit` polls.
-__device__ inline bool wait_equal_gpu(const int *p, int want, uint32_t limit = kSpinLimit)
+__device__ inline bool wait_equal_gpu(const int *p, int want, uint32_t limit = kPollLimit)
 {
     for (uint32_t i = 0; i < limit; ++i) {
         if (ld_acquire_gpu(p) == want) return true;
-        __nanosleep(200);
+        __nanosleep(40);
     }
     return false;
 }

@@ -488,9 +488,10 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             // CTAs queue for the SMs.
             if (iterate && (long long)grid.x * grid.y <= 2LL * plan->sm_count)
                 scores_done = (uint32_t *)(ws + L.scores_done);
-            if (!c.ok(launch_pdl(scores_umma_kernel, grid, dim3(kScThreads), kScSmemBytes, st, 1u, tmapX, tmapXp,
+            const int ring = (long long)grid.x * grid.y <= plan->sm_count ? kScRingBytesAlone : kScRingBytes;
+            if (!c.ok(launch_pdl(scores_umma_kernel, grid, dim3(kScThreads), (size_t)scores_smem_bytes(ring), st, 1u, tmapX, tmapXp,
                                  offsets, plan->d, o.counts, order, (const int32_t *)(ws + L.kpos), norms, kmat,
-                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, use_reg ? 0 : 1)))
+                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, use_reg ? 0 : 1, ring)))
                 return RTPRUNE_ERR_CUDA;
         } else {
             const int btiles = (maxB + kF3Tile - 1) / kF3Tile, mtiles = (maxN + kF3Tile - 1) / kF3Tile;
@@ -972,7 +973,7 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
     if (dtype == RTPRUNE_BF16) {
         if (!p->encode_tiled ||
             !c.ok(cudaFuncSetAttribute(scores_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kScSmemBytes)) ||
+                                       scores_smem_bytes(kScRingBytesAlone))) ||
             !c.ok(cudaFuncSetAttribute(merge_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kMgSmemBytes))) {
             if (!p->last_cuda_error) p->last_cuda_error = (int)cudaErrorNotSupported;

@@ -12,7 +12,7 @@
 // Warp roles (192 threads): warps 0-3 run the epilogue (TMEM -> registers -> divide by the two norms
 // -> global); warp 4 issues the TMA loads (those of a k-block from several lanes at once); warp 5 owns TMEM and its
 // lane 0 issues the UMMAs.  A
-// ring of shared-memory stages (as many as fit in 96 KB: 4 for B <= 64, 2 for B = 256) is handed over
+// ring of shared-memory stages (as many as fit in 96 KB: 4 for B <= 64, 2 for B = 256; twice that in small grids) is handed over
 // with mbarriers.  The ring is sized so that two CTAs share an SM: a whole Large batch is one wave.
 #pragma once
 #include "common.cuh"
@@ -28,8 +28,11 @@ constexpr int kScBBoxRows = 64;      // rows per TMA box of the B operand
 constexpr int kScThreads = 192;
 constexpr int kScABytes = kScTileM * 128;    // 16 KB
 constexpr int kScBBoxBytes = kScBBoxRows * 128;  // 8 KB
+// Ring of a run whose CTAs share an SM in pairs, and of one whose CTAs have an SM each: there a tile is a chain of trips to
+// memory, and twenty k-blocks through eight stages are three trips instead of five.
 constexpr int kScRingBytes = 96 * 1024;
-constexpr int kScSmemBytes = kScRingBytes + 1024 /*alignment*/ + 2048 /*barriers, norms*/;
+constexpr int kScRingBytesAlone = 192 * 1024;
+__host__ __device__ constexpr int scores_smem_bytes(int ring) { return ring + 1024 /*alignment*/ + 2048 /*barriers, norms*/; }
 
 struct ScoresBarriers {
     uint64_t full[kScMaxStages];
@@ -47,37 +50,21 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                    const int32_t *__restrict__ order, const int32_t *__restrict__ kpos,
                    const float *__restrict__ norms, float *__restrict__ kmat, int kmat_stride,
                    int max_tokens, int total, WsHeader *__restrict__ hdr, uint32_t *__restrict__ scores_done,
-                   int bulk_readers)
+                   int bulk_readers, int ring_bytes)
 {
     extern __shared__ uint8_t smem_raw[];
     const int img = blockIdx.y, mt = blockIdx.x;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    ScoresBarriers *bars = reinterpret_cast<ScoresBarriers *>(smem + ring_bytes);
+    // what needs nothing from the kernels ahead comes before the wait for them (the offsets are inputs of the run)
     ptx::grid_dep_launch();
-    ptx::grid_dep_wait();     // counts, order, norms and the compact copy come from the kernels ahead
     int t_begin, N;
-    const int M = __ldcg(counts + img);       // (issued with the two offsets: one trip to L2)
-    if (!image_range(offsets, img, max_tokens, total, t_begin, N)) return;
-    const int B = N - M;
-    if (mt * kScTileM >= N) return;
-    // With scores_done, every tile of a valid image is counted when it is complete (at once if nothing is
-    // pruned): the Sinkhorn kernel, launched as a programmatic dependent, starts on an image when its
-    // tiles are in.
-    if (B == 0) {
-        if (scores_done && threadIdx.x == 0) atomicAdd(&scores_done[img], 1u);
+    const bool in_image = image_range(offsets, img, max_tokens, total, t_begin, N) && mt * kScTileM < N;
+    if (!in_image) {
+        ptx::grid_dep_wait();
         return;
     }
-
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    ScoresBarriers *bars = reinterpret_cast<ScoresBarriers *>(smem + kScRingBytes);
-    // stage = A tile + the B boxes of the widest pass; as many stages as fit in the ring
-    const int boxes_max = (min(kScBNMax, B) + kScBBoxRows - 1) / kScBBoxRows;
-    const int stage_bytes = kScABytes + boxes_max * kScBBoxBytes;
-    const int kScStages = min(kScMaxStages, kScRingBytes / stage_bytes);   // 2 .. 4
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nkb = (d + kScBK - 1) / kScBK;
-    const int nbt = (B + kScBNMax - 1) / kScBNMax;
-    const int32_t *ord = order + t_begin;
-    const int xp0 = xp_row0(t_begin, img);
-
     if (tid == 0) {
         for (int s = 0; s < kScMaxStages; ++s) {
             ptx::mbar_init(&bars->full[s], 1);
@@ -87,6 +74,8 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
         ptx::mbar_init(&bars->tmem_empty, 128);
         bars->abort_flag = 0;
         ptx::fence_mbar_init();
+        ptx::prefetch_tensormap(&tmapX);
+        ptx::prefetch_tensormap(&tmapXp);
     }
     if (warp == 5) {
         ptx::tmem_alloc(&bars->tmem_base, kScBNMax);
@@ -97,16 +86,31 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
     ptx::tc_fence_after();
     const uint32_t tmem_base = bars->tmem_base;
     const uint32_t smem_base = ptx::smem_u32(smem);
+    ptx::grid_dep_wait();     // counts, order, norms and the compact copy come from the kernels ahead
+    const int B = N - __ldcg(counts + img), M = N - B;
+    // With scores_done, every tile of a valid image is counted when it is complete (at once if nothing is
+    // pruned): the Sinkhorn kernel, launched as a programmatic dependent, starts on an image when its
+    // tiles are in.
+    if (B == 0) {
+        if (scores_done && tid == 0) atomicAdd(&scores_done[img], 1u);
+        if (warp == 5) ptx::tmem_dealloc(tmem_base, kScBNMax);
+        return;
+    }
+
+    // stage = A tile + the B boxes of the widest pass; as many stages as fit in the ring
+    const int boxes_max = (min(kScBNMax, B) + kScBBoxRows - 1) / kScBBoxRows;
+    const int stage_bytes = kScABytes + boxes_max * kScBBoxBytes;
+    const int kScStages = min(kScMaxStages, ring_bytes / stage_bytes);   // 2 .. 8
+    const int nkb = (d + kScBK - 1) / kScBK;
+    const int nbt = (B + kScBNMax - 1) / kScBNMax;
+    const int32_t *ord = order + t_begin;
+    const int xp0 = xp_row0(t_begin, img);
 
     if (warp == 4) {
         // ---------------- producer: tiled TMA for both operands -----------------------------------
         // The whole warp walks the k-blocks in step; the loads of a k-block are issued by as many lanes at
         // once (lane 0: the A tile, lanes 1-4: the B boxes) instead of by one thread one after the other.
         {
-            if (lane == 0) {
-                ptx::prefetch_tensormap(&tmapX);
-                ptx::prefetch_tensormap(&tmapXp);
-            }
             uint32_t it = 0;
             bool alive = true;
             for (int bt = 0; bt < nbt && alive && !bars->abort_flag; ++bt) {

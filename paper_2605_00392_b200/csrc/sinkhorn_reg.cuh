@@ -112,9 +112,9 @@ sinkhorn_reg_kernel(const int32_t *__restrict__ offsets, const int32_t *__restri
             const uint32_t want = (uint32_t)((N + 127) / 128);     // the scores kernel's 128-token tiles
             const bool tagged = ptx::wait_equal_gpu(&hdr->run_tag, ptx::ld_acquire_gpu(&hdr->launch_seq));
             bool ok = false;
-            for (uint32_t i = 0; tagged && i < ptx::kSpinLimit && !ok; ++i) {
+            for (uint32_t i = 0; tagged && i < ptx::kPollLimit && !ok; ++i) {
                 ok = (uint32_t)ptx::ld_acquire_gpu(reinterpret_cast<const int *>(scores_done + img)) >= want;
-                if (!ok) __nanosleep(200);
+                if (!ok) __nanosleep(40);
             }
             if (!ok) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
         }

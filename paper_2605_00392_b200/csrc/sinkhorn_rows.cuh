@@ -674,9 +674,9 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
             // first the run's number: before it is there the counts are what the run before left
             const bool tagged = ptx::wait_equal_gpu(&hdr->run_tag, ptx::ld_acquire_gpu(&hdr->launch_seq));
             bool ok = false;
-            for (uint32_t i = 0; tagged && i < ptx::kSpinLimit && !ok; ++i) {
+            for (uint32_t i = 0; tagged && i < ptx::kPollLimit && !ok; ++i) {
                 ok = (uint32_t)ptx::ld_acquire_gpu(reinterpret_cast<const int *>(scores_done + img)) >= want;
-                if (!ok) __nanosleep(100);
+                if (!ok) __nanosleep(40);
             }
             if (!ok) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
         }

@@ -18,6 +18,9 @@ constexpr int kS1Warps = kS1Threads / 32;
 
 constexpr int kS1StageRows = kS1Warps;   // rows per stage of the streaming ring: one per warp
 constexpr int kS1MaxStages = 4;
+// Counting ranks costs N compares per token: ahead of the four passes over the digits while a thread has one token (64
+// tokens: 2 us less), behind them at two (64 images of 400 tokens: stage 1 34.8 -> 36.9 us, 1024 of them 238 -> 254).
+constexpr int kRankMax = kS1Threads;
 
 // Stages of the streaming ring for rows of row_bytes: as many as fit in 96 KB, 2 to 4.
 __host__ __device__ inline int stage1_stages(size_t row_bytes)
@@ -67,7 +70,7 @@ __device__ inline int block_excl_scan(int v, int *scratch)
 // Selection of one image by one CTA (256 threads): phi from the chunk partials; r and
 // B = floor(r N + 1/2) clamped to [0, N-1], M = N - B; the M tokens of largest criterion (`norms`: the
 // l2 norms, or the variance / entropy values of a run that ranks by those; ties to the lower
-// index) are T_kept.  The M-th largest value is found by a radix select over its bits (four
+// index) are T_kept.  Up to kRankMax tokens every token's rank is counted; beyond that the M-th largest value is found by a radix select over its bits (four
 // 8-bit digits, a 256-bin histogram each), tokens equal to it are admitted in index order.  Writes
 // order[] = kept indices ascending, then pruned indices ascending, and its inverse kpos[]; counts,
 // stats.
@@ -159,6 +162,46 @@ __device__ inline void select_image(int img, int t_begin, int N, int d, int chun
         s_keys[k] = key_bits(key);
         if (norms_out) norms_out[t_begin + k] = key;
     }
+    // Up to kRankMax tokens: every thread counts how many tokens rank ahead of its own (larger, or equal and earlier): one
+    // pass over the keys, no histogram, and it needs neither phi nor M.  A warp's 32 tokens are consecutive, so only
+    // against one another do ties look at the index.
+    const bool by_rank = N <= kRankMax;
+    constexpr int kOwn = kRankMax / nth;
+    int rank[kOwn];
+    if (by_rank) {
+        for (int k = N + tid; k < ((N + 31) & ~31); k += nth) s_keys[k] = 0u;       // (only ever compared past N)
+        __syncthreads();
+        const uint4 *k4 = reinterpret_cast<const uint4 *>(s_keys);
+#pragma unroll
+        for (int q = 0; q < kOwn; ++q) {
+            rank[q] = 0;
+            const int base = 32 * warp + q * nth;
+            if (base < N) {
+                const uint32_t key = s_keys[base + lane];
+                int ahead[4] = {0, 0, 0, 0};
+                for (int j = 0; j < base >> 2; ++j) {
+                    const uint4 o = k4[j];
+                    ahead[0] += o.x >= key;
+                    ahead[1] += o.y >= key;
+                    ahead[2] += o.z >= key;
+                    ahead[3] += o.w >= key;
+                }
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const uint32_t o = __shfl_sync(0xffffffffu, key, j);
+                    ahead[j & 3] += (base + j < N) && (o > key || (o == key && j < lane));
+                }
+                for (int j = (base >> 2) + 8; j < (N + 3) >> 2; ++j) {               // (zeros past N are never larger)
+                    const uint4 o = k4[j];
+                    ahead[0] += o.x > key;
+                    ahead[1] += o.y > key;
+                    ahead[2] += o.z > key;
+                    ahead[3] += o.w > key;
+                }
+                rank[q] = (ahead[0] + ahead[1]) + (ahead[2] + ahead[3]);
+            }
+        }
+    }
     const float ssum = block_sum(local, s_redf);
     if (tid == 0) {
         const float Nf = (float)N;
@@ -188,6 +231,42 @@ __device__ inline void select_image(int img, int t_begin, int N, int d, int chun
     }
     __syncthreads();
     const int M = s_M;
+
+    int32_t *ord = order + t_begin;
+    if (by_rank) {
+        // positions of the kept tokens in ascending index: over the warp's 32 tokens by ballot, over the groups of 32
+        // (in s_hist) by a warp's scan
+        uint32_t mask[kOwn];
+#pragma unroll
+        for (int q = 0; q < kOwn; ++q) {
+            const int k = tid + q * nth;
+            mask[q] = __ballot_sync(0xffffffffu, k < N && rank[q] < M);
+            if (lane == 0) s_hist[q * kS1Warps + warp] = __popc(mask[q]);
+        }
+        __syncthreads();
+        const int c = lane < kOwn * kS1Warps ? s_hist[lane] : 0;
+        int before = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, before, o);
+            if (lane >= o) before += u;
+        }
+        before -= c;
+#pragma unroll
+        for (int q = 0; q < kOwn; ++q) {
+            const int k = tid + q * nth;
+            const int run = __shfl_sync(0xffffffffu, before, q * kS1Warps + warp) + __popc(mask[q] & ((1u << lane) - 1u));
+            if (k < N) {
+                const bool kept = (mask[q] >> lane) & 1u;
+                const int pos = kept ? run : M + (k - run);
+                ord[pos] = k;
+                kpos[t_begin + k] = kept ? run : -1 - (k - run);
+                if (order_out) order_out[t_begin + pos] = k;
+            }
+        }
+        __syncthreads();
+        return;
+    }
 
     // radix select: after the four digits `prefix` is the M-th largest key and `need` is how many
     // tokens equal to it are kept
@@ -256,7 +335,6 @@ __device__ inline void select_image(int img, int t_begin, int N, int d, int chun
         }
     }
     int kpos_run = block_excl_scan(nkept, s_redi);   // kept tokens before k0
-    int32_t *ord = order + t_begin;
     for (int k = k0; k < k1; ++k) {
         const bool kept = (keptmask >> (k - k0)) & 1u;
         const int pos = kept ? kpos_run : (M + (k - kpos_run));
@@ -335,27 +413,31 @@ stage1_kernel(const T *__restrict__ X, const int32_t *__restrict__ offsets, int 
     __shared__ uint64_t s_full[kS1MaxStages], s_empty[kS1MaxStages];
     const int img = blockIdx.y, chunk = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (blockIdx.x == 0 && blockIdx.y == 0) {
-        // This CTA numbers the run: the kernels behind tell this run's counters and lists in the workspace from
-        // the last run's by the number.  It is counted up here, on the device, after the run ahead in the stream
-        // has ended and BEFORE this CTA lets the dependents go (they are scheduled once every CTA of this grid
-        // has done so), so every kernel of the run reads the new number, also in a replayed CUDA graph.
-        ptx::grid_dep_wait();
-        if (tid == 0) {
-            int seq = hdr->launch_seq + 1;
-            if (seq == 0) seq = 1;         // 0 is what a fresh workspace holds
-            ptx::st_release_gpu(&hdr->launch_seq, seq);
-            __threadfence();
+    // CTA (0, 0) numbers the run: the kernels behind tell this run's counters and lists in the workspace from
+    // the last run's by the number.  It is counted up here, on the device, after the run ahead in the stream
+    // has ended and BEFORE this CTA lets the dependents go (they are scheduled once every CTA of this grid
+    // has done so), so every kernel of the run reads the new number, also in a replayed CUDA graph.  Its first
+    // copies are on their way by then; the warp that does it (and alone lets the dependents go) has no part in issuing
+    // them.
+    const bool numbers = blockIdx.x == 0 && blockIdx.y == 0;
+    auto number_run = [&]() {
+        if (warp == kS1Warps - 1) {
+            if (lane == 0) {
+                int seq = hdr->launch_seq + 1;
+                if (seq == 0) seq = 1;         // 0 is what a fresh workspace holds
+                ptx::st_release_gpu(&hdr->launch_seq, seq);
+                __threadfence();
+            }
+            __syncwarp();
+            ptx::grid_dep_launch();
         }
-        __syncthreads();
-        ptx::grid_dep_launch();
-    } else {
-        ptx::grid_dep_launch();
-        ptx::grid_dep_wait();     // the workspace may still be in use by the run ahead in the stream
-    }
+    };
+    if (!numbers) ptx::grid_dep_launch();
+    ptx::grid_dep_wait();         // the workspace may still be in use by the run ahead in the stream
     int t_begin, n_img;
     const bool valid = image_range(offsets, img, max_tokens, total, t_begin, n_img);
     if (!valid) {
+        if (numbers) number_run();
         if (chunk != 0) return;
         if (tid == 0) {   // offsets broke the contract: the image yields no output
             atomicOr(&hdr->status, RTPRUNE_DEV_BAD_OFFSETS);
@@ -401,6 +483,7 @@ stage1_kernel(const T *__restrict__ X, const int32_t *__restrict__ offsets, int 
         int issued = 0;           // thread 0: copies issued so far
         if (tid == 0)
             for (int it = 0; it < min(nstage, nit); ++it, ++issued) issue(it);
+        if (numbers) number_run();
         for (int it = 0; it < nit; ++it) {
             const int s = it % nstage;
             {   // a warp goes on or gives up as one (the row's reductions below are warp-wide)
@@ -613,15 +696,19 @@ gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restri
                    int32_t *__restrict__ out_offsets, uint32_t *__restrict__ scores_done)
 {
     __shared__ int s_scan[32];
-    const int img = blockIdx.y;
+    // the last images first: what stage 1 read last is what L2 still holds
+    const int img = (int)gridDim.y - 1 - (int)blockIdx.y;
     ptx::grid_dep_launch();
+    int t_begin, N;
+    const bool valid = image_range(offsets, img, max_tokens, total, t_begin, N);     // (inputs of the run)
     ptx::grid_dep_wait();     // counts and order come from the kernel ahead
+    const int M_img = __ldcg(counts + img);
     // One CTA prepares what the kernels behind this one share through the workspace, while the others
     // copy: it empties the per-image counters and the list of finished plans, then publishes the run's
     // number.  Kernels launched as programmatic dependents may already be resident and must not read
     // those words before they see that number: until then they hold what the run before left.  (That
     // run has ended: it is ahead of stage 1 in the stream.)  It also turns the counts into out_offsets.
-    if (blockIdx.x == 0 && img == 0) {
+    if (blockIdx.x == 0 && blockIdx.y == 0) {
         for (int i = threadIdx.x; i < batch; i += 128) {
             sink_done[i] = 0;
             scores_done[i] = 0;
@@ -636,9 +723,8 @@ gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restri
         if (threadIdx.x == 0) ptx::st_release_gpu(&hdr->run_tag, ptx::ld_acquire_gpu(&hdr->launch_seq));
         scan_counts<128>(counts, out_offsets, batch, s_scan);
     }
-    int t_begin, N;
-    if (!image_range(offsets, img, max_tokens, total, t_begin, N)) return;
-    const int M = counts[img], B = N - M, Bpad = (B + 63) & ~63;
+    if (!valid) return;
+    const int M = M_img, B = N - M, Bpad = (B + 63) & ~63;
     const int j0 = blockIdx.x * kGpRows + (threadIdx.x >> 5) * 2;
     if (j0 >= Bpad) return;
     const int lane = threadIdx.x & 31;
