@@ -440,6 +440,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
     __nv_bfloat16 *pbuf = kTensor ? (__nv_bfloat16 *)(ws + L.pbuf) : nullptr;
     const int pbuf_pitch = (std::max(maxB, 1) + 63) / 64 * 64;   // <= L.pbuf_pitch_max
     int32_t *ready_list = nullptr;   // images in the order their plans are finished, when the merge follows it
+    int split = 1;                   // CTAs per tile of the scores
     uint32_t *scores_done = nullptr; // per-image counts of finished score tiles, when the scores kernel keeps them
     const bool iterate = params->form != RTPRUNE_SINKHORN_EXACT;   // Sinkhorn iterations, else the exact pairing
 
@@ -488,10 +489,13 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             // CTAs queue for the SMs.
             if (iterate && (long long)grid.x * grid.y <= 2LL * plan->sm_count)
                 scores_done = (uint32_t *)(ws + L.scores_done);
-            const int ring = (long long)grid.x * grid.y <= plan->sm_count ? kScRingBytesAlone : kScRingBytes;
-            if (!c.ok(launch_pdl(scores_umma_kernel, grid, dim3(kScThreads), (size_t)scores_smem_bytes(ring), st, 1u, tmapX, tmapXp,
+            // a tile's contraction over 8, 4 or 2 CTAs while the device has SMs for them all
+            while (split < 8 && maxB <= kScBNMax && (long long)grid.x * grid.y * split * 2 <= plan->sm_count) split *= 2;
+            const int ring = split == 1 && (long long)grid.x * grid.y <= plan->sm_count ? kScRingBytesAlone : kScRingBytes;
+            grid.x *= (unsigned)split;
+            if (!c.ok(launch_pdl(scores_umma_kernel, grid, dim3(kScThreads), (size_t)(scores_smem_bytes(ring) + scores_split_bytes(split)), st, (unsigned)split, tmapX, tmapXp,
                                  offsets, plan->d, o.counts, order, (const int32_t *)(ws + L.kpos), norms, kmat,
-                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, use_reg ? 0 : 1, ring)))
+                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, use_reg ? 0 : 1, ring, split)))
                 return RTPRUNE_ERR_CUDA;
         } else {
             const int btiles = (maxB + kF3Tile - 1) / kF3Tile, mtiles = (maxN + kF3Tile - 1) / kF3Tile;
@@ -527,7 +531,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                                  (const int32_t *)order, (const float *)kmat, L.kmat_stride, maxN, total, op, pbuf,
                                  pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight, o.stats,
                                  (uint32_t *)(ws + L.sink_done), ready_list, (WsHeader *)(ws + L.header),
-                                 (const uint32_t *)scores_done)))
+                                 (const uint32_t *)scores_done, split)))
                 return RTPRUNE_ERR_CUDA;
             launched(plan, st, "sinkhorn_reg");
             all_fast = true;
@@ -565,7 +569,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                                  (unsigned)cc, offsets, (const int32_t *)o.counts, (const int32_t *)o.out_offsets,
                                  (const int32_t *)order, kmat, L.kmat_stride, maxN, total, op, cc, spread, smem_floats_rows,
                                  pbuf, pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight, o.stats,
-                                 (uint32_t *)(ws + L.sink_done), ready_list, (WsHeader *)(ws + L.header), sd)))
+                                 (uint32_t *)(ws + L.sink_done), ready_list, (WsHeader *)(ws + L.header), sd, split)))
                 return RTPRUNE_ERR_CUDA;
             // the name in a profile says what the launch was for: the instance for wide tiles, or whole images of more
             // than 32 768 cells on one CTA in a batch that fills the device; else the common case
@@ -973,7 +977,8 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
     if (dtype == RTPRUNE_BF16) {
         if (!p->encode_tiled ||
             !c.ok(cudaFuncSetAttribute(scores_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       scores_smem_bytes(kScRingBytesAlone))) ||
+                                       std::max(scores_smem_bytes(kScRingBytesAlone),
+                                                scores_smem_bytes(kScRingBytes) + scores_split_bytes(8)))) ||
             !c.ok(cudaFuncSetAttribute(merge_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kMgSmemBytes))) {
             if (!p->last_cuda_error) p->last_cuda_error = (int)cudaErrorNotSupported;

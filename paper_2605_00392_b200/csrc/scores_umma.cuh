@@ -13,7 +13,10 @@
 // -> global); warp 4 issues the TMA loads (those of a k-block from several lanes at once); warp 5 owns TMEM and its
 // lane 0 issues the UMMAs.  A
 // ring of shared-memory stages (as many as fit in 96 KB: 4 for B <= 64, 2 for B = 256; twice that in small grids) is handed over
-// with mbarriers.  The ring is sized so that two CTAs share an SM: a whole Large batch is one wave.
+// with mbarriers.  Small grids (split > 1): a tile's k-blocks are dealt out to a cluster of `split` CTAs, since one SM's
+// TMA unit takes in about 31 bytes per clock (480 KB of a 128 x 64 tile: 8 us).  Their partial sums are reduce-scattered
+// over the cluster by units of 16 columns through distributed shared memory and added in rank order.
+// The ring is sized so that two CTAs share an SM: a whole Large batch is one wave.
 #pragma once
 #include "common.cuh"
 #include "ptx.cuh"
@@ -34,6 +37,13 @@ constexpr int kScRingBytes = 96 * 1024;
 constexpr int kScRingBytesAlone = 192 * 1024;
 __host__ __device__ constexpr int scores_smem_bytes(int ring) { return ring + 1024 /*alignment*/ + 2048 /*barriers, norms*/; }
 
+constexpr int kScUnit = 16;          // columns per unit of the reduction over a cluster
+// Shared memory for the CTAs' partial sums: of each, the units this CTA owns.
+__host__ __device__ constexpr int scores_split_bytes(int split)
+{
+    return split > 1 ? split * ((kScBNMax / kScUnit + split - 1) / split) * kScTileM * kScUnit * 4 : 0;
+}
+
 struct ScoresBarriers {
     uint64_t full[kScMaxStages];
     uint64_t empty[kScMaxStages];
@@ -50,13 +60,15 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                    const int32_t *__restrict__ order, const int32_t *__restrict__ kpos,
                    const float *__restrict__ norms, float *__restrict__ kmat, int kmat_stride,
                    int max_tokens, int total, WsHeader *__restrict__ hdr, uint32_t *__restrict__ scores_done,
-                   int bulk_readers, int ring_bytes)
+                   int bulk_readers, int ring_bytes, int split)
 {
     extern __shared__ uint8_t smem_raw[];
-    const int img = blockIdx.y, mt = blockIdx.x;
+    const int img = blockIdx.y, mt = split > 1 ? blockIdx.x / split : blockIdx.x;
+    const int rank = blockIdx.x - mt * split;     // in the cluster of a split tile
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     ScoresBarriers *bars = reinterpret_cast<ScoresBarriers *>(smem + ring_bytes);
+    float4 *parts = reinterpret_cast<float4 *>(smem + ring_bytes + 2048);        // [rank][own unit][4 columns][row]
     // what needs nothing from the kernels ahead comes before the wait for them (the offsets are inputs of the run)
     ptx::grid_dep_launch();
     int t_begin, N;
@@ -101,11 +113,13 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
     const int boxes_max = (min(kScBNMax, B) + kScBBoxRows - 1) / kScBBoxRows;
     const int stage_bytes = kScABytes + boxes_max * kScBBoxBytes;
     const int kScStages = min(kScMaxStages, ring_bytes / stage_bytes);   // 2 .. 8
-    const int nkb = (d + kScBK - 1) / kScBK;
+    const int nkb_all = (d + kScBK - 1) / kScBK, nkb_per = (nkb_all + split - 1) / split;
+    const int kb_lo = rank * nkb_per, nkb = max(0, min(nkb_all, kb_lo + nkb_per) - kb_lo);       // this CTA's k-blocks
     const int nbt = (B + kScBNMax - 1) / kScBNMax;
     const int32_t *ord = order + t_begin;
     const int xp0 = xp_row0(t_begin, img);
 
+    bool sync_due = split > 1;                    // every warp takes one barrier of the cluster
     if (warp == 4) {
         // ---------------- producer: tiled TMA for both operands -----------------------------------
         // The whole warp walks the k-blocks in step; the loads of a k-block are issued by as many lanes at
@@ -128,10 +142,10 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                     if (lane == 0) ptx::mbar_arrive_expect_tx(&bars->full[s], kScABytes + nbox * kScBBoxBytes);
                     __syncwarp();
                     if (lane == 0)
-                        ptx::tma_load_2d(a_dst, &tmapX, &bars->full[s], kb * kScBK, t_begin + mt * kScTileM);
+                        ptx::tma_load_2d(a_dst, &tmapX, &bars->full[s], (kb_lo + kb) * kScBK, t_begin + mt * kScTileM);
                     else if (lane <= nbox)
                         ptx::tma_load_2d(a_dst + kScABytes + (lane - 1) * kScBBoxBytes, &tmapXp, &bars->full[s],
-                                         kb * kScBK, xp0 + bt * kScBNMax + (lane - 1) * kScBBoxRows);
+                                         (kb_lo + kb) * kScBK, xp0 + bt * kScBNMax + (lane - 1) * kScBBoxRows);
                 }
             }
         }
@@ -199,6 +213,45 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                 continue;
             }
             ptx::tc_fence_after();
+            if (split > 1) {
+                // (one pass: B <= 256.  Compact loops: a small run waits for instructions more than for arithmetic.)
+                const int units = (kScBNMax / kScUnit + split - 1) / split;
+                const uint32_t mine = ptx::smem_u32(parts + rank * units * 4 * kScTileM + row);
+#pragma unroll 1
+                for (int u = 0; u < BN / kScUnit && nkb > 0; ++u) {
+                    uint32_t r[16];
+                    ptx::tmem_ld16(tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(u * kScUnit), r);
+                    ptx::tmem_ld_wait();
+                    const uint32_t to = ptx::map_to_rank(mine + (uint32_t)(u / split * 4 * kScTileM * 16), (uint32_t)(u % split));
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) ptx::st_cluster_v4(to + (uint32_t)(g * kScTileM * 16), r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+                }
+                ptx::cluster_sync_all();               // every part has landed
+                sync_due = false;
+                const int active = (nkb_all + nkb_per - 1) / nkb_per;       // ranks with k-blocks
+                if (p >= 0) {
+#pragma unroll 1
+                    for (int v = 0; v < 4 * units; ++v) {
+                        const int j = ((v >> 2) * split + rank) * kScUnit + 4 * (v & 3);
+                        if (j >= B) continue;
+                        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+                        for (int q = 0; q < active; ++q) {
+                            const float4 x = parts[(q * units * 4 + v) * kScTileM + row];
+                            o.x += x.x;
+                            o.y += x.y;
+                            o.z += x.z;
+                            o.w += x.w;
+                        }
+                        o.x *= inv_ni * bars->inv_nj[j];
+                        o.y *= inv_ni * bars->inv_nj[min(j + 1, B - 1)];
+                        o.z *= inv_ni * bars->inv_nj[min(j + 2, B - 1)];
+                        o.w *= inv_ni * bars->inv_nj[min(j + 3, B - 1)];
+                        *reinterpret_cast<float4 *>(Simg + (size_t)p * ldS + j) = o;
+                    }
+                }
+                break;
+            }
             for (int c0 = 0; c0 < BN; c0 += 32) {
                 uint32_t r[32];
                 ptx::tmem_ld32(tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
@@ -225,6 +278,8 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
         }
     }
 
+    __syncwarp();
+    if (sync_due) ptx::cluster_sync_all();
     ptx::tc_fence_before();
     if (scores_done) {                         // the epilogue's stores, before the count below
         if (bulk_readers) ptx::fence_proxy_async_all();      // (they are read by bulk copies)

@@ -651,7 +651,7 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
                      int spread, int smem_floats, __nv_bfloat16 *__restrict__ pbuf, int pbuf_pitch,
                      int32_t *__restrict__ merged_idx, int32_t *__restrict__ merge_partner,
                      float *__restrict__ merge_weight, float *__restrict__ stats, uint32_t *__restrict__ sink_done,
-                     int32_t *__restrict__ ready_list, WsHeader *__restrict__ hdr, const uint32_t *scores_done)
+                     int32_t *__restrict__ ready_list, WsHeader *__restrict__ hdr, const uint32_t *scores_done, int tile_ctas)
 {
     extern __shared__ __align__(16) float sm[];
     __shared__ uint64_t s_xbar[2], s_cbar[kSrChunks];
@@ -670,7 +670,7 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
     const bool valid = image_range(offsets, img, max_tokens, total, t_begin, N);
     if (valid && scores_done) {
         if (tid == 0) {
-            const uint32_t want = (uint32_t)((N + 127) / 128);     // the scores kernel's 128-token tiles
+            const uint32_t want = (uint32_t)((N + 127) / 128 * tile_ctas);     // the scores kernel's CTAs, by 128-token tile
             // first the run's number: before it is there the counts are what the run before left
             const bool tagged = ptx::wait_equal_gpu(&hdr->run_tag, ptx::ld_acquire_gpu(&hdr->launch_seq));
             bool ok = false;
