@@ -141,7 +141,7 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
                   int batch, int mtiles, const int32_t *__restrict__ counts,
                   const int32_t *__restrict__ out_offsets, const int32_t *__restrict__ kpos,
                   int max_tokens, int total, __nv_bfloat16 *__restrict__ Y, int32_t *__restrict__ kept_idx,
-                  WsHeader *__restrict__ hdr, const int32_t *ready_list)
+                  WsHeader *__restrict__ hdr, const int32_t *ready_list, int by_image)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -288,11 +288,13 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
             bool ok = !ready_list || ptx::wait_equal_gpu(&hdr->run_tag, ptx::ld_acquire_gpu(&hdr->launch_seq));
             while (ok && !bars->abort_flag) {
                 // next unit: from the shared counter when the units follow the list of finished images
-                const int u = ready_list ? (int)atomicAdd(&hdr->merge_next, 1u)
-                                         : (int)(blockIdx.x + drawn++ * gridDim.x);
+                const bool drawn_units = ready_list && !by_image;
+                const int u = drawn_units ? (int)atomicAdd(&hdr->merge_next, 1u) : (int)(blockIdx.x + drawn++ * gridDim.x);
                 if (u >= nunits) break;
-                const MergeUnit q = merge_unit(u, mtiles, nct, offsets, counts, out_offsets, max_tokens, total,
-                                               ready_list);
+                MergeUnit q = merge_unit(u, mtiles, nct, offsets, counts, out_offsets, max_tokens, total,
+                                         drawn_units ? ready_list : nullptr);
+                // (by image: what the unit needs to know is there before the image is)
+                if (by_image && q.valid && merge_wait_image(ready_list, q.img) < 0) q.timed_out = true;
                 if (q.timed_out) ok = false;
                 else if (q.valid) ok = push(q);
             }

@@ -47,6 +47,27 @@ __device__ inline bool mbar_try_wait(uint64_t *bar, uint32_t parity)
         : "memory");
     return ok != 0;
 }
+// The same, ordered after what the other CTAs of the cluster did before their arrivals; bounded.
+__device__ inline bool mbar_wait_cluster(uint64_t *bar, uint32_t parity)
+{
+    for (uint32_t i = 0; i < kSpinLimit; ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+// Arrival on a barrier of another CTA of the cluster (address from map_to_rank).
+__device__ inline void mbar_arrive_remote(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 // Bounded wait for the phase with the given parity to complete.  false = gave up after `limit` polls.
 __device__ inline bool mbar_wait(uint64_t *bar, uint32_t parity, uint32_t limit = kSpinLimit)
 {

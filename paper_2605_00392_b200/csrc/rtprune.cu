@@ -441,6 +441,9 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
     const int pbuf_pitch = (std::max(maxB, 1) + 63) / 64 * 64;   // <= L.pbuf_pitch_max
     int32_t *ready_list = nullptr;   // images in the order their plans are finished, when the merge follows it
     int split = 1;                   // CTAs per tile of the scores
+    // the merge has a CTA for every unit: each waits for its own image, no order of completion
+    const long long merge_units = (long long)batch * ((maxN + kMgTileM - 1) / kMgTileM) * ((plan->d + kMgTileN - 1) / kMgTileN);
+    const int by_image = merge_units <= plan->sm_count ? 1 : 0;
     uint32_t *scores_done = nullptr; // per-image counts of finished score tiles, when the scores kernel keeps them
     const bool iterate = params->form != RTPRUNE_SINKHORN_EXACT;   // Sinkhorn iterations, else the exact pairing
 
@@ -489,13 +492,14 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             // CTAs queue for the SMs.
             if (iterate && (long long)grid.x * grid.y <= 2LL * plan->sm_count)
                 scores_done = (uint32_t *)(ws + L.scores_done);
-            // a tile's contraction over 8, 4 or 2 CTAs while the device has SMs for them all
-            while (split < 8 && maxB <= kScBNMax && (long long)grid.x * grid.y * split * 2 <= plan->sm_count) split *= 2;
+            // a tile's contraction over 4 or 2 CTAs while the device has SMs for them all (not for the one-CTA kernels of
+            // the log form and the exact pairing, which take far longer than the scores)
+            while (iterate && !use_log_form(params) && split < 4 && maxB <= kScBNMax && (long long)grid.x * grid.y * split * 2 <= plan->sm_count) split *= 2;
             const int ring = split == 1 && (long long)grid.x * grid.y <= plan->sm_count ? kScRingBytesAlone : kScRingBytes;
             grid.x *= (unsigned)split;
             if (!c.ok(launch_pdl(scores_umma_kernel, grid, dim3(kScThreads), (size_t)(scores_smem_bytes(ring) + scores_split_bytes(split)), st, (unsigned)split, tmapX, tmapXp,
                                  offsets, plan->d, o.counts, order, (const int32_t *)(ws + L.kpos), norms, kmat,
-                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, use_reg ? 0 : 1, ring, split)))
+                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, ring, split)))
                 return RTPRUNE_ERR_CUDA;
         } else {
             const int btiles = (maxB + kF3Tile - 1) / kF3Tile, mtiles = (maxN + kF3Tile - 1) / kF3Tile;
@@ -531,7 +535,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                                  (const int32_t *)order, (const float *)kmat, L.kmat_stride, maxN, total, op, pbuf,
                                  pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight, o.stats,
                                  (uint32_t *)(ws + L.sink_done), ready_list, (WsHeader *)(ws + L.header),
-                                 (const uint32_t *)scores_done, split)))
+                                 (const uint32_t *)scores_done, split, by_image)))
                 return RTPRUNE_ERR_CUDA;
             launched(plan, st, "sinkhorn_reg");
             all_fast = true;
@@ -569,7 +573,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                                  (unsigned)cc, offsets, (const int32_t *)o.counts, (const int32_t *)o.out_offsets,
                                  (const int32_t *)order, kmat, L.kmat_stride, maxN, total, op, cc, spread, smem_floats_rows,
                                  pbuf, pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight, o.stats,
-                                 (uint32_t *)(ws + L.sink_done), ready_list, (WsHeader *)(ws + L.header), sd, split)))
+                                 (uint32_t *)(ws + L.sink_done), ready_list, (WsHeader *)(ws + L.header), sd, split, by_image)))
                 return RTPRUNE_ERR_CUDA;
             // the name in a profile says what the launch was for: the instance for wide tiles, or whole images of more
             // than 32 768 cells on one CTA in a batch that fills the device; else the common case
@@ -657,7 +661,8 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
         if (!c.ok(launch_pdl(merge_umma_kernel, dim3((unsigned)grid), dim3(kMgThreads), kMgSmemBytes, st, 1u,
                              tmapXm, tmapXpm, tmapP, offsets, plan->d, batch, mtiles_m, o.counts, o.out_offsets,
                              (const int32_t *)(ws + L.kpos), maxN, total, (__nv_bfloat16 *)o.Y, o.kept_idx,
-                             (WsHeader *)(ws + L.header), (const int32_t *)ready_list)))
+                             (WsHeader *)(ws + L.header), (const int32_t *)ready_list,
+                             ready_list ? by_image : 0)))
             return RTPRUNE_ERR_CUDA;
     } else {
         const int mtiles = (maxN + kF3Tile - 1) / kF3Tile, nct = (plan->d + kM3N - 1) / kM3N;
@@ -978,7 +983,7 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
         if (!p->encode_tiled ||
             !c.ok(cudaFuncSetAttribute(scores_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        std::max(scores_smem_bytes(kScRingBytesAlone),
-                                                scores_smem_bytes(kScRingBytes) + scores_split_bytes(8)))) ||
+                                                scores_smem_bytes(kScRingBytes) + scores_split_bytes(4)))) ||
             !c.ok(cudaFuncSetAttribute(merge_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kMgSmemBytes))) {
             if (!p->last_cuda_error) p->last_cuda_error = (int)cudaErrorNotSupported;

@@ -60,7 +60,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                    const int32_t *__restrict__ order, const int32_t *__restrict__ kpos,
                    const float *__restrict__ norms, float *__restrict__ kmat, int kmat_stride,
                    int max_tokens, int total, WsHeader *__restrict__ hdr, uint32_t *__restrict__ scores_done,
-                   int bulk_readers, int ring_bytes, int split)
+                   int ring_bytes, int split)
 {
     extern __shared__ uint8_t smem_raw[];
     const int img = blockIdx.y, mt = split > 1 ? blockIdx.x / split : blockIdx.x;
@@ -282,7 +282,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
     if (sync_due) ptx::cluster_sync_all();
     ptx::tc_fence_before();
     if (scores_done) {                         // the epilogue's stores, before the count below
-        if (bulk_readers) ptx::fence_proxy_async_all();      // (they are read by bulk copies)
+        ptx::fence_proxy_async_all();          // (they are read by bulk copies)
         __threadfence();
     }
     __syncthreads();

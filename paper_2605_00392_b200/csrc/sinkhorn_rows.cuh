@@ -475,8 +475,15 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
 // This CTA has written everything it contributes to image `img`; the last of the C CTAs to say so
 // appends the image to the list that the merge kernel consumes in order of completion (it may already
 // be running: it was launched as a programmatic dependent).  Called by every thread of the CTA.
+// by_image: the merge kernel has a CTA for every unit, which waits for its own image: the entry's place is the image's
+// number, and nobody counts.
+__device__ inline void sinkhorn_list(int img, int32_t *__restrict__ ready_list, WsHeader *__restrict__ hdr, bool by_image)
+{
+    const uint32_t slot = by_image ? (uint32_t)img : atomicAdd(&hdr->n_ready, 1u);
+    ptx::st_release_gpu(ready_list + slot, img + 1);
+}
 __device__ inline void sinkhorn_publish(int img, uint32_t C, uint32_t *__restrict__ sink_done,
-                                        int32_t *__restrict__ ready_list, WsHeader *__restrict__ hdr)
+                                        int32_t *__restrict__ ready_list, WsHeader *__restrict__ hdr, bool by_image)
 {
     if (!ready_list) return;
     ptx::fence_proxy_async_all();     // the plan rows are read by TMA over there
@@ -486,8 +493,7 @@ __device__ inline void sinkhorn_publish(int img, uint32_t C, uint32_t *__restric
         const uint32_t prev = C > 1u ? atomicAdd(&sink_done[img], 1u) : 0u;
         if (prev == C - 1u) {
             __threadfence();
-            const uint32_t slot = atomicAdd(&hdr->n_ready, 1u);
-            ptx::st_release_gpu(ready_list + slot, img + 1);
+            sinkhorn_list(img, ready_list, hdr, by_image);
         }
     }
 }
@@ -502,6 +508,7 @@ struct SrOut {
     float *weight_seg;
     uint32_t *sink_done;
     int32_t *ready_list;
+    bool by_image;
 };
 
 // Plan P = U K V of this CTA's rows: alpha P in bf16 (row = the kept token's position in X, columns up to the next
@@ -566,7 +573,7 @@ __device__ inline void sr_finish(const SrTile &t, const OtParams &p, const SrOut
             }
         }
     }
-    sinkhorn_publish(o.img, (uint32_t)t.C, o.sink_done, o.ready_list, hdr);
+    sinkhorn_publish(o.img, (uint32_t)t.C, o.sink_done, o.ready_list, hdr, o.by_image);
 
     // pairs: over the row slots of a warp, the warps, the CTAs (ranks hold ascending rows)
 #pragma unroll
@@ -651,7 +658,7 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
                      int spread, int smem_floats, __nv_bfloat16 *__restrict__ pbuf, int pbuf_pitch,
                      int32_t *__restrict__ merged_idx, int32_t *__restrict__ merge_partner,
                      float *__restrict__ merge_weight, float *__restrict__ stats, uint32_t *__restrict__ sink_done,
-                     int32_t *__restrict__ ready_list, WsHeader *__restrict__ hdr, const uint32_t *scores_done, int tile_ctas)
+                     int32_t *__restrict__ ready_list, WsHeader *__restrict__ hdr, const uint32_t *scores_done, int tile_ctas, int by_image)
 {
     extern __shared__ __align__(16) float sm[];
     __shared__ uint64_t s_xbar[2], s_cbar[kSrChunks];
@@ -688,7 +695,7 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
     t.B = valid ? N - t.M : 0;
     if (t.B == 0 || t.B > kSrMaxB) {           // nothing to solve, or another kernel's tile (then no list is kept)
         if (rank == 0) {
-            sinkhorn_publish(img, 1u, sink_done, ready_list, hdr);
+            sinkhorn_publish(img, 1u, sink_done, ready_list, hdr, by_image != 0);
             if (scores_done) ptx::grid_dep_wait();
         }
         return;
@@ -728,7 +735,7 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
     const float v_init = expf(shift * inv_eps);            // v = 0
     const int seg = t_begin - out0;
     const SrOut o{img, order + t_begin, pbuf ? pbuf + (size_t)t_begin * pbuf_pitch : nullptr, pbuf_pitch,
-                  merged_idx + seg, merge_partner + seg, merge_weight + seg, sink_done, ready_list};
+                  merged_idx + seg, merge_partner + seg, merge_weight + seg, sink_done, ready_list, by_image != 0};
     auto solve = [&](auto lr, auto nq, auto rb) {
         constexpr int LR = decltype(lr)::value, NQ = decltype(nq)::value, RB = decltype(rb)::value;
         sr_build(t, shift, inv_eps, 1.f / kappa, hdr);

@@ -509,7 +509,7 @@ sinkhorn_stream_kernel(const int32_t *__restrict__ offsets, const int32_t *__res
     ptx::cluster_sync_all();
     const int seg = t_begin - __ldcg(out_offsets + img);
     const SrOut o{img, order + t_begin, pbuf ? pbuf + (size_t)t_begin * pbuf_pitch : nullptr, pbuf_pitch,
-                  merged_idx + seg, merge_partner + seg, merge_weight + seg, nullptr, nullptr};
+                  merged_idx + seg, merge_partner + seg, merge_weight + seg, nullptr, nullptr, false};
     float *st = stats + (size_t)img * kStats;
     switch (W >> 8) {
     case 3: st_solve<6, TH>(t, p, o, st, hdr); break;

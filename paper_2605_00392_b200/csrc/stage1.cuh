@@ -704,10 +704,10 @@ gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restri
     ptx::grid_dep_wait();     // counts and order come from the kernel ahead
     const int M_img = __ldcg(counts + img);
     // One CTA prepares what the kernels behind this one share through the workspace, while the others
-    // copy: it empties the per-image counters and the list of finished plans, then publishes the run's
-    // number.  Kernels launched as programmatic dependents may already be resident and must not read
+    // copy: it empties the per-image counters and the list of finished plans, turns the counts into out_offsets, then
+    // publishes the run's number.  Kernels launched as programmatic dependents may already be resident and must not read
     // those words before they see that number: until then they hold what the run before left.  (That
-    // run has ended: it is ahead of stage 1 in the stream.)  It also turns the counts into out_offsets.
+    // run has ended: it is ahead of stage 1 in the stream.)
     if (blockIdx.x == 0 && blockIdx.y == 0) {
         for (int i = threadIdx.x; i < batch; i += 128) {
             sink_done[i] = 0;
@@ -718,10 +718,10 @@ gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restri
             hdr->n_ready = 0;
             hdr->merge_next = 0;
         }
+        scan_counts<128>(counts, out_offsets, batch, s_scan);
         __threadfence();
         __syncthreads();
         if (threadIdx.x == 0) ptx::st_release_gpu(&hdr->run_tag, ptx::ld_acquire_gpu(&hdr->launch_seq));
-        scan_counts<128>(counts, out_offsets, batch, s_scan);
     }
     if (!valid) return;
     const int M = M_img, B = N - M, Bpad = (B + 63) & ~63;
