@@ -69,7 +69,7 @@ struct FuShared {
     uint64_t sc_full[kFuScStages], sc_empty[kFuScStages], sc_accum;
     uint64_t mg_full[kFuMgStages], mg_empty[kFuMgStages];
     uint64_t acc_full[kFuAccStages], acc_empty[kFuAccStages];
-    uint64_t kbar, pubbar;                      // sinkhorn_reg_kernel: the scores have landed; the other CTA has written its plan
+    uint64_t pubbar;                            // sinkhorn_reg_kernel: the other CTA has written its plan
     uint64_t xbar[2];                           // the other CTA's column sums of an iteration have arrived (by parity)
     uint32_t tmem_base;
     volatile int abort_flag;

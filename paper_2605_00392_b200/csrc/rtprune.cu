@@ -440,7 +440,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
     __nv_bfloat16 *pbuf = kTensor ? (__nv_bfloat16 *)(ws + L.pbuf) : nullptr;
     const int pbuf_pitch = (std::max(maxB, 1) + 63) / 64 * 64;   // <= L.pbuf_pitch_max
     int32_t *ready_list = nullptr;   // images in the order their plans are finished, when the merge follows it
-    int split = 1;                   // CTAs per tile of the scores
+    int split = 1;                   // CTAs per tile of the scores (1 or 4)
     // the merge has a CTA for every unit: each waits for its own image, no order of completion
     const long long merge_units = (long long)batch * ((maxN + kMgTileM - 1) / kMgTileM) * ((plan->d + kMgTileN - 1) / kMgTileN);
     const int by_image = merge_units <= plan->sm_count ? 1 : 0;
@@ -492,14 +492,15 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             // CTAs queue for the SMs.
             if (iterate && (long long)grid.x * grid.y <= 2LL * plan->sm_count)
                 scores_done = (uint32_t *)(ws + L.scores_done);
-            // a tile's contraction over 4 or 2 CTAs while the device has SMs for them all (not for the one-CTA kernels of
-            // the log form and the exact pairing, which take far longer than the scores)
-            while (iterate && !use_log_form(params) && split < 4 && maxB <= kScBNMax && (long long)grid.x * grid.y * split * 2 <= plan->sm_count) split *= 2;
+            // a tile's contraction over 4 CTAs while the device has SMs for them all (over 2 it gains nothing: 32 images of
+            // 256 tokens 18.4 us either way; not for the one-CTA kernels of the log form and the exact pairing, which take
+            // far longer than the scores)
+            if (iterate && !use_log_form(params) && maxB <= kScBNMax && (long long)grid.x * grid.y * 4 <= plan->sm_count) split = 4;
             const int ring = split == 1 && (long long)grid.x * grid.y <= plan->sm_count ? kScRingBytesAlone : kScRingBytes;
             grid.x *= (unsigned)split;
             if (!c.ok(launch_pdl(scores_umma_kernel, grid, dim3(kScThreads), (size_t)(scores_smem_bytes(ring) + scores_split_bytes(split)), st, (unsigned)split, tmapX, tmapXp,
                                  offsets, plan->d, o.counts, order, (const int32_t *)(ws + L.kpos), norms, kmat,
-                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, ring, split)))
+                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, use_reg ? 0 : 1, ring, split)))
                 return RTPRUNE_ERR_CUDA;
         } else {
             const int btiles = (maxB + kF3Tile - 1) / kF3Tile, mtiles = (maxN + kF3Tile - 1) / kF3Tile;

@@ -13,7 +13,7 @@
 // -> global); warp 4 issues the TMA loads (those of a k-block from several lanes at once); warp 5 owns TMEM and its
 // lane 0 issues the UMMAs.  A
 // ring of shared-memory stages (as many as fit in 96 KB: 4 for B <= 64, 2 for B = 256; twice that in small grids) is handed over
-// with mbarriers.  Small grids (split > 1): a tile's k-blocks are dealt out to a cluster of `split` CTAs, since one SM's
+// with mbarriers.  Small grids (split > 1): a tile's k-blocks are dealt out to a cluster of `split` (4) CTAs, since one SM's
 // TMA unit takes in about 31 bytes per clock (480 KB of a 128 x 64 tile: 8 us).  Their partial sums are reduce-scattered
 // over the cluster by units of 16 columns through distributed shared memory and added in rank order.
 // The ring is sized so that two CTAs share an SM: a whole Large batch is one wave.
@@ -60,7 +60,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                    const int32_t *__restrict__ order, const int32_t *__restrict__ kpos,
                    const float *__restrict__ norms, float *__restrict__ kmat, int kmat_stride,
                    int max_tokens, int total, WsHeader *__restrict__ hdr, uint32_t *__restrict__ scores_done,
-                   int ring_bytes, int split)
+                   int bulk_readers, int ring_bytes, int split)
 {
     extern __shared__ uint8_t smem_raw[];
     const int img = blockIdx.y, mt = split > 1 ? blockIdx.x / split : blockIdx.x;
@@ -282,7 +282,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
     if (sync_due) ptx::cluster_sync_all();
     ptx::tc_fence_before();
     if (scores_done) {                         // the epilogue's stores, before the count below
-        ptx::fence_proxy_async_all();          // (they are read by bulk copies)
+        if (bulk_readers) ptx::fence_proxy_async_all();      // (they are read by bulk copies)
         __threadfence();
     }
     __syncthreads();

@@ -1,4 +1,4 @@
-"""The scores of small batches, whose contraction is shared out over clusters of 2 and 4 CTAs: pruned counts around the
+"""The scores of small batches, whose contraction is shared out over clusters of 4 CTAs: pruned counts around the
 units of 16 columns, widths whose k-blocks do not share out evenly (or are fewer than the CTAs), images that end within a
 tile.  Marked gpu."""
 import pytest
