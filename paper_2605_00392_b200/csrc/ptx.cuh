@@ -245,6 +245,10 @@ __device__ inline void cluster_sync_all()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// The same in two halves that publish nothing: after the wait every thread of the cluster has arrived, so every CTA is
+// running and its shared memory may be written.
+__device__ inline void cluster_started() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ inline void cluster_wait_started() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
 
 // ---- tcgen05: tensor memory and UMMA ------------------------------------------------------------
 // Executed by one full warp.  ncols: power of two in [32, 512].  The TMEM base address is written to

@@ -77,6 +77,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
         ptx::grid_dep_wait();
         return;
     }
+    if (split > 1) ptx::cluster_started();        // (waited for before anything is stored into another CTA)
     if (tid == 0) {
         for (int s = 0; s < kScMaxStages; ++s) {
             ptx::mbar_init(&bars->full[s], 1);
@@ -104,6 +105,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
     // pruned): the Sinkhorn kernel, launched as a programmatic dependent, starts on an image when its
     // tiles are in.
     if (B == 0) {
+        if (split > 1) ptx::cluster_wait_started();
         if (scores_done && tid == 0) atomicAdd(&scores_done[img], 1u);
         if (warp == 5) ptx::tmem_dealloc(tmem_base, kScBNMax);
         return;
@@ -119,7 +121,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
     const int32_t *ord = order + t_begin;
     const int xp0 = xp_row0(t_begin, img);
 
-    bool sync_due = split > 1;                    // every warp takes one barrier of the cluster
+    bool sync_due = split > 1;                    // every warp takes both barriers of the cluster
     if (warp == 4) {
         // ---------------- producer: tiled TMA for both operands -----------------------------------
         // The whole warp walks the k-blocks in step; the loads of a k-block are issued by as many lanes at
@@ -217,6 +219,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                 // (one pass: B <= 256.  Compact loops: a small run waits for instructions more than for arithmetic.)
                 const int units = (kScBNMax / kScUnit + split - 1) / split;
                 const uint32_t mine = ptx::smem_u32(parts + rank * units * 4 * kScTileM + row);
+                ptx::cluster_wait_started();           // the other CTAs' shared memory is theirs to be written
 #pragma unroll 1
                 for (int u = 0; u < BN / kScUnit && nkb > 0; ++u) {
                     uint32_t r[16];
@@ -279,7 +282,10 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
     }
 
     __syncwarp();
-    if (sync_due) ptx::cluster_sync_all();
+    if (sync_due) {
+        ptx::cluster_wait_started();
+        ptx::cluster_sync_all();
+    }
     ptx::tc_fence_before();
     if (scores_done) {                         // the epilogue's stores, before the count below
         if (bulk_readers) ptx::fence_proxy_async_all();      // (they are read by bulk copies)
