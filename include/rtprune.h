@@ -251,7 +251,8 @@ rtprune_status_t rtprune_query_status_static(rtprune_plan_t *plan, void *cuda_st
 /*
  * The same run, from and to HOST buffers (pinned memory recommended): copies X, offsets and rho to
  * the device arena, runs, and copies every output back, all asynchronously on the stream; the
- * caller synchronises the stream before reading.  `rho_host` may be NULL (params->rho is ignored
+ * caller synchronises the stream before reading (also after an error, before it frees or reuses the
+ * buffers: what was enqueued up to then is on the stream, or ordered before its end).  `rho_host` may be NULL (params->rho is ignored
  * here).  Y_host has room for total_tokens rows; the first out_offsets[batch] are written when the ratio is
  * fixed (the kept counts are then known on the host before the launch), all total_tokens rows when it is
  * dynamic (only the first out_offsets[batch] are meaningful).
@@ -332,6 +333,15 @@ rtprune_status_t rtprune_test_expire_waits(rtprune_plan_t *plan, void *cuda_stre
  * faults, nothing is read that never arrived, and the next run with the default limit is clean.
  */
 rtprune_status_t rtprune_test_set_poll_limit(rtprune_plan_t *plan, int64_t polls);
+
+/*
+ * Test aid for the error path of rtprune_run_host, which takes a large batch with a fixed ratio through in groups
+ * of images on several streams: its group number `group` (from 0; negative: none, the default) fails with
+ * RTPRUNE_ERR_CUDA once the copy of its tokens is on its way, as if the next call had been refused.  As after any error
+ * everything enqueued before is ordered ahead of what the caller's stream takes next: once that stream has been waited
+ * for, nothing reads or writes the buffers any more.
+ */
+rtprune_status_t rtprune_test_fail_group(rtprune_plan_t *plan, int32_t group);
 
 /* Kernels launched by the most recent run / select / run_host call on this plan. */
 int32_t rtprune_last_launch_count(const rtprune_plan_t *plan);

@@ -70,6 +70,7 @@ def lib() -> ctypes.CDLL:
     L.rtprune_query_status_static.argtypes = [vp, vp, ctypes.POINTER(ctypes.c_uint32)]
     L.rtprune_test_expire_waits.argtypes = [vp, vp, vp, sz, ctypes.c_uint32, vp]
     L.rtprune_test_set_poll_limit.argtypes = [vp, ctypes.c_int64]
+    L.rtprune_test_fail_group.argtypes = [vp, i32]
     L.rtprune_run_host.argtypes = [vp, vp, vp, vp, vp, i32, i64, pp, vp, sz,
                                    vp, vp, vp, vp, vp, vp, vp, vp]
     L.rtprune_host_arena_bytes.argtypes = [vp, ctypes.POINTER(sz)]
@@ -242,6 +243,10 @@ class Plan:
     def set_poll_limit(self, polls: int) -> None:
         """Test aid: polls after which stage 1's waits on its copies give up (negative: the default)."""
         _check(lib().rtprune_test_set_poll_limit(self.handle, int(polls)), "rtprune_test_set_poll_limit")
+
+    def fail_group(self, group: int) -> None:
+        """Test aid: run_host's group of images of this number fails before its launches (negative: none)."""
+        _check(lib().rtprune_test_fail_group(self.handle, int(group)), "rtprune_test_fail_group")
 
     # -- rtprune_host_arena_bytes / rtprune_run_host
     def host_arena_bytes(self) -> int:

@@ -72,6 +72,7 @@ struct rtprune_plan_s {
     int map_next;           // entry the next miss replaces
     int64_t last_host_ns;   // host time the most recent rtprune_run call spent inside the library
     HostPipe *host_pipe;    // rtprune_run_host's, from its first pipelined call on
+    int fail_group;         // group of rtprune_run_host that fails once its tokens are on their way (-1: none; tests set it)
     uint32_t poll_limit;    // polls after which stage 1's waits on its copies give up (ptx::kSpinLimit; tests lower it)
 };
 
@@ -906,6 +907,7 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
     p->map_next = 0;
     p->last_host_ns = 0;
     p->host_pipe = nullptr;
+    p->fail_group = -1;
     p->poll_limit = ptx::kSpinLimit;
     p->profiling = false;
     p->ev_count = 0;
@@ -1217,6 +1219,13 @@ rtprune_status_t rtprune_test_set_poll_limit(rtprune_plan_t *plan, int64_t polls
     return RTPRUNE_OK;
 }
 
+rtprune_status_t rtprune_test_fail_group(rtprune_plan_t *plan, int32_t group)
+{
+    if (!plan) return RTPRUNE_ERR_INVALID_ARG;
+    plan->fail_group = group < 0 ? -1 : group;
+    return RTPRUNE_OK;
+}
+
 rtprune_status_t rtprune_host_arena_bytes(const rtprune_plan_t *plan, size_t *arena_bytes)
 {
     if (!plan || !arena_bytes) return RTPRUNE_ERR_INVALID_ARG;
@@ -1285,62 +1294,77 @@ rtprune_status_t rtprune_run_host(rtprune_plan_t *plan, void *cuda_stream, const
     }
     HostPipe *pipe = plan->host_pipe;
     cudaStream_t in = groups > 1 ? pipe->in : st, out = groups > 1 ? pipe->out : st;
-    if (groups > 1 && (!c.ok(cudaEventRecord(pipe->begin, st)) || !c.ok(cudaStreamWaitEvent(in, pipe->begin, 0)) ||
-                       !c.ok(cudaStreamWaitEvent(out, pipe->begin, 0))))
-        return RTPRUNE_ERR_CUDA;
-    if (!c.ok(cudaMemcpyAsync(d_offsets, offsets_host, ((size_t)batch + 1) * 4, cudaMemcpyHostToDevice, in)) ||
-        (rho_host && !c.ok(cudaMemcpyAsync(base + a.rho, rho_host, (size_t)batch * 4, cudaMemcpyHostToDevice, in))) ||
-        !c.ok(cudaMemsetAsync(base + a.ws + plan->ws.header, 0, plan->ws.clear_bytes, st)))
-        return RTPRUNE_ERR_CUDA;
-    int i0 = 0;
-    size_t kept0 = 0;                      // output rows of the groups before (fixed ratio)
-    for (int g = 0; g < groups; ++g) {
-        // images [i0, i1): the cut nearest to equal shares of the tokens, at least one image each
-        int i1 = g == groups - 1 ? batch : i0 + 1;
-        while (i1 < batch - (groups - 1 - g) && (long long)offsets_host[i1] * groups < (g + 1LL) * total_tokens) ++i1;
-        const size_t t0 = (size_t)offsets_host[i0], t1 = (size_t)offsets_host[i1];
-        if (!c.ok(cudaMemcpyAsync(base + a.X + t0 * row, (const char *)X_host + t0 * row, (t1 - t0) * row, cudaMemcpyHostToDevice, in)))
+    // Whatever goes wrong on the way, the side streams are joined to the caller's below: a caller that has waited for its
+    // stream may free the buffers.
+    auto enqueue = [&]() -> rtprune_status_t {
+        if (groups > 1 && (!c.ok(cudaEventRecord(pipe->begin, st)) || !c.ok(cudaStreamWaitEvent(in, pipe->begin, 0)) ||
+                           !c.ok(cudaStreamWaitEvent(out, pipe->begin, 0))))
             return RTPRUNE_ERR_CUDA;
-        if (groups > 1 && (!c.ok(cudaEventRecord(pipe->copied[g], in)) || !c.ok(cudaStreamWaitEvent(st, pipe->copied[g], 0))))
+        if (!c.ok(cudaMemcpyAsync(d_offsets, offsets_host, ((size_t)batch + 1) * 4, cudaMemcpyHostToDevice, in)) ||
+            (rho_host && !c.ok(cudaMemcpyAsync(base + a.rho, rho_host, (size_t)batch * 4, cudaMemcpyHostToDevice, in))) ||
+            !c.ok(cudaMemsetAsync(base + a.ws + plan->ws.header, 0, plan->ws.clear_bytes, st)))
             return RTPRUNE_ERR_CUDA;
-        // the group's images keep their places in X and in the workspace; its outputs are packed behind the groups' before
-        rtprune_params_t pg = p;
-        if (pg.rho) pg.rho += i0;
-        DevOut o{base + a.Y + kept0 * row, groups > 1 ? (int32_t *)(base + a.group_offsets) + i0 + g : d_out, d_counts + i0,
-                 d_kept + kept0, d_merged - kept0, d_partner - kept0, d_weight - kept0, d_stats + (size_t)i0 * kStats};
-        const rtprune_status_t rs = run_device(plan, st, base + a.X, d_offsets + i0, i1 - i0, (int)total_tokens, &pg, base + a.ws, o);
-        if (rs != RTPRUNE_OK) return rs;
-        // Rows of Y to bring back: with a fixed ratio every image's kept count is known here; a dynamic ratio is
-        // decided on the device, so all rows are copied.
-        size_t rows = (size_t)total_tokens;
-        if (!p.dynamic) {
-            rows = 0;
-            for (int i = i0; i < i1; ++i) rows += (size_t)fixed_kept(p.r_fixed, offsets_host[i + 1] - offsets_host[i]);
+        int i0 = 0;
+        size_t kept0 = 0;                      // output rows of the groups before (fixed ratio)
+        for (int g = 0; g < groups; ++g) {
+            // images [i0, i1): the cut nearest to equal shares of the tokens, at least one image each
+            int i1 = g == groups - 1 ? batch : i0 + 1;
+            while (i1 < batch - (groups - 1 - g) && (long long)offsets_host[i1] * groups < (g + 1LL) * total_tokens) ++i1;
+            const size_t t0 = (size_t)offsets_host[i0], t1 = (size_t)offsets_host[i1];
+            if (!c.ok(cudaMemcpyAsync(base + a.X + t0 * row, (const char *)X_host + t0 * row, (t1 - t0) * row, cudaMemcpyHostToDevice, in)) ||
+                g == plan->fail_group)
+                return RTPRUNE_ERR_CUDA;
+            if (groups > 1 && (!c.ok(cudaEventRecord(pipe->copied[g], in)) || !c.ok(cudaStreamWaitEvent(st, pipe->copied[g], 0))))
+                return RTPRUNE_ERR_CUDA;
+            // the group's images keep their places in X and in the workspace; its outputs are packed behind the groups' before
+            rtprune_params_t pg = p;
+            if (pg.rho) pg.rho += i0;
+            DevOut o{base + a.Y + kept0 * row, groups > 1 ? (int32_t *)(base + a.group_offsets) + i0 + g : d_out, d_counts + i0,
+                     d_kept + kept0, d_merged - kept0, d_partner - kept0, d_weight - kept0, d_stats + (size_t)i0 * kStats};
+            const rtprune_status_t rs = run_device(plan, st, base + a.X, d_offsets + i0, i1 - i0, (int)total_tokens, &pg, base + a.ws, o);
+            if (rs != RTPRUNE_OK) return rs;
+            // Rows of Y to bring back: with a fixed ratio every image's kept count is known here; a dynamic ratio is
+            // decided on the device, so all rows are copied.
+            size_t rows = (size_t)total_tokens;
+            if (!p.dynamic) {
+                rows = 0;
+                for (int i = i0; i < i1; ++i) rows += (size_t)fixed_kept(p.r_fixed, offsets_host[i + 1] - offsets_host[i]);
+            }
+            if (groups > 1 && (!c.ok(cudaEventRecord(pipe->solved[g], st)) || !c.ok(cudaStreamWaitEvent(out, pipe->solved[g], 0))))
+                return RTPRUNE_ERR_CUDA;
+            if (rows && !c.ok(cudaMemcpyAsync((char *)Y_host + kept0 * row, base + a.Y + kept0 * row, rows * row, cudaMemcpyDeviceToHost, out)))
+                return RTPRUNE_ERR_CUDA;
+            kept0 += rows;
+            i0 = i1;
         }
-        if (groups > 1 && (!c.ok(cudaEventRecord(pipe->solved[g], st)) || !c.ok(cudaStreamWaitEvent(out, pipe->solved[g], 0))))
+        if (groups > 1) {
+            scan_counts_kernel<<<1, 256, 0, st>>>(d_counts, d_out, batch);
+            ++plan->last_launches;
+        }
+        const size_t tot4 = (size_t)total_tokens * 4;
+        if (!c.ok(cudaGetLastError()) ||
+            !c.ok(cudaMemcpyAsync(out_offsets_host, d_out, ((size_t)batch + 1) * 4, cudaMemcpyDeviceToHost, st)) ||
+            !c.ok(cudaMemcpyAsync(counts_host, d_counts, (size_t)batch * 4, cudaMemcpyDeviceToHost, st)) ||
+            !c.ok(cudaMemcpyAsync(kept_idx_host, d_kept, tot4, cudaMemcpyDeviceToHost, st)) ||
+            !c.ok(cudaMemcpyAsync(merged_idx_host, d_merged, tot4, cudaMemcpyDeviceToHost, st)) ||
+            !c.ok(cudaMemcpyAsync(merge_partner_host, d_partner, tot4, cudaMemcpyDeviceToHost, st)) ||
+            !c.ok(cudaMemcpyAsync(merge_weight_host, d_weight, tot4, cudaMemcpyDeviceToHost, st)) ||
+            !c.ok(cudaMemcpyAsync(stats_host, d_stats, (size_t)batch * kStats * 4, cudaMemcpyDeviceToHost, st)))
             return RTPRUNE_ERR_CUDA;
-        if (rows && !c.ok(cudaMemcpyAsync((char *)Y_host + kept0 * row, base + a.Y + kept0 * row, rows * row, cudaMemcpyDeviceToHost, out)))
-            return RTPRUNE_ERR_CUDA;
-        kept0 += rows;
-        i0 = i1;
-    }
+        return RTPRUNE_OK;
+    };
+    s = enqueue();
     if (groups > 1) {
-        scan_counts_kernel<<<1, 256, 0, st>>>(d_counts, d_out, batch);
-        ++plan->last_launches;
+        // (a run that went through has waited for every copy in already)
+        bool joined = c.ok(cudaEventRecord(pipe->end, out)) && c.ok(cudaStreamWaitEvent(st, pipe->end, 0));
+        if (s != RTPRUNE_OK) joined = joined && c.ok(cudaEventRecord(pipe->begin, in)) && c.ok(cudaStreamWaitEvent(st, pipe->begin, 0));
+        if (!joined) {
+            (void)cudaStreamSynchronize(in);
+            (void)cudaStreamSynchronize(out);
+            s = RTPRUNE_ERR_CUDA;
+        }
     }
-    const size_t tot4 = (size_t)total_tokens * 4;
-    if (!c.ok(cudaGetLastError()) ||
-        !c.ok(cudaMemcpyAsync(out_offsets_host, d_out, ((size_t)batch + 1) * 4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(counts_host, d_counts, (size_t)batch * 4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(kept_idx_host, d_kept, tot4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(merged_idx_host, d_merged, tot4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(merge_partner_host, d_partner, tot4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(merge_weight_host, d_weight, tot4, cudaMemcpyDeviceToHost, st)) ||
-        !c.ok(cudaMemcpyAsync(stats_host, d_stats, (size_t)batch * kStats * 4, cudaMemcpyDeviceToHost, st)))
-        return RTPRUNE_ERR_CUDA;
-    if (groups > 1 && (!c.ok(cudaEventRecord(pipe->end, out)) || !c.ok(cudaStreamWaitEvent(st, pipe->end, 0))))
-        return RTPRUNE_ERR_CUDA;
-    return RTPRUNE_OK;
+    return s;
 }
 
 rtprune_status_t rtprune_query_status(rtprune_plan_t *plan, void *cuda_stream, void *workspace,

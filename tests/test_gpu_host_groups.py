@@ -33,3 +33,32 @@ def test_groups_equal_the_device_entry_point(lengths, dtype, r):
             torch.testing.assert_close(a.merge_weight[:nb], b.merge_weight[:nb], rtol=1e-5, atol=0)
     finally:
         plan.close()
+
+
+def test_an_error_between_the_groups_leaves_nothing_in_flight():
+    """A group that fails after others have been enqueued: the error is returned, and once the caller's stream has been
+    waited for no copy is on its way any more (the last group before the failure copies 15 MB out)."""
+    w = synth.ragged([400] * 8, params=dict(r_fixed=0.25))
+    X, batch, kept = w.X.repeat(20, 1).pin_memory(), 160, 300
+    offsets = (torch.arange(batch + 1) * 400).to(torch.int32).pin_memory()
+    plan = binding.Plan(w.d, X.dtype, batch, X.shape[0], 400)
+    try:
+        out = binding.Outputs.allocate(X.shape[0], batch, w.d, X.dtype, "cpu", pin=True)
+        params = binding.make_params(None, dynamic=0, r_fixed=0.25)
+        rows = 4 * (batch // 8) * kept                       # of the four groups ahead of the failure
+        for _ in range(3):
+            out.Y.fill_(77.0)
+            plan.fail_group(4)
+            with pytest.raises(binding.RtpruneError):
+                plan.run_host(X, offsets, None, params, out)
+            torch.cuda.current_stream().synchronize()
+            last = out.Y[rows - 1].clone()
+            torch.cuda.synchronize()
+            assert torch.equal(out.Y[rows - 1], last) and not (last == 77.0).any()
+            assert (out.Y[rows:] == 77.0).all()              # the failed group and those after it
+        plan.fail_group(-1)
+        plan.run_host(X, offsets, None, params, out)         # the plan stays usable
+        torch.cuda.current_stream().synchronize()
+        assert int(out.out_offsets[batch]) == batch * kept and not (out.Y[:batch * kept] == 77.0).any()
+    finally:
+        plan.close()
