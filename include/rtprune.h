@@ -304,12 +304,19 @@ rtprune_status_t rtprune_profile_read(rtprune_plan_t *plan, int32_t *n, float *m
  *   image_counts DEVICE [batch] uint32 scratch of the caller, written: edge pixels of each image
  *   edge_counts  DEVICE [batch][height/patch][width/patch] int32, written: edge pixels of each patch
  *                (rho_k = edge_counts / patch^2); may be NULL
- * Asynchronous on the stream (one memset, two kernels), allocates nothing.  Host-detectable errors
- * are returned before any launch.
+ * Asynchronous on the stream (three kernels), allocates nothing.  Host-detectable errors are returned
+ * before any launch.  There is no workspace and so no status word: an image for some of whose pixels a bounded
+ * device-side wait gave up gets rho = NaN and image_counts = UINT32_MAX, and its edge_counts mean nothing.
  */
 rtprune_status_t rtprune_density(void *cuda_stream, const uint8_t *images, int32_t batch, int32_t height,
                                  int32_t width, int32_t patch, float tau, float *rho,
                                  uint32_t *image_counts, int32_t *edge_counts);
+
+/* Test aid: rtprune_density whose waits give up at once, although the pixels are on their way: each CTA marks its
+ * image, waits its copy out with the default limit and leaves.  Every image comes back marked as above; nothing faults. */
+rtprune_status_t rtprune_test_density_expired(void *cuda_stream, const uint8_t *images, int32_t batch, int32_t height,
+                                              int32_t width, int32_t patch, float tau, float *rho,
+                                              uint32_t *image_counts, int32_t *edge_counts);
 
 /*
  * Test aid: makes the library's bounded device-side waits run out without any fault.  Launches one small

@@ -76,6 +76,7 @@ def lib() -> ctypes.CDLL:
     L.rtprune_host_arena_bytes.argtypes = [vp, ctypes.POINTER(sz)]
     L.rtprune_query_status.argtypes = [vp, vp, vp, ctypes.POINTER(ctypes.c_uint32)]
     L.rtprune_density.argtypes = [vp, vp, i32, i32, i32, i32, ctypes.c_float, vp, vp, vp]
+    L.rtprune_test_density_expired.argtypes = L.rtprune_density.argtypes
     L.rtprune_profile_enable.argtypes = [vp, i32]
     L.rtprune_profile_read.argtypes = [vp, ctypes.POINTER(i32), ctypes.POINTER(ctypes.c_float),
                                        ctypes.POINTER(ctypes.c_char_p)]

@@ -163,21 +163,26 @@ __device__ __noinline__ int dn_exact_pair(f32x2 gx, f32x2 gy, float T, unsigned 
     return corr;
 }
 
-// Zeroes the counters the tile kernel adds to (its grid dependency).
-__global__ void density_clear_kernel(uint32_t *__restrict__ image_counts, int batch, int32_t *__restrict__ edge_counts,
-                                     int patches)
+// Zeroes the counters the tile kernel adds to and the place of its marks (its grid dependency).
+__global__ void density_clear_kernel(uint32_t *__restrict__ image_counts, float *__restrict__ rho, int batch,
+                                     int32_t *__restrict__ edge_counts, int patches)
 {
     ptx::grid_dep_launch();
     const int n = blockDim.x * gridDim.x, i0 = blockIdx.x * blockDim.x + threadIdx.x;
-    for (int i = i0; i < batch; i += n) image_counts[i] = 0;
+    for (int i = i0; i < batch; i += n) {
+        image_counts[i] = 0;
+        rho[i] = 0.f;
+    }
     for (int i = i0; i < patches; i += n) edge_counts[i] = 0;
 }
 
 // grid = (segments of seg_w columns, bands of band_h rows, batch).  Launched as a programmatic dependent of
-// density_clear_kernel.
+// density_clear_kernel.  A CTA whose wait for its pixels runs out (poll_limit) marks its image's rho with NaN and waits
+// once more, with the full limit, for the copy that is on its way into its shared memory.
 __global__ void __launch_bounds__(kDnThreads, 4)
 density_tile_kernel(const __grid_constant__ CUtensorMap map, int H, int W, int p, int seg_w, int band_h,
-                    unsigned long long thr2, int32_t *__restrict__ edge_counts, uint32_t *__restrict__ image_counts)
+                    unsigned long long thr2, int32_t *__restrict__ edge_counts, uint32_t *__restrict__ image_counts,
+                    float *__restrict__ rho, uint32_t poll_limit)
 {
     extern __shared__ __align__(128) uint8_t tile[];
     __shared__ uint64_t s_full;
@@ -203,7 +208,12 @@ density_tile_kernel(const __grid_constant__ CUtensorMap map, int H, int W, int p
         ptx::mbar_arrive_expect_tx(&s_full, (uint32_t)((band_h + 2) * kDnRowPitch));
         ptx::tma_load_3d(ptx::smem_u32(tile), &map, &s_full, (3 * x0 - 16) / 4, y0 - 1, img);
     }
-    const bool landed = ptx::mbar_wait(&s_full, 0);
+    const bool landed = ptx::mbar_wait(&s_full, 0, poll_limit);
+    if (!landed) {
+        (void)ptx::mbar_wait(&s_full, 0);
+        ptx::grid_dep_wait();                         // (rho has been cleared)
+        rho[img] = __int_as_float(0x7fffffff);
+    }
     if (landed && kDnWalk * walk < bh && xt < sw) {
         const bool first_col = x0 + xt == 0, last_col = x0 + xt + 16 == W;
         const uint8_t *base = tile + kDnWalk * walk * kDnRowPitch + 16 + 3 * xt;
@@ -277,13 +287,15 @@ density_tile_kernel(const __grid_constant__ CUtensorMap map, int H, int W, int p
 }
 
 // rho = average over the patches of (edge pixels / patch pixels); the patches are equal, so this is the
-// image's edge pixels over its pixels.
-__global__ void density_finish_kernel(const uint32_t *__restrict__ image_counts, int batch, float inv_pixels,
+// image's edge pixels over its pixels.  A marked image (NaN) stays so and counts UINT32_MAX.
+__global__ void density_finish_kernel(uint32_t *__restrict__ image_counts, int batch, float inv_pixels,
                                       float *__restrict__ rho)
 {
     ptx::grid_dep_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < batch) rho[i] = (float)image_counts[i] * inv_pixels;
+    if (i >= batch) return;
+    if (isnan(rho[i])) image_counts[i] = 0xffffffffu;
+    else rho[i] = (float)image_counts[i] * inv_pixels;
 }
 
 // Launch that may begin while the kernel ahead of it in the stream drains (it waits for it itself).
@@ -326,13 +338,11 @@ static bool pages_map(CUtensorMap *map, const uint8_t *images, int batch, int H,
                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-}  // namespace rtp
-
-extern "C" rtprune_status_t rtprune_density(void *cuda_stream, const uint8_t *images, int32_t batch, int32_t height,
-                                            int32_t width, int32_t patch, float tau, float *rho,
-                                            uint32_t *image_counts, int32_t *edge_counts)
+// rtprune_density, the waits for pixels giving up after poll_limit polls.
+static rtprune_status_t launch_density(void *cuda_stream, const uint8_t *images, int32_t batch, int32_t height, int32_t width,
+                                       int32_t patch, float tau, float *rho, uint32_t *image_counts, int32_t *edge_counts,
+                                       uint32_t poll_limit)
 {
-    using namespace rtp;
     if (batch < 0 || height <= 0 || width <= 0) return RTPRUNE_ERR_INVALID_ARG;
     if (patch != 16 && patch != 32 && patch != 64) return RTPRUNE_ERR_UNSUPPORTED;
     if (height % patch || width % patch) return RTPRUNE_ERR_UNSUPPORTED;
@@ -355,7 +365,7 @@ extern "C" rtprune_status_t rtprune_density(void *cuda_stream, const uint8_t *im
     while (band_h > 16 && (long long)batch * nx * ((height + band_h - 1) / band_h) < 2 * 148) band_h >>= 1;
     const int patches = (edge_counts && band_h < patch) ? batch * (height / patch) * (width / patch) : 0;
     const int n_clear = std::max((int)batch, patches);
-    density_clear_kernel<<<std::min((n_clear + 255) / 256, 148), 256, 0, st>>>(image_counts, batch, edge_counts, patches);
+    density_clear_kernel<<<std::min((n_clear + 255) / 256, 148), 256, 0, st>>>(image_counts, rho, batch, edge_counts, patches);
     CUtensorMap map;
     if (!pages_map(&map, images, batch, height, width, band_h)) return RTPRUNE_ERR_CUDA;
     // the attribute is the function's, per device: set once on each (a bit of the mask)
@@ -371,10 +381,27 @@ extern "C" rtprune_status_t rtprune_density(void *cuda_stream, const uint8_t *im
     const dim3 threads((unsigned)(std::min(seg_w, (int)width) / 16), (unsigned)(band_h / kDnWalk));
     const dim3 grid((unsigned)nx, (unsigned)((height + band_h - 1) / band_h), (unsigned)batch);
     if (launch_dependent(density_tile_kernel, grid, threads, (size_t)kDnSmemBytes, st, map, height, width, patch,
-                         seg_w, band_h, thr2, edge_counts, image_counts) != cudaSuccess)
+                         seg_w, band_h, thr2, edge_counts, image_counts, rho, poll_limit) != cudaSuccess)
         return RTPRUNE_ERR_CUDA;
     if (launch_dependent(density_finish_kernel, dim3((unsigned)(batch + 255) / 256), dim3(256), (size_t)0, st,
-                         (const uint32_t *)image_counts, batch, 1.f / ((float)height * (float)width), rho) != cudaSuccess)
+                         image_counts, batch, 1.f / ((float)height * (float)width), rho) != cudaSuccess)
         return RTPRUNE_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? RTPRUNE_OK : RTPRUNE_ERR_CUDA;
+}
+
+}  // namespace rtp
+
+extern "C" rtprune_status_t rtprune_density(void *cuda_stream, const uint8_t *images, int32_t batch, int32_t height,
+                                            int32_t width, int32_t patch, float tau, float *rho,
+                                            uint32_t *image_counts, int32_t *edge_counts)
+{
+    return rtp::launch_density(cuda_stream, images, batch, height, width, patch, tau, rho, image_counts, edge_counts,
+                               rtp::ptx::kSpinLimit);
+}
+
+extern "C" rtprune_status_t rtprune_test_density_expired(void *cuda_stream, const uint8_t *images, int32_t batch,
+                                                         int32_t height, int32_t width, int32_t patch, float tau,
+                                                         float *rho, uint32_t *image_counts, int32_t *edge_counts)
+{
+    return rtp::launch_density(cuda_stream, images, batch, height, width, patch, tau, rho, image_counts, edge_counts, 0u);
 }

@@ -36,3 +36,20 @@ def test_gradients_next_to_the_threshold():
             tau = np.nextafter(tau, np.float32(10.0 if k > 0 else 0.0), dtype=np.float32)
         _, counts, _ = binding.density(torch.from_numpy(page).to(DEV), 64, float(tau))
         assert int(counts[0]) == (128 if float(g) ** 2 >= np.ceil((float(tau) * 255000.0) ** 2) else 0), k
+
+
+def test_a_wait_that_gives_up_marks_its_image():
+    # every CTA of every image gives up at once: no count may pass for a result
+    pages = torch.randint(0, 256, (3, 128, 320, 3), dtype=torch.uint8, device=DEV)
+    for patch in (16, 64):
+        rho = torch.zeros(3, device=DEV)
+        counts = torch.zeros(3, dtype=torch.int32, device=DEV)
+        per_patch = torch.zeros(3 * (128 // patch) * (320 // patch), dtype=torch.int32, device=DEV)
+        assert binding.lib().rtprune_test_density_expired(None, pages.data_ptr(), 3, 128, 320, patch, 0.2, rho.data_ptr(),
+                                                          counts.data_ptr(), per_patch.data_ptr()) == 0
+        torch.cuda.synchronize()
+        assert torch.isnan(rho).all() and (counts == -1).all()             # (UINT32_MAX)
+        rho, counts, per_patch = binding.density(pages, patch, 0.2, want_patch_counts=True)
+        _, ref = od.density_batch(pages.cpu().numpy(), patch, float(np.float32(0.2)))
+        np.testing.assert_array_equal(per_patch.cpu().numpy(), ref)
+        assert torch.isfinite(rho).all()
