@@ -350,6 +350,10 @@ rtprune_status_t rtprune_test_set_poll_limit(rtprune_plan_t *plan, int64_t polls
  */
 rtprune_status_t rtprune_test_fail_group(rtprune_plan_t *plan, int32_t group);
 
+/* Test aid: the plan's later runs behave as on a device that can run no cluster of the Sinkhorn kernel for tiles of 640 to
+ * 2047 pruned tokens (the kernels for wider tiles then take them). */
+rtprune_status_t rtprune_test_no_stream_clusters(rtprune_plan_t *plan);
+
 /* Kernels launched by the most recent run / select / run_host call on this plan. */
 int32_t rtprune_last_launch_count(const rtprune_plan_t *plan);
 

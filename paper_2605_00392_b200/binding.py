@@ -71,6 +71,7 @@ def lib() -> ctypes.CDLL:
     L.rtprune_test_expire_waits.argtypes = [vp, vp, vp, sz, ctypes.c_uint32, vp]
     L.rtprune_test_set_poll_limit.argtypes = [vp, ctypes.c_int64]
     L.rtprune_test_fail_group.argtypes = [vp, i32]
+    L.rtprune_test_no_stream_clusters.argtypes = [vp]
     L.rtprune_run_host.argtypes = [vp, vp, vp, vp, vp, i32, i64, pp, vp, sz,
                                    vp, vp, vp, vp, vp, vp, vp, vp]
     L.rtprune_host_arena_bytes.argtypes = [vp, ctypes.POINTER(sz)]
@@ -248,6 +249,10 @@ class Plan:
     def fail_group(self, group: int) -> None:
         """Test aid: run_host's group of images of this number fails before its launches (negative: none)."""
         _check(lib().rtprune_test_fail_group(self.handle, int(group)), "rtprune_test_fail_group")
+
+    def no_stream_clusters(self) -> None:
+        """Test aid: this plan's runs do without the Sinkhorn kernel for tiles of 640 to 2047 pruned tokens."""
+        _check(lib().rtprune_test_no_stream_clusters(self.handle), "rtprune_test_no_stream_clusters")
 
     # -- rtprune_host_arena_bytes / rtprune_run_host
     def host_arena_bytes(self) -> int:

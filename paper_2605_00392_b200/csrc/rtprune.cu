@@ -585,25 +585,25 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
         const size_t tall_smem = (size_t)std::max(plan->smem_optin - 1024, 0);
         // Up to kStMaxB columns: clusters that stream K from the workspace, of the size (2 to 16) that needs the least
         // time when a wave of images takes work / CTAs and a little for the exchanges
-        const bool stream = iterate && !use_log_form(params) && !all_fast && maxB <= kStMaxB;
-        if (stream) {
-            const int threads = st_threads(st_width(maxB));
-            int best = -1;
+        int stream_c = 0;                   // 0: not such a run, or the device runs no cluster of the kernel
+        const int stream_threads = st_threads(st_width(std::min(maxB, kStMaxB)));
+        if (iterate && !use_log_form(params) && !all_fast && maxB <= kStMaxB) {
             double least = 0.0;
             for (int cc = kStMaxC; cc >= 2; --cc) {
                 const int nc = plan->stream_clusters[cc];
                 const int rows = (maxN - kSrMaxB - 1 + cc - 1) / cc + 1;
-                if (nc < 1 || sizeof(float) * (size_t)st_min_floats(st_width(maxB), cc, rows, threads / 32) > tall_smem) continue;
+                if (nc < 1 || sizeof(float) * (size_t)st_min_floats(st_width(maxB), cc, rows, stream_threads / 32) > tall_smem) continue;
                 const double t = ((batch + nc - 1) / nc) * (1.0 / cc + 0.01);
-                if (best < 0 || t < least) {
-                    best = cc;
+                if (stream_c == 0 || t < least) {
+                    stream_c = cc;
                     least = t;
                 }
             }
-            if (best < 0) return RTPRUNE_ERR_CUDA;
-            if (!c.ok(launch_pdl(threads == 512 ? sinkhorn_stream_kernel<512> : sinkhorn_stream_kernel<256>,
-                                 dim3((unsigned)(batch * best)), dim3((unsigned)threads), tall_smem, st,
-                                 (unsigned)best, offsets, (const int32_t *)o.counts, (const int32_t *)o.out_offsets,
+        }
+        if (stream_c > 0) {
+            if (!c.ok(launch_pdl(stream_threads == 512 ? sinkhorn_stream_kernel<512> : sinkhorn_stream_kernel<256>,
+                                 dim3((unsigned)(batch * stream_c)), dim3((unsigned)stream_threads), tall_smem, st,
+                                 (unsigned)stream_c, offsets, (const int32_t *)o.counts, (const int32_t *)o.out_offsets,
                                  (const int32_t *)order, kmat, L.kmat_stride, maxN, total, op,
                                  (int)(tall_smem / sizeof(float)), pbuf, pbuf_pitch, o.merged_idx, o.merge_partner,
                                  o.merge_weight, o.stats, rows_max_b, (WsHeader *)(ws + L.header))))
@@ -611,9 +611,9 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             launched(plan, st, "sinkhorn_tall");
             all_fast = true;
         }
-        // Wider tiles: clusters of 8 CTAs iterate on K in the workspace tile with a block barrier per block of rows; the
-        // general kernel keeps only what is wider still.  It takes all the shared memory a CTA can have: what its
-        // fixed regions leave is the ring of row blocks.
+        // Wider tiles (any over kSrMaxB columns if the kernel that streams cannot run): clusters of 8 CTAs iterate on K in
+        // the workspace tile with a block barrier per block of rows; the general kernel keeps only what is wider still.  It
+        // takes all the shared memory a CTA can have: what its fixed regions leave is the ring of row blocks.
         const bool tall = iterate && !use_log_form(params) && !all_fast &&
                           sizeof(float) * (sinkhorn_tall_smem_floats(std::min(maxB, kTallMaxB), maxN) +
                                            kTallStageFloatsMax) <= tall_smem;
@@ -1223,6 +1223,13 @@ rtprune_status_t rtprune_test_fail_group(rtprune_plan_t *plan, int32_t group)
 {
     if (!plan) return RTPRUNE_ERR_INVALID_ARG;
     plan->fail_group = group < 0 ? -1 : group;
+    return RTPRUNE_OK;
+}
+
+rtprune_status_t rtprune_test_no_stream_clusters(rtprune_plan_t *plan)
+{
+    if (!plan) return RTPRUNE_ERR_INVALID_ARG;
+    std::fill(plan->stream_clusters, plan->stream_clusters + kStMaxC + 1, 0);
     return RTPRUNE_OK;
 }
 

@@ -25,3 +25,17 @@ def test_all_iterations_and_tolerance():
     a = parity.run_gpu(w, overrides=dict(stop_at_fixed_point=0)).out
     b = parity.run_gpu(w, overrides=dict(tol=1e-3)).out
     assert float(a.stats[0, 5]) == 100.0 and 1.0 <= float(b.stats[0, 5]) <= 5.0 and float(b.stats[0, 6]) <= 1e-3
+
+
+@pytest.mark.parametrize("lengths,d,dtype,r,iters", [([1400, 700, 30], 1280, torch.bfloat16, 0.5, 100), ([2137], 1280, torch.bfloat16, 0.4207, 100),
+                                                     ([1400] * 20, 64, torch.float32, 0.5, 30), ([3000, 4094], 64, torch.float32, 0.5, 6)])
+def test_without_a_cluster_of_the_kernel_the_one_for_wider_tiles_runs(lengths, d, dtype, r, iters):
+    import parity
+    from paper_2605_00392_b200 import binding
+    w = synth.ragged(lengths, d=d, dtype=dtype, params=dict(r_fixed=r, iters=iters))
+    plan = binding.Plan(w.d, w.X.dtype, w.batch, w.total_tokens, w.max_tokens)
+    try:
+        plan.no_stream_clusters()
+        parity.check_workload(w, plan=plan, images=list(range(min(len(lengths), 3))))
+    finally:
+        plan.close()
