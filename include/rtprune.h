@@ -109,14 +109,14 @@ typedef struct {
     float eps;            /* entropic regularisation: Z = S-bar / eps; > 0 (1 uses S-bar itself)     */
     int32_t iters;        /* Sinkhorn iterations T, >= 0 (paper: 100)                                */
     int32_t form;         /* rtprune_sinkhorn_form_t                                                 */
-    int32_t stop_at_fixed_point; /* 1: leave the loop once an iteration reproduces its input: the duals
-                             of the scaling form all within one unit in the last place of their
-                             previous values (bit-identical log-domain duals in the LOG form) -- later
-                             iterations could only move them within rounding, so the result is that
-                             of all `iters` iterations to fp32 accuracy.  (A dual that keeps cycling
-                             within four units also counts, from its third such iteration on; images with
-                             more than 639 pruned tokens: within four units, the rounding noise of their
-                             long sums.)
+    int32_t stop_at_fixed_point; /* 1: leave the loop once an iteration reproduces its input, whatever the
+                             batch size and storage type: every dual of the scaling form within one unit in
+                             the last place of its previous value, or in a cycle of rounding (within four
+                             units of it and back within one unit of the value before that; images with more
+                             than 639 pruned tokens: within four units, the rounding noise of their long
+                             sums); bit-identical log-domain duals in the LOG form.  Later iterations could
+                             only move them within rounding, so the result is that of all `iters`
+                             iterations to fp32 accuracy.
                              0: always run `iters`.                                                  */
     float tol;            /* > 0: also stop once no dual moved by more than tol (log units) in an
                              iteration.  0 (default): never stop on a tolerance.                    */

@@ -29,6 +29,7 @@
 #pragma once
 #include "common.cuh"
 #include "ptx.cuh"
+#include "settled.h"
 #include "sinkhorn.cuh"
 #include "sinkhorn_rows.cuh"
 
@@ -188,6 +189,7 @@ __device__ inline FuIterState fused_iterate(const float4 (&k)[NS][CPL / 4], floa
     const uint32_t xusum_peer = ptx::map_to_rank(ptx::smem_u32(&sh->xusum[0][0]), peer);
     const uint32_t xbar_peer = ptx::map_to_rank(ptx::smem_u32(&sh->xbar[0]), peer);
     FuIterState st{0, 0.f};
+    int before = 0;                                // the thread's column (the last thread: the dustbin's) two iterations ago
 
     for (int it = 0; it < p.iters; ++it, ++round) {
         const uint32_t par = round & 1u, phase = (round >> 1) & 1u;
@@ -259,8 +261,8 @@ __device__ inline FuIterState fused_iterate(const float4 (&k)[NS][CPL / 4], floa
         __syncthreads();
 
         // V: thread j completes column j over the warps, sends the sum to the other CTA, waits for that CTA's
-        int cont = 0;
         float move = 0.f;
+        int now = 0, last = 0;                     // the thread's dual before and after (none: nothing moves)
         if (tid < ldk) {
             float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
 #pragma unroll
@@ -280,9 +282,10 @@ __device__ inline FuIterState fused_iterate(const float4 (&k)[NS][CPL / 4], floa
             if (tid < B) {
                 nv = rcp_fast((cs + sh->xpart[par][tid]) + kappa * Ud);
                 const float ov = sh->vs[tid];
-                move = fabsf(nv - ov) * rcp_fast(ov);
-                cont = p.tol > 0.f ? (move > p.tol) : (p.stop_fp ? ulp_far(nv, ov) : 1);
                 sh->vs[tid] = nv;
+                move = fabsf(nv - ov) * rcp_fast(ov);
+                now = __float_as_int(nv);
+                last = __float_as_int(ov);
             }
         }
         if (tid == kFuThreads - 1) {              // the dustbin column
@@ -295,14 +298,16 @@ __device__ inline FuIterState fused_iterate(const float4 (&k)[NS][CPL / 4], floa
                 atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
             }
             const float nVd = Mf * rcp_fast(kappa * ((su + sh->xusum[par][0]) + Ud));
-            const float mj = fabsf(nVd - Vd) * rcp_fast(Vd);
-            move = fmaxf(move, mj);
-            cont |= p.tol > 0.f ? (mj > p.tol) : (p.stop_fp ? ulp_far(nVd, Vd) : 1);
+            move = fabsf(nVd - Vd) * rcp_fast(Vd);
+            now = __float_as_int(nVd);
+            last = __float_as_int(Vd);
             sh->vs[ldk] = nVd;
         }
+        const bool moves = p.tol > 0.f ? move > p.tol : !p.stop_fp || !dual_settled(now, last, before);
+        before = last;
         st.last_move = move;
         ++st.done;
-        if (!__syncthreads_or(cont)) {
+        if (!__syncthreads_or(moves)) {
             ++round;
             break;
         }

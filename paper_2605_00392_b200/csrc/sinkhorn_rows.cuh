@@ -31,6 +31,7 @@
 
 #include "common.cuh"
 #include "ptx.cuh"
+#include "settled.h"
 #include "sinkhorn.cuh"
 
 namespace rtp {
@@ -376,11 +377,11 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
     __syncthreads();                                   // K, V
     constexpr int kCols = (W + kSrThreads - 1) / kSrThreads;
     float nv[kCols], ov[kCols];                        // this thread's columns
-    int near[kCols];
+    int before[kCols];                                 // and their values two iterations ago
 #pragma unroll
     for (int e = 0; e < kCols; ++e) {
         nv[e] = ov[e] = tid + e * kSrThreads < t.B ? v_init : kappa * v_init;
-        near[e] = 0;
+        before[e] = 0;
     }
     SrState st{0, 0.f};
     Pass ps;
@@ -448,11 +449,9 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
                     ov[e] = nv[e];
                     nv[e] = (j < t.B ? 1.f : Mf) * rcp_fast(tot[e]);
                     t.vs[j] = nv[e];
-                    // settled: within a unit in the last place of the last value, or within four for the third time in
-                    // a row (sums of a few hundred terms may keep cycling by two or three units)
-                    const int d = abs(__float_as_int(nv[e]) - __float_as_int(ov[e]));
-                    near[e] = d <= 4 ? near[e] + 1 : 0;
-                    cont |= p.tol > 0.f ? (fabsf(nv[e] - ov[e]) > p.tol * ov[e]) : (!p.stop_fp || (d > 1 && near[e] < 3));
+                    cont |= p.tol > 0.f ? (fabsf(nv[e] - ov[e]) > p.tol * ov[e])
+                                        : (!p.stop_fp || !dual_settled(__float_as_int(nv[e]), __float_as_int(ov[e]), before[e]));
+                    before[e] = __float_as_int(ov[e]);
                 }
             }
         }

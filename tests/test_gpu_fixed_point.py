@@ -87,3 +87,35 @@ def test_exit_at_fixed_point_equals_all_iterations(binding, case):
         assert float((ya != yb).float().mean()) < 2e-3
     else:
         torch.testing.assert_close(ya, yb, rtol=1e-5, atol=1e-6)
+
+
+# Where the iterations are many (eps below 1) the exit saves most and is reached slowly.  Once every dual settles, an
+# iteration moves V and with it U by a unit in the last place at most, by four on images with more than 639 pruned tokens
+# (the recursion does not expand a move), so what the 100 - k iterations that were saved can change in a weight is
+# 2 (100 - k) such moves and the noise of its own factors.
+@pytest.mark.parametrize("lengths,dtype,d,r", [([400] * 6, torch.bfloat16, 1280, 0.3), ([256, 300] * 40, torch.bfloat16, 1280, 0.2),
+                                               ([1156, 456, 900], torch.bfloat16, 1280, 0.35), ([400, 256] * 4, torch.float32, 64, 0.25),
+                                               ([2137], torch.bfloat16, 1280, 0.4207)], ids=["reg", "rows", "rows_wide", "fp32", "stream"])
+@pytest.mark.parametrize("eps", [1.0, 0.3, 0.1, 0.05])
+def test_exit_at_small_eps(binding, lengths, dtype, d, r, eps):
+    dev = torch.device("cuda", 0)
+    w = synth.ragged(lengths, d=d, dtype=dtype, params=dict(r_fixed=r))
+    plan = binding.Plan(w.d, w.X.dtype, w.batch, w.total_tokens, w.max_tokens, device=dev)
+    plan.profile_enable(True)
+    try:
+        a, names = _run(binding, plan, w, dev, stop_at_fixed_point=1, eps=eps)
+        b, _ = _run(binding, plan, w, dev, stop_at_fixed_point=0, eps=eps)
+    finally:
+        plan.profile_enable(False)
+        plan.close()
+    nb = w.batch
+    k = a.stats[:nb, 5].cpu().numpy()
+    assert np.all(b.stats[:nb, 5].cpu().numpy() == 100.0) and k.min() >= 1.0
+    move, units = a.stats[:nb, 6].cpu().numpy(), 2.0 ** -23
+    step = 4 if float(a.stats[:nb, 4].max()) > 639 else 1
+    assert np.all(move[k < 100] <= 4 * units) and (eps < 0.3 or np.all(k < 100)), (k, move)
+    offs, kept = w.offsets.astype(np.int64), a.out_offsets.cpu().numpy().astype(np.int64)
+    wa, wb = a.merge_weight.cpu().numpy().astype(np.float64), b.merge_weight.cpu().numpy().astype(np.float64)
+    for i in range(nb):
+        s = slice(int(offs[i] - kept[i]), int(offs[i + 1] - kept[i + 1]))
+        assert np.all(np.abs(wa[s] - wb[s]) <= (2 * step * (100 - k[i]) + 16) * units * wb[s]), (i, k[i], np.max(np.abs(wa[s] / wb[s] - 1)) / units)
