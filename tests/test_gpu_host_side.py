@@ -1,5 +1,6 @@
 """Host-side behaviour of the library on a GPU: a bounded device-side wait that runs out is reported and leaves
 the context usable; function attributes set by one plan survive a later, smaller plan.  Marked gpu."""
+import numpy as np
 import pytest
 import torch
 
@@ -65,12 +66,20 @@ def test_smaller_plan_does_not_shrink_an_earlier_plans_kernels(parity, binding):
         plan_big.close()
 
 
-def test_two_slices_concatenate_to_the_one_call_result(binding):
+@pytest.mark.parametrize("batch,same_kernels", [(7, True), (16, False), (148, False)])
+def test_two_slices_concatenate_to_the_one_call_result(binding, batch, same_kernels):
     """What two ranks would do, on one GPU: each slice of the batch (the package's shard_slice) through a plan
     of its own, the second slice's offsets shifted by the first one's kept rows; the concatenation must equal
-    the one-call result bit for bit (counts, offsets, indices, pairs, Y)."""
+    the one-call result: counts, offsets and indices exactly; Y, pairs and weights bit for bit where slices and whole
+    take the same kernels in the same split (7 = 4 + 3 images), else to the rounding of sums in another order: the
+    scores of 16 images of 400 tokens are summed in one piece, those of 8 in four; 148 images are beyond the
+    register-resident Sinkhorn kernel's clusters, 74 are not."""
     dev = torch.device("cuda", 0)
-    w = synth.make("large", batch=7)                     # dynamic ratio, 4 + 3 images
+    w = synth.make("large", batch=min(batch, 16))        # dynamic ratio
+    if batch > 16:                                       # the same images again and again
+        reps = -(-batch // 16)
+        w = synth.Workload(**{**w.__dict__, "X": w.X.repeat(reps, 1)[:400 * batch], "rho": np.tile(w.rho, reps)[:batch],
+                              "offsets": (np.arange(batch + 1) * 400).astype(w.offsets.dtype)})
     fields = {k: (int(v) if k in ("dynamic", "iters") else float(v)) for k, v in w.params.items()}
 
     def run(X, offsets, rho):
@@ -89,23 +98,35 @@ def test_two_slices_concatenate_to_the_one_call_result(binding):
         (lo, hi), (row_lo, row_hi), local_offsets = binding.shard_slice(w.offsets, 2, rank)
         parts.append(((lo, hi), (row_lo, row_hi), run(w.X[row_lo:row_hi], local_offsets, w.rho[lo:hi])))
         kept_rows.append(int(parts[-1][2].out_offsets[hi - lo]))
-    assert parts[0][0] == (0, 4) and parts[1][0] == (4, 7)
-    nb = w.batch
-    total_kept = int(whole.out_offsets[nb])
+    first = (batch + 1) // 2
+    assert parts[0][0] == (0, first) and parts[1][0] == (first, batch)
+    total_kept = int(whole.out_offsets[batch])
     assert sum(kept_rows) == total_kept
     counts = torch.cat([p[2].counts[:p[0][1] - p[0][0]] for p in parts])
-    assert torch.equal(counts, whole.counts[:nb])
-    offs = torch.cat([parts[0][2].out_offsets[:4] + binding.packed_row_base(kept_rows, 0),
-                      parts[1][2].out_offsets[:4] + binding.packed_row_base(kept_rows, 1)])
-    assert torch.equal(offs, whole.out_offsets[:nb + 1])
-    Y = torch.cat([p[2].Y[:k] for p, k in zip(parts, kept_rows)])
-    assert torch.equal(Y, whole.Y[:total_kept])
+    assert torch.equal(counts, whole.counts[:batch])
+    offs = torch.cat([parts[0][2].out_offsets[:first] + binding.packed_row_base(kept_rows, 0),
+                      parts[1][2].out_offsets[:batch - first + 1] + binding.packed_row_base(kept_rows, 1)])
+    assert torch.equal(offs, whole.out_offsets[:batch + 1])
     kept_idx = torch.cat([p[2].kept_idx[:k] for p, k in zip(parts, kept_rows)])
     assert torch.equal(kept_idx, whole.kept_idx[:total_kept])
     pruned = [(p[1][1] - p[1][0]) - k for p, k in zip(parts, kept_rows)]
-    for name in ("merged_idx", "merge_partner"):
-        got = torch.cat([getattr(p[2], name)[:n] for p, n in zip(parts, pruned)])
-        assert torch.equal(got, getattr(whole, name)[:sum(pruned)]), name
+    got = {name: torch.cat([getattr(p[2], name)[:n] for p, n in zip(parts, pruned)])
+           for name in ("merged_idx", "merge_partner", "merge_weight")}
+    ref = {name: getattr(whole, name)[:sum(pruned)] for name in got}
+    assert torch.equal(got["merged_idx"], ref["merged_idx"])
+    Y, Y_ref = torch.cat([p[2].Y[:k] for p, k in zip(parts, kept_rows)]), whole.Y[:total_kept]
+    if same_kernels:
+        assert torch.equal(Y, Y_ref)
+        for name in got:
+            assert torch.equal(got[name], ref[name]), name
+    else:
+        # a rounding of the plan can tip an element of Y over to its bf16 neighbour, and a column whose largest entries lie
+        # within rounding of one another (background tokens are near-duplicates) to another partner: the entry it names is
+        # the largest to 1e-5 all the same, which the weights show
+        assert not (torch.equal(Y, Y_ref) and torch.equal(got["merge_weight"], ref["merge_weight"]))
+        y, yr = Y.float(), Y_ref.float()
+        assert ((y - yr).abs() <= 2.0 ** -7 * yr.abs() + 1e-6 * yr.abs().max()).all() and float((y != yr).float().mean()) < 1e-3
+        torch.testing.assert_close(got["merge_weight"], ref["merge_weight"], rtol=1e-5, atol=0)
 
 
 @pytest.mark.parametrize("name,batch", [("large", 16), ("base", 32), ("ragged", 6)])
@@ -115,7 +136,7 @@ def test_run_captured_into_a_cuda_graph_replays(binding, name, batch):
     bit for bit: the run number the kernels tell their hand-over lists by is counted on the device, not
     baked into the launches."""
     dev = torch.device("cuda", 0)
-    if name == "ragged":      # tiles of up to 578 pruned tokens: the cluster kernel's instance for wide tiles
+    if name == "ragged":      # tiles of up to 578 pruned tokens: sinkhorn_rows_wide
         sets = [synth.ragged([456, 1156, 700, 64, 300, 900], seed=40 + s, params=dict(r_fixed=0.5)) for s in range(3)]
     else:
         sets = [synth.make(name, seed_offset=s, batch=batch) for s in range(3)]
