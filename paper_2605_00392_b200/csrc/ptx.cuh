@@ -196,6 +196,15 @@ template <int N> __device__ inline void bulk_wait()
 __device__ inline void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ inline void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// 16 bytes of read-only global memory.  Volatile: a run of such loads stays a run, all in flight before the first use,
+// where the compiler is free to take __ldg loads one by one to save registers.
+__device__ inline uint4 ld_nc_v4(const uint4 *p)
+{
+    uint4 v;
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 // ---- thread-block clusters: ranks, distributed shared memory, cluster barrier ------------------------
 __device__ inline uint32_t cluster_ctarank()
 {

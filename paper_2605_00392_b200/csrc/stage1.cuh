@@ -685,7 +685,9 @@ stage1_kernel(const T *__restrict__ X, const int32_t *__restrict__ offsets, int 
 // Compact copy of T_prop for the tensor-core kernels (bf16 storage): image i's B pruned rows, in
 // ascending token order, at rows xp_row0(offsets[i], i) .., then rows of zeros up to a multiple of
 // 64 so that whole 64-row tiles can be fetched.  grid = (ceil(max rows / 8), batch), 128 threads:
-// a warp copies two rows, all loads of a row issued before the stores.
+// a warp copies two rows, all ten loads of a lane issued before the stores.  (As __ldg loads they were at the compiler's
+// mercy: with the fp32 kernels in the same translation unit it took them a few at a time, 40 registers instead of 62, and
+// 64 x 400 tokens 106.2 us instead of 105.3.)
 // ---------------------------------------------------------------------------------------------
 constexpr int kGpRows = 8;     // rows per CTA: four warps, two rows each
 __global__ void __launch_bounds__(128)
@@ -741,9 +743,9 @@ gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restri
 #pragma unroll
             for (int b = 0; b < 5; ++b) {
                 const int v = v0 + 32 * b;
-                t[a][b] = (src_row[a] >= 0 && v < nvec)
-                              ? __ldg(reinterpret_cast<const uint4 *>(Xb + (size_t)src_row[a] * d) + v)
-                              : make_uint4(0, 0, 0, 0);
+                t[a][b] = make_uint4(0, 0, 0, 0);
+                if (src_row[a] >= 0 && v < nvec)
+                    t[a][b] = ptx::ld_nc_v4(reinterpret_cast<const uint4 *>(Xb + (size_t)src_row[a] * d) + v);
             }
 #pragma unroll
         for (int a = 0; a < 2; ++a)
