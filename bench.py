@@ -223,7 +223,7 @@ LARGE_N = {   # token counts before -> after pruning of the OCR models with larg
 
 def run_large_n(args) -> None:
     """`--step largen`: the whole path on images of thousands of tokens (score tiles of 4 to 19 MB that
-    no cluster's shared memory holds: the Sinkhorn kernel for wide tiles).  One GPU; one JSON line with
+    no cluster's shared memory holds: the Sinkhorn kernel that streams them).  One GPU; one JSON line with
     one entry per shape."""
     print(json.dumps(large_n_line(args)), flush=True)
 
@@ -264,18 +264,19 @@ def large_n_line(args) -> dict:
         M, B, it = st[:, 3].astype(np.int64), st[:, 4].astype(np.int64), st[:, 5]
         avg = {k: float(np.mean(v)) for k, v in per_kernel.items()}
         ms_step = total_ms / steps
-        # the wide-tile Sinkhorn kernel must read K (M rows of pitch (B+4)&~3 floats) once per iteration
+        # the Sinkhorn kernel of these tiles must read K (M rows of pitch (B+4)&~3 floats) once per iteration
         k_bytes = float(np.sum(it * M * ((B + 4) & ~3) * 4))
-        tall_ms = avg.get("sinkhorn_tall", 0.0)
+        kernel = next((k for k in ("sinkhorn_stream", "sinkhorn_tall") if k in avg), None)
+        k_ms = avg.get(kernel, 0.0)
         path_bytes = w.total_tokens * w.d * 2 + int(M.sum()) * w.d * 2 + 12 * w.total_tokens
         shapes[name] = {
             "workload": "%d images x %d tokens x %d bf16, fixed r = %.4f (%d kept), T=100" % (batch, n, w.d, r, int(M[0])),
             "ms_per_step": ms_step, "images_per_s": batch / (ms_step / 1e3),
             "tokens_per_s": w.total_tokens / (ms_step / 1e3), "kernel_ms": avg,
             "mean_iterations_run": float(it.mean()), "max_iterations_run": float(it.max()),
-            "roofline": {"kernel": "sinkhorn_tall", "bound": "hbm", "achieved": k_bytes / (tall_ms / 1e3) / 1e9 if tall_ms else None,
-                         "peak": hbm_peak, "unit": "GB/s", "frac": k_bytes / (tall_ms / 1e3) / 1e9 / hbm_peak if tall_ms else None,
-                         "peak_source": peak_kind, "traffic": None, "avg_launch_ms": tall_ms,
+            "roofline": {"kernel": kernel, "bound": "hbm", "achieved": k_bytes / (k_ms / 1e3) / 1e9 if k_ms else None,
+                         "peak": hbm_peak, "unit": "GB/s", "frac": k_bytes / (k_ms / 1e3) / 1e9 / hbm_peak if k_ms else None,
+                         "peak_source": peak_kind, "traffic": None, "avg_launch_ms": k_ms,
                          "note": "bytes = executed iterations x the image's K tile; the tiles of a batch stay in L2 when they fit"},
             "path_roofline": {"bound": "hbm", "algorithmic_bytes": path_bytes,
                               "frac": path_bytes / (ms_step / 1e3) / 1e9 / hbm_peak},
@@ -647,8 +648,8 @@ def main() -> None:
             "stage1": ("hbm", x_bytes + total * 4 * 3 + batch * 48),
             "gather": ("hbm", 2 * xp_bytes),
             "scores": ("hbm", x_bytes + xp_bytes + 4 * sumMB),
-            "sinkhorn_cluster": ("alu", sink_flops),
-            "sinkhorn_wide": ("alu", sink_flops),
+            "sinkhorn_rows": ("alu", sink_flops),
+            "sinkhorn_rows_wide": ("alu", sink_flops),
             "sinkhorn_reg": ("alu", sink_flops),
             "sinkhorn": ("alu", sink_flops),
             "merge": ("hbm", x_bytes + y_bytes + sumM * 4),

@@ -558,8 +558,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             };
             const long long limit = plan->fast_smem_bytes / (int)sizeof(float);
             const long long cells = (long long)(maxN - std::min(mb, maxN / 2)) * std::min(mb, maxN / 2);
-            const bool spare = 2LL * batch <= plan->sm_count;
-            const int spread = spare ? 10000 : 40000;
+            const int spread = 2LL * batch <= plan->sm_count ? 10000 : 40000;
             int cc = 1;
             while (cc < kSrMaxC && floats(cc) > limit) cc *= 2;
             while (cc < kSrMaxC && (long long)batch * cc * 2 <= plan->sm_count && cells > (long long)spread * cc) cc *= 2;
@@ -577,9 +576,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                                  pbuf, pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight, o.stats,
                                  (uint32_t *)(ws + L.sink_done), ready_list, (WsHeader *)(ws + L.header), sd, split, by_image)))
                 return RTPRUNE_ERR_CUDA;
-            // the name in a profile says what the launch was for: the instance for wide tiles, or whole images of more
-            // than 32 768 cells on one CTA in a batch that fills the device; else the common case
-            launched(plan, st, mb > 255 || (!spare && cells > 32768LL * cc) ? "sinkhorn_wide" : "sinkhorn_cluster");
+            launched(plan, st, mb > 255 ? "sinkhorn_rows_wide" : "sinkhorn_rows");
         }
         // Scaling form, tiles left (more than kSrMaxB columns)
         const size_t tall_smem = (size_t)std::max(plan->smem_optin - 1024, 0);
@@ -608,7 +605,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                                  (int)(tall_smem / sizeof(float)), pbuf, pbuf_pitch, o.merged_idx, o.merge_partner,
                                  o.merge_weight, o.stats, rows_max_b, (WsHeader *)(ws + L.header))))
                 return RTPRUNE_ERR_CUDA;
-            launched(plan, st, "sinkhorn_tall");
+            launched(plan, st, "sinkhorn_stream");
             all_fast = true;
         }
         // Wider tiles (any over kSrMaxB columns if the kernel that streams cannot run): clusters of 8 CTAs iterate on K in

@@ -105,12 +105,12 @@ def test_large_tile_leaves_shared_memory(parity):
 
 
 def test_tile_wider_than_the_cluster_kernel_takes(parity):
-    # N = 1400 at r = 0.5: 700 pruned tokens, more than the 640 columns the cluster kernels cover, so
-    # this image is solved by the kernel for wide tiles (clusters of 8 CTAs, K iterated in the workspace)
-    # while the other two are solved by the two instances of the cluster kernel in the same run
+    # N = 1400 at r = 0.5: 700 pruned tokens, more than the 639 columns sinkhorn_rows covers, so this image is
+    # solved by the kernel that streams K from the workspace while the other two are solved by sinkhorn_rows_wide
+    # in the same run
     w = synth.ragged([1400, 300, 1000], params=dict(r_fixed=0.5))
     rep = parity.check_workload(w)
-    assert rep["launches"] == 6      # stage1, gather, scores, sinkhorn_wide, sinkhorn_tall, merge
+    assert rep["launches"] == 6      # stage1, gather, scores, sinkhorn_rows_wide, sinkhorn_stream, merge
 
 
 def test_exact_ties_keep_lower_index(parity):
@@ -284,8 +284,8 @@ def test_many_runs_in_bursts_reproduce_bit_for_bit(binding, name, batch, bursts)
     # without a synchronisation, on inputs that alternate, must each reproduce the first result of
     # their input bit for bit: a kernel that reads a counter left by the run before shows up here (the
     # small batch leaves SMs free for dependents to become resident early).  The ragged batch and the batch
-    # of 160 images take the cluster kernel's instance for wide tiles, which then also feeds the merge
-    # kernel image by image (clusters of 4 and single CTAs, the largest tiles iterating in the workspace).
+    # of 160 images take sinkhorn_rows_wide and sinkhorn_rows, which then also feed the merge
+    # kernel image by image (clusters and single CTAs, the largest tiles in part in the workspace).
     dev = torch.device("cuda", 0)
     sets = [synth.make(name, seed_offset=s, batch=batch) for s in range(3)]
     w0 = sets[0]

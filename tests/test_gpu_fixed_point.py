@@ -39,18 +39,20 @@ def _run(binding, plan, w, dev, **over):
 CASES = [
     # register-resident K, clusters of two: 200 x 200, the largest tile of a 400-token image
     ("reg", [400] * 6, torch.bfloat16, 1280, 0.5, {}, "sinkhorn_reg", 2e-6),
-    # more images than clusters of the register kernel fit at once: the shared-memory cluster kernel
-    ("cluster", [400] * 80, torch.bfloat16, 1280, 0.25, {}, "sinkhorn_cluster", 2e-6),
-    # the same batch at the ratio cap: 200 x 200 tiles no longer fit one CTA each, the instance for wide tiles takes them
-    ("cluster_at_cap", [400] * 80, torch.bfloat16, 1280, 0.5, {}, "sinkhorn_wide", 2e-6),
-    # 578 columns (more than 256): the cluster kernel's instance for wide tiles, K in the workspace
-    ("wide", [1156, 1156, 900], torch.bfloat16, 1280, 0.5, {}, "sinkhorn_wide", 2e-6),
-    # 1729 columns: clusters of 8 or 16 CTAs iterate on K in the workspace (exit within 4 ulp: long sums)
-    ("tall", [4512], torch.bfloat16, 1280, 0.3832, {}, "sinkhorn_tall", 2e-5),
+    # more images than clusters of the register kernel fit at once: rows over warps, a CTA per image
+    ("rows", [400] * 80, torch.bfloat16, 1280, 0.25, {}, "sinkhorn_rows", 2e-6),
+    # the same batch at the ratio cap: 200 x 200 tiles no longer fit one CTA's shared memory, two CTAs per image
+    ("rows_at_cap", [400] * 80, torch.bfloat16, 1280, 0.5, {}, "sinkhorn_rows", 2e-6),
+    # 578 columns (more than 255): the instance for wide tiles, eight CTAs per image
+    ("rows_wide", [1156, 1156, 900], torch.bfloat16, 1280, 0.5, {}, "sinkhorn_rows_wide", 2e-6),
+    # 1729 columns: warps stream rows of K from the workspace (exit within 4 units: long sums)
+    ("stream", [4512], torch.bfloat16, 1280, 0.3832, {}, "sinkhorn_stream", 2e-5),
+    # 2256 columns, beyond that kernel: clusters of 8 or 16 CTAs iterate on K in the workspace (exit within 4 units)
+    ("tall", [4512], torch.bfloat16, 1280, 0.5, {}, "sinkhorn_tall", 2e-5),
     # log-domain form, one CTA per image (exit when the duals repeat bit for bit)
     ("log", [400, 256], torch.bfloat16, 1280, 0.5, dict(form=1), "sinkhorn", 2e-5),
-    # fp32 storage takes the cluster kernel with the plan written in place
-    ("fp32", [400] * 4, torch.float32, 64, 0.5, {}, "sinkhorn_cluster", 2e-6),
+    # fp32 storage: rows over warps, the plan written in place
+    ("fp32", [400] * 4, torch.float32, 64, 0.5, {}, "sinkhorn_rows", 2e-6),
 ]
 
 
@@ -93,11 +95,14 @@ def test_exit_at_fixed_point_equals_all_iterations(binding, case):
 # iteration moves V and with it U by a unit in the last place at most, by four on images with more than 639 pruned tokens
 # (the recursion does not expand a move), so what the 100 - k iterations that were saved can change in a weight is
 # 2 (100 - k) such moves and the noise of its own factors.
-@pytest.mark.parametrize("lengths,dtype,d,r", [([400] * 6, torch.bfloat16, 1280, 0.3), ([256, 300] * 40, torch.bfloat16, 1280, 0.2),
-                                               ([1156, 456, 900], torch.bfloat16, 1280, 0.35), ([400, 256] * 4, torch.float32, 64, 0.25),
-                                               ([2137], torch.bfloat16, 1280, 0.4207)], ids=["reg", "rows", "rows_wide", "fp32", "stream"])
+@pytest.mark.parametrize("lengths,dtype,d,r,kernel", [([400] * 6, torch.bfloat16, 1280, 0.3, "sinkhorn_reg"),
+                                                      ([256, 300] * 40, torch.bfloat16, 1280, 0.2, "sinkhorn_rows"),
+                                                      ([1156, 456, 900], torch.bfloat16, 1280, 0.35, "sinkhorn_rows_wide"),
+                                                      ([400, 256] * 4, torch.float32, 64, 0.25, "sinkhorn_rows"),
+                                                      ([2137], torch.bfloat16, 1280, 0.4207, "sinkhorn_stream"),
+                                                      ([4512], torch.bfloat16, 1280, 0.5, "sinkhorn_tall")])
 @pytest.mark.parametrize("eps", [1.0, 0.3, 0.1, 0.05])
-def test_exit_at_small_eps(binding, lengths, dtype, d, r, eps):
+def test_exit_at_small_eps(binding, lengths, dtype, d, r, kernel, eps):
     dev = torch.device("cuda", 0)
     w = synth.ragged(lengths, d=d, dtype=dtype, params=dict(r_fixed=r))
     plan = binding.Plan(w.d, w.X.dtype, w.batch, w.total_tokens, w.max_tokens, device=dev)
@@ -108,6 +113,7 @@ def test_exit_at_small_eps(binding, lengths, dtype, d, r, eps):
     finally:
         plan.profile_enable(False)
         plan.close()
+    assert kernel in names, names
     nb = w.batch
     k = a.stats[:nb, 5].cpu().numpy()
     assert np.all(b.stats[:nb, 5].cpu().numpy() == 100.0) and k.min() >= 1.0

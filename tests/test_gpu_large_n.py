@@ -1,7 +1,7 @@
 """Parity on images with thousands of visual tokens (the token counts of the OCR models with large
 visual token sets in the paper's cross-model table: 2137 -> 1238 and 4512 -> 2783 tokens), whose
-score tiles are far wider than one CTA's or one cluster's shared memory: the Sinkhorn kernel for wide
-tiles iterates on K in the workspace with a cluster of 8 CTAs per image."""
+score tiles are far wider than one CTA's or one cluster's shared memory: two Sinkhorn kernels iterate on K in the
+workspace with a cluster of CTAs per image, sinkhorn_stream (640 to 2047 pruned tokens) and sinkhorn_tall (up to 4092)."""
 import numpy as np
 import pytest
 import torch
@@ -29,16 +29,24 @@ def _names(plan):
 
 def test_2137_tokens_to_1238(parity):
     # r = 1 - 1238 / 2137: B = 899 pruned tokens, a 1238 x 899 tile (4.4 MB); the second image is solved by
-    # the cluster kernel in the same run
+    # sinkhorn_rows_wide in the same run
     w = synth.ragged([2137, 700], params=dict(r_fixed=0.4207))
     rep = parity.check_workload(w)
-    assert rep["launches"] == 6      # stage1, gather, scores, sinkhorn_wide, sinkhorn_tall, merge
+    assert rep["launches"] == 6      # stage1, gather, scores, sinkhorn_rows_wide, sinkhorn_stream, merge
 
 
 def test_4512_tokens_to_2783(parity):
-    # B = 1729: one 16-byte chunk per thread over all 512 threads of a row group
+    # B = 1729: a 2783 x 1729 tile (19.3 MB)
     w = synth.ragged([4512], params=dict(r_fixed=0.3832))
     parity.check_workload(w)
+
+
+def test_4512_tokens_to_half(parity):
+    # B = 2256, wider than sinkhorn_stream takes: sinkhorn_tall, two 16-byte chunks per thread; beside it an image for each
+    # of the other kernels' widths (sinkhorn_tall takes the one of 1000 columns too)
+    w = synth.ragged([4512, 700, 2000], params=dict(r_fixed=0.5))
+    rep = parity.check_workload(w)
+    assert rep["launches"] == 6      # stage1, gather, scores, sinkhorn_rows_wide, sinkhorn_tall, merge
 
 
 def test_two_chunks_per_thread_and_fp32_storage(parity):
@@ -50,8 +58,8 @@ def test_two_chunks_per_thread_and_fp32_storage(parity):
     parity.check_workload(w)
 
 
-def test_many_images_with_narrow_wide_tiles_take_clusters_of_four(parity):
-    # 20 images whose clusters of 8 would not all run at once, tiles of 700 columns: clusters of 4 CTAs
+def test_many_images_with_narrow_wide_tiles(parity):
+    # 20 images whose clusters of 8 would not all run at once, tiles of 700 columns: smaller clusters
     w = synth.ragged([1400] * 20, d=64, dtype=torch.float32, params=dict(r_fixed=0.5, iters=30))
     parity.check_workload(w)
     w = synth.ragged([1400] * 19 + [700], params=dict(r_fixed=0.5))
@@ -65,18 +73,22 @@ def test_single_kept_row_leaves_seven_ctas_without_rows(parity):
 
 
 def test_largest_image_goes_to_the_general_kernel(parity):
-    # N = 8192, the plan's limit, with more than 4092 pruned tokens: wider than the wide-tile kernel takes
+    # N = 8192, the plan's limit, with more than 4092 pruned tokens: wider than sinkhorn_tall takes
     w = synth.ragged([8192], d=64, dtype=torch.float32, params=dict(r_fixed=0.55, iters=8))
     rep = parity.check_workload(w)
-    assert rep["launches"] == 6      # stage1, scores, sinkhorn_wide, sinkhorn_tall (leaves it), sinkhorn, merge
+    assert rep["launches"] == 6      # stage1, scores, sinkhorn_rows_wide, sinkhorn_tall (leaves it), sinkhorn, merge
 
 
-def test_wide_tile_runs_reproduce_bit_for_bit(parity, binding):
+@pytest.mark.parametrize("lengths,r,kernel", [([2137, 1500], 0.45, "sinkhorn_stream"), ([4512, 1500], 0.5, "sinkhorn_tall")])
+def test_wide_tile_runs_reproduce_bit_for_bit(parity, binding, lengths, r, kernel):
     dev = torch.device("cuda", 0)
-    w = synth.ragged([2137, 1500], params=dict(r_fixed=0.45))
+    w = synth.ragged(lengths, params=dict(r_fixed=r))
     plan = binding.Plan(w.d, w.X.dtype, w.batch, w.total_tokens, w.max_tokens, device=dev)
     a = parity.run_gpu(w, plan=plan).out
+    plan.profile_enable(True)
     b = parity.run_gpu(w, plan=plan).out
+    assert kernel in _names(plan)
+    plan.profile_enable(False)
     n = int(a.out_offsets[w.batch])                  # rows of Y and entries of kept_idx that are written
     nb = w.total_tokens - n
     assert torch.equal(a.out_offsets, b.out_offsets) and torch.equal(a.counts, b.counts)
@@ -89,7 +101,7 @@ def test_wide_tile_runs_reproduce_bit_for_bit(parity, binding):
 
 
 def test_wide_tile_fixed_point_stop_equals_all_iterations(parity):
-    # leaving the loop once no dual moves by more than one unit in the last place gives the result of all
+    # leaving the loop once no dual moves by more than four units in the last place gives the result of all
     # T = 100 iterations to fp32 accuracy
     w = synth.ragged([2137], params=dict(r_fixed=0.4207))
     a = parity.run_gpu(w, overrides=dict(stop_at_fixed_point=1)).out
