@@ -15,13 +15,12 @@ struct OtParams {
 
 constexpr int kSinkThreads = 512;
 
-// Row pitch (floats) of K in the fused stage-2 kernel and the register kernel (fused.cuh): the widths their lane layouts
-// cover.
+// Row pitch (floats) of K in the fused stage-2 kernel and the register kernel (fused.cuh), at most 256 columns: the widths
+// their lane layouts cover.
 __host__ __device__ inline int sinkhorn_ldk(int B)
 {
     if (B <= 128) return B <= 32 ? 32 : (B <= 64 ? 64 : 128);
-    if (B <= 256) return B <= 192 ? 192 : 256;
-    return B <= 384 ? 384 : (B <= 512 ? 512 : 640);
+    return B <= 192 ? 192 : 256;
 }
 
 // True if two positive floats differ by more than one unit in the last place.

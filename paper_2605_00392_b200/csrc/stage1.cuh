@@ -166,40 +166,35 @@ __device__ inline void select_image(int img, int t_begin, int N, int d, int chun
     // pass over the keys, no histogram, and it needs neither phi nor M.  A warp's 32 tokens are consecutive, so only
     // against one another do ties look at the index.
     const bool by_rank = N <= kRankMax;
-    constexpr int kOwn = kRankMax / nth;
-    int rank[kOwn];
+    int rank = 0;                                  // (a token per thread)
     if (by_rank) {
         for (int k = N + tid; k < ((N + 31) & ~31); k += nth) s_keys[k] = 0u;       // (only ever compared past N)
         __syncthreads();
         const uint4 *k4 = reinterpret_cast<const uint4 *>(s_keys);
-#pragma unroll
-        for (int q = 0; q < kOwn; ++q) {
-            rank[q] = 0;
-            const int base = 32 * warp + q * nth;
-            if (base < N) {
-                const uint32_t key = s_keys[base + lane];
-                int ahead[4] = {0, 0, 0, 0};
-                for (int j = 0; j < base >> 2; ++j) {
-                    const uint4 o = k4[j];
-                    ahead[0] += o.x >= key;
-                    ahead[1] += o.y >= key;
-                    ahead[2] += o.z >= key;
-                    ahead[3] += o.w >= key;
-                }
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const uint32_t o = __shfl_sync(0xffffffffu, key, j);
-                    ahead[j & 3] += (base + j < N) && (o > key || (o == key && j < lane));
-                }
-                for (int j = (base >> 2) + 8; j < (N + 3) >> 2; ++j) {               // (zeros past N are never larger)
-                    const uint4 o = k4[j];
-                    ahead[0] += o.x > key;
-                    ahead[1] += o.y > key;
-                    ahead[2] += o.z > key;
-                    ahead[3] += o.w > key;
-                }
-                rank[q] = (ahead[0] + ahead[1]) + (ahead[2] + ahead[3]);
+        const int base = 32 * warp;
+        if (base < N) {
+            const uint32_t key = s_keys[base + lane];
+            int ahead[4] = {0, 0, 0, 0};
+            for (int j = 0; j < base >> 2; ++j) {
+                const uint4 o = k4[j];
+                ahead[0] += o.x >= key;
+                ahead[1] += o.y >= key;
+                ahead[2] += o.z >= key;
+                ahead[3] += o.w >= key;
             }
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const uint32_t o = __shfl_sync(0xffffffffu, key, j);
+                ahead[j & 3] += (base + j < N) && (o > key || (o == key && j < lane));
+            }
+            for (int j = (base >> 2) + 8; j < (N + 3) >> 2; ++j) {               // (zeros past N are never larger)
+                const uint4 o = k4[j];
+                ahead[0] += o.x > key;
+                ahead[1] += o.y > key;
+                ahead[2] += o.z > key;
+                ahead[3] += o.w > key;
+            }
+            rank = (ahead[0] + ahead[1]) + (ahead[2] + ahead[3]);
         }
     }
     const float ssum = block_sum(local, s_redf);
@@ -236,15 +231,10 @@ __device__ inline void select_image(int img, int t_begin, int N, int d, int chun
     if (by_rank) {
         // positions of the kept tokens in ascending index: over the warp's 32 tokens by ballot, over the groups of 32
         // (in s_hist) by a warp's scan
-        uint32_t mask[kOwn];
-#pragma unroll
-        for (int q = 0; q < kOwn; ++q) {
-            const int k = tid + q * nth;
-            mask[q] = __ballot_sync(0xffffffffu, k < N && rank[q] < M);
-            if (lane == 0) s_hist[q * kS1Warps + warp] = __popc(mask[q]);
-        }
+        const uint32_t mask = __ballot_sync(0xffffffffu, tid < N && rank < M);
+        if (lane == 0) s_hist[warp] = __popc(mask);
         __syncthreads();
-        const int c = lane < kOwn * kS1Warps ? s_hist[lane] : 0;
+        const int c = lane < kS1Warps ? s_hist[lane] : 0;
         int before = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -252,17 +242,13 @@ __device__ inline void select_image(int img, int t_begin, int N, int d, int chun
             if (lane >= o) before += u;
         }
         before -= c;
-#pragma unroll
-        for (int q = 0; q < kOwn; ++q) {
-            const int k = tid + q * nth;
-            const int run = __shfl_sync(0xffffffffu, before, q * kS1Warps + warp) + __popc(mask[q] & ((1u << lane) - 1u));
-            if (k < N) {
-                const bool kept = (mask[q] >> lane) & 1u;
-                const int pos = kept ? run : M + (k - run);
-                ord[pos] = k;
-                kpos[t_begin + k] = kept ? run : -1 - (k - run);
-                if (order_out) order_out[t_begin + pos] = k;
-            }
+        const int run = __shfl_sync(0xffffffffu, before, warp) + __popc(mask & ((1u << lane) - 1u));
+        if (tid < N) {
+            const bool kept = (mask >> lane) & 1u;
+            const int pos = kept ? run : M + (tid - run);
+            ord[pos] = tid;
+            kpos[t_begin + tid] = kept ? run : -1 - (tid - run);
+            if (order_out) order_out[t_begin + pos] = tid;
         }
         __syncthreads();
         return;

@@ -36,6 +36,10 @@ def test_without_a_cluster_of_the_kernel_the_one_for_wider_tiles_runs(lengths, d
     plan = binding.Plan(w.d, w.X.dtype, w.batch, w.total_tokens, w.max_tokens)
     try:
         plan.no_stream_clusters()
+        plan.profile_enable(True)
         parity.check_workload(w, plan=plan, images=list(range(min(len(lengths), 3))))
+        names = [n for n, _ in plan.profile_read()]
+        assert "sinkhorn_tall" in names and "sinkhorn_stream" not in names
+        plan.profile_enable(False)
     finally:
         plan.close()
