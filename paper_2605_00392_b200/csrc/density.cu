@@ -355,6 +355,9 @@ static rtprune_status_t launch_density(void *cuda_stream, const uint8_t *images,
     const double t2 = std::ceil(t * t);
     const unsigned long long thr2 = t2 >= 1.8e19 ? ~0ull : (unsigned long long)t2;
     if (batch > 65535 || (height + kDnBand - 1) / kDnBand > 65535) return RTPRUNE_ERR_UNSUPPORTED;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return RTPRUNE_ERR_CUDA;
     // columns: equal segments, multiples of 64 (whole patches)
     const int nseg = (width + kDnSeg - 1) / kDnSeg;
     const int seg_w = std::min(kDnSeg, ((width + nseg - 1) / nseg + 63) / 64 * 64);
@@ -362,16 +365,14 @@ static rtprune_status_t launch_density(void *cuda_stream, const uint8_t *images,
     // rows: bands of 64; of 16 when those would leave half the device idle (the two extra rows of a band then cost
     // an eighth instead of a thirty-second)
     int band_h = kDnBand;
-    while (band_h > 16 && (long long)batch * nx * ((height + band_h - 1) / band_h) < 2 * 148) band_h >>= 1;
+    while (band_h > 16 && (long long)batch * nx * ((height + band_h - 1) / band_h) < 2LL * sms) band_h >>= 1;
     const int patches = (edge_counts && band_h < patch) ? batch * (height / patch) * (width / patch) : 0;
     const int n_clear = std::max((int)batch, patches);
-    density_clear_kernel<<<std::min((n_clear + 255) / 256, 148), 256, 0, st>>>(image_counts, rho, batch, edge_counts, patches);
+    density_clear_kernel<<<std::min((n_clear + 255) / 256, sms), 256, 0, st>>>(image_counts, rho, batch, edge_counts, patches);
     CUtensorMap map;
     if (!pages_map(&map, images, batch, height, width, band_h)) return RTPRUNE_ERR_CUDA;
     // the attribute is the function's, per device: set once on each (a bit of the mask)
     static std::atomic<unsigned long long> attribute_set{0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return RTPRUNE_ERR_CUDA;
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(attribute_set.load(std::memory_order_relaxed) & bit)) {
         if (cudaFuncSetAttribute(density_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDnSmemBytes) != cudaSuccess)
