@@ -36,8 +36,8 @@ FP32_FMA_PEAK_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12   # SMs x FP32 lanes x 2 f
 REFERENCE_SAMPLE = 64      # images per step of the --impl reference arm: the whole Large batch, as cpu_baseline
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from an ncu capture (profiles/), by kernel
 # (kernels changed since their capture, or never captured, have no entry and report null)
-NCU_TRAFFIC_BYTES = {"stage1": 66078208, "gather": 10355200, "scores": 87525888, "sinkhorn_reg": 4935424,
-                     "merge": 118104064, "density_tile": None}
+NCU_TRAFFIC_BYTES = {"stage1": 65876224, "gather": 10372864, "scores": 86270720, "sinkhorn_reg": 4948992,
+                     "merge": 117271040, "density_tile": 318164992}
 
 
 def cpu_threads() -> int:
@@ -194,7 +194,7 @@ def density_line(args) -> dict:
     nbytes = batch * H * W * 3
     line = {"metric": "pages/sec (textual density)", "value": batch / ms * 1e3, "unit": "images/s", "n_gpus": 1,
             "steps": args.steps, "warmup": warm, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": "u8 -> int64 (exact)", "data": "synthetic",
+            "vs_baseline": None, "dtype": "u8 -> fp32, int64 near the threshold (exact)", "data": "synthetic",
             "config": {"workload": "density: 64 pages x 1280 x 1280 x RGB8, patch 64, tau 0.2",
                        "l2": "pages rotate over 2 buffer sets (629 MB > L2)"},
             "roofline": {"kernel": "density_tile", "bound": "hbm", "achieved": nbytes / ms / 1e6, "peak": hbm_peak,

@@ -22,10 +22,10 @@
 // image is decided per image (sr_ctas): an exchange costs about as much as a pass over 20 000 cells.
 //
 // What bounds it: shared-memory reads of K and instruction latency; on a 300 x 100 tile on one CTA an iteration is
-// 4200 cycles (pass 3000, column sums, V and two barriers the rest).  Measured on the kernel alone, against the kernel
-// before it (16 warps walking rows one by one, a cluster barrier per iteration): 128 images of 456-1156 tokens
-// 240 -> 141 us, 1024 x 400 at r = 0.25 284 -> 213 us, 256 x 400 in fp32 storage 124 -> 70 us, 64 images of 456-1156
-// tokens at eps = 0.1 (25 iterations) 972 -> 348 us.
+// 4200 cycles (pass 3000, column sums, V and two barriers the rest).  Measured by events around the kernel, against the
+// kernel before it (16 warps walking rows one by one, a cluster barrier per iteration): 128 images of 456-1156 tokens
+// 209 -> 149 us, 1024 x 400 at r = 0.25 288 -> 243 us, 256 x 400 in fp32 storage 119 -> 78 us, 64 images of 456-1156
+// tokens at eps = 0.1 (31 iterations on average) 834 -> 475 us.
 #pragma once
 #include <type_traits>
 

@@ -1,7 +1,8 @@
 // Dustbin-augmented optimal transport by Sinkhorn iterations (Eq. 5, Appendix C) in scaling form for
-// score tiles too wide for the kernel of sinkhorn_rows.cuh: images with many tokens (thousands
-// per image, as the OCR models with large visual token sets produce), up to 4092 pruned tokens.  One
-// cluster of 8 CTAs per image (16 when the batch is small enough to leave SMs idle otherwise); the tile's rows (kept tokens) are split over the CTAs; K =
+// score tiles too wide for the kernels of sinkhorn_rows.cuh and sinkhorn_stream.cuh: images with many tokens (thousands
+// per image, as the OCR models with large visual token sets produce), up to 4092 pruned tokens; narrower ones of the same
+// run, or of a device that runs no cluster of the streaming kernel, from 640 up.  One cluster of 8 CTAs per image (16 when
+// the batch is small enough to leave SMs idle otherwise); the tile's rows (kept tokens) are split over the CTAs; K =
 // exp((S - c)/eps) is built in place in the image's workspace tile and read once per iteration
 // through L2: a CTA's rows are contiguous there, so one thread streams them block by block into a ring
 // of shared-memory stages with 1-D bulk copies, a few blocks ahead of the threads (the tile does not
@@ -533,7 +534,7 @@ __device__ inline void sinkhorn_tall_solve(float *Kg, int ldS, int M, int B, int
     }
 }
 
-// grid = batch * 8 CTAs, clusters of 8 along x.  Takes the images that the kernel ahead of it
+// grid = batch * C CTAs, clusters of C (8 or 16) along x.  Takes the images that the kernel ahead of it
 // left (those with B > rows_max_b) and whose B <= kTallMaxB; every
 // early return depends on the image only, so a cluster leaves as a whole.
 __global__ void __launch_bounds__(kTallThreads, 1)

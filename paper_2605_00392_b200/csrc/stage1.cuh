@@ -672,8 +672,8 @@ stage1_kernel(const T *__restrict__ X, const int32_t *__restrict__ offsets, int 
 // ascending token order, at rows xp_row0(offsets[i], i) .., then rows of zeros up to a multiple of
 // 64 so that whole 64-row tiles can be fetched.  grid = (ceil(max rows / 8), batch), 128 threads:
 // a warp copies two rows, all ten loads of a lane issued before the stores.  (As __ldg loads they were at the compiler's
-// mercy: with the fp32 kernels in the same translation unit it took them a few at a time, 40 registers instead of 62, and
-// 64 x 400 tokens 106.2 us instead of 105.3.)
+// mercy: with the fp32 kernels in the same translation unit it took them a few at a time, in 40 registers, and 64 x 400
+// tokens 106.2 us instead of 105.3.)
 // ---------------------------------------------------------------------------------------------
 constexpr int kGpRows = 8;     // rows per CTA: four warps, two rows each
 __global__ void __launch_bounds__(128)
