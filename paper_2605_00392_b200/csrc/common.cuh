@@ -123,6 +123,20 @@ __device__ inline float warp_max(float x)
     return x;
 }
 
+// Smallest and largest value over a warp, in one instruction each (a NaN counts as no value).
+__device__ inline float warp_min_redux(float x)
+{
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ inline float warp_max_redux(float x)
+{
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // Sum over a CTA; `red` is shared scratch of at least 32 floats; every thread gets the result.
 __device__ inline float block_sum(float x, float *red)
 {

@@ -77,6 +77,7 @@ struct FuShared {
     int out0;
     float vsum[kFuWarps];
     float wsum[kFuWarps];
+    float2 range[kFuWarps];                     // smallest and largest relative move of a warp's columns
     __align__(16) float xusum[2][4];            // the other CTA's sum of U, by iteration parity
     __align__(16) float inv_nj[kFuMaxB];        // 1 / |x_j| of the pruned tokens
     __align__(16) float inv_ni[kFuMaxRows];     // 1 / |x_i| of this CTA's kept rows
@@ -261,7 +262,7 @@ __device__ inline FuIterState fused_iterate(const float4 (&k)[NS][CPL / 4], floa
         __syncthreads();
 
         // V: thread j completes column j over the warps, sends the sum to the other CTA, waits for that CTA's
-        float move = 0.f;
+        float move = 0.f, lo = INFINITY, hi = -INFINITY;
         int now = 0, last = 0;                     // the thread's dual before and after (none: nothing moves)
         if (tid < ldk) {
             float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
@@ -283,7 +284,8 @@ __device__ inline FuIterState fused_iterate(const float4 (&k)[NS][CPL / 4], floa
                 nv = rcp_fast((cs + sh->xpart[par][tid]) + kappa * Ud);
                 const float ov = sh->vs[tid];
                 sh->vs[tid] = nv;
-                move = fabsf(nv - ov) * rcp_fast(ov);
+                lo = hi = (nv - ov) * rcp_fast(ov);
+                move = fabsf(lo);
                 now = __float_as_int(nv);
                 last = __float_as_int(ov);
             }
@@ -298,29 +300,28 @@ __device__ inline FuIterState fused_iterate(const float4 (&k)[NS][CPL / 4], floa
                 atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
             }
             const float nVd = Mf * rcp_fast(kappa * ((su + sh->xusum[par][0]) + Ud));
-            move = fabsf(nVd - Vd) * rcp_fast(Vd);
+            lo = hi = (nVd - Vd) * rcp_fast(Vd);
+            move = fabsf(lo);
             now = __float_as_int(nVd);
             last = __float_as_int(Vd);
             sh->vs[ldk] = nVd;
         }
         const bool moves = p.tol > 0.f ? move > p.tol : !p.stop_fp || !dual_settled(now, last, before);
         before = last;
-        st.last_move = move;
+        lo = warp_min_redux(lo);
+        hi = warp_max_redux(hi);
+        if (lane == 0) sh->range[warp] = make_float2(lo, hi);
         ++st.done;
-        if (!__syncthreads_or(moves)) {
+        const int go = __syncthreads_or(moves);
+        const float2 range = sh->range[lane % kFuWarps];       // (written again after the next iteration's first barrier)
+        lo = warp_min_redux(range.x);
+        hi = warp_max_redux(range.y);
+        st.last_move = 0.5f * (hi - lo);
+        if (!go || (p.tol == 0.f && p.stop_fp && plan_settled(lo, hi))) {
             ++round;
             break;
         }
     }
-    // largest relative dual move of the last executed iteration, over the CTA
-    float mv = warp_max(st.last_move);
-    __syncthreads();
-    if (lane == 0) sh->wsum[warp] = mv;
-    __syncthreads();
-    mv = 0.f;
-#pragma unroll
-    for (int w = 0; w < kFuWarps; ++w) mv = fmaxf(mv, sh->wsum[w]);
-    st.last_move = mv;
     return st;
 }
 

@@ -369,7 +369,7 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
     constexpr int W = Pass::W, BR = Pass::BR;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float Mf = (float)t.M;
-    __shared__ float s_move[kSrWarps];
+    __shared__ float2 s_range[kSrWarps];               // smallest and largest relative move of a warp's columns
     for (int j = tid; j < W; j += kSrThreads) t.vs[j] = j < t.B ? v_init : (j == t.B ? kappa * v_init : 0.f);
     const int nbatch = (t.Mr + BR - 1) / BR, nsmem = min(nbatch, t.cap / BR);
     const int nwarps = min(kSrWarps, nbatch);          // warps with rows; the others' column sums stay zero
@@ -431,6 +431,7 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
 
         // V: a thread completes a column (or two) over the warps and the CTAs
         int cont = 0;
+        float lo = INFINITY, hi = -INFINITY;
         if (tid <= t.B) {
             float tot[kCols];
 #pragma unroll
@@ -449,25 +450,26 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
                     ov[e] = nv[e];
                     nv[e] = (j < t.B ? 1.f : Mf) * rcp_fast(tot[e]);
                     t.vs[j] = nv[e];
+                    const float rel = (nv[e] - ov[e]) * rcp_fast(ov[e]);
+                    lo = fminf(lo, rel);
+                    hi = fmaxf(hi, rel);
                     cont |= p.tol > 0.f ? (fabsf(nv[e] - ov[e]) > p.tol * ov[e])
                                         : (!p.stop_fp || !dual_settled(__float_as_int(nv[e]), __float_as_int(ov[e]), before[e]));
                     before[e] = __float_as_int(ov[e]);
                 }
             }
         }
+        lo = warp_min_redux(lo);
+        hi = warp_max_redux(hi);
+        if (lane == 0) s_range[warp] = make_float2(lo, hi);
         ++st.done;
-        if (!__syncthreads_or(cont)) break;
+        const int go = __syncthreads_or(cont);
+        const float2 range = s_range[lane % kSrWarps];         // (written again after the next iteration's first barrier)
+        lo = warp_min_redux(range.x);
+        hi = warp_max_redux(range.y);
+        st.last_move = 0.5f * (hi - lo);
+        if (!go || (p.tol == 0.f && p.stop_fp && plan_settled(lo, hi))) break;
     }
-    // largest relative dual move of the last executed iteration, over the CTA
-#pragma unroll
-    for (int e = 0; e < kCols; ++e)
-        if (tid + e * kSrThreads <= t.B && st.done > 0) st.last_move = fmaxf(st.last_move, fabsf(nv[e] - ov[e]) / ov[e]);
-    const float mv = warp_max(st.last_move);
-    if (lane == 0) s_move[warp] = mv;
-    __syncthreads();
-    st.last_move = 0.f;
-#pragma unroll
-    for (int w = 0; w < kSrWarps; ++w) st.last_move = fmaxf(st.last_move, s_move[w]);
     return st;
 }
 
