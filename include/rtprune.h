@@ -128,8 +128,7 @@ typedef struct {
 /* Number of floats per image in the `stats` output. */
 #define RTPRUNE_STATS_STRIDE 8
 /* stats[i*8 + ..]: 0 phi, 1 rho, 2 r, 3 M (kept), 4 B (pruned), 5 Sinkhorn iterations executed,
- *                  6 largest dual change of the last executed iteration (log units; images with at most 639 pruned
- *                  tokens in the scaling form: a common factor of all V aside), 7 reserved */
+ *                  6 largest dual change of the last executed iteration (log units), 7 reserved */
 
 /* Bits of the device status word (rtprune_query_status). */
 #define RTPRUNE_DEV_NONFINITE 1u

@@ -42,7 +42,7 @@ struct WsLayout {
     size_t xp;         // bf16 [total + 64 batch][d] compact copy of the pruned tokens (bf16 mode): image
                        //                          i's B rows start at row xp_row0(offsets[i], i), followed
                        //                          by zero rows up to a multiple of 64
-    size_t pbuf;       // bf16 [total][pbuf_pitch] plan rows for the tensor-core merge (bf16 mode)
+    size_t pbuf;       // bf16 [total][pbuf_pitch] alpha P (bf16 mode): row = offset + position among the kept
     int pbuf_pitch_max;  // elements; a run uses round_up(its largest possible B, 64) <= this
     size_t total;      // bytes
     int chunks;        // chunks per image = ceil(max_tokens_per_image / kChunkTokens)

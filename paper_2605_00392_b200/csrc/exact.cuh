@@ -274,18 +274,18 @@ exact_pairing_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
     }
 
     if (pbuf) {
-        // alpha P in bf16: rows by the kept token's position in X, columns up to the next multiple of 64
+        // alpha P in bf16: rows by position among the kept tokens, columns up to the next multiple of 64
         const int kpad = (B + 63) & ~63;
         const int vec_per_row = kpad >> 3;
         __nv_bfloat16 *Pimg = pbuf + (size_t)t_begin * pbuf_pitch;
         for (int idx = tid; idx < M * vec_per_row; idx += kExThreads) {
             const int i = idx / vec_per_row, q = idx - i * vec_per_row;
-            *reinterpret_cast<uint4 *>(Pimg + (size_t)ord[i] * pbuf_pitch + 8 * q) = make_uint4(0u, 0u, 0u, 0u);
+            *reinterpret_cast<uint4 *>(Pimg + (size_t)i * pbuf_pitch + 8 * q) = make_uint4(0u, 0u, 0u, 0u);
         }
         __syncthreads();
         const __nv_bfloat16 a = __float2bfloat16_rn(prm.alpha);
         for (int j = tid; j < B; j += kExThreads)
-            if (match[j] >= 0) Pimg[(size_t)ord[match[j]] * pbuf_pitch + j] = a;
+            if (match[j] >= 0) Pimg[(size_t)match[j] * pbuf_pitch + j] = a;
     } else {
         // fp32: the plan in place of the scores in the workspace tile (every read of S is behind the barrier above)
         for (int idx = tid; idx < M * B; idx += kExThreads) {

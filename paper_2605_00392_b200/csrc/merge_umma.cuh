@@ -1,29 +1,33 @@
 // Merge + pack (Eq. 7 and the output of Algorithm 1): Y = T_k + alpha * P T_p, written packed, on the
-// tcgen05 tensor cores (bf16 inputs, fp32 accumulation in TMEM), every operand fetched by tiled TMA.
+// tcgen05 tensor cores (bf16 inputs, fp32 accumulation in TMEM).
 //
-// A work unit is (image, tile of 128 CONSECUTIVE tokens, tile of 256 output columns).  The kept
-// token's own row enters through the tensor cores too: the contraction of a unit is
-//     D = [ I_128 | alpha P_tok ] . [ T_v rows of the token tile ; T_p ]
-// so the accumulator already holds T_k + alpha P T_p (1.0 x bf16 is exact in the fp32 accumulator) and
-// the epilogue reads no global memory.  Rows of pruned tokens are computed and dropped.
-//   * A operand: two constant identity tiles (built once in shared memory), then the plan rows
-//     alpha P[token][0..B) in bf16, K-major, from the plan buffer whose rows are token positions.
-//   * B operand, MN-major (row = contraction index, 64-column slabs of 128 bytes, 128-byte swizzle):
-//     the token tile's rows of X (k-blocks 0, 1), then the image's pruned rows from the compact copy,
-//     whose zero rows pad B to a multiple of 64.
+// A work unit is (image, tile of 128 consecutive KEPT tokens, tile of 256 output columns).  The contraction
+// is alpha P . T_p; the kept tokens' own rows join in the epilogue, in fp32.
+//   * A operand: the plan rows alpha P[p][0..B) in bf16, K-major, by tiled TMA from the plan buffer, whose
+//     rows are positions among the kept tokens.
+//   * B operand: the image's pruned rows from the compact copy by tiled TMA, MN-major (row = contraction
+//     index, 64-column slabs of 128 bytes, 128-byte swizzle); its zero rows pad B to a multiple of 64.
 //   * D: two 128-lane x 256-column fp32 accumulators in TMEM, so that the epilogue of one unit
 //     overlaps the loads and UMMAs of the next.
+//   * The kept tokens' rows: gathered from X by token index with 16-byte cp.async, coalesced, half a unit's
+//     columns at a time into a tile; a thread of the epilogue adds its row's accumulator in place, then its warp
+//     stores the rows, coalesced.
+// What bounds it is what an SM takes in through TMA (about 31 bytes per clock), so nothing comes that way that
+// need not: tiles of kept rows instead of token tiles with their pruned rows (a quarter of a corpus image, two
+// fifths of a long one), own rows by another path instead of as UMMA operands against an identity tile.
+// Against token tiles with own rows through the tensor cores (event times): 1024 x 400 at r = 0.25 426 -> 344 us,
+// 128 images of 456-1156 tokens 141 -> 113, 16 x 2137 133 -> 71, 8 x 4512 223 -> 111, 64 x 400 39 -> 37; 1014 images of 69
+// tokens 90 -> 102 (half-empty tiles: too few own rows in flight).
 // The kernel is persistent: CTA c takes units c, c + gridDim.x, ...  When the Sinkhorn kernel ahead
 // publishes a list of finished images, the units follow that list (its s-th entry takes the place of
 // image s), the CTAs draw them from a counter, and the scheduler waits, bounded, for the entry it
 // needs: the kernel is launched as a programmatic dependent and merges the first images on whatever
-// SMs are free while the last ones still iterate.  Warp roles (224 threads):
-// warps 0-3 epilogue (TMEM -> registers -> bf16 -> own row of a padded staging tile -> one bulk store
-// per kept row); warp 4 issues the TMA loads (the loads of a k-block from several lanes at once); warp 5 owns TMEM and
+// SMs are free while the last ones still iterate.  Warp roles (480 threads):
+// warps 0-7 epilogue (two warpgroups, one for each half of a unit's columns); warp 8 issues the TMA loads (the loads of a k-block from several lanes at once); warp 9 owns TMEM and
 // its lane 0 issues the UMMAs;
-// warp 6 lane 0 is the scheduler: it draws the units, looks up what the other roles need to know about
+// warp 10 lane 0 is the scheduler: it draws the units, looks up what the other roles need to know about
 // them (a chain of dependent loads from L2) a few units ahead and hands them over through a small queue
-// in shared memory.
+// in shared memory; warps 11-14 fetch the kept tokens' rows.
 #pragma once
 #include "common.cuh"
 #include "ptx.cuh"
@@ -33,28 +37,34 @@ namespace rtp {
 constexpr int kMgTileM = 128;
 constexpr int kMgTileN = 256;        // output columns per unit
 constexpr int kMgBK = 64;            // contraction rows per k-block
-constexpr int kMgBStages = 3;        // ring of B tiles (every k-block)
-constexpr int kMgAStages = 2;        // ring of plan tiles (k-blocks after the identity ones)
-constexpr int kMgThreads = 224;
+constexpr int kMgLoaders = 128;      // threads that fetch the kept tokens' rows
+constexpr int kMgEpilogue = 256;
+constexpr int kMgThreads = kMgEpilogue + 96 + kMgLoaders;
 constexpr int kMgLookahead = 1;       // units the scheduler may be ahead of the producer
 constexpr int kMgABytes = kMgTileM * 128;            // A tile: 128 rows x 64 bf16
 constexpr int kMgBBytes = kMgBK * kMgTileN * 2;      // B tile: 64 rows x 256 bf16 = 32 KB
 constexpr int kMgBBoxBytes = kMgBK * 128;            // one 64-column slab of it
-// I_128 as two 128 x 64 K-major views of [64 zero rows][I_64][64 zero rows]: the view that starts at
-// the I_64 block has its ones in rows 0-63, the view that starts 64 rows earlier in rows 64-127.
-constexpr int kMgIdentBytes = 3 * (kMgABytes / 2);
-constexpr int kMgIdentKb = 2;                        // k-blocks that carry the token tile's own rows (one, if
-                                                     // the image ends within the tile's first 64 rows)
-constexpr int kMgStagePitch = kMgTileN * 2 + 16;     // bytes per staging row: padded, conflict-free
-constexpr int kMgStagingBytes = kMgTileM * kMgStagePitch;
-constexpr int kMgSmemBytes = kMgBStages * kMgBBytes + kMgAStages * kMgABytes + kMgIdentBytes +
-                             kMgStagingBytes + 1024 /*alignment*/ + 1024 /*barriers, unit queue*/;
+constexpr int kMgStageBytes = kMgABytes + kMgBBytes; // a k-block: a plan tile and a tile of pruned rows
+constexpr int kMgOwnCols = 128;                      // columns of a tile of own rows: 256 bytes a row, the 16-byte pieces
+constexpr int kMgOwnBytes = kMgTileM * kMgOwnCols * 2;   // of row r at places xor (r & 7), conflict-free either way
+// Shared memory is shared out between k-blocks in flight and tiles of own rows by what a unit has of each: two k-blocks (B up to
+// 128) to two tiles of own rows, or many k-blocks.
+constexpr int kMgMaxStages = 3, kMgMaxBufs = 4;
+constexpr int kMgDeepB = 256;
+__host__ __device__ constexpr int merge_smem_bytes(int stages, int bufs)
+{
+    return stages * kMgStageBytes + bufs * kMgOwnBytes + 1024 /*alignment*/ + 1024 /*barriers, unit queue*/;
+}
+constexpr int kMgSmemMax = merge_smem_bytes(2, 4) > merge_smem_bytes(3, 2) ? merge_smem_bytes(2, 4) : merge_smem_bytes(3, 2);
+static_assert(kMgSmemMax <= 227 * 1024, "one CTA per SM");
 
 constexpr int kMgQueue = 16;         // ring of units between the producer and the other roles (about 6 in flight)
 
 struct MergeBarriers {
-    uint64_t full[kMgBStages];       // B tile (and, for plan k-blocks, the A tile) of a k-block has landed
-    uint64_t empty[kMgBStages];      // the k-block's UMMAs have read them
+    uint64_t full[kMgMaxStages];        // a k-block's tiles have landed
+    uint64_t empty[kMgMaxStages];       // its UMMAs have read them
+    uint64_t own_full[kMgMaxBufs];   // the kept tokens' rows are there
+    uint64_t own_empty[kMgMaxBufs];  // their sums have been stored
     uint64_t accum_full[2];
     uint64_t accum_empty[2];
     uint32_t tmem_base;
@@ -65,7 +75,6 @@ struct MergeBarriers {
 struct MergeUnit {
     int img, mt, ct;
     int t_begin, N, M, B, out0;
-    int nident;       // identity k-blocks: 64-row blocks of the tile that hold tokens of the image
     bool valid;
     bool timed_out;   // the image's list entry never came
 };
@@ -127,52 +136,43 @@ __device__ inline MergeUnit merge_unit(int u, int mtiles, int nct, const int32_t
     const int m_img = __ldcg(counts + q.img), out0 = __ldcg(out_offsets + q.img);
     q.t_begin = o_lo;
     q.N = o_hi - o_lo;
-    q.valid = q.N >= 1 && q.N <= max_tokens && o_lo >= 0 && o_hi <= total && q.mt * kMgTileM < q.N;
+    q.valid = q.N >= 1 && q.N <= max_tokens && o_lo >= 0 && o_hi <= total && q.mt * kMgTileM < m_img;
     q.M = q.valid ? m_img : 0;
     q.B = q.N - q.M;
     q.out0 = q.valid ? out0 : 0;
-    q.nident = (q.N - q.mt * kMgTileM <= kMgBK) ? 1 : kMgIdentKb;
     return q;
 }
 
 __global__ void __launch_bounds__(kMgThreads, 1)
-merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_constant__ CUtensorMap tmapXp,
-                  const __grid_constant__ CUtensorMap tmapP, const int32_t *__restrict__ offsets, int d,
+merge_umma_kernel(const __grid_constant__ CUtensorMap tmapXp, const __grid_constant__ CUtensorMap tmapP,
+                  const __nv_bfloat16 *__restrict__ X, const int32_t *__restrict__ offsets, int d,
                   int batch, int mtiles, const int32_t *__restrict__ counts,
-                  const int32_t *__restrict__ out_offsets, const int32_t *__restrict__ kpos,
+                  const int32_t *__restrict__ out_offsets, const int32_t *__restrict__ order,
                   int max_tokens, int total, __nv_bfloat16 *__restrict__ Y, int32_t *__restrict__ kept_idx,
-                  WsHeader *__restrict__ hdr, const int32_t *ready_list, int by_image)
+                  WsHeader *__restrict__ hdr, const int32_t *ready_list, int by_image, int stages, int bufs)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t *a_ring = smem + kMgBStages * kMgBBytes;
-    uint8_t *ident = a_ring + kMgAStages * kMgABytes;
-    uint8_t *staging = ident + kMgIdentBytes;
-    MergeBarriers *bars = reinterpret_cast<MergeBarriers *>(staging + kMgStagingBytes);
-    MergeQueue *mq = reinterpret_cast<MergeQueue *>(staging + kMgStagingBytes + 256);
+    uint8_t *own = smem + stages * kMgStageBytes;
+    MergeBarriers *bars = reinterpret_cast<MergeBarriers *>(own + bufs * kMgOwnBytes);
+    MergeQueue *mq = reinterpret_cast<MergeQueue *>(own + bufs * kMgOwnBytes + 256);
+    static_assert(sizeof(MergeBarriers) <= 256 && sizeof(MergeQueue) <= 768, "");
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nct = (d + kMgTileN - 1) / kMgTileN;
     const int nunits = batch * mtiles * nct;
 
-    // identity block: rows 64 .. 127 of the 192-row region hold I_64 (ones at (64 + r, k = r)), in the
-    // swizzled K-major layout; the other rows are zero
-    for (int v = tid; v < kMgIdentBytes / 16; v += kMgThreads)
-        reinterpret_cast<uint4 *>(ident)[v] = make_uint4(0, 0, 0, 0);
-    __syncthreads();
-    if (tid < 64) {
-        const int r = 64 + tid, k = tid;
-        const uint32_t off = (r >> 3) * 1024 + (r & 7) * 128 + (((k >> 3) ^ (r & 7)) << 4) + (k & 7) * 2;
-        *reinterpret_cast<uint16_t *>(ident + off) = 0x3F80;   // bf16 1.0
-    }
-    ptx::fence_proxy_async_smem();
     if (tid == 0) {
-        for (int s = 0; s < kMgBStages; ++s) {
+        for (int s = 0; s < stages; ++s) {
             ptx::mbar_init(&bars->full[s], 1);
             ptx::mbar_init(&bars->empty[s], 1);
         }
+        for (int b = 0; b < bufs; ++b) {
+            ptx::mbar_init(&bars->own_full[b], kMgLoaders);
+            ptx::mbar_init(&bars->own_empty[b], 128);
+        }
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(&bars->accum_full[b], 1);
-            ptx::mbar_init(&bars->accum_empty[b], 128);
+            ptx::mbar_init(&bars->accum_empty[b], kMgEpilogue);
         }
         bars->abort_flag = 0;
         mq->head = 0;
@@ -180,7 +180,7 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
         mq->tail = 0;
         ptx::fence_mbar_init();
     }
-    if (warp == 5) {
+    if (warp == 9) {
         ptx::tmem_alloc(&bars->tmem_base, 512);
         ptx::tmem_relinquish();
     }
@@ -195,78 +195,58 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
     ptx::grid_dep_launch();
     if (!ready_list) ptx::grid_dep_wait();
 
-    if (warp == 4) {
-        // ---------------- producer: tiled TMA for every operand -------------------------------------
+    if (warp == 8) {
+        // ---------------- producer: tiled TMA for both operands -------------------------------------
         // The whole warp walks the units and k-blocks in step (every lane takes the same waits); the loads of a
         // k-block are issued by as many lanes at once, one load each (lanes 0-3: the 64-column slabs of the B
         // tile, lane 4: the plan tile): one thread issuing them one after the other spent about 145 cycles in
         // each issue, 40 % of the kernel's time.
-        {
-            if (lane == 0) {
-                ptx::prefetch_tensormap(&tmapX);
-                ptx::prefetch_tensormap(&tmapXp);
-                ptx::prefetch_tensormap(&tmapP);
+        if (lane == 0) {
+            ptx::prefetch_tensormap(&tmapXp);
+            ptx::prefetch_tensormap(&tmapP);
+        }
+        int s = 0;                                    // place in the ring of k-blocks, and its phase
+        uint32_t phase = 1;                           // (the first wait on each place returns at once)
+        bool alive = true;
+        for (uint32_t n = 0; alive && !bars->abort_flag; ++n) {
+            MergeUnit q;
+            const bool got = merge_pop(mq, bars, n, q);
+            if (!__all_sync(0xffffffffu, got)) {
+                bars->abort_flag = 1;
+                if (lane == 0) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
+                break;
             }
-            // `it` counts k-blocks (B ring), `ia` plan k-blocks (A ring).  a_user[slot] is the k-block that
-            // last read the A slot: its UMMAs must have finished before the slot is refilled.
-            uint32_t it = 0, ia = 0;
-            uint32_t a_user[kMgAStages];
-            for (int s = 0; s < kMgAStages; ++s) a_user[s] = 0xffffffffu;
-            bool alive = true;
-            for (uint32_t n = 0; alive && !bars->abort_flag; ++n) {
-                MergeUnit q;
-                const bool got = merge_pop(mq, bars, n, q);
-                if (!__all_sync(0xffffffffu, got)) {
+            if (q.img < 0) break;
+            __syncwarp();                             // every lane has read the entry before it may be reused
+            if (lane == 0) mq->prod = n + 1;
+            if (ready_list) ptx::fence_proxy_async_all();   // the plan was written with ordinary stores
+            const int nkb = (q.B + kMgBK - 1) / kMgBK;
+            const int row0 = q.t_begin + q.mt * kMgTileM;
+            const int xp0 = xp_row0(q.t_begin, q.img);
+            const int col0 = q.ct * kMgTileN;
+            const int nslab = min(kMgTileN, d - col0 + 63) / 64;   // 64-column slabs with any column < d
+            for (int kb = 0; kb < nkb; ++kb) {
+                const bool ok = ptx::mbar_wait(&bars->empty[s], phase);
+                if (!__all_sync(0xffffffffu, ok)) {
                     bars->abort_flag = 1;
                     if (lane == 0) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
+                    alive = false;
                     break;
                 }
-                if (q.img < 0) break;
-                __syncwarp();                         // every lane has read the entry before it may be reused
-                if (lane == 0) mq->prod = n + 1;
-                if (ready_list) ptx::fence_proxy_async_all();   // the plan was written with ordinary stores
-                const int nkb = q.nident + (q.B + kMgBK - 1) / kMgBK;
-                const int row0 = q.t_begin + q.mt * kMgTileM;
-                const int xp0 = xp_row0(q.t_begin, q.img);
-                const int col0 = q.ct * kMgTileN;
-                const int nslab = min(kMgTileN, d - col0 + 63) / 64;   // 64-column slabs with any column < d
-                for (int kb = 0; kb < nkb; ++kb, ++it) {
-                    const int s = it % kMgBStages;
-                    bool ok = it < (uint32_t)kMgBStages || ptx::mbar_wait(&bars->empty[s], ((it / kMgBStages) - 1) & 1);
-                    const uint32_t b_dst = smem_base + s * kMgBBytes;
-                    const bool own = kb < q.nident;         // the token tile's own rows: A is the identity
-                    int sa = 0;
-                    if (!own) {
-                        sa = ia % kMgAStages;
-                        const uint32_t prev = a_user[sa];
-                        // k-blocks up to it - kMgBStages are known to be done (the wait above); a younger
-                        // reader of this A slot is the latest user of its B slot: wait for that phase
-                        if (ok && prev != 0xffffffffu && prev + kMgBStages > it)
-                            ok = ptx::mbar_wait(&bars->empty[prev % kMgBStages], (prev / kMgBStages) & 1);
-                        a_user[sa] = it;
-                        ++ia;
-                    }
-                    if (!__all_sync(0xffffffffu, ok)) {
-                        bars->abort_flag = 1;
-                        if (lane == 0) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
-                        alive = false;
-                        break;
-                    }
-                    if (lane == 0)
-                        ptx::mbar_arrive_expect_tx(&bars->full[s], (own ? 0 : kMgABytes) + nslab * kMgBBoxBytes);
-                    __syncwarp();
-                    if (lane < nslab) {
-                        const CUtensorMap *bm = own ? &tmapX : &tmapXp;
-                        const int brow = own ? row0 + kb * kMgBK : xp0 + (kb - q.nident) * kMgBK;
-                        ptx::tma_load_2d(b_dst + lane * kMgBBoxBytes, bm, &bars->full[s], col0 + lane * 64, brow);
-                    } else if (lane == 4 && !own) {
-                        ptx::tma_load_2d(ptx::smem_u32(a_ring) + sa * kMgABytes, &tmapP, &bars->full[s],
-                                         (kb - q.nident) * kMgBK, row0);
-                    }
+                if (lane == 0) ptx::mbar_arrive_expect_tx(&bars->full[s], kMgABytes + nslab * kMgBBoxBytes);
+                __syncwarp();
+                const uint32_t a_dst = smem_base + s * kMgStageBytes;
+                if (lane < nslab)
+                    ptx::tma_load_2d(a_dst + kMgABytes + lane * kMgBBoxBytes, &tmapXp, &bars->full[s], col0 + lane * 64, xp0 + kb * kMgBK);
+                else if (lane == 4)
+                    ptx::tma_load_2d(a_dst, &tmapP, &bars->full[s], kb * kMgBK, row0);
+                if (++s == stages) {
+                    s = 0;
+                    phase ^= 1u;
                 }
             }
         }
-    } else if (warp == 6) {
+    } else if (warp == 10) {
         // ---------------- scheduler -------------------------------------------------------------------
         if (lane == 0) {
             uint32_t pushed = 0, drawn = 0;
@@ -306,11 +286,12 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
                 atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
             }
         }
-    } else if (warp == 5) {
+    } else if (warp == 9) {
         // ---------------- UMMA issuer -----------------------------------------------------------------
         if (lane == 0) {
             const uint32_t idesc = ptx::idesc_bf16(kMgTileM, kMgTileN, false, true);
-            uint32_t it = 0, ia = 0, acc = 0;
+            int s = 0;
+            uint32_t phase = 0;
             for (uint32_t n = 0; !bars->abort_flag; ++n) {
                 MergeUnit q;
                 if (!merge_pop(mq, bars, n, q)) {
@@ -319,10 +300,10 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
                     break;
                 }
                 if (q.img < 0) break;
-                const int nkb = q.nident + (q.B + kMgBK - 1) / kMgBK;
-                const int buf = acc & 1;
-                if (acc >= 2) {
-                    if (!ptx::mbar_wait(&bars->accum_empty[buf], ((acc >> 1) - 1) & 1)) {
+                const int nkb = (q.B + kMgBK - 1) / kMgBK;
+                const int buf = n & 1;
+                if (n >= 2) {
+                    if (!ptx::mbar_wait(&bars->accum_empty[buf], ((n >> 1) - 1) & 1)) {
                         bars->abort_flag = 1;
                         atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
                         break;
@@ -331,22 +312,13 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
                 }
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * kMgTileN);
                 bool failed = false;
-                for (int kb = 0; kb < nkb; ++kb, ++it) {
-                    const int s = it % kMgBStages;
-                    if (!ptx::mbar_wait(&bars->full[s], (it / kMgBStages) & 1)) {
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!ptx::mbar_wait(&bars->full[s], phase)) {
                         failed = true;
                         break;
                     }
                     ptx::tc_fence_after();
-                    // identity k-block 0: the view whose rows 0-63 are I_64; k-block 1: rows 64-127
-                    uint32_t a_base;
-                    if (kb < q.nident) {
-                        a_base = ptx::smem_u32(ident) + (1 - kb) * (kMgABytes / 2);
-                    } else {
-                        a_base = ptx::smem_u32(a_ring) + (ia % kMgAStages) * kMgABytes;
-                        ++ia;
-                    }
-                    const uint32_t b_base = smem_base + s * kMgBBytes;
+                    const uint32_t a_base = smem_base + s * kMgStageBytes, b_base = a_base + kMgABytes;
 #pragma unroll
                     for (int k = 0; k < kMgBK / 16; ++k) {
                         // A: K-major, 32 bytes further along the 128-byte row per 16 k.
@@ -357,22 +329,72 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
                         ptx::umma_bf16(d_tmem, da, db, idesc, (kb | k) != 0);
                     }
                     ptx::umma_commit(&bars->empty[s]);
+                    if (++s == stages) {
+                        s = 0;
+                        phase ^= 1u;
+                    }
                 }
                 if (failed) {
                     bars->abort_flag = 1;
                     atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
                     break;
                 }
-                ptx::umma_commit(&bars->accum_full[buf]);
-                ++acc;
+                ptx::umma_commit(&bars->accum_full[buf]);    // (at once for an image with nothing pruned)
             }
         }
+    } else if (warp >= 11) {
+        // ---------------- loaders: the kept tokens' own rows ------------------------------------------
+        // A warp fetches 32 rows, two at a time (16 lanes x 16 bytes = 128 columns each).
+        const int lrow = (warp - 11) * 32, sub = lane >> 4, piece = lane & 15;
+        const uint32_t own_base = ptx::smem_u32(own) + (uint32_t)((lrow + sub) * 256);
+        int buf = 0;                                  // tile of own rows, and its phase
+        uint32_t phase = 1;
+        bool alive = true;
+        for (uint32_t n = 0; alive; ++n) {
+            MergeUnit q;
+            const bool got = merge_pop(mq, bars, n, q);
+            if (!__all_sync(0xffffffffu, got)) {
+                bars->abort_flag = 1;
+                if (lane == 0) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
+                break;
+            }
+            if (q.img < 0) break;
+            const int p = q.mt * kMgTileM + lrow + lane;     // position among the kept tokens
+            const int tok = p < q.M ? __ldcg(order + q.t_begin + p) : -1;
+            if (q.ct == 0 && tok >= 0) kept_idx[q.out0 + p] = tok;
+            const int nrows = max(0, min(32, q.M - (q.mt * kMgTileM + lrow)));
+            const int col_end = min(d, (q.ct + 1) * kMgTileN);
+            for (int col = q.ct * kMgTileN; col < col_end; col += kMgOwnCols) {
+                const bool ok = ptx::mbar_wait(&bars->own_empty[buf], phase);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    bars->abort_flag = 1;
+                    if (lane == 0) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
+                    alive = false;
+                    break;
+                }
+                const int c = col + piece * 8;
+                const __nv_bfloat16 *src = X + (size_t)q.t_begin * d + c;
+                const uint32_t dst = own_base + (uint32_t)(buf * kMgOwnBytes);
+#pragma unroll 4
+                for (int r = 0; r < nrows; r += 2) {
+                    const int t = __shfl_sync(0xffffffffu, tok, r + sub);
+                    if (t >= 0 && c < col_end)
+                        ptx::cp_async_16(dst + (uint32_t)(r * 256 + ((piece ^ ((r + sub) & 7)) << 4)), src + (size_t)t * d, 16u);
+                }
+                ptx::cp_async_arrive(&bars->own_full[buf]);  // once this thread's copies have landed
+                if (++buf == bufs) {
+                    buf = 0;
+                    phase ^= 1u;
+                }
+            }
+        }
+        ptx::cp_async_commit();
+        ptx::cp_async_wait<0>();
     } else {
-        // ---------------- warps 0-3: epilogue ---------------------------------------------------------
-        const int row = tid;                                  // TMEM lane = row of the token tile
-        uint8_t *srow = staging + row * kMgStagePitch;        // this thread's staging row, nobody else's
-        const uint32_t srow_u32 = ptx::smem_u32(srow);
-        uint32_t acc = 0;
+        // ---------------- warps 0-7: epilogue ---------------------------------------------------------
+        const int row = tid & 127, half = tid >> 7;           // TMEM lane = row of the tile; which half of the columns
+        int ob = 0;                                           // tile of own rows of the unit's first half, and its phase
+        uint32_t phase = 0;
         for (uint32_t n = 0;; ++n) {
             MergeUnit q;
             const bool got = merge_pop(mq, bars, n, q);
@@ -382,11 +404,25 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
                 break;
             }
             if (q.img < 0) break;
-            const int tok = q.mt * kMgTileM + row;            // image-local token of this row
-            const int p = (tok < q.N) ? __ldcg(kpos + q.t_begin + tok) : -1;   // >= 0: position among kept
-            const int buf = acc & 1;
+            const int buf = n & 1;
+            const int col = q.ct * kMgTileN + half * kMgOwnCols, ncols = min(kMgOwnCols, d - col);    // (may be <= 0)
+            // own rows: the tile of this thread's half
+            int mine = ob;
+            uint32_t mine_phase = phase;
+            const int tiles = d - q.ct * kMgTileN > kMgOwnCols ? 2 : 1;
+            for (int k = 0; k < tiles; ++k) {
+                if (k == half) {
+                    mine = ob;
+                    mine_phase = phase;
+                }
+                if (++ob == bufs) {
+                    ob = 0;
+                    phase ^= 1u;
+                }
+            }
             // the TMEM loads below are warp-collective: take the go / no-go decision per warp
-            bool ok = !bars->abort_flag && ptx::mbar_wait(&bars->accum_full[buf], (acc >> 1) & 1);
+            bool ok = !bars->abort_flag && ptx::mbar_wait(&bars->accum_full[buf], (n >> 1) & 1) &&
+                      (ncols <= 0 || ptx::mbar_wait(&bars->own_full[mine], mine_phase));
             if (!__all_sync(0xffffffffu, ok)) {
                 bars->abort_flag = 1;
                 if (lane == 0) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
@@ -394,43 +430,54 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_consta
             }
             ptx::tc_fence_after();
             // unit n's accumulator is complete, so every epilogue thread is done with unit n - 2 (its
-            // accumulator buffer was handed back) and the UMMA issuer is past it: those entries are free
+            // accumulator buffer was handed back) and the producer, the UMMA issuer and the loaders are past it:
+            // those entries are free
             if (tid == 0 && n >= 1) mq->tail = n - 1;
-            ptx::bulk_wait_read<0>();                         // the previous unit's store has read this row
-            const int col0 = q.ct * kMgTileN;
-            const int ncols = min(kMgTileN, d - col0);
-            // a warp whose 32 rows all lie past the image's end has nothing to convert or store
-            const bool warp_has_rows = q.mt * kMgTileM + warp * 32 < q.N;
-            for (int c0 = 0; c0 < (warp_has_rows ? ncols : 0); c0 += 32) {
-                uint32_t r[32];
-                ptx::tmem_ld32(tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * kMgTileN + c0), r);
-                ptx::tmem_ld_wait();
+            const int w0 = row & ~31, prow0 = q.mt * kMgTileM + w0;      // the warp's first row of the tile, and of the kept ones
+            uint8_t *const tile = own + mine * kMgOwnBytes;
+            // a warp whose 32 rows all lie past the kept ones has nothing to add or store
+            if (prow0 < q.M && q.B > 0) {
+                uint8_t *const srow = tile + row * 256;
+                for (int c0 = 0; c0 < ncols; c0 += 32) {
+                    uint32_t r[32];
+                    ptx::tmem_ld32(tmem_base + ((uint32_t)w0 << 16) + (uint32_t)(buf * kMgTileN + half * kMgOwnCols + c0), r);
+                    uint4 x[4];
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    __nv_bfloat162 o[4];
+                    for (int g = 0; g < 4; ++g) x[g] = *reinterpret_cast<const uint4 *>(srow + (((c0 / 8 + g) ^ (row & 7)) << 4));
+                    ptx::tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        o[e] = __floats2bfloat162_rn(__uint_as_float(r[8 * g + 2 * e]),
-                                                     __uint_as_float(r[8 * g + 2 * e + 1]));
-                    *reinterpret_cast<uint4 *>(srow + (c0 + 8 * g) * 2) = *reinterpret_cast<uint4 *>(o);
+                    for (int g = 0; g < 4; ++g) {
+                        float f[8];
+                        Elem<__nv_bfloat16>::unpack(x[g], f);
+                        __nv_bfloat162 o[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            o[e] = __floats2bfloat162_rn(f[2 * e] + __uint_as_float(r[8 * g + 2 * e]),
+                                                         f[2 * e + 1] + __uint_as_float(r[8 * g + 2 * e + 1]));
+                        *reinterpret_cast<uint4 *>(srow + (((c0 / 8 + g) ^ (row & 7)) << 4)) = *reinterpret_cast<uint4 *>(o);
+                    }
                 }
             }
             ptx::tc_fence_before();
             ptx::mbar_arrive(&bars->accum_empty[buf]);
-            ++acc;
-            if (p >= 0) {
-                ptx::fence_proxy_async_smem();
-                ptx::bulk_store(Y + (size_t)(q.out0 + p) * d + col0, srow_u32, (uint32_t)ncols * 2u);
-                if (q.ct == 0) kept_idx[q.out0 + p] = tok;
+            __syncwarp();                                     // the warp's rows are complete
+            if (ncols > 0) {
+                const int sub = lane >> 4, piece = lane & 15, nrows = min(32, q.M - prow0);      // (may be <= 0)
+                __nv_bfloat16 *dst = Y + (size_t)(q.out0 + prow0) * d + col + piece * 8;
+                if (piece * 8 < ncols) {
+#pragma unroll 8
+                    for (int r = sub; r < nrows; r += 2)
+                        *reinterpret_cast<uint4 *>(dst + (size_t)r * d) =
+                            *reinterpret_cast<const uint4 *>(tile + (w0 + r) * 256 + ((piece ^ (r & 7)) << 4));
+                }
+                ptx::mbar_arrive(&bars->own_empty[mine]);     // (after this thread's reads)
             }
-            ptx::bulk_commit();
         }
-        ptx::bulk_wait<0>();                                  // stores complete before the CTA retires
     }
 
     ptx::tc_fence_before();
     __syncthreads();
-    if (warp == 5) {
+    if (warp == 9) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem_base, 512);
     }

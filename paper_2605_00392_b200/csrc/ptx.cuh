@@ -132,6 +132,11 @@ __device__ inline void cp_async_16(uint32_t dst_smem, const void *src, uint32_t 
                  : "memory");
 }
 __device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// One of the mbarrier's expected arrivals, made when this thread's cp.async copies so far have landed.
+__device__ inline void cp_async_arrive(uint64_t *bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 template <int N> __device__ inline void cp_async_wait()
 {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");

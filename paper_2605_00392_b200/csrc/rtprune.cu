@@ -65,7 +65,7 @@ struct rtprune_plan_s {
         const void *ws;
         int total, batch, pbuf_pitch;
         bool valid;
-        CUtensorMap scX, scXp, mgX, mgXp, mgP;
+        CUtensorMap scX, scXp, mgXp, mgP;
     };
     static constexpr int kMapSets = 8;
     MapSet maps[kMapSets];
@@ -247,7 +247,7 @@ bool scaling_in_range(const rtprune_params_t *p)
     return (2.f * c - lo) / p->eps <= 62.f;
 }
 
-// The five tensor maps of a bf16 run over (X, workspace): from the plan's cache, or encoded into it.
+// The four tensor maps of a bf16 run over (X, workspace): from the plan's cache, or encoded into it.
 const rtprune_plan_s::MapSet *tensor_maps(rtprune_plan_t *plan, const void *X, char *ws, int total, int batch,
                                           int pbuf_pitch)
 {
@@ -263,7 +263,6 @@ const rtprune_plan_s::MapSet *tensor_maps(rtprune_plan_t *plan, const void *X, c
     const uint64_t d = (uint64_t)plan->d, rows_xp = (uint64_t)total + 64 * (uint64_t)batch;
     if (!make_tmap_bf16(plan, &m.scX, X, (uint64_t)total, d, d * 2, kScBK, kScTileM) ||
         !make_tmap_bf16(plan, &m.scXp, ws + L.xp, rows_xp, d, d * 2, kScBK, kScBBoxRows) ||
-        !make_tmap_bf16(plan, &m.mgX, X, (uint64_t)total, d, d * 2, 64, kMgBK) ||
         !make_tmap_bf16(plan, &m.mgXp, ws + L.xp, rows_xp, d, d * 2, 64, kMgBK) ||
         !make_tmap_bf16(plan, &m.mgP, ws + L.pbuf, (uint64_t)total, (uint64_t)pbuf_pitch, (uint64_t)pbuf_pitch * 2,
                         kMgBK, kMgTileM))
@@ -644,19 +643,21 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
     }
 
     if constexpr (kTensor) {
-        // every operand by tiled TMA: X rows (token tiles), the compact copy of pruned rows, the plan
+        // operands by tiled TMA: the plan, the compact copy of pruned rows
         const rtprune_plan_s::MapSet *ms = tensor_maps(plan, X, ws, total, batch, pbuf_pitch);
         if (!ms) return RTPRUNE_ERR_CUDA;
-        const CUtensorMap &tmapXm = ms->mgX, &tmapXpm = ms->mgXp, &tmapP = ms->mgP;
+        const CUtensorMap &tmapXpm = ms->mgXp, &tmapP = ms->mgP;
         const int mtiles_m = (maxN + kMgTileM - 1) / kMgTileM;
         const int nct = (plan->d + kMgTileN - 1) / kMgTileN;
         const long long nunits = (long long)batch * mtiles_m * nct;
         const int grid = (int)std::min<long long>(nunits, plan->sm_count);
-        if (!c.ok(launch_pdl(merge_umma_kernel, dim3((unsigned)grid), dim3(kMgThreads), kMgSmemBytes, st, 1u,
-                             tmapXm, tmapXpm, tmapP, offsets, plan->d, batch, mtiles_m, o.counts, o.out_offsets,
-                             (const int32_t *)(ws + L.kpos), maxN, total, (__nv_bfloat16 *)o.Y, o.kept_idx,
+        // shared memory for a deep ring of k-blocks where an image has many, else for more tiles of own rows
+        const int mg_stages = maxB > kMgDeepB ? 3 : 2, mg_bufs = maxB > kMgDeepB ? 2 : 4;
+        if (!c.ok(launch_pdl(merge_umma_kernel, dim3((unsigned)grid), dim3(kMgThreads), (size_t)merge_smem_bytes(mg_stages, mg_bufs), st, 1u,
+                             tmapXpm, tmapP, (const __nv_bfloat16 *)X, offsets, plan->d, batch, mtiles_m, o.counts, o.out_offsets,
+                             (const int32_t *)order, maxN, total, (__nv_bfloat16 *)o.Y, o.kept_idx,
                              (WsHeader *)(ws + L.header), (const int32_t *)ready_list,
-                             ready_list ? by_image : 0)))
+                             ready_list ? by_image : 0, mg_stages, mg_bufs)))
             return RTPRUNE_ERR_CUDA;
     } else {
         const int mtiles = (maxN + kF3Tile - 1) / kF3Tile, nct = (plan->d + kM3N - 1) / kM3N;
@@ -980,7 +981,7 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
                                        std::max(scores_smem_bytes(kScRingBytesAlone),
                                                 scores_smem_bytes(kScRingBytes) + scores_split_bytes(4)))) ||
             !c.ok(cudaFuncSetAttribute(merge_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kMgSmemBytes))) {
+                                       kMgSmemMax))) {
             if (!p->last_cuda_error) p->last_cuda_error = (int)cudaErrorNotSupported;
             delete p;
             return RTPRUNE_ERR_CUDA;

@@ -42,7 +42,7 @@ __device__ inline FuIterState reg_sinkhorn(FuShared *sh, const float *kbuf, floa
         for (int s = 0; s < NS; ++s) U[s] = ((s * kFuWarps + warp) * RPS + slot < Ml) ? 1.f : 0.f;   // u = 0
     }
 
-    // alpha P = alpha U K V in bf16: row = the kept token's position in X, columns up to the next multiple
+    // alpha P = alpha U K V in bf16: row = position among the kept tokens, columns up to the next multiple
     // of 64 (zeros past B: K is zero there), 4 columns = 8 bytes per store
     const int kpad = (B + 63) & ~63;
     float4 V[NQ];
@@ -52,7 +52,7 @@ __device__ inline FuIterState reg_sinkhorn(FuShared *sh, const float *kbuf, floa
     for (int s = 0; s < NS; ++s) {
         const int i = (s * kFuWarps + warp) * RPS + slot;
         if (i < Ml) {
-            __nv_bfloat16 *prow = Pimg + (size_t)sh->rowtok[i] * pbuf_pitch;
+            __nv_bfloat16 *prow = Pimg + (size_t)(row_lo + i) * pbuf_pitch;
             const float au = p.alpha * U[s];
 #pragma unroll
             for (int q = 0; q < NQ; ++q) {
@@ -138,7 +138,6 @@ sinkhorn_reg_kernel(const int32_t *__restrict__ offsets, const int32_t *__restri
     const float v_init = expf(shift * inv_eps);
     const float *Sg = kmat + kmat_offset(kmat_stride, t_begin, img);
 
-    for (int i = tid; i < Ml; i += kFuThreads) sh->rowtok[i] = __ldcg(order + t_begin + row_lo + i);
     // both CTAs are running and have their barriers in place before anything is sent to the other
     ptx::cluster_sync_all();
     if (scores_done) {

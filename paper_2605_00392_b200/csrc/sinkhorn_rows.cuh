@@ -61,7 +61,7 @@ __host__ __device__ inline int sr_batch_rows(int B) { return B < 64 ? 32 : (B < 
 __host__ __device__ inline int sr_aux_floats(int B, int C, int rows)
 {
     const int w = sr_width(B);
-    return 2 * kSrWarps * w + (C > 1 ? 2 * C * w : 0) + w + 2 * ((rows + 33) & ~3);
+    return 2 * kSrWarps * w + (C > 1 ? 2 * C * w : 0) + w + ((rows + 33) & ~3);
 }
 // Shared-memory rows of K for `rows` kept tokens: those and the dustbin's, in whole batches.
 __host__ __device__ inline int sr_smem_rows(int B, int rows)
@@ -93,7 +93,6 @@ struct SrTile {
     float *Ks;                  // [cap][ld]
     float *Kg;                  // this CTA's first row in the workspace tile
     float *part, *xpart, *vs, *us;
-    int *toks;
     uint64_t *xbar, *cbar;      // [2] column sums of the other CTAs; [kSrChunks] copies of S
 };
 
@@ -467,7 +466,7 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
         const float2 range = s_range[lane % kSrWarps];         // (written again after the next iteration's first barrier)
         lo = warp_min_redux(range.x);
         hi = warp_max_redux(range.y);
-        st.last_move = 0.5f * (hi - lo);
+        st.last_move = fmaxf(-lo, hi);
         if (!go || (p.tol == 0.f && p.stop_fp && plan_settled(lo, hi))) break;
     }
     return st;
@@ -503,7 +502,7 @@ __device__ inline void sinkhorn_publish(int img, uint32_t C, uint32_t *__restric
 struct SrOut {
     int img;
     const int32_t *ord;                        // kept tokens, then pruned tokens
-    __nv_bfloat16 *Pimg;                       // plan rows by token position (bf16 storage), else nullptr
+    __nv_bfloat16 *Pimg;                       // plan rows of this CTA (bf16 storage), else nullptr
     int pbuf_pitch;
     int32_t *merged_seg, *partner_seg;
     float *weight_seg;
@@ -512,7 +511,7 @@ struct SrOut {
     bool by_image;
 };
 
-// Plan P = U K V of this CTA's rows: alpha P in bf16 (row = the kept token's position in X, columns up to the next
+// Plan P = U K V of this CTA's rows: alpha P in bf16 (row = position among the kept tokens, columns up to the next
 // multiple of 64) or P in fp32 in place in the workspace tile.  In the same pass the pairing: partner_j = argmax_i P_ij
 // = argmax_i K_ij U_i, ties to the lower i.  The merge kernel may take the image before the pairs are out.
 template <int LR, int NQ, int RB>
@@ -548,7 +547,7 @@ __device__ inline void sr_finish(const SrTile &t, const OtParams &p, const SrOut
         if (i >= t.Ml) continue;
         const float *krow = i < t.cap ? t.Ks + (size_t)i * t.ld : t.Kg + (size_t)i * t.ld;
         const float u = t.us[i];
-        __nv_bfloat16 *prow = o.Pimg ? o.Pimg + (size_t)t.toks[i] * o.pbuf_pitch : nullptr;
+        __nv_bfloat16 *prow = o.Pimg ? o.Pimg + (size_t)i * o.pbuf_pitch : nullptr;
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
             const int col = 4 * (q * LR + sub);
@@ -718,24 +717,20 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
     t.xpart = t.part + 2 * kSrWarps * w;
     t.vs = t.xpart + (t.C > 1 ? 2 * t.C * w : 0);
     t.us = t.vs + w;
-    t.toks = reinterpret_cast<int *>(t.us + ((rows_per + 33) & ~3));
-    t.Ks = t.us + 2 * ((rows_per + 33) & ~3);
+    t.Ks = t.us + ((rows_per + 33) & ~3);
     t.xbar = s_xbar;
     t.cbar = s_cbar;
     if (tid < kSrChunks) {
         ptx::fence_proxy_async_all();          // the scores were written with ordinary stores
         sr_fetch(t, tid);
     }
-    for (int i = tid; i < t.Ml; i += kSrThreads) {
-        t.toks[i] = __ldcg(order + t_begin + t.row_lo + i);
-        t.us[i] = 1.f;                                     // u = 0
-    }
+    for (int i = tid; i < t.Ml; i += kSrThreads) t.us[i] = 1.f;      // u = 0
     const float inv_eps = 1.f / p.eps;
     const float shift = fmaxf(1.f, p.z);
     const float kappa = expf((p.z - shift) * inv_eps);
     const float v_init = expf(shift * inv_eps);            // v = 0
     const int seg = t_begin - out0;
-    const SrOut o{img, order + t_begin, pbuf ? pbuf + (size_t)t_begin * pbuf_pitch : nullptr, pbuf_pitch,
+    const SrOut o{img, order + t_begin, pbuf ? pbuf + (size_t)(t_begin + t.row_lo) * pbuf_pitch : nullptr, pbuf_pitch,
                   merged_idx + seg, merge_partner + seg, merge_weight + seg, sink_done, ready_list, by_image != 0};
     auto solve = [&](auto lr, auto nq, auto rb) {
         constexpr int LR = decltype(lr)::value, NQ = decltype(nq)::value, RB = decltype(rb)::value;

@@ -41,10 +41,10 @@ constexpr float kStFixedPointTol = 4.76837158e-7f;
 __host__ __device__ inline int st_width(int B) { return (B + 256) & ~255; }
 __host__ __device__ inline int st_slice(int W, int C) { return (W + C - 1) / C; }
 // Floats of shared memory besides the ring of rows: V, the warps' column sums (two of them share a row), the parts
-// received (values, and indices for the pairing), U and token of every row.
+// received (values, and indices for the pairing), U of every row.
 __host__ __device__ inline int st_fixed_floats(int W, int C, int rows, int warps)
 {
-    return W + (warps / 2) * W + 2 * C * st_slice(W, C) + 2 * ((rows + 3) & ~3);
+    return W + (warps / 2) * W + 2 * C * st_slice(W, C) + ((rows + 3) & ~3);
 }
 // The ring: at least two rows per warp; the pairing needs a value and an index per warp and column.
 __host__ __device__ inline int st_min_floats(int W, int C, int rows, int warps) { return st_fixed_floats(W, C, rows, warps) + 2 * warps * W; }
@@ -56,7 +56,6 @@ struct StTile {
     uint32_t rank;
     float *Kg;                                 // this CTA's first row in the workspace tile
     float *vs, *part, *xrecv, *us, *ring;
-    int *toks;
     uint64_t *full, *sbar, *vbar;              // [warps][stages] rows; column sums; V
     int stages;
 };
@@ -380,7 +379,7 @@ __device__ inline void st_solve(const StTile &t, const OtParams &p, const SrOut 
             for (int q = 0; q < NH; ++q) k[q] = kn[q];
             if (r + 1 < nrows) fetch(i + step);
             const float u = t.us[i];
-            __nv_bfloat16 *prow = o.Pimg ? o.Pimg + (size_t)t.toks[i] * o.pbuf_pitch + col0 : nullptr;
+            __nv_bfloat16 *prow = o.Pimg ? o.Pimg + (size_t)i * o.pbuf_pitch + col0 : nullptr;
             float *krow = t.Kg + (size_t)i * t.ld + col0;
 #pragma unroll
             for (int q = 0; q < NH; ++q) {
@@ -493,7 +492,6 @@ sinkhorn_stream_kernel(const int32_t *__restrict__ offsets, const int32_t *__res
     t.part = t.vs + W;
     t.xrecv = t.part + (kWarps / 2) * W;
     t.us = t.xrecv + 2 * t.C * st_slice(W, t.C);
-    t.toks = reinterpret_cast<int *>(t.us + ((rows_per + 3) & ~3));
     const int fixed = (st_fixed_floats(W, t.C, rows_per, kWarps) + 3) & ~3;
     t.ring = sm + fixed;
     t.stages = min(kStMaxStages, (smem_floats - fixed) / (kWarps * t.ld));
@@ -502,13 +500,12 @@ sinkhorn_stream_kernel(const int32_t *__restrict__ offsets, const int32_t *__res
     t.vbar = &s_bar[1];
     const float v_init = expf(fmaxf(1.f, p.z) / p.eps), kappa = expf((p.z - fmaxf(1.f, p.z)) / p.eps);
     for (int j = tid; j < W; j += TH) t.vs[j] = j < t.B ? v_init : (j == t.B ? kappa * v_init : 0.f);
-    for (int i = tid; i < t.Ml; i += TH) t.toks[i] = __ldcg(order + t_begin + t.row_lo + i);
     ptx::fence_proxy_async_all();          // the scores were written with ordinary stores
     __syncthreads();
     // every CTA of the cluster is running and has its barriers and V in place before anything is sent to it
     ptx::cluster_sync_all();
     const int seg = t_begin - __ldcg(out_offsets + img);
-    const SrOut o{img, order + t_begin, pbuf ? pbuf + (size_t)t_begin * pbuf_pitch : nullptr, pbuf_pitch,
+    const SrOut o{img, order + t_begin, pbuf ? pbuf + (size_t)(t_begin + t.row_lo) * pbuf_pitch : nullptr, pbuf_pitch,
                   merged_idx + seg, merge_partner + seg, merge_weight + seg, nullptr, nullptr, false};
     float *st = stats + (size_t)img * kStats;
     switch (W >> 8) {

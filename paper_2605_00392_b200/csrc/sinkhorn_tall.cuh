@@ -41,7 +41,7 @@ __host__ __device__ inline size_t sinkhorn_tall_smem_floats(int maxB, int maxM, 
     const size_t qpr = (size_t)score_pitch(maxB) / 4;
     const size_t sl = (qpr + C - 1) / C;
     const size_t rows_cap = ((size_t)maxM + C - 1) / C;
-    return (4 * qpr + 4) + 2 * C * 4 * sl + 2048 + 256 + 64 + 64 + 2 * (rows_cap + 4) + 4;
+    return (4 * qpr + 4) + 2 * C * 4 * sl + 2048 + 256 + 64 + 64 + (rows_cap + 4) + 4;
 }
 constexpr int kTallMaxStages = 4;
 constexpr int kTallStageFloatsMax = 16384;      // a block of rows is at most 64 KB (see the three layouts)
@@ -116,8 +116,7 @@ __device__ inline void sinkhorn_tall_solve(float *Kg, int ldS, int M, int B, int
     float *wred = red + 256;                  // [2][16] + [2]  per-warp sums of V and moves; the groups' sums of U
     float *xs = wred + 64;                    // [4][C]         per-CTA sums of U, sums of V, continue flags, moves
     float *us = xs + 64;                      // [rows_cap + 4] U of this CTA's rows
-    int *toks = reinterpret_cast<int *>(us + rows_cap + 4);   // [rows_cap] token position of this CTA's rows
-    const int fixed_floats = (int)((us + rows_cap + 4 + rows_cap) - sm + 3) & ~3;
+    const int fixed_floats = (int)((us + rows_cap + 4) - sm + 3) & ~3;
     float *ring = sm + fixed_floats;          // [NS][G R ldS]  blocks of rows of K on their way to the threads
     const int stage_floats = G * R * ldS;
     const int NS = max(1, min(kTallMaxStages, (smem_floats - fixed_floats) / stage_floats));
@@ -135,10 +134,7 @@ __device__ inline void sinkhorn_tall_solve(float *Kg, int ldS, int M, int B, int
     const float v_init = expf(shift * inv_eps);       // v = 0
     const float Bf = (float)B, Mf = (float)M;
 
-    for (int i = tid; i < Ml; i += kTallThreads) {
-        toks[i] = __ldcg(ord + row_lo + i);
-        us[i] = 1.f;                                  // u = 0
-    }
+    for (int i = tid; i < Ml; i += kTallThreads) us[i] = 1.f;      // u = 0
     // ---- K = exp((S - c)/eps) of this CTA's rows, in place, zero from column B on ---------------------
     {
         const int total_q = Ml * qpr;
@@ -173,7 +169,7 @@ __device__ inline void sinkhorn_tall_solve(float *Kg, int ldS, int M, int B, int
         ptx::fence_mbar_init();
     }
     ptx::fence_proxy_async_all();     // K was stored through the generic proxy; the bulk copies read it
-    __syncthreads();              // K (re-read from L2 below by other threads of this CTA), vs, us, toks
+    __syncthreads();              // K (re-read from L2 below by other threads of this CTA), vs, us
     // every CTA of the cluster is running and has its shared memory laid out before anyone writes into it
     ptx::cluster_sync_all();
 
@@ -441,7 +437,6 @@ __device__ inline void sinkhorn_tall_solve(float *Kg, int ldS, int M, int B, int
                 const int i = (blk * G + g) * R + r;
                 if (i >= Ml) continue;
                 const float U = us[i];
-                const int tok = toks[i];
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) {
                     if (!cv[q]) continue;
@@ -455,11 +450,11 @@ __device__ inline void sinkhorn_tall_solve(float *Kg, int ldS, int M, int B, int
                     }
                     const float4 P = make_float4(ku[0] * V[q].x, ku[1] * V[q].y, ku[2] * V[q].z, ku[3] * V[q].w);
                     if (Pimg) {
-                        if (4 * cq[q] < kpad) {          // alpha P in bf16, row = the kept token's position in X
+                        if (4 * cq[q] < kpad) {          // alpha P in bf16, row = position among the kept tokens
                             __nv_bfloat162 o[2];
                             o[0] = __floats2bfloat162_rn(p.alpha * P.x, p.alpha * P.y);
                             o[1] = __floats2bfloat162_rn(p.alpha * P.z, p.alpha * P.w);
-                            *reinterpret_cast<uint2 *>(Pimg + (size_t)tok * pbuf_pitch + 4 * cq[q]) =
+                            *reinterpret_cast<uint2 *>(Pimg + (size_t)(row_lo + i) * pbuf_pitch + 4 * cq[q]) =
                                 *reinterpret_cast<uint2 *>(o);
                         }
                     } else {
@@ -472,7 +467,7 @@ __device__ inline void sinkhorn_tall_solve(float *Kg, int ldS, int M, int B, int
             const int zq = (kpad - ldc) >> 2;
             for (int idx = tid; idx < Ml * zq; idx += kTallThreads) {
                 const int i = idx / zq, c = idx - i * zq;
-                *reinterpret_cast<uint2 *>(Pimg + (size_t)toks[i] * pbuf_pitch + ldc + 4 * c) = make_uint2(0u, 0u);
+                *reinterpret_cast<uint2 *>(Pimg + (size_t)(row_lo + i) * pbuf_pitch + ldc + 4 * c) = make_uint2(0u, 0u);
             }
         }
         // pairing: the row groups meet in group 0, the CTAs in the owner of the column
