@@ -546,30 +546,51 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             // tile's image uses fewer, see sr_ctas), more while the device has SMs to spare and a CTA would have more
             // than 10 000 cells (an exchange of column sums costs less than a pass over that many).  A batch that would
             // then take more than four waves of CTAs halves it: the few tiles that do not fit read a part of K from L2.
+            // Batches of more CTAs than SMs take CTAs of half the threads and half the shared memory, two to an SM, for tiles of
+            // up to 255 columns: what one spends on its set-up, barriers and results the other iterates in.  Two CTAs per image for
+            // one only in batches of four waves or more and with a fixed ratio, when most tiles are as large as the largest possible
+            // one.  Event times, 512 threads -> 256: 1014 x 69 at a dynamic ratio 90 -> 51 us, 1024 x 400 at r = 0.25 197 -> 172 (2
+            // CTAs per image); whole runs of 700 images of 150-400 tokens at r = 0.25 588 -> 562, but 300 x 400 at r = 0.25 394 ->
+            // 401, 250 of 200-400 in fp32 storage at r = 0.3 522 -> 531, and 479 of 199-304 at a dynamic ratio 379 -> 392.
             const int mb = std::min(maxB, kSrMaxB);
-            auto floats = [&](int cc) {
-                long long most = 0;
-                for (int b = 1; b <= mb; ++b) {
-                    const int rows = (std::max(maxN - b, 1) + cc - 1) / cc;
-                    most = std::max(most, (long long)sr_smem_rows(b, rows) * score_pitch(b) + sr_aux_floats(b, cc, rows));
-                }
-                return most;
-            };
-            const long long limit = plan->fast_smem_bytes / (int)sizeof(float);
             const long long cells = (long long)(maxN - std::min(mb, maxN / 2)) * std::min(mb, maxN / 2);
             const int spread = 2LL * batch <= plan->sm_count ? 10000 : 40000;
-            int cc = 1;
-            while (cc < kSrMaxC && floats(cc) > limit) cc *= 2;
-            while (cc < kSrMaxC && (long long)batch * cc * 2 <= plan->sm_count && cells > (long long)spread * cc) cc *= 2;
-            if (cc > 1 && (long long)batch * cc > 4LL * plan->sm_count) cc /= 2;
-            const int smem_floats_rows = (int)std::min(limit, floats(cc)) & ~3;
+            int sr_threads = kSrThreads, cc = 1, full_cc = 0, smem_floats_rows = 0;
+            for (;; sr_threads /= 2) {
+                const bool half = sr_threads < kSrThreads;
+                auto floats = [&](int c1) {
+                    long long most = 0;
+                    for (int b = 1; b <= mb; ++b) {
+                        const int rows = (std::max(maxN - b, 1) + c1 - 1) / c1;
+                        most = std::max(most, (long long)sr_smem_rows(b, rows) * score_pitch(b) + sr_aux_floats(b, c1, rows, sr_threads / 32));
+                    }
+                    return most;
+                };
+                const long long limit = (half ? std::min(plan->fast_smem_bytes, kSrHalfSmemBytes) : plan->fast_smem_bytes) / (int)sizeof(float);
+                cc = 1;
+                while (cc < kSrMaxC && floats(cc) > limit) cc *= 2;
+                while (cc < kSrMaxC && (long long)batch * cc * 2 <= plan->sm_count && cells > (long long)spread * cc) cc *= 2;
+                if (!half && full_cc == 0 && mb <= 255 && (long long)batch * cc > plan->sm_count) {
+                    full_cc = cc;
+                    continue;
+                }
+                if (half && cc > full_cc && (params->dynamic || full_cc > 1 || (long long)batch < 4LL * plan->sm_count)) {     // back to the whole SM
+                    sr_threads = 2 * kSrThreads;
+                    continue;
+                }
+                if (cc > 1 && (long long)batch * cc > (half ? 8LL : 4LL) * plan->sm_count) cc /= 2;
+                smem_floats_rows = (int)std::min(limit, floats(cc)) & ~3;
+                break;
+            }
+            const bool half = sr_threads < kSrThreads;
             all_fast = maxB <= kSrMaxB;
             rows_max_b = kSrMaxB;
             // When one kernel solves every image, it hands them to the merge kernel one by one
             ready_list = (kTensor && all_fast) ? (int32_t *)(ws + L.ready_list) : nullptr;
             const uint32_t *sd = ready_list ? (const uint32_t *)scores_done : (const uint32_t *)nullptr;
-            if (!c.ok(launch_pdl(mb > 255 ? sinkhorn_rows_kernel<true> : sinkhorn_rows_kernel<false>,
-                                 dim3((unsigned)(batch * cc)), dim3(kSrThreads), sizeof(float) * (size_t)smem_floats_rows, st,
+            if (!c.ok(launch_pdl(half ? sinkhorn_rows_kernel<false, kSrThreads / 2>
+                                 : mb > 255 ? sinkhorn_rows_kernel<true, kSrThreads> : sinkhorn_rows_kernel<false, kSrThreads>,
+                                 dim3((unsigned)(batch * cc)), dim3((unsigned)sr_threads), sizeof(float) * (size_t)smem_floats_rows, st,
                                  (unsigned)cc, offsets, (const int32_t *)o.counts, (const int32_t *)o.out_offsets,
                                  (const int32_t *)order, kmat, L.kmat_stride, maxN, total, op, cc, spread, smem_floats_rows,
                                  pbuf, pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight, o.stats,
@@ -958,10 +979,12 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
         delete p;
         return RTPRUNE_ERR_CUDA;
     }
-    if (!c.ok(cudaFuncSetAttribute(sinkhorn_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (!c.ok(cudaFuncSetAttribute(sinkhorn_rows_kernel<false, kSrThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    p->fast_smem_bytes)) ||
-        !c.ok(cudaFuncSetAttribute(sinkhorn_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   p->fast_smem_bytes))) {
+        !c.ok(cudaFuncSetAttribute(sinkhorn_rows_kernel<true, kSrThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   p->fast_smem_bytes)) ||
+        !c.ok(cudaFuncSetAttribute(sinkhorn_rows_kernel<false, kSrThreads / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   std::min(p->fast_smem_bytes, kSrHalfSmemBytes)))) {
         delete p;
         return RTPRUNE_ERR_CUDA;
     }

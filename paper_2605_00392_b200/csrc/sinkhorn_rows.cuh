@@ -20,6 +20,8 @@
 // A CTA keeps as many of its rows of K as fit in shared memory (they are fetched by bulk copies, being contiguous, and
 // exponentiated in place), the rest lies in the workspace tile (L2).  How many CTAs of the launched cluster work on an
 // image is decided per image (sr_ctas): an exchange costs about as much as a pass over 20 000 cells.
+// Large batches of narrow tiles run with half the threads and shared memory per CTA, two to an SM (the rule is where the kernel
+// is launched).
 //
 // What bounds it: shared-memory reads of K and instruction latency; on a 300 x 100 tile on one CTA an iteration is
 // 4200 cycles (pass 3000, column sums, V and two barriers the rest).  Measured by events around the kernel, against the
@@ -46,8 +48,8 @@ __device__ inline float rcp_fast(float x)
 // exp(x) by the hardware base-2 exponential (relative error about 2^-22).
 __device__ inline float exp_fast(float x) { return exp2f(x * 1.4426950408889634f); }
 
-constexpr int kSrThreads = 512;
-constexpr int kSrWarps = kSrThreads / 32;
+constexpr int kSrThreads = 512;                // of a CTA that has an SM to itself; half as many where two share one,
+constexpr int kSrHalfSmemBytes = 111 * 1024;   // and half of its 228 KB then (1 KB per CTA is the system's, 1 KB static)
 constexpr int kSrMaxB = 639;
 constexpr int kSrMaxC = 8;                     // CTAs per image at most
 constexpr int kSrChunks = 8;                   // bulk copies a CTA's rows of S arrive in
@@ -58,10 +60,10 @@ __host__ __device__ inline int sr_width(int B) { return B < 32 ? 32 : (B < 64 ? 
 __host__ __device__ inline int sr_batch_rows(int B) { return B < 64 ? 32 : (B < 128 ? 16 : (B < 256 ? 8 : 4)); }
 // Floats of shared memory besides K: the warps' column sums (the pairing's values and indices take their place), the
 // CTAs' column sums of two iterations, V, and per row (of whole batches) U and its token.
-__host__ __device__ inline int sr_aux_floats(int B, int C, int rows)
+__host__ __device__ inline int sr_aux_floats(int B, int C, int rows, int warps)
 {
     const int w = sr_width(B);
-    return 2 * kSrWarps * w + (C > 1 ? 2 * C * w : 0) + w + ((rows + 33) & ~3);
+    return 2 * warps * w + (C > 1 ? 2 * C * w : 0) + w + ((rows + 33) & ~3);
 }
 // Shared-memory rows of K for `rows` kept tokens: those and the dustbin's, in whole batches.
 __host__ __device__ inline int sr_smem_rows(int B, int rows)
@@ -71,13 +73,13 @@ __host__ __device__ inline int sr_smem_rows(int B, int rows)
 }
 // CTAs (1, 2, 4 or 8, at most C) that work on an M x B tile: enough for K to fit in their shared memory and for each to
 // have at most `spread` cells.
-__host__ __device__ inline int sr_ctas(int M, int B, int C, int smem_floats, int spread)
+__host__ __device__ inline int sr_ctas(int M, int B, int C, int smem_floats, int spread, int warps)
 {
     int c = 1;
     while (c < C) {
         const int rows = (M + c - 1) / c;
         const long long cells = (long long)sr_smem_rows(B, rows) * score_pitch(B);
-        if (cells + sr_aux_floats(B, c, rows) <= smem_floats && cells <= spread) break;
+        if (cells + sr_aux_floats(B, c, rows, warps) <= smem_floats && cells <= spread) break;
         c *= 2;
     }
     return c;
@@ -194,19 +196,20 @@ __device__ inline void sr_fetch(const SrTile &t, int c)
     ptx::mbar_arrive_expect_tx(&t.cbar[c], bytes);
     ptx::bulk_load(ptx::smem_u32(t.Ks + (size_t)lo * t.ld), t.Kg + (size_t)lo * t.ld, bytes, &t.cbar[c]);
 }
+template <int TH>
 __device__ inline void sr_build(const SrTile &t, float shift, float inv_eps, float inv_kappa, WsHeader *hdr)
 {
     const int tid = threadIdx.x;
     const float a = inv_eps * 1.4426950408889634f, b = -shift * a;
     const int qpr = t.ld >> 2;
-    const int dq = kSrThreads % qpr, q0 = tid % qpr;       // place in a row: of the thread's first chunk, and what a step adds
+    const int dq = TH % qpr, q0 = tid % qpr;       // place in a row: of the thread's first chunk, and what a step adds
     for (int c = 0; c < kSrChunks; ++c) {
         int lo, hi;
         if (!sr_chunk_rows(t, c, lo, hi)) break;
         if (!ptx::mbar_wait(&t.cbar[c], 0)) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
         float4 *k = reinterpret_cast<float4 *>(t.Ks + (size_t)lo * t.ld);
         int q = q0;
-        for (int i = tid; i < (hi - lo) * qpr; i += kSrThreads) {
+        for (int i = tid; i < (hi - lo) * qpr; i += TH) {
             k[i] = sr_k4(k[i], a, b, 4 * q, t.B);
             q += dq;
             if (q >= qpr) q -= qpr;
@@ -217,7 +220,7 @@ __device__ inline void sr_build(const SrTile &t, float shift, float inv_eps, flo
         float4 *k = reinterpret_cast<float4 *>(t.Kg + (size_t)t.cap * t.ld);
         const int n = (t.Ml - t.cap) * qpr;
         int q = q0;
-        for (int i = tid; i < n; i += 4 * kSrThreads) {
+        for (int i = tid; i < n; i += 4 * TH) {
             float4 v[4];
             int qq[4];
 #pragma unroll
@@ -225,20 +228,20 @@ __device__ inline void sr_build(const SrTile &t, float shift, float inv_eps, flo
                 qq[e] = q;
                 q += dq;
                 if (q >= qpr) q -= qpr;
-                v[e] = i + e * kSrThreads < n ? __ldcg(k + i + e * kSrThreads) : make_float4(0.f, 0.f, 0.f, 0.f);
+                v[e] = i + e * TH < n ? __ldcg(k + i + e * TH) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                if (i + e * kSrThreads < n) k[i + e * kSrThreads] = sr_k4(v[e], a, b, 4 * qq[e], t.B);
+                if (i + e * TH < n) k[i + e * TH] = sr_k4(v[e], a, b, 4 * qq[e], t.B);
         }
     }
     // the dustbin's row, and zeros up to a whole batch
     if (t.Mr > t.Ml) {
         float *p = (t.Ml < t.cap ? t.Ks : t.Kg) + (size_t)t.Ml * t.ld;
-        for (int j = tid; j < t.ld; j += kSrThreads) p[j] = j < t.B ? 1.f : (j == t.B ? inv_kappa : 0.f);
+        for (int j = tid; j < t.ld; j += TH) p[j] = j < t.B ? 1.f : (j == t.B ? inv_kappa : 0.f);
     }
     if (t.Mr < t.cap)
-        for (int j = tid; j < (t.cap - t.Mr) * t.ld; j += kSrThreads) t.Ks[(size_t)t.Mr * t.ld + j] = 0.f;
+        for (int j = tid; j < (t.cap - t.Mr) * t.ld; j += TH) t.Ks[(size_t)t.Mr * t.ld + j] = 0.f;
 }
 
 // A warp's work on a batch of BR rows: lane group `slot` takes the RB rows from base + RB * slot on.
@@ -336,7 +339,7 @@ struct SrPass {
 };
 
 // This CTA's column sums to the other CTAs at work on the image, theirs added to them, in rank order.
-template <int COLS, int W>
+template <int TH, int COLS, int W>
 __device__ inline void sr_exchange(const SrTile &t, int it, float (&tot)[COLS], WsHeader *hdr)
 {
     const int tid = threadIdx.x;
@@ -348,38 +351,38 @@ __device__ inline void sr_exchange(const SrTile &t, int it, float (&tot)[COLS], 
         const uint32_t to = ptx::map_to_rank(at, r), tobar = ptx::map_to_rank(bar, r);
 #pragma unroll
         for (int e = 0; e < COLS; ++e)
-            if (tid + e * kSrThreads <= t.B) sr_send(to + (uint32_t)(e * kSrThreads) * 4u, tot[e], tobar);
+            if (tid + e * TH <= t.B) sr_send(to + (uint32_t)(e * TH) * 4u, tot[e], tobar);
     }
     if (!ptx::mbar_wait(&t.xbar[par], ((uint32_t)it >> 1) & 1u)) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
 #pragma unroll
     for (int e = 0; e < COLS; ++e) {
-        if (tid + e * kSrThreads > t.B) continue;
+        if (tid + e * TH > t.B) continue;
         float sum = 0.f;
-        for (uint32_t r = 0; r < C; ++r) sum += r == t.rank ? tot[e] : t.xpart[(par * C + r) * W + tid + e * kSrThreads];
+        for (uint32_t r = 0; r < C; ++r) sum += r == t.rank ? tot[e] : t.xpart[(par * C + r) * W + tid + e * TH];
         tot[e] = sum;
     }
 }
 
 // The iterations.  On return vs[] holds the final V (kappa V_d at [B]) and us[] the U of this CTA's rows.
-template <int LR, int NQ, int RB>
+template <int TH, int LR, int NQ, int RB>
 __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float kappa, float v_init, WsHeader *hdr)
 {
     typedef SrPass<LR, NQ, RB> Pass;
     constexpr int W = Pass::W, BR = Pass::BR;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float Mf = (float)t.M;
-    __shared__ float2 s_range[kSrWarps];               // smallest and largest relative move of a warp's columns
-    for (int j = tid; j < W; j += kSrThreads) t.vs[j] = j < t.B ? v_init : (j == t.B ? kappa * v_init : 0.f);
+    __shared__ float2 s_range[(TH / 32)];               // smallest and largest relative move of a warp's columns
+    for (int j = tid; j < W; j += TH) t.vs[j] = j < t.B ? v_init : (j == t.B ? kappa * v_init : 0.f);
     const int nbatch = (t.Mr + BR - 1) / BR, nsmem = min(nbatch, t.cap / BR);
-    const int nwarps = min(kSrWarps, nbatch);          // warps with rows; the others' column sums stay zero
-    for (int j = nwarps * W + tid; j < kSrWarps * W; j += kSrThreads) t.part[j] = 0.f;
+    const int nwarps = min((TH / 32), nbatch);          // warps with rows; the others' column sums stay zero
+    for (int j = nwarps * W + tid; j < (TH / 32) * W; j += TH) t.part[j] = 0.f;
     __syncthreads();                                   // K, V
-    constexpr int kCols = (W + kSrThreads - 1) / kSrThreads;
+    constexpr int kCols = (W + TH - 1) / TH;
     float nv[kCols], ov[kCols];                        // this thread's columns
     int before[kCols];                                 // and their values two iterations ago
 #pragma unroll
     for (int e = 0; e < kCols; ++e) {
-        nv[e] = ov[e] = tid + e * kSrThreads < t.B ? v_init : kappa * v_init;
+        nv[e] = ov[e] = tid + e * TH < t.B ? v_init : kappa * v_init;
         before[e] = 0;
     }
     SrState st{0, 0.f};
@@ -391,14 +394,14 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
             ptx::mbar_arrive_expect_tx(&t.xbar[it & 1], (uint32_t)(t.C - 1) * (uint32_t)((t.B + 1) * 4));
         if (warp < nwarps) {
             ps.begin(t.vs);
-            for (int g = warp; g < nsmem; g += kSrWarps) {
+            for (int g = warp; g < nsmem; g += (TH / 32)) {
                 float4 k[RB][NQ];
                 ps.load_smem(t, g * BR, k);
                 ps.batch(t, g * BR, k);
             }
             if (nsmem < nbatch) {
                 // (the first batch past shared memory that is this warp's)
-                for (int g = nsmem + (warp - nsmem % kSrWarps + kSrWarps) % kSrWarps; g < nbatch; g += kSrWarps) {
+                for (int g = nsmem + (warp - nsmem % (TH / 32) + (TH / 32)) % (TH / 32); g < nbatch; g += (TH / 32)) {
                     float4 k[RB][NQ];
                     ps.load_global(t, g * BR, k);
                     ps.batch(t, g * BR, k);
@@ -435,16 +438,16 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
             float tot[kCols];
 #pragma unroll
             for (int e = 0; e < kCols; ++e) {
-                const float *part = t.part + min(tid + e * kSrThreads, W - 1);
+                const float *part = t.part + min(tid + e * TH, W - 1);
                 float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int w = 0; w < kSrWarps; ++w) c[w & 3] += part[w * W];
+                for (int w = 0; w < (TH / 32); ++w) c[w & 3] += part[w * W];
                 tot[e] = (c[0] + c[1]) + (c[2] + c[3]);
             }
-            if (t.C > 1) sr_exchange<kCols, W>(t, it, tot, hdr);
+            if (t.C > 1) sr_exchange<TH, kCols, W>(t, it, tot, hdr);
 #pragma unroll
             for (int e = 0; e < kCols; ++e) {
-                const int j = tid + e * kSrThreads;
+                const int j = tid + e * TH;
                 if (j <= t.B) {
                     ov[e] = nv[e];
                     nv[e] = (j < t.B ? 1.f : Mf) * rcp_fast(tot[e]);
@@ -463,7 +466,7 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
         if (lane == 0) s_range[warp] = make_float2(lo, hi);
         ++st.done;
         const int go = __syncthreads_or(cont);
-        const float2 range = s_range[lane % kSrWarps];         // (written again after the next iteration's first barrier)
+        const float2 range = s_range[lane % (TH / 32)];         // (written again after the next iteration's first barrier)
         lo = warp_min_redux(range.x);
         hi = warp_max_redux(range.y);
         st.last_move = fmaxf(-lo, hi);
@@ -514,7 +517,7 @@ struct SrOut {
 // Plan P = U K V of this CTA's rows: alpha P in bf16 (row = position among the kept tokens, columns up to the next
 // multiple of 64) or P in fp32 in place in the workspace tile.  In the same pass the pairing: partner_j = argmax_i P_ij
 // = argmax_i K_ij U_i, ties to the lower i.  The merge kernel may take the image before the pairs are out.
-template <int LR, int NQ, int RB>
+template <int TH, int LR, int NQ, int RB>
 __device__ inline void sr_finish(const SrTile &t, const OtParams &p, const SrOut &o, WsHeader *hdr)
 {
     typedef SrPass<LR, NQ, RB> Pass;
@@ -542,7 +545,7 @@ __device__ inline void sr_finish(const SrTile &t, const OtParams &p, const SrOut
     }
     // (rows one by one: this code runs once per image, and fetching it costs more than its latencies)
     constexpr int RPW = 32 / LR;
-    for (int i0 = warp * RPW; i0 < t.Ml; i0 += kSrWarps * RPW) {
+    for (int i0 = warp * RPW; i0 < t.Ml; i0 += (TH / 32) * RPW) {
         const int i = i0 + slot;
         if (i >= t.Ml) continue;
         const float *krow = i < t.cap ? t.Ks + (size_t)i * t.ld : t.Kg + (size_t)i * t.ld;
@@ -591,7 +594,7 @@ __device__ inline void sr_finish(const SrTile &t, const OtParams &p, const SrOut
             }
     }
     float *pv = t.part;
-    int *pi = reinterpret_cast<int *>(t.part + kSrWarps * W);
+    int *pi = reinterpret_cast<int *>(t.part + (TH / 32) * W);
     if (slot == 0) {
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
@@ -603,11 +606,11 @@ __device__ inline void sr_finish(const SrTile &t, const OtParams &p, const SrOut
     if (t.C > 1) ptx::cluster_sync_all();      // nobody reads xpart as column sums any more
     else __syncthreads();
     const uint32_t xp0 = ptx::smem_u32(t.xpart);
-    for (int j = tid; j < t.B; j += kSrThreads) {
+    for (int j = tid; j < t.B; j += TH) {
         float b = pv[j];
         int ib = pi[j];
 #pragma unroll
-        for (int w = 1; w < kSrWarps; ++w) {
+        for (int w = 1; w < (TH / 32); ++w) {
             const float ob = pv[w * W + j];
             const int oi = pi[w * W + j];
             if (ob > b || (ob == b && oi < ib)) {
@@ -629,7 +632,7 @@ __device__ inline void sr_finish(const SrTile &t, const OtParams &p, const SrOut
         ptx::cluster_sync_all();                   // after this barrier nothing is written into another CTA any more
         if (t.rank == 0) {
             const int *xi = reinterpret_cast<const int *>(t.xpart + t.C * W);
-            for (int j = tid; j < t.B; j += kSrThreads) {
+            for (int j = tid; j < t.B; j += TH) {
                 float b = t.xpart[j];
                 int ib = xi[j];
                 for (int r = 1; r < t.C; ++r) {
@@ -650,8 +653,8 @@ __device__ inline void sr_finish(const SrTile &t, const OtParams &p, const SrOut
 // grid = batch * C CTAs, clusters of C along x (C = 1: no cluster).  WIDE: tiles of up to 639 pruned tokens, else up to
 // 255.  With scores_done (per-image counts of finished score tiles) a CTA starts when its image's are in; otherwise, and
 // before rank 0 leaves, it waits for the grid ahead, so that this grid's end still implies that one's.
-template <bool WIDE>
-__global__ void __launch_bounds__(kSrThreads, 1)
+template <bool WIDE, int TH>
+__global__ void __launch_bounds__(TH, kSrThreads / TH)
 sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restrict__ counts,
                      const int32_t *__restrict__ out_offsets, const int32_t *__restrict__ order,
                      float *__restrict__ kmat, int kmat_stride, int max_tokens, int total, OtParams p, int C,
@@ -700,7 +703,7 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
         }
         return;
     }
-    t.C = sr_ctas(t.M, t.B, C, smem_floats, spread);
+    t.C = sr_ctas(t.M, t.B, C, smem_floats, spread, TH / 32);
     t.rank = rank;
     if ((int)rank >= t.C) return;
     const int rows_per = (t.M + t.C - 1) / t.C;
@@ -709,12 +712,12 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
     t.Mr = t.Ml + ((int)rank == t.C - 1 ? 1 : 0);
     t.ld = score_pitch(t.B);
     const int br = sr_batch_rows(t.B);
-    const int room = (smem_floats - sr_aux_floats(t.B, t.C, rows_per)) / t.ld;      // rows of K
+    const int room = (smem_floats - sr_aux_floats(t.B, t.C, rows_per, TH / 32)) / t.ld;      // rows of K
     t.cap = min(room / br, (t.Mr + br - 1) / br) * br;
     t.Kg = kmat + kmat_offset(kmat_stride, t_begin, img) + (size_t)t.row_lo * t.ld;
     const int w = sr_width(t.B);
     t.part = sm;
-    t.xpart = t.part + 2 * kSrWarps * w;
+    t.xpart = t.part + 2 * (TH / 32) * w;
     t.vs = t.xpart + (t.C > 1 ? 2 * t.C * w : 0);
     t.us = t.vs + w;
     t.Ks = t.us + ((rows_per + 33) & ~3);
@@ -724,7 +727,7 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
         ptx::fence_proxy_async_all();          // the scores were written with ordinary stores
         sr_fetch(t, tid);
     }
-    for (int i = tid; i < t.Ml; i += kSrThreads) t.us[i] = 1.f;      // u = 0
+    for (int i = tid; i < t.Ml; i += TH) t.us[i] = 1.f;      // u = 0
     const float inv_eps = 1.f / p.eps;
     const float shift = fmaxf(1.f, p.z);
     const float kappa = expf((p.z - shift) * inv_eps);
@@ -734,15 +737,15 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
                   merged_idx + seg, merge_partner + seg, merge_weight + seg, sink_done, ready_list, by_image != 0};
     auto solve = [&](auto lr, auto nq, auto rb) {
         constexpr int LR = decltype(lr)::value, NQ = decltype(nq)::value, RB = decltype(rb)::value;
-        sr_build(t, shift, inv_eps, 1.f / kappa, hdr);
+        sr_build<TH>(t, shift, inv_eps, 1.f / kappa, hdr);
         // every CTA at work is running and has its barriers in place before anything is sent to it
         if (t.C > 1) ptx::cluster_sync_all();
-        const SrState st = sr_iterate<LR, NQ, RB>(t, p, kappa, v_init, hdr);
+        const SrState st = sr_iterate<TH, LR, NQ, RB>(t, p, kappa, v_init, hdr);
         if (tid == 0 && rank == 0) {
             stats[(size_t)img * kStats + 5] = (float)st.done;
             stats[(size_t)img * kStats + 6] = st.last_move;
         }
-        sr_finish<LR, NQ, RB>(t, p, o, hdr);
+        sr_finish<TH, LR, NQ, RB>(t, p, o, hdr);
     };
     using std::integral_constant;
     if (t.B < 32) solve(integral_constant<int, 8>(), integral_constant<int, 1>(), integral_constant<int, 8>());
