@@ -65,7 +65,7 @@ struct rtprune_plan_s {
         const void *ws;
         int total, batch, pbuf_pitch;
         bool valid;
-        CUtensorMap scX, scXp, mgXp, mgP;
+        CUtensorMap scX, scXp, scK, mgXp, mgP;       // scK: only where kept_copy_fits
     };
     static constexpr int kMapSets = 8;
     MapSet maps[kMapSets];
@@ -247,7 +247,11 @@ bool scaling_in_range(const rtprune_params_t *p)
     return (2.f * c - lo) / p->eps <= 62.f;
 }
 
-// The four tensor maps of a bf16 run over (X, workspace): from the plan's cache, or encoded into it.
+// The copy of the kept rows that the scores of long images read lies where the plan will be: the kernels that write the plan of
+// such images start when the scores are complete.
+bool kept_copy_fits(const rtprune_plan_t *plan) { return plan->ws.pbuf_pitch_max >= plan->d; }
+
+// The tensor maps of a bf16 run over (X, workspace): from the plan's cache, or encoded into it.
 const rtprune_plan_s::MapSet *tensor_maps(rtprune_plan_t *plan, const void *X, char *ws, int total, int batch,
                                           int pbuf_pitch)
 {
@@ -267,6 +271,7 @@ const rtprune_plan_s::MapSet *tensor_maps(rtprune_plan_t *plan, const void *X, c
         !make_tmap_bf16(plan, &m.mgP, ws + L.pbuf, (uint64_t)total, (uint64_t)pbuf_pitch, (uint64_t)pbuf_pitch * 2,
                         kMgBK, kMgTileM))
         return nullptr;
+    if (kept_copy_fits(plan) && !make_tmap_bf16(plan, &m.scK, ws + L.pbuf, (uint64_t)total, d, d * 2, kScBK, kScTileM)) return nullptr;
     m.X = X;
     m.ws = ws;
     m.total = total;
@@ -469,38 +474,42 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
     }
     if (maxB > 0) {
         if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-            // compact copy of the pruned rows for the tensor-core kernels
+            // compact copy of the pruned rows for the tensor-core kernels, and of the kept ones where the scores take those
+            const bool dense = iterate && !use_log_form(params) && maxB > kSrMaxB && kept_copy_fits(plan);
             {
                 const int rows_max = (maxB + 63) & ~63;
-                dim3 ggrid((rows_max + kGpRows - 1) / kGpRows, batch);
+                const unsigned prop_ctas = (unsigned)((rows_max + kGpRows - 1) / kGpRows);
+                dim3 ggrid(prop_ctas + (dense ? (unsigned)((maxN + kGpRows - 1) / kGpRows) : 0u), batch);
                 if (!c.ok(launch_pdl(gather_prop_kernel, ggrid, dim3(128), 0, st, 1u,
                                      (const __nv_bfloat16 *)X, offsets, o.counts, order, plan->d, maxN, total,
                                      (__nv_bfloat16 *)(ws + L.xp), (uint32_t *)(ws + L.sink_done),
                                      (int32_t *)(ws + L.ready_list), (WsHeader *)(ws + L.header), batch,
-                                     o.out_offsets, (uint32_t *)(ws + L.scores_done))))
+                                     o.out_offsets, (uint32_t *)(ws + L.scores_done),
+                                     dense ? (__nv_bfloat16 *)(ws + L.pbuf) : (__nv_bfloat16 *)nullptr, (int)prop_ctas)))
                     return RTPRUNE_ERR_CUDA;
                 launched(plan, st, "gather");
             }
             // scores: one CTA per (128 consecutive tokens, image)
             const rtprune_plan_s::MapSet *ms = tensor_maps(plan, X, ws, total, batch, pbuf_pitch);
             if (!ms) return RTPRUNE_ERR_CUDA;
-            const CUtensorMap &tmapX = ms->scX, &tmapXp = ms->scXp;
+            const CUtensorMap &tmapX = dense ? ms->scK : ms->scX, &tmapXp = ms->scXp;
             dim3 grid((maxN + kScTileM - 1) / kScTileM, batch);
             // The Sinkhorn kernel can start on an image as soon as that image's score tiles are in.  That
             // costs each scores CTA a release (its stores made visible before it counts itself), which
             // pays when the grid is one wave of CTAs and its end is a tail of a few slow CTAs, not when
             // CTAs queue for the SMs.
-            if (iterate && (long long)grid.x * grid.y <= 2LL * plan->sm_count)
+            if (iterate && !dense && (long long)grid.x * grid.y <= 2LL * plan->sm_count)
                 scores_done = (uint32_t *)(ws + L.scores_done);
             // a tile's contraction over 4 CTAs while the device has SMs for them all (over 2 it gains nothing: 32 images of
             // 256 tokens 18.4 us either way; not for the one-CTA kernels of the log form and the exact pairing, which take
             // far longer than the scores)
             if (iterate && !use_log_form(params) && maxB <= kScBNMax && (long long)grid.x * grid.y * 4 <= plan->sm_count) split = 4;
-            const int ring = split == 1 && (long long)grid.x * grid.y <= plan->sm_count ? kScRingBytesAlone : kScRingBytes;
-            grid.x *= (unsigned)split;
+            const int passes = dense ? (maxB + kScBNMax - 1) / kScBNMax : 0;
+            const int ring = split == 1 && !dense && (long long)grid.x * grid.y <= plan->sm_count ? kScRingBytesAlone : kScRingBytes;
+            grid.x *= (unsigned)(dense ? passes : split);
             if (!c.ok(launch_pdl(scores_umma_kernel, grid, dim3(kScThreads), (size_t)(scores_smem_bytes(ring) + scores_split_bytes(split)), st, (unsigned)split, tmapX, tmapXp,
                                  offsets, plan->d, o.counts, order, (const int32_t *)(ws + L.kpos), norms, kmat,
-                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, use_reg ? 0 : 1, ring, split)))
+                                 L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, use_reg ? 0 : 1, ring, split, passes)))
                 return RTPRUNE_ERR_CUDA;
         } else {
             const int btiles = (maxB + kF3Tile - 1) / kF3Tile, mtiles = (maxN + kF3Tile - 1) / kF3Tile;

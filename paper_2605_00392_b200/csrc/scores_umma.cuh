@@ -17,6 +17,9 @@
 // TMA unit takes in about 31 bytes per clock (480 KB of a 128 x 64 tile: 8 us).  Their partial sums are reduce-scattered
 // over the cluster by units of 16 columns through distributed shared memory and added in rank order.
 // The ring is sized so that two CTAs share an SM: a whole Large batch is one wave.
+// Dense (passes > 0): tiles of 128 kept tokens, from a copy of the kept rows that the kernel ahead made, and a CTA per tile and
+// pass of 256 pruned columns.  For images of more than 639 pruned tokens, where a copy costs less than the contraction of the
+// pruned rows with themselves (two fifths of it at r = 0.4), and a CTA with all the passes of a tile would leave SMs idle.
 #pragma once
 #include "common.cuh"
 #include "ptx.cuh"
@@ -60,11 +63,12 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                    const int32_t *__restrict__ order, const int32_t *__restrict__ kpos,
                    const float *__restrict__ norms, float *__restrict__ kmat, int kmat_stride,
                    int max_tokens, int total, WsHeader *__restrict__ hdr, uint32_t *__restrict__ scores_done,
-                   int bulk_readers, int ring_bytes, int split)
+                   int bulk_readers, int ring_bytes, int split, int passes)
 {
     extern __shared__ uint8_t smem_raw[];
-    const int img = blockIdx.y, mt = split > 1 ? blockIdx.x / split : blockIdx.x;
-    const int rank = blockIdx.x - mt * split;     // in the cluster of a split tile
+    const bool dense = passes > 0;
+    const int img = blockIdx.y, mt = dense ? blockIdx.x / passes : split > 1 ? blockIdx.x / split : blockIdx.x;
+    const int rank = dense ? 0 : blockIdx.x - mt * split;     // in the cluster of a split tile
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     ScoresBarriers *bars = reinterpret_cast<ScoresBarriers *>(smem + ring_bytes);
@@ -104,7 +108,8 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
     // With scores_done, every tile of a valid image is counted when it is complete (at once if nothing is
     // pruned): the Sinkhorn kernel, launched as a programmatic dependent, starts on an image when its
     // tiles are in.
-    if (B == 0) {
+    const int pass0 = dense ? blockIdx.x - mt * passes : 0;       // first pass of this CTA
+    if (B == 0 || (dense && (mt * kScTileM >= M || pass0 * kScBNMax >= B))) {
         if (split > 1) ptx::cluster_wait_started();
         if (scores_done && tid == 0) atomicAdd(&scores_done[img], 1u);
         if (warp == 5) ptx::tmem_dealloc(tmem_base, kScBNMax);
@@ -117,7 +122,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
     const int kScStages = min(kScMaxStages, ring_bytes / stage_bytes);   // 2 .. 8
     const int nkb_all = (d + kScBK - 1) / kScBK, nkb_per = (nkb_all + split - 1) / split;
     const int kb_lo = rank * nkb_per, nkb = max(0, min(nkb_all, kb_lo + nkb_per) - kb_lo);       // this CTA's k-blocks
-    const int nbt = (B + kScBNMax - 1) / kScBNMax;
+    const int nbt = dense ? 1 : (B + kScBNMax - 1) / kScBNMax;      // passes of this CTA
     const int32_t *ord = order + t_begin;
     const int xp0 = xp_row0(t_begin, img);
 
@@ -130,7 +135,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
             uint32_t it = 0;
             bool alive = true;
             for (int bt = 0; bt < nbt && alive && !bars->abort_flag; ++bt) {
-                const int nbox = (min(kScBNMax, B - bt * kScBNMax) + kScBBoxRows - 1) / kScBBoxRows;
+                const int j0 = (pass0 + bt) * kScBNMax, nbox = (min(kScBNMax, B - j0) + kScBBoxRows - 1) / kScBBoxRows;
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % kScStages;
                     const bool ok = it < (uint32_t)kScStages || ptx::mbar_wait(&bars->empty[s], ((it / kScStages) - 1) & 1);
@@ -147,7 +152,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                         ptx::tma_load_2d(a_dst, &tmapX, &bars->full[s], (kb_lo + kb) * kScBK, t_begin + mt * kScTileM);
                     else if (lane <= nbox)
                         ptx::tma_load_2d(a_dst + kScABytes + (lane - 1) * kScBBoxBytes, &tmapXp, &bars->full[s],
-                                         (kb_lo + kb) * kScBK, xp0 + bt * kScBNMax + (lane - 1) * kScBBoxRows);
+                                         (kb_lo + kb) * kScBK, xp0 + j0 + (lane - 1) * kScBBoxRows);
                 }
             }
         }
@@ -156,7 +161,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
         if (lane == 0) {
             uint32_t it = 0;
             for (int bt = 0; bt < nbt && !bars->abort_flag; ++bt) {
-                const int BN = min(kScBNMax, (B - bt * kScBNMax + 15) & ~15);
+                const int BN = min(kScBNMax, (B - (pass0 + bt) * kScBNMax + 15) & ~15);
                 const uint32_t idesc = ptx::idesc_bf16(kScTileM, BN, false, false);
                 if (bt > 0) {
                     if (!ptx::mbar_wait(&bars->tmem_empty, (bt - 1) & 1)) {
@@ -193,11 +198,11 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
         const int ldS = score_pitch(B);
         const int row = tid;                       // TMEM lane = tile row
         const int k_tok = mt * kScTileM + row;
-        const int p = (k_tok < N) ? kpos[t_begin + k_tok] : -1;
-        const float inv_ni = (p >= 0) ? 1.f / fmaxf(norms[t_begin + k_tok], kNormFloor) : 1.f;
+        const int p = dense ? (k_tok < M ? k_tok : -1) : (k_tok < N) ? kpos[t_begin + k_tok] : -1;
+        const float inv_ni = (p >= 0) ? 1.f / fmaxf(norms[t_begin + (dense ? ord[p] : k_tok)], kNormFloor) : 1.f;
         bool dead = false;     // a wait gave up: keep taking the named barriers, skip the rest
         for (int bt = 0; bt < nbt; ++bt) {
-            const int j0 = bt * kScBNMax;
+            const int j0 = (pass0 + bt) * kScBNMax;
             const int BN = min(kScBNMax, (B - j0 + 15) & ~15);
             // 1/|x_j| of this pass's columns, shared by the 128 epilogue threads (the first barrier
             // keeps a fast warp from overwriting values a slow one still reads)

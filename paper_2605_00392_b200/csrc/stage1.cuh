@@ -671,7 +671,8 @@ stage1_kernel(const T *__restrict__ X, const int32_t *__restrict__ offsets, int 
 // Compact copy of T_prop for the tensor-core kernels (bf16 storage): image i's B pruned rows, in
 // ascending token order, at rows xp_row0(offsets[i], i) .., then rows of zeros up to a multiple of
 // 64 so that whole 64-row tiles can be fetched.  grid = (ceil(max rows / 8), batch), 128 threads:
-// a warp copies two rows, all ten loads of a lane issued before the stores.  (As __ldg loads they were at the compiler's
+// a warp copies two rows, all ten loads of a lane issued before the stores.  With xk, further CTAs copy the kept rows too: row
+// offsets[i] + position among the kept.  (As __ldg loads they were at the compiler's
 // mercy: with the fp32 kernels in the same translation unit it took them a few at a time, in 40 registers, and 64 x 400
 // tokens 106.2 us instead of 105.3.)
 // ---------------------------------------------------------------------------------------------
@@ -681,7 +682,7 @@ gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restri
                    const int32_t *__restrict__ counts, const int32_t *__restrict__ order, int d,
                    int max_tokens, int total, __nv_bfloat16 *__restrict__ xp, uint32_t *__restrict__ sink_done,
                    int32_t *__restrict__ ready_list, WsHeader *__restrict__ hdr, int batch,
-                   int32_t *__restrict__ out_offsets, uint32_t *__restrict__ scores_done)
+                   int32_t *__restrict__ out_offsets, uint32_t *__restrict__ scores_done, __nv_bfloat16 *__restrict__ xk, int prop_ctas)
 {
     __shared__ int s_scan[32];
     // the last images first: what stage 1 read last is what L2 still holds
@@ -712,16 +713,18 @@ gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restri
         if (threadIdx.x == 0) ptx::st_release_gpu(&hdr->run_tag, ptx::ld_acquire_gpu(&hdr->launch_seq));
     }
     if (!valid) return;
-    const int M = M_img, B = N - M, Bpad = (B + 63) & ~63;
-    const int j0 = blockIdx.x * kGpRows + (threadIdx.x >> 5) * 2;
-    if (j0 >= Bpad) return;
+    const bool kept = (int)blockIdx.x >= prop_ctas;
+    const int M = M_img, rows = kept ? M : N - M, rows_pad = kept ? M : (N - M + 63) & ~63;
+    const int j0 = ((int)blockIdx.x - (kept ? prop_ctas : 0)) * kGpRows + (threadIdx.x >> 5) * 2;
+    if (j0 >= rows_pad) return;
     const int lane = threadIdx.x & 31;
     const int nvec = d >> 3;
-    uint4 *seg = reinterpret_cast<uint4 *>(xp + (size_t)xp_row0(t_begin, img) * d);
+    uint4 *seg = reinterpret_cast<uint4 *>(kept ? xk + (size_t)t_begin * d : xp + (size_t)xp_row0(t_begin, img) * d);
+    const int32_t *ord = order + t_begin + (kept ? 0 : M);
     int src_row[2];
 #pragma unroll
     for (int a = 0; a < 2; ++a)
-        src_row[a] = (j0 + a < B) ? t_begin + __ldg(order + t_begin + M + j0 + a) : -1;
+        src_row[a] = (j0 + a < rows) ? t_begin + __ldg(ord + j0 + a) : -1;
     for (int v0 = lane; v0 < nvec; v0 += 32 * 5) {
         uint4 t[2][5];
 #pragma unroll
@@ -738,7 +741,7 @@ gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restri
 #pragma unroll
             for (int b = 0; b < 5; ++b) {
                 const int v = v0 + 32 * b;
-                if (j0 + a < Bpad && v < nvec) seg[(size_t)(j0 + a) * nvec + v] = t[a][b];
+                if (j0 + a < rows_pad && v < nvec) seg[(size_t)(j0 + a) * nvec + v] = t[a][b];
             }
     }
 }

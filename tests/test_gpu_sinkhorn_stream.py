@@ -43,3 +43,13 @@ def test_without_a_cluster_of_the_kernel_the_one_for_wider_tiles_runs(lengths, d
         plan.profile_enable(False)
     finally:
         plan.close()
+
+
+# Scores from the copy of the kept rows (more than 639 pruned tokens possible, room for d columns in a plan row of max_tokens
+# rounded up to 64): kept rows around a whole number of 128-row tiles, pruned ones around whole passes of 256 columns, an image
+# that another kernel solves and some with next to nothing to prune beside them; the last has no room for the copy.
+@pytest.mark.parametrize("lengths,r,d", [([1536, 1538, 1300, 1, 40], 0.5, 1280), ([1408, 1406], 0.5, 1408), ([1400, 60], 0.5, 1416)])
+def test_scores_of_kept_rows(lengths, r, d):
+    import parity
+    w = synth.ragged(lengths, d=d, dtype=torch.bfloat16, params=dict(r_fixed=r, iters=10))
+    parity.check_workload(w)
