@@ -480,12 +480,15 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                 const int rows_max = (maxB + 63) & ~63;
                 const unsigned prop_ctas = (unsigned)((rows_max + kGpRows - 1) / kGpRows);
                 dim3 ggrid(prop_ctas + (dense ? (unsigned)((maxN + kGpRows - 1) / kGpRows) : 0u), batch);
-                if (!c.ok(launch_pdl(gather_prop_kernel, ggrid, dim3(128), 0, st, 1u,
+                // in the smallest batches the bookkeeping has a CTA to itself: 1 x 64 tokens 37.3 -> 36.6 us, 1 x 400 47.2 -> 46.4, 4 x
+                // 300-400 54.5 -> 53.8; 32 x 256 the same, 36 x 400 would lose 1.2
+                const int book = batch <= 8 ? (int)ggrid.x++ : 0;
+                if (!c.ok(launch_pdl(dense ? gather_prop_kernel<true> : gather_prop_kernel<false>, ggrid, dim3(128), 0, st, 1u,
                                      (const __nv_bfloat16 *)X, offsets, o.counts, order, plan->d, maxN, total,
                                      (__nv_bfloat16 *)(ws + L.xp), (uint32_t *)(ws + L.sink_done),
                                      (int32_t *)(ws + L.ready_list), (WsHeader *)(ws + L.header), batch,
                                      o.out_offsets, (uint32_t *)(ws + L.scores_done),
-                                     dense ? (__nv_bfloat16 *)(ws + L.pbuf) : (__nv_bfloat16 *)nullptr, (int)prop_ctas)))
+                                     dense ? (__nv_bfloat16 *)(ws + L.pbuf) : (__nv_bfloat16 *)nullptr, (int)prop_ctas, book)))
                     return RTPRUNE_ERR_CUDA;
                 launched(plan, st, "gather");
             }
@@ -507,7 +510,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             const int passes = dense ? (maxB + kScBNMax - 1) / kScBNMax : 0;
             const int ring = split == 1 && !dense && (long long)grid.x * grid.y <= plan->sm_count ? kScRingBytesAlone : kScRingBytes;
             grid.x *= (unsigned)(dense ? passes : split);
-            if (!c.ok(launch_pdl(scores_umma_kernel, grid, dim3(kScThreads), (size_t)(scores_smem_bytes(ring) + scores_split_bytes(split)), st, (unsigned)split, tmapX, tmapXp,
+            if (!c.ok(launch_pdl(dense ? scores_umma_kernel<true> : scores_umma_kernel<false>, grid, dim3(kScThreads), (size_t)(scores_smem_bytes(ring) + scores_split_bytes(split)), st, (unsigned)split, tmapX, tmapXp,
                                  offsets, plan->d, o.counts, order, (const int32_t *)(ws + L.kpos), norms, kmat,
                                  L.kmat_stride, maxN, total, (WsHeader *)(ws + L.header), scores_done, use_reg ? 0 : 1, ring, split, passes)))
                 return RTPRUNE_ERR_CUDA;
@@ -681,8 +684,11 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
         const int nct = (plan->d + kMgTileN - 1) / kMgTileN;
         const long long nunits = (long long)batch * mtiles_m * nct;
         const int grid = (int)std::min<long long>(nunits, plan->sm_count);
-        // shared memory for a deep ring of k-blocks where an image has many, else for more tiles of own rows
-        const int mg_stages = maxB > kMgDeepB ? 3 : 2, mg_bufs = maxB > kMgDeepB ? 2 : 4;
+        // shared memory for a deep ring of k-blocks where an image has many, else for more tiles of own rows (with a dynamic ratio
+        // most images prune far less than the most they may: 128 of 456-1156 tokens 418 -> 416 us with the latter, but 40 of
+        // 1000-1156 at r = 0.48 323 -> 332)
+        const bool deep = maxB > kSrMaxB || (maxB > kMgDeepB && !params->dynamic);
+        const int mg_stages = deep ? 3 : 2, mg_bufs = deep ? 2 : 4;
         if (!c.ok(launch_pdl(merge_umma_kernel, dim3((unsigned)grid), dim3(kMgThreads), (size_t)merge_smem_bytes(mg_stages, mg_bufs), st, 1u,
                              tmapXpm, tmapP, (const __nv_bfloat16 *)X, offsets, plan->d, batch, mtiles_m, o.counts, o.out_offsets,
                              (const int32_t *)order, maxN, total, (__nv_bfloat16 *)o.Y, o.kept_idx,
@@ -1009,7 +1015,8 @@ rtprune_status_t rtprune_plan(rtprune_plan_t **plan_out, int32_t d, rtprune_dtyp
     }
     if (dtype == RTPRUNE_BF16) {
         if (!p->encode_tiled ||
-            !c.ok(cudaFuncSetAttribute(scores_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            !c.ok(cudaFuncSetAttribute(scores_umma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, scores_smem_bytes(kScRingBytes))) ||
+            !c.ok(cudaFuncSetAttribute(scores_umma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        std::max(scores_smem_bytes(kScRingBytesAlone),
                                                 scores_smem_bytes(kScRingBytes) + scores_split_bytes(4)))) ||
             !c.ok(cudaFuncSetAttribute(merge_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

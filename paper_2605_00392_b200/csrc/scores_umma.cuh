@@ -17,7 +17,7 @@
 // TMA unit takes in about 31 bytes per clock (480 KB of a 128 x 64 tile: 8 us).  Their partial sums are reduce-scattered
 // over the cluster by units of 16 columns through distributed shared memory and added in rank order.
 // The ring is sized so that two CTAs share an SM: a whole Large batch is one wave.
-// Dense (passes > 0): tiles of 128 kept tokens, from a copy of the kept rows that the kernel ahead made, and a CTA per tile and
+// DENSE: tiles of 128 kept tokens, from a copy of the kept rows that the kernel ahead made, and a CTA per tile and
 // pass of 256 pruned columns.  For images of more than 639 pruned tokens, where a copy costs less than the contraction of the
 // pruned rows with themselves (two fifths of it at r = 0.4), and a CTA with all the passes of a tile would leave SMs idle.
 #pragma once
@@ -57,6 +57,7 @@ struct ScoresBarriers {
     float inv_nj[kScBNMax];          // 1 / |x_j| of the current pass's pruned tokens
 };
 
+template <bool DENSE>
 __global__ void __launch_bounds__(kScThreads, 2)
 scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_constant__ CUtensorMap tmapXp,
                    const int32_t *__restrict__ offsets, int d, const int32_t *__restrict__ counts,
@@ -66,7 +67,7 @@ scores_umma_kernel(const __grid_constant__ CUtensorMap tmapX, const __grid_const
                    int bulk_readers, int ring_bytes, int split, int passes)
 {
     extern __shared__ uint8_t smem_raw[];
-    const bool dense = passes > 0;
+    constexpr bool dense = DENSE;
     const int img = blockIdx.y, mt = dense ? blockIdx.x / passes : split > 1 ? blockIdx.x / split : blockIdx.x;
     const int rank = dense ? 0 : blockIdx.x - mt * split;     // in the cluster of a split tile
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;

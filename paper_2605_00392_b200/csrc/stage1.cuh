@@ -671,18 +671,19 @@ stage1_kernel(const T *__restrict__ X, const int32_t *__restrict__ offsets, int 
 // Compact copy of T_prop for the tensor-core kernels (bf16 storage): image i's B pruned rows, in
 // ascending token order, at rows xp_row0(offsets[i], i) .., then rows of zeros up to a multiple of
 // 64 so that whole 64-row tiles can be fetched.  grid = (ceil(max rows / 8), batch), 128 threads:
-// a warp copies two rows, all ten loads of a lane issued before the stores.  With xk, further CTAs copy the kept rows too: row
+// a warp copies two rows, all ten loads of a lane issued before the stores.  KEPT: further CTAs copy the kept rows to xk: row
 // offsets[i] + position among the kept.  (As __ldg loads they were at the compiler's
 // mercy: with the fp32 kernels in the same translation unit it took them a few at a time, in 40 registers, and 64 x 400
 // tokens 106.2 us instead of 105.3.)
 // ---------------------------------------------------------------------------------------------
 constexpr int kGpRows = 8;     // rows per CTA: four warps, two rows each
+template <bool KEPT>
 __global__ void __launch_bounds__(128)
 gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restrict__ offsets,
                    const int32_t *__restrict__ counts, const int32_t *__restrict__ order, int d,
                    int max_tokens, int total, __nv_bfloat16 *__restrict__ xp, uint32_t *__restrict__ sink_done,
                    int32_t *__restrict__ ready_list, WsHeader *__restrict__ hdr, int batch,
-                   int32_t *__restrict__ out_offsets, uint32_t *__restrict__ scores_done, __nv_bfloat16 *__restrict__ xk, int prop_ctas)
+                   int32_t *__restrict__ out_offsets, uint32_t *__restrict__ scores_done, __nv_bfloat16 *__restrict__ xk, int prop_ctas, int book)
 {
     __shared__ int s_scan[32];
     // the last images first: what stage 1 read last is what L2 still holds
@@ -692,12 +693,13 @@ gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restri
     const bool valid = image_range(offsets, img, max_tokens, total, t_begin, N);     // (inputs of the run)
     ptx::grid_dep_wait();     // counts and order come from the kernel ahead
     const int M_img = __ldcg(counts + img);
-    // One CTA prepares what the kernels behind this one share through the workspace, while the others
+    // One CTA (book: the first, which then copies like the others, or one of its own) prepares what the kernels behind this one
+    // share through the workspace, while the others
     // copy: it empties the per-image counters and the list of finished plans, turns the counts into out_offsets, then
     // publishes the run's number.  Kernels launched as programmatic dependents may already be resident and must not read
     // those words before they see that number: until then they hold what the run before left.  (That
     // run has ended: it is ahead of stage 1 in the stream.)
-    if (blockIdx.x == 0 && blockIdx.y == 0) {
+    if ((int)blockIdx.x == book && blockIdx.y == 0) {
         for (int i = threadIdx.x; i < batch; i += 128) {
             sink_done[i] = 0;
             scores_done[i] = 0;
@@ -712,8 +714,8 @@ gather_prop_kernel(const __nv_bfloat16 *__restrict__ Xb, const int32_t *__restri
         __syncthreads();
         if (threadIdx.x == 0) ptx::st_release_gpu(&hdr->run_tag, ptx::ld_acquire_gpu(&hdr->launch_seq));
     }
-    if (!valid) return;
-    const bool kept = (int)blockIdx.x >= prop_ctas;
+    if (!valid || (book > 0 && (int)blockIdx.x == book)) return;
+    const bool kept = KEPT && (int)blockIdx.x >= prop_ctas;
     const int M = M_img, rows = kept ? M : N - M, rows_pad = kept ? M : (N - M + 63) & ~63;
     const int j0 = ((int)blockIdx.x - (kept ? prop_ctas : 0)) * kGpRows + (threadIdx.x >> 5) * 2;
     if (j0 >= rows_pad) return;
