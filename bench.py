@@ -36,8 +36,8 @@ FP32_FMA_PEAK_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12   # SMs x FP32 lanes x 2 f
 REFERENCE_SAMPLE = 64      # images per step of the --impl reference arm: the whole Large batch, as cpu_baseline
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from an ncu capture (profiles/), by kernel
 # (kernels changed since their capture, or never captured, have no entry and report null)
-NCU_TRAFFIC_BYTES = {"stage1": 65876224, "gather": 10372864, "scores": 86270720, "sinkhorn_reg": 4948992,
-                     "merge": 117271040, "density_tile": 318164992}
+NCU_TRAFFIC_BYTES = {"stage1": 65616128, "gather": 17652480, "scores": 89325568, "sinkhorn_reg": 7470336,
+                     "merge": 91571712, "density_tile": 318164992}
 
 
 def cpu_threads() -> int:
