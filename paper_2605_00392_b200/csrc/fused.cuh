@@ -316,7 +316,7 @@ __device__ inline FuIterState fused_iterate(const float4 (&k)[NS][CPL / 4], floa
         const float2 range = sh->range[lane % kFuWarps];       // (written again after the next iteration's first barrier)
         lo = warp_min_redux(range.x);
         hi = warp_max_redux(range.y);
-        st.last_move = fmaxf(-lo, hi);
+        st.last_move = fmaxf(0.f, fmaxf(-lo, hi));              // (0 where every dual is NaN)
         if (!go || (p.tol == 0.f && p.stop_fp && plan_settled(lo, hi))) {
             ++round;
             break;

@@ -469,7 +469,7 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
         const float2 range = s_range[lane % (TH / 32)];         // (written again after the next iteration's first barrier)
         lo = warp_min_redux(range.x);
         hi = warp_max_redux(range.y);
-        st.last_move = fmaxf(-lo, hi);
+        st.last_move = fmaxf(0.f, fmaxf(-lo, hi));              // (0 where every dual is NaN)
         if (!go || (p.tol == 0.f && p.stop_fp && plan_settled(lo, hi))) break;
     }
     return st;

@@ -125,3 +125,27 @@ def test_exit_at_small_eps(binding, lengths, dtype, d, r, kernel, eps):
     for i in range(nb):
         s = slice(int(offs[i] - kept[i]), int(offs[i + 1] - kept[i + 1]))
         assert np.all(np.abs(wa[s] - wb[s]) <= (2 * step * (100 - k[i]) + 16) * units * wb[s]), (i, k[i], np.max(np.abs(wa[s] / wb[s] - 1)) / units)
+
+
+# A token that is not a number (reported by the status word): its image leaves the loop when its duals, all NaN, repeat, and
+# reports no move; the other images are what they are without it.
+@pytest.mark.parametrize("batch,kernel", [(4, "sinkhorn_reg"), (160, "sinkhorn_rows")])
+def test_an_image_that_is_not_a_number(binding, batch, kernel):
+    dev = torch.device("cuda", 0)
+    w = synth.ragged([100] * batch, d=1280, params=dict(r_fixed=0.25))
+    plan = binding.Plan(w.d, w.X.dtype, w.batch, w.total_tokens, w.max_tokens, device=dev)
+    X, offs = w.X.to(dev), torch.from_numpy(w.offsets.copy()).to(dev)
+    params = binding.make_params(None, r_fixed=0.25)
+    outs = [binding.Outputs.allocate(w.total_tokens, w.batch, w.d, w.X.dtype, dev) for _ in range(2)]
+    plan.profile_enable(True)
+    plan.run(X, offs, params, outs[0])
+    assert plan.query_status() == 0 and kernel in [n for n, _ in plan.profile_read()]
+    X[int(outs[0].merged_idx[3]), 5] = float("nan")            # a pruned token of the first image
+    plan.run(X, offs, params, outs[1])
+    assert plan.query_status() == binding.DEV_NONFINITE
+    plan.profile_enable(False)
+    plan.close()
+    a, b = outs
+    assert torch.isnan(b.stats[0, 0]) and b.stats[0, 5:7].tolist() == [2.0, 0.0]
+    assert torch.equal(a.stats[1:], b.stats[1:]) and torch.equal(a.kept_idx[75:], b.kept_idx[75:])
+    assert torch.equal(a.Y[75:75 * batch], b.Y[75:75 * batch]) and torch.equal(a.merge_weight[25:25 * batch], b.merge_weight[25:25 * batch])

@@ -24,7 +24,13 @@ def settled(tmp_path_factory):
     def run(now, last):
         rel = (now - last) / last                     # float32, as the kernels take it
         return bool(fn(float(rel.min()), float(rel.max())))
+    run.rule = lambda lo, hi: bool(fn(lo, hi))
     return run
+
+
+def test_columns_without_a_number_leave_the_rule_for_single_duals_to_decide(settled):
+    assert not settled.rule(float("inf"), float("-inf")) and not settled.rule(float("nan"), float("nan"))
+    assert settled.rule(0.0, 0.0) and settled.rule(-1e-7, 1e-7) and not settled.rule(-1e-6, 1e-6)
 
 
 @pytest.mark.parametrize("columns", [2, 17, 640])
