@@ -251,6 +251,24 @@ bool scaling_in_range(const rtprune_params_t *p)
 // such images start when the scores are complete.
 bool kept_copy_fits(const rtprune_plan_t *plan) { return plan->ws.pbuf_pitch_max >= plan->d; }
 
+// Whether the scores of a run that may prune more than kSrMaxB tokens of an image read such a copy, a CTA per tile and pass.  What
+// may be pruned follows from the plan; what there is to gain from the images, of which the host knows the mean length n.  In the
+// first case the CTAs are few and the passes spread the work.  In the others the CTAs beyond an image's own tiles and passes must
+// not be most of them (plan made for longer images), and either the tiles alone would leave half the device idle, or the copy (of
+// n - b rows) has to cost less than the pruned rows' contraction with themselves (b of them; with a dynamic ratio images prune
+// about 0.4 of the most they may).  Copy + scores, event times, token tiles -> kept rows: 2 x 1000 tokens, plan for 4512, 40 -> 31 us;
+// 16 x 1400 dynamic 68 -> 58; 16 x 2700, plan for 4512, 230 -> 154; 32 x 2137 at r = 0.31 186 -> 175; but 64 x 400, plan for
+// 4512, 64 -> 190, 200 x 100 likewise 121 -> 526, 32 x 4512 at r = 0.15 382 -> 407, 64 x 1400 dynamic 148 -> 170.
+bool scores_of_kept_rows(const rtprune_plan_t *plan, const rtprune_params_t *p, int batch, int total, int maxB)
+{
+    if (maxB <= kSrMaxB || !kept_copy_fits(plan)) return false;
+    const long long tiles = (long long)batch * ((plan->max_tokens + kScTileM - 1) / kScTileM);
+    const long long slots = 2LL * plan->sm_count;
+    if (tiles * ((maxB + kScBNMax - 1) / kScBNMax) <= 2 * slots) return true;
+    const double n = (double)total / batch, b = n * (p->dynamic ? 0.4 * std::fmin(p->r_max, 1.f) : p->r_fixed);
+    return 2.0 * n >= plan->max_tokens && (tiles <= slots || b * b >= 150.0 * (n - b));
+}
+
 // The tensor maps of a bf16 run over (X, workspace): from the plan's cache, or encoded into it.
 const rtprune_plan_s::MapSet *tensor_maps(rtprune_plan_t *plan, const void *X, char *ws, int total, int batch,
                                           int pbuf_pitch)
@@ -451,6 +469,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
     const int pbuf_pitch = (std::max(maxB, 1) + 63) / 64 * 64;   // <= L.pbuf_pitch_max
     int32_t *ready_list = nullptr;   // images in the order their plans are finished, when the merge follows it
     int split = 1;                   // CTAs per tile of the scores (1 or 4)
+    bool dense = false;              // the scores read a copy of the kept rows
     // the merge has a CTA for every unit: each waits for its own image, no order of completion
     const long long merge_units = (long long)batch * ((maxN + kMgTileM - 1) / kMgTileM) * ((plan->d + kMgTileN - 1) / kMgTileN);
     const int by_image = merge_units <= plan->sm_count ? 1 : 0;
@@ -480,7 +499,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
     if (maxB > 0) {
         if constexpr (std::is_same<T, __nv_bfloat16>::value) {
             // compact copy of the pruned rows for the tensor-core kernels, and of the kept ones where the scores take those
-            const bool dense = iterate && !use_log_form(params) && maxB > kSrMaxB && kept_copy_fits(plan);
+            dense = iterate && !use_log_form(params) && scores_of_kept_rows(plan, params, batch, total, maxB);
             {
                 const int rows_max = (maxB + 63) & ~63;
                 const unsigned prop_ctas = (unsigned)((rows_max + kGpRows - 1) / kGpRows);
@@ -528,7 +547,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                 return RTPRUNE_ERR_CUDA;
         }
         if (!c.ok(cudaGetLastError())) return RTPRUNE_ERR_CUDA;
-        launched(plan, st, "scores");
+        launched(plan, st, dense ? "scores_kept" : "scores");
 
         OtParams op{params->z, params->alpha, params->eps, params->iters,
                     params->stop_at_fixed_point, params->tol};
