@@ -123,17 +123,29 @@ __device__ inline float warp_max(float x)
     return x;
 }
 
-// Smallest and largest value over a warp, in one instruction each (a NaN counts as no value).
+// Smallest and largest value over a warp, in one instruction each, and of two values (NaN if one of them is).
 __device__ inline float warp_min_redux(float x)
 {
     float r;
-    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    asm volatile("redux.sync.min.NaN.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
     return r;
 }
 __device__ inline float warp_max_redux(float x)
 {
     float r;
-    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ inline float min_nan(float a, float b)
+{
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ inline float max_nan(float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
     return r;
 }
 

@@ -316,7 +316,7 @@ __device__ inline FuIterState fused_iterate(const float4 (&k)[NS][CPL / 4], floa
         const float2 range = sh->range[lane % kFuWarps];       // (written again after the next iteration's first barrier)
         lo = warp_min_redux(range.x);
         hi = warp_max_redux(range.y);
-        st.last_move = fmaxf(0.f, fmaxf(-lo, hi));              // (0 where every dual is NaN)
+        st.last_move = fmaxf(-lo, hi);
         if (!go || (p.tol == 0.f && p.stop_fp && plan_settled(lo, hi))) {
             ++round;
             break;
@@ -784,7 +784,7 @@ stage2_fused_kernel(const __nv_bfloat16 *__restrict__ X, const int32_t *__restri
 #undef RTP_FU
             if (tid == 0 && rank == 0) {
                 stats[(size_t)img * kStats + 5] = (float)ist.done;
-                stats[(size_t)img * kStats + 6] = ist.last_move;
+                stats[(size_t)img * kStats + 6] = fmaxf(ist.last_move, 0.f);      // (0 where every dual is NaN)
             }
             ptx::fence_proxy_async_smem();     // the plan arrays (ordinary stores) feed UMMAs
         }

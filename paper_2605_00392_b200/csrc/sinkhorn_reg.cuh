@@ -213,7 +213,7 @@ sinkhorn_reg_kernel(const int32_t *__restrict__ offsets, const int32_t *__restri
 #undef RTP_RG
     if (tid == 0 && rank == 0) {
         stats[(size_t)img * kStats + 5] = (float)ist.done;
-        stats[(size_t)img * kStats + 6] = ist.last_move;
+        stats[(size_t)img * kStats + 6] = fmaxf(ist.last_move, 0.f);      // (0 where every dual is NaN)
     }
     ptx::cluster_sync_all();          // the pairing partials are with rank 0; nothing is sent to another CTA after this
     if (rank == 0) {

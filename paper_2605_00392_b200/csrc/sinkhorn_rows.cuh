@@ -453,8 +453,8 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
                     nv[e] = (j < t.B ? 1.f : Mf) * rcp_fast(tot[e]);
                     t.vs[j] = nv[e];
                     const float rel = (nv[e] - ov[e]) * rcp_fast(ov[e]);
-                    lo = fminf(lo, rel);
-                    hi = fmaxf(hi, rel);
+                    lo = e == 0 ? rel : min_nan(lo, rel);
+                    hi = e == 0 ? rel : max_nan(hi, rel);
                     cont |= p.tol > 0.f ? (fabsf(nv[e] - ov[e]) > p.tol * ov[e])
                                         : (!p.stop_fp || !dual_settled(__float_as_int(nv[e]), __float_as_int(ov[e]), before[e]));
                     before[e] = __float_as_int(ov[e]);
@@ -469,7 +469,7 @@ __device__ inline SrState sr_iterate(const SrTile &t, const OtParams &p, float k
         const float2 range = s_range[lane % (TH / 32)];         // (written again after the next iteration's first barrier)
         lo = warp_min_redux(range.x);
         hi = warp_max_redux(range.y);
-        st.last_move = fmaxf(0.f, fmaxf(-lo, hi));              // (0 where every dual is NaN)
+        st.last_move = fmaxf(-lo, hi);
         if (!go || (p.tol == 0.f && p.stop_fp && plan_settled(lo, hi))) break;
     }
     return st;
@@ -743,7 +743,7 @@ sinkhorn_rows_kernel(const int32_t *__restrict__ offsets, const int32_t *__restr
         const SrState st = sr_iterate<TH, LR, NQ, RB>(t, p, kappa, v_init, hdr);
         if (tid == 0 && rank == 0) {
             stats[(size_t)img * kStats + 5] = (float)st.done;
-            stats[(size_t)img * kStats + 6] = st.last_move;
+            stats[(size_t)img * kStats + 6] = fmaxf(st.last_move, 0.f);      // (0 where every dual is NaN)
         }
         sr_finish<TH, LR, NQ, RB>(t, p, o, hdr);
     };
