@@ -650,6 +650,7 @@ def main() -> None:
             "scores": ("hbm", x_bytes + xp_bytes + 4 * sumMB),
             "sinkhorn_rows": ("alu", sink_flops),
             "sinkhorn_rows_wide": ("alu", sink_flops),
+            "sinkhorn_rows_half": ("alu", sink_flops),
             "sinkhorn_reg": ("alu", sink_flops),
             "sinkhorn": ("alu", sink_flops),
             "merge": ("hbm", x_bytes + y_bytes + sumM * 4),

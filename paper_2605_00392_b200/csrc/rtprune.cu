@@ -582,43 +582,46 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
             // tile's image uses fewer, see sr_ctas), more while the device has SMs to spare and a CTA would have more
             // than 10 000 cells (an exchange of column sums costs less than a pass over that many).  A batch that would
             // then take more than four waves of CTAs halves it: the few tiles that do not fit read a part of K from L2.
-            // Batches of more CTAs than SMs take CTAs of half the threads and half the shared memory, two to an SM, for tiles of
-            // up to 255 columns: what one spends on its set-up, barriers and results the other iterates in.  Two CTAs per image for
-            // one only in batches of four waves or more and with a fixed ratio, when most tiles are as large as the largest possible
-            // one.  Event times, 512 threads -> 256: 1014 x 69 at a dynamic ratio 90 -> 51 us, 1024 x 400 at r = 0.25 197 -> 172 (2
-            // CTAs per image); whole runs of 700 images of 150-400 tokens at r = 0.25 588 -> 562, but 300 x 400 at r = 0.25 394 ->
-            // 401, 250 of 200-400 in fp32 storage at r = 0.3 522 -> 531, and 479 of 199-304 at a dynamic ratio 379 -> 392.
             const int mb = std::min(maxB, kSrMaxB);
+            auto floats = [&](int c1, int warps) {
+                long long most = 0;
+                for (int b = 1; b <= mb; ++b) {
+                    const int rows = (std::max(maxN - b, 1) + c1 - 1) / c1;
+                    most = std::max(most, (long long)sr_smem_rows(b, rows) * score_pitch(b) + sr_aux_floats(b, c1, rows, warps));
+                }
+                return most;
+            };
             const long long cells = (long long)(maxN - std::min(mb, maxN / 2)) * std::min(mb, maxN / 2);
             const int spread = 2LL * batch <= plan->sm_count ? 10000 : 40000;
-            int sr_threads = kSrThreads, cc = 1, full_cc = 0, smem_floats_rows = 0;
-            for (;; sr_threads /= 2) {
-                const bool half = sr_threads < kSrThreads;
-                auto floats = [&](int c1) {
-                    long long most = 0;
-                    for (int b = 1; b <= mb; ++b) {
-                        const int rows = (std::max(maxN - b, 1) + c1 - 1) / c1;
-                        most = std::max(most, (long long)sr_smem_rows(b, rows) * score_pitch(b) + sr_aux_floats(b, c1, rows, sr_threads / 32));
-                    }
-                    return most;
-                };
-                const long long limit = (half ? std::min(plan->fast_smem_bytes, kSrHalfSmemBytes) : plan->fast_smem_bytes) / (int)sizeof(float);
-                cc = 1;
-                while (cc < kSrMaxC && floats(cc) > limit) cc *= 2;
-                while (cc < kSrMaxC && (long long)batch * cc * 2 <= plan->sm_count && cells > (long long)spread * cc) cc *= 2;
-                if (!half && full_cc == 0 && mb <= 255 && (long long)batch * cc > plan->sm_count) {
-                    full_cc = cc;
-                    continue;
-                }
-                if (half && cc > full_cc && (params->dynamic || full_cc > 1 || (long long)batch < 4LL * plan->sm_count)) {     // back to the whole SM
-                    sr_threads = 2 * kSrThreads;
-                    continue;
-                }
-                if (cc > 1 && (long long)batch * cc > (half ? 8LL : 4LL) * plan->sm_count) cc /= 2;
-                smem_floats_rows = (int)std::min(limit, floats(cc)) & ~3;
-                break;
-            }
-            const bool half = sr_threads < kSrThreads;
+            long long limit = plan->fast_smem_bytes / (int)sizeof(float);
+            int cc = 1;
+            while (cc < kSrMaxC && floats(cc, kSrThreads / 32) > limit) cc *= 2;
+            while (cc < kSrMaxC && (long long)batch * cc * 2 <= plan->sm_count && cells > (long long)spread * cc) cc *= 2;
+            // More images than SMs, a CTA each, tiles of up to 255 columns: CTAs of half the threads and half the shared memory, two
+            // to an SM: what one spends on its set-up, barriers and results the other iterates in.  A part of the largest tile's K may
+            // then lie in L2, three eighths with a fixed ratio, any with a dynamic one, under which most tiles are far smaller: that
+            // takes two images per SM nearly (four in fp32 storage, which has no merge to overlap).  At a small eps images run
+            // 30 to 100 iterations, each slower beside another, and the slowest hold up a batch of a wave or two: only small tiles there,
+            // tiles that fit in larger batches, and larger ones with a fixed ratio and four images per SM.  Whole runs, a CTA per SM -> two:
+            // eps = 1: 1014 x 69 tokens dynamic 346 -> 305 us, 180 x 200 at r = 0.25 136 -> 132, 260 x 400 at r = 0.25 312 -> 306, 1024 x
+            // 400 at r = 0.25 1119 -> 1096, at r = 0.35 1328 -> 1314, dynamic 1089 -> 1057; but 150 x 400 at r = 0.25 214 -> 225, 700 x 400 at
+            // r = 0.5 (40 % in L2) 945 -> 951, 250 x 200-400 in fp32 storage at r = 0.3 519 -> 522.
+            // eps = 0.2: 220 x 300 at r = 0.25 258 -> 249, but 260 x 400 dynamic 344 -> 370.
+            // eps = 0.1: 160 x 69 at r = 0.25 144 -> 120, 310 x 256 at r = 0.4 410 -> 383, 592 x 400 at r = 0.25 956 -> 900, 400 x 256 dynamic
+            // 412 -> 400; but 160 x 200 dynamic 221 -> 245, 310 x 256 dynamic 326 -> 339, 310 x 400 at r = 0.25 576 -> 592, 450 x 400
+            // dynamic 736 -> 810.
+            // Where a tile takes several CTAs on whole SMs: 128 x 1156 at r = 0.2 576 -> 610, 100 x 1000 at r = 0.25 396 -> 417.  Two halves
+            // for one whole: 1024 x 400 at r = 0.25 1119 -> 1135, at r = 0.5 1348 -> 1368.
+            const long long half_limit = std::min(plan->fast_smem_bytes, kSrHalfSmemBytes) / (int)sizeof(float);
+            const float per_sm = (float)batch / plan->sm_count;
+            int percent = 100;                   // of half an SM: the largest tile
+            if (per_sm >= (kTensor ? 1.7f : 4.f)) percent = !params->dynamic ? 160 : params->eps >= 0.25f ? 200 : 100;
+            if (params->eps < 0.15f && per_sm < 4.f) percent = per_sm <= (params->dynamic ? 2.5f : 2.f) ? 45 : 100;
+            const bool half = cc == 1 && mb <= 255 && batch > plan->sm_count && 100 * floats(1, kSrThreads / 64) <= percent * half_limit;
+            if (half) limit = half_limit;
+            if (cc > 1 && (long long)batch * cc > 4LL * plan->sm_count) cc /= 2;
+            const int sr_threads = half ? kSrThreads / 2 : kSrThreads;
+            const int smem_floats_rows = (int)std::min(limit, floats(cc, sr_threads / 32)) & ~3;
             all_fast = maxB <= kSrMaxB;
             rows_max_b = kSrMaxB;
             // When one kernel solves every image, it hands them to the merge kernel one by one
@@ -632,7 +635,7 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
                                  pbuf, pbuf_pitch, o.merged_idx, o.merge_partner, o.merge_weight, o.stats,
                                  (uint32_t *)(ws + L.sink_done), ready_list, (WsHeader *)(ws + L.header), sd, split, by_image)))
                 return RTPRUNE_ERR_CUDA;
-            launched(plan, st, mb > 255 ? "sinkhorn_rows_wide" : "sinkhorn_rows");
+            launched(plan, st, half ? "sinkhorn_rows_half" : mb > 255 ? "sinkhorn_rows_wide" : "sinkhorn_rows");
         }
         // Scaling form, tiles left (more than kSrMaxB columns)
         const size_t tall_smem = (size_t)std::max(plan->smem_optin - 1024, 0);

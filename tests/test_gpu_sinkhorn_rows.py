@@ -25,11 +25,38 @@ def test_hand_over_to_the_merge_with_mixed_cluster_sizes():
     parity.check_workload(w)
 
 
-# More CTAs than SMs and tiles of up to 255 columns: CTAs of 256 threads, two to an SM, at the same edges of lane layouts, one per
-# image or (600 images) two; tiles that half an SM does not hold go to the whole one.
-@pytest.mark.parametrize("lengths,r,iters", [([62, 64, 66, 126, 128, 200, 3, 2] * 20, 0.5, 100), ([69] * 150, 0.5, 100),
-                                             ([254, 256, 30] * 60, 0.4, 30), ([400] * 600, 0.25, 30), ([510] * 150, 0.5, 20)])
-def test_half_size_ctas(lengths, r, iters):
+# More images than SMs and tiles of up to 255 columns: CTAs of 256 threads, two to an SM, at the same edges of lane layouts, with K in
+# shared memory or (400 tokens) partly in L2; in bf16 storage plans and the hand-over to the merge too, ragged and dynamic.  A CTA
+# per SM again (no length has r N within 32 bits' rounding of a half, 0.35 x 30 = 10.5 would):
+# more than three eighths in L2, or any in a batch of little more than a wave, tiles of more than one CTA, more than 255 columns, and large
+# tiles of a small batch at a small eps.
+RAGGED = [62, 64, 66, 126, 128, 200, 3, 2]
+
+
+@pytest.mark.parametrize("lengths,d,dtype,params,kernel", [
+    (RAGGED * 20, 64, torch.float32, dict(r_fixed=0.5), "sinkhorn_rows_half"),
+    ([69] * 150, 64, torch.float32, dict(r_fixed=0.5), "sinkhorn_rows_half"),
+    ([254, 256, 30] * 60, 64, torch.float32, dict(r_fixed=0.4, iters=30), "sinkhorn_rows_half"),
+    ([400] * 600, 64, torch.float32, dict(r_fixed=0.25, iters=30), "sinkhorn_rows_half"),
+    (RAGGED * 20, 1280, torch.bfloat16, dict(r_fixed=0.5), "sinkhorn_rows_half"),
+    ([400, 31, 280, 1, 333] * 52, 1280, torch.bfloat16, dict(r_fixed=0.35), "sinkhorn_rows_half"),
+    ([256, 99, 180] * 51, 1280, torch.bfloat16, dict(dynamic=1, phi_lo=0.0, phi_hi=0.5, r_max=0.5), "sinkhorn_rows_half"),
+    (RAGGED * 20, 1280, torch.bfloat16, dict(r_fixed=0.25, eps=0.1), "sinkhorn_rows_half"),
+    (RAGGED * 20, 1280, torch.bfloat16, dict(r_fixed=0.5, eps=0.1), "sinkhorn_rows"),
+    ([400] * 150, 1280, torch.bfloat16, dict(r_fixed=0.25, iters=20), "sinkhorn_rows"),
+    ([400] * 260, 1280, torch.bfloat16, dict(r_fixed=0.5, iters=20), "sinkhorn_rows"),
+    ([508] * 150, 64, torch.float32, dict(r_fixed=0.5, iters=20), "sinkhorn_rows"),
+    ([510] * 150, 64, torch.float32, dict(r_fixed=0.5, iters=20), "sinkhorn_rows_wide")])
+def test_half_size_ctas(lengths, d, dtype, params, kernel):
     import parity
-    w = synth.ragged(lengths, d=64, dtype=torch.float32, params=dict(r_fixed=r, iters=iters))
-    parity.check_workload(w, images=list(range(8)) + [len(lengths) - 1])
+    from paper_2605_00392_b200 import binding
+    w = synth.ragged(lengths, d=d, dtype=dtype, params=params)
+    plan = binding.Plan(w.d, w.X.dtype, w.batch, w.total_tokens, w.max_tokens)
+    try:
+        plan.profile_enable(True)
+        parity.check_workload(w, plan=plan, images=list(range(8)) + [len(lengths) - 1])
+        names = [n for n, _ in plan.profile_read()]
+        assert [n for n in names if n.startswith("sinkhorn")] == [kernel], names
+        plan.profile_enable(False)
+    finally:
+        plan.close()
