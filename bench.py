@@ -692,7 +692,7 @@ def main() -> None:
             "graph_replay": {"ms_per_step": ms_graph, "value": world * batch / (ms_graph / 1e3), "unit": "images/s",
                              "note": "the K steps as replays of CUDA graphs, one captured rtprune_run per buffer set"},
             "config": {"workload": WORKLOAD_DESC, "global_batch": world * batch,
-                       "accumulate": "fp32", "sinkhorn": "T=100 with exit at the fixed point (no dual moves by more than 1 ulp)",
+                       "accumulate": "fp32", "sinkhorn": "T=100 with exit at the fixed point (no dual moves by more than 1 ulp, or all V by one factor within 2^-23)",
                        "mean_iterations_run": float(iters_run.mean()),
                        "mean_retention": float(sumM) / total,
                        "l2": "inputs and outputs rotate over %d buffer sets (%.0f MB > L2)"

@@ -3,7 +3,7 @@
 // iterations, and the two CTAs' column sums exchanged by asynchronous stores counted on a barrier (no
 // cluster-wide barrier in the loop).  The iteration itself is fused_iterate (fused.cuh); this kernel is
 // its stand-alone form for the schedule of separate kernels: it reads the scores from the workspace tile,
-// writes alpha P (bf16, row = token position) for the tensor-core merge, hands the image to the merge
+// writes alpha P (bf16, row = position among the kept tokens) for the tensor-core merge, hands the image to the merge
 // kernel as soon as that is done, and then writes the pairs.  Taken instead of sinkhorn_rows_kernel when
 // every tile the run can hold fits: at most 256 pruned tokens, 64 K values per thread.
 #pragma once

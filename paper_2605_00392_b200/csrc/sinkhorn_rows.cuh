@@ -59,7 +59,7 @@ __host__ __device__ inline int sr_width(int B) { return B < 32 ? 32 : (B < 64 ? 
 // Rows of a warp's batch (at most): K in shared memory is padded to whole batches.
 __host__ __device__ inline int sr_batch_rows(int B) { return B < 64 ? 32 : (B < 128 ? 16 : (B < 256 ? 8 : 4)); }
 // Floats of shared memory besides K: the warps' column sums (the pairing's values and indices take their place), the
-// CTAs' column sums of two iterations, V, and per row (of whole batches) U and its token.
+// CTAs' column sums of two iterations, V, and U per row (of whole batches).
 __host__ __device__ inline int sr_aux_floats(int B, int C, int rows, int warps)
 {
     const int w = sr_width(B);
