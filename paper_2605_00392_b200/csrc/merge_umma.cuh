@@ -364,7 +364,9 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapXp, const __grid_const
             if (q.ct == 0 && tok >= 0) kept_idx[q.out0 + p] = tok;
             const int nrows = max(0, min(32, q.M - (q.mt * kMgTileM + lrow)));
             const int col_end = min(d, (q.ct + 1) * kMgTileN);
-            for (int col = q.ct * kMgTileN; col < col_end; col += kMgOwnCols) {
+            // (the second half's tile also where a unit has no such columns: a thread of the epilogue that passed a tile by could
+            // take an earlier phase of its barrier for a later one)
+            for (int col = q.ct * kMgTileN; col < (q.ct + 1) * kMgTileN; col += kMgOwnCols) {
                 const bool ok = ptx::mbar_wait(&bars->own_empty[buf], phase);
                 if (!__all_sync(0xffffffffu, ok)) {
                     bars->abort_flag = 1;
@@ -407,22 +409,16 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapXp, const __grid_const
             const int buf = n & 1;
             const int col = q.ct * kMgTileN + half * kMgOwnCols, ncols = min(kMgOwnCols, d - col);    // (may be <= 0)
             // own rows: the tile of this thread's half
-            int mine = ob;
-            uint32_t mine_phase = phase;
-            const int tiles = d - q.ct * kMgTileN > kMgOwnCols ? 2 : 1;
-            for (int k = 0; k < tiles; ++k) {
-                if (k == half) {
-                    mine = ob;
-                    mine_phase = phase;
-                }
-                if (++ob == bufs) {
-                    ob = 0;
-                    phase ^= 1u;
-                }
+            const int mine = ob + half;                          // (there is an even number of them)
+            const uint32_t mine_phase = phase;
+            ob += 2;
+            if (ob == bufs) {
+                ob = 0;
+                phase ^= 1u;
             }
             // the TMEM loads below are warp-collective: take the go / no-go decision per warp
             bool ok = !bars->abort_flag && ptx::mbar_wait(&bars->accum_full[buf], (n >> 1) & 1) &&
-                      (ncols <= 0 || ptx::mbar_wait(&bars->own_full[mine], mine_phase));
+                      ptx::mbar_wait(&bars->own_full[mine], mine_phase);
             if (!__all_sync(0xffffffffu, ok)) {
                 bars->abort_flag = 1;
                 if (lane == 0) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
@@ -461,17 +457,15 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapXp, const __grid_const
             ptx::tc_fence_before();
             ptx::mbar_arrive(&bars->accum_empty[buf]);
             __syncwarp();                                     // the warp's rows are complete
-            if (ncols > 0) {
-                const int sub = lane >> 4, piece = lane & 15, nrows = min(32, q.M - prow0);      // (may be <= 0)
-                __nv_bfloat16 *dst = Y + (size_t)(q.out0 + prow0) * d + col + piece * 8;
-                if (piece * 8 < ncols) {
+            const int sub = lane >> 4, piece = lane & 15, nrows = min(32, q.M - prow0);      // (may be <= 0)
+            __nv_bfloat16 *dst = Y + (size_t)(q.out0 + prow0) * d + col + piece * 8;
+            if (piece * 8 < ncols) {
 #pragma unroll 8
-                    for (int r = sub; r < nrows; r += 2)
-                        *reinterpret_cast<uint4 *>(dst + (size_t)r * d) =
-                            *reinterpret_cast<const uint4 *>(tile + (w0 + r) * 256 + ((piece ^ (r & 7)) << 4));
-                }
-                ptx::mbar_arrive(&bars->own_empty[mine]);     // (after this thread's reads)
+                for (int r = sub; r < nrows; r += 2)
+                    *reinterpret_cast<uint4 *>(dst + (size_t)r * d) =
+                        *reinterpret_cast<const uint4 *>(tile + (w0 + r) * 256 + ((piece ^ (r & 7)) << 4));
             }
+            ptx::mbar_arrive(&bars->own_empty[mine]);     // (after this thread's reads)
         }
     }
 

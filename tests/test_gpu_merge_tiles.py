@@ -40,3 +40,59 @@ def test_tiles(lengths, r, d):
     # the scores' own rounding
     bound = 2.0 ** -8 * (Y32.abs() + X.float().abs().max())
     assert bool(((Y.float() - Y32).abs() <= bound)[same].all())
+
+
+# Tokens in clusters and a small eps: rows of the plan that differ from one another, so that a row taken for another, or a k-block left
+# out, shows.  Kept tokens around multiples of 64 (tiles of own rows) and 128, in batches that leave SMs idle and in larger ones, where a CTA
+# has many units one after another, with a ring of four tiles of own rows and (1100 tokens) of two; widths whose last unit has no
+# columns in its second half.  Reference: the recursion in 64 bits
+# on the tokens that were kept.
+@pytest.mark.parametrize("lengths", [[84, 85, 87, 170, 171, 172, 3, 1], [84, 85, 87, 170, 171, 172, 3, 1] * 30, [64] * 200,
+                                     [255, 257, 340, 343], [400] * 40, [1100, 84] * 25])
+@pytest.mark.parametrize("d", [64, 136, 264, 392, 1096, 1280])
+def test_rows_of_the_plan(lengths, d):
+    dev, r, alpha, eps = torch.device("cuda", 0), 0.25, 0.5, 0.1
+    gen = torch.Generator(device=dev).manual_seed(d + len(lengths))
+    total = sum(lengths)
+    X = torch.randn(8, d, generator=gen, device=dev)[torch.randint(0, 8, (total,), generator=gen, device=dev)]
+    X = (X + 0.3 * torch.randn(total, d, generator=gen, device=dev)) * torch.exp(0.5 * torch.randn(total, 1, generator=gen, device=dev))
+    X = X.bfloat16()
+    start = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    offs = torch.from_numpy(start).to(dev)
+    plan = binding.Plan(d, X.dtype, len(lengths), total, max(lengths), device=dev)
+    out = binding.Outputs.allocate(total, len(lengths), d, X.dtype, dev)
+    plan.run(X, offs, binding.make_params(None, dynamic=0, r_fixed=r, alpha=alpha, eps=eps), out)
+    assert plan.query_status() == 0
+    plan.close()
+    first = out.out_offsets.cpu().numpy()
+    for n in sorted(set(lengths)):
+        images = [i for i, m in enumerate(lengths) if m == n]
+        M = int(first[images[0] + 1] - first[images[0]])
+        B = n - M
+        assert M == max(1, n - int(np.floor(r * n + 0.5)))
+        x = torch.stack([X[start[i]:start[i + 1]] for i in images]).double()
+        kept = torch.stack([out.kept_idx[first[i]:first[i] + M] for i in images]).long()
+        pruned = torch.stack([out.merged_idx[start[i] - first[i]:start[i] - first[i] + B] for i in images]).long()
+        Y = torch.stack([out.Y[first[i]:first[i] + M] for i in images]).double()
+        own = torch.gather(x, 1, kept[:, :, None].expand(-1, -1, d))
+        if B == 0:
+            assert torch.equal(Y, own)
+            continue
+        away = torch.gather(x, 1, pruned[:, :, None].expand(-1, -1, d))
+        K = torch.full((len(images), M + 1, B + 1), 0.2, dtype=torch.float64, device=dev)
+        K[:, :M, :B] = torch.nn.functional.normalize(own, dim=2) @ torch.nn.functional.normalize(away, dim=2).transpose(1, 2)
+        K = torch.exp((K - 1.0) / eps)
+        V = torch.full((len(images), B + 1, 1), float(np.exp(1.0 / eps)), dtype=torch.float64, device=dev)
+        a, b = torch.ones(M + 1, 1, dtype=torch.float64, device=dev), torch.ones(B + 1, 1, dtype=torch.float64, device=dev)
+        a[M], b[B] = B, M
+        for _ in range(100):
+            U = a / (K @ V)
+            V = b / (K.transpose(1, 2) @ U)
+        P = (alpha * U * K * V.transpose(1, 2))[:, :M, :B]
+        # bf16 rounds alpha P and the result by 2^-8 of them at most; the scores' fp32 sums of d terms, divided by eps, and the fp32
+        # recursion move P by 1e-4 of itself at most
+        bound = 2.0 ** -8 * own.abs() + (2.0 ** -7 + 1e-4) * (P @ away.abs())
+        assert bool(((Y - (own + P @ away)).abs() <= bound).all()), n
+        if M >= 60:                                            # (the bound tells rows apart: with the next row's plan most rows break it)
+            wrong = ((Y - (own + P.roll(1, 1) @ away)).abs() > bound).any(2)
+            assert float(wrong.double().mean()) > 0.5, n
