@@ -47,6 +47,7 @@ constexpr int kMgBBoxBytes = kMgBK * 128;            // one 64-column slab of it
 constexpr int kMgStageBytes = kMgABytes + kMgBBytes; // a k-block: a plan tile and a tile of pruned rows
 constexpr int kMgOwnCols = 128;                      // columns of a tile of own rows: 256 bytes a row, the 16-byte pieces
 constexpr int kMgOwnBytes = kMgTileM * kMgOwnCols * 2;   // of row r at places xor (r & 7), conflict-free either way
+constexpr int kMgShortRows = 64;                     // a unit of up to so many rows: both halves of its columns in one tile
 // Shared memory is shared out between k-blocks in flight and tiles of own rows by what a unit has of each: two k-blocks (B up to
 // 128) to two tiles of own rows, or many k-blocks.
 constexpr int kMgMaxStages = 3, kMgMaxBufs = 4;
@@ -85,6 +86,15 @@ struct MergeQueue {
     volatile uint32_t tail;          // units every role is done with
     MergeUnit e[kMgQueue];
 };
+
+// Whether a unit's own rows take one tile instead of two.  The threads of the epilogue without a row then pass the tile by, and a
+// thread that has passed a phase of a barrier by must know it complete before it waits for the next (a wait tells phases apart by
+// parity only): with four tiles the one before belongs to unit n - 2 or an earlier one, which the accumulator's barrier has shown to
+// be done; with two it can belong to unit n - 1.
+__device__ inline bool merge_few_rows(const MergeUnit &q, int bufs)
+{
+    return bufs >= 4 && q.M - q.mt * kMgTileM <= kMgShortRows;
+}
 
 // Bounded wait for the n-th unit of the queue.  false = gave up, or the kernel is being abandoned.
 __device__ inline bool merge_pop(MergeQueue *mq, const MergeBarriers *bars, uint32_t n, MergeUnit &q)
@@ -344,9 +354,10 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapXp, const __grid_const
         }
     } else if (warp >= 11) {
         // ---------------- loaders: the kept tokens' own rows ------------------------------------------
-        // A warp fetches 32 rows, two at a time (16 lanes x 16 bytes = 128 columns each).
-        const int lrow = (warp - 11) * 32, sub = lane >> 4, piece = lane & 15;
-        const uint32_t own_base = ptx::smem_u32(own) + (uint32_t)((lrow + sub) * 256);
+        // A warp fetches 32 rows, two at a time (16 lanes x 16 bytes = 128 columns each).  In a unit of up to 64 rows the second two
+        // warps take the second half of the columns, into the second half of the same tile: four such units are in flight, not two.
+        const int sub = lane >> 4, piece = lane & 15;
+        const uint32_t own_base = ptx::smem_u32(own) + (uint32_t)(((warp - 11) * 32 + sub) * 256);
         int buf = 0;                                  // tile of own rows, and its phase
         uint32_t phase = 1;
         bool alive = true;
@@ -359,14 +370,16 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapXp, const __grid_const
                 break;
             }
             if (q.img < 0) break;
+            const bool few = merge_few_rows(q, bufs);
+            const int right = few ? (warp - 11) >> 1 : 0, lrow = (few ? (warp - 11) & 1 : warp - 11) * 32;
             const int p = q.mt * kMgTileM + lrow + lane;     // position among the kept tokens
             const int tok = p < q.M ? __ldcg(order + q.t_begin + p) : -1;
-            if (q.ct == 0 && tok >= 0) kept_idx[q.out0 + p] = tok;
+            if (q.ct == 0 && right == 0 && tok >= 0) kept_idx[q.out0 + p] = tok;
             const int nrows = max(0, min(32, q.M - (q.mt * kMgTileM + lrow)));
             const int col_end = min(d, (q.ct + 1) * kMgTileN);
             // (the second half's tile also where a unit has no such columns: a thread of the epilogue that passed a tile by could
             // take an earlier phase of its barrier for a later one)
-            for (int col = q.ct * kMgTileN; col < (q.ct + 1) * kMgTileN; col += kMgOwnCols) {
+            for (int col = q.ct * kMgTileN; col < (q.ct + 1) * kMgTileN; col += few ? kMgTileN : kMgOwnCols) {
                 const bool ok = ptx::mbar_wait(&bars->own_empty[buf], phase);
                 if (!__all_sync(0xffffffffu, ok)) {
                     bars->abort_flag = 1;
@@ -374,7 +387,7 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapXp, const __grid_const
                     alive = false;
                     break;
                 }
-                const int c = col + piece * 8;
+                const int c = col + right * kMgOwnCols + piece * 8;
                 const __nv_bfloat16 *src = X + (size_t)q.t_begin * d + c;
                 const uint32_t dst = own_base + (uint32_t)(buf * kMgOwnBytes);
 #pragma unroll 4
@@ -408,17 +421,22 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapXp, const __grid_const
             if (q.img < 0) break;
             const int buf = n & 1;
             const int col = q.ct * kMgTileN + half * kMgOwnCols, ncols = min(kMgOwnCols, d - col);    // (may be <= 0)
-            // own rows: the tile of this thread's half
-            const int mine = ob + half;                          // (there is an even number of them)
-            const uint32_t mine_phase = phase;
-            ob += 2;
-            if (ob == bufs) {
-                ob = 0;
+            // own rows: the tile of this thread's half (rows past the kept ones of a unit of up to 64 have none)
+            const bool few = merge_few_rows(q, bufs), has_own = !few || row < kMgShortRows;
+            int mine = few ? ob : ob + half;
+            uint32_t mine_phase = phase;
+            if (mine >= bufs) {
+                mine -= bufs;
+                mine_phase ^= 1u;
+            }
+            ob += few ? 1 : 2;
+            if (ob >= bufs) {
+                ob -= bufs;
                 phase ^= 1u;
             }
             // the TMEM loads below are warp-collective: take the go / no-go decision per warp
             bool ok = !bars->abort_flag && ptx::mbar_wait(&bars->accum_full[buf], (n >> 1) & 1) &&
-                      ptx::mbar_wait(&bars->own_full[mine], mine_phase);
+                      (!has_own || ptx::mbar_wait(&bars->own_full[mine], mine_phase));
             if (!__all_sync(0xffffffffu, ok)) {
                 bars->abort_flag = 1;
                 if (lane == 0) atomicOr(&hdr->status, RTPRUNE_DEV_TIMEOUT);
@@ -430,7 +448,7 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapXp, const __grid_const
             // those entries are free
             if (tid == 0 && n >= 1) mq->tail = n - 1;
             const int w0 = row & ~31, prow0 = q.mt * kMgTileM + w0;      // the warp's first row of the tile, and of the kept ones
-            uint8_t *const tile = own + mine * kMgOwnBytes;
+            uint8_t *const tile = own + mine * kMgOwnBytes + (few ? half * (kMgShortRows * 256) : 0);
             // a warp whose 32 rows all lie past the kept ones has nothing to add or store
             if (prow0 < q.M && q.B > 0) {
                 uint8_t *const srow = tile + row * 256;
@@ -465,7 +483,7 @@ merge_umma_kernel(const __grid_constant__ CUtensorMap tmapXp, const __grid_const
                     *reinterpret_cast<uint4 *>(dst + (size_t)r * d) =
                         *reinterpret_cast<const uint4 *>(tile + (w0 + r) * 256 + ((piece ^ (r & 7)) << 4));
             }
-            ptx::mbar_arrive(&bars->own_empty[mine]);     // (after this thread's reads)
+            if (has_own) ptx::mbar_arrive(&bars->own_empty[mine]);     // (after this thread's reads)
         }
     }
 
