@@ -359,10 +359,12 @@ cudaError_t launch_stage1_kernel(const rtprune_plan_t *pl, cudaStream_t st, cons
     const int per_image = std::max(1, slots / std::max(batch, 1));
     int chunk_tokens = (pl->max_tokens + per_image - 1) / per_image;
     // Images of different lengths: by their mean, each with half a chunk to spare (64 of 456-1156 tokens 59 -> 49 us, 200 of
-    // 150-400 69 -> 57, 64 of 200-400 32 -> 29).  A little more than a wave of whole images: halves of them (300 x 400 118 -> 98; 500 x
-    // 400, 1.7 waves, would go from 133 to 139, 1024 x 400 from 241 to 252).
+    // 150-400 69 -> 57, 64 of 200-400 32 -> 29).  More than a wave of whole images and at most one and a half: halves of them, three
+    // waves of those at most against two whole ones; images so short that a CTA is mostly set-up up to a wave and a quarter.  Whole
+    // runs, whole -> halves: 300 x 400 tokens 385 -> 363 us, 400 x 400 481 -> 464, 444 x 400 523 -> 509, 444 x 256 328 -> 325, 430 x 700
+    // 940 -> 922, 350 x 100 149.9 -> 148.2; but 470 x 400 544 -> 550, 430 x 100 169.9 -> 172.5, 430 x 69 145.7 -> 149.5.
     if (10LL * total < 9LL * batch * pl->max_tokens) chunk_tokens = total / std::max(slots - batch / 2, slots / 2);
-    else if (batch > slots && 4 * batch <= 5 * slots) chunk_tokens = (pl->max_tokens + 1) / 2;
+    else if (batch > slots && 4 * batch <= (pl->max_tokens >= 256 ? 6 : 5) * slots) chunk_tokens = (pl->max_tokens + 1) / 2;
     chunk_tokens = std::min(512, std::max(kChunkTokens, (chunk_tokens + 7) / 8 * 8));
     const int chunks_run = (pl->max_tokens + chunk_tokens - 1) / chunk_tokens;   // <= L.chunks
     dim3 grid(chunks_run, batch);
