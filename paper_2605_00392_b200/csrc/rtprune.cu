@@ -713,10 +713,11 @@ rtprune_status_t launch_stage2(rtprune_plan_t *plan, cudaStream_t st, const void
         const int nct = (plan->d + kMgTileN - 1) / kMgTileN;
         const long long nunits = (long long)batch * mtiles_m * nct;
         const int grid = (int)std::min<long long>(nunits, plan->sm_count);
-        // shared memory for a deep ring of k-blocks where an image has many, else for more tiles of own rows (with a dynamic ratio
-        // most images prune far less than the most they may: 128 of 456-1156 tokens 418 -> 416 us with the latter, but 40 of
-        // 1000-1156 at r = 0.48 323 -> 332)
-        const bool deep = maxB > kSrMaxB || (maxB > kMgDeepB && !params->dynamic);
+        // shared memory for a deep ring of k-blocks where an image has many, else for more tiles of own rows.  Whole runs, tiles -> ring:
+        // 100 x 700 tokens at r = 0.4 364 -> 359 us, 40 x 1156 at r = 0.48 360 -> 351, 100 x 1156 at r = 0.25 580 -> 573, 16 x 2137 dynamic
+        // 393 -> 387.  With a dynamic ratio most images prune far less than the most they may, and up to there it is all one (64 x 1156 364,
+        // 366; 16 x 900 108.3, 107.7); batches of images short against the plan have few k-blocks (64 x 400, plan for 1400, 160 -> 163).
+        const bool deep = (maxB > kSrMaxB && 2LL * total >= (long long)batch * maxN) || (maxB > kMgDeepB && !params->dynamic);
         const int mg_stages = deep ? 3 : 2, mg_bufs = deep ? 2 : 4;
         if (!c.ok(launch_pdl(merge_umma_kernel, dim3((unsigned)grid), dim3(kMgThreads), (size_t)merge_smem_bytes(mg_stages, mg_bufs), st, 1u,
                              tmapXpm, tmapP, (const __nv_bfloat16 *)X, offsets, plan->d, batch, mtiles_m, o.counts, o.out_offsets,
