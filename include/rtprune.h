@@ -112,9 +112,9 @@ typedef struct {
     int32_t stop_at_fixed_point; /* 1: leave the loop once an iteration reproduces its input, whatever the
                              batch size and storage type: every dual of the scaling form within one unit in
                              the last place of its previous value, or in a cycle of rounding (within four
-                             units of it and back within one unit of the value before that), or all column
-                             duals V within one unit of their previous values times a common factor (V -> cV,
-                             U -> U/c is the same plan); images with more than 639 pruned tokens: every dual
+                             units of it and back within one unit of the value before that), or the relative
+                             moves of all column duals V within 2^-22 of each other, each within 2^-23 of a
+                             common factor (V -> cV, U -> U/c is the same plan); images with more than 639 pruned tokens: every dual
                              within four units, the rounding noise of their long sums; bit-identical log-domain
                              duals in the LOG form.  Later iterations could only move the plan within
                              rounding, so the result is that of all `iters` iterations to fp32 accuracy.
@@ -128,7 +128,8 @@ typedef struct {
 /* Number of floats per image in the `stats` output. */
 #define RTPRUNE_STATS_STRIDE 8
 /* stats[i*8 + ..]: 0 phi, 1 rho, 2 r, 3 M (kept), 4 B (pruned), 5 Sinkhorn iterations executed,
- *                  6 largest dual change of the last executed iteration (log units), 7 reserved */
+ *                  6 largest dual change of the last executed iteration (log units; a factor common to all
+ *                  V, see stop_at_fixed_point, counts), 7 reserved */
 
 /* Bits of the device status word (rtprune_query_status). */
 #define RTPRUNE_DEV_NONFINITE 1u

@@ -24,13 +24,13 @@ __host__ __device__ inline bool dual_settled(int now, int last, int before)
 
 // The recursion leaves U -> U/c, V -> cV free, and rounding moves c by a unit or two per iteration long after the plan U K V
 // has settled.  lo and hi: the smallest and largest relative move (V - V_last) / V_last of an iteration over all columns, the
-// dustbin's among them.  Settled: they lie within two units of 2^-23 of each other, that is every column within one unit of a
-// common factor: what single duals that each move by one unit at most, up or down, can spread over.  A column that still
-// drifts against the others keeps the loop going.  Measured against 64 bits on the device, 64 to 1156 tokens, eps 1, 0.3 and
-// 0.1: the weights' rms error is that of the rule for single duals within 2 % either way (bf16 storage 0.2 to 2.2e-6, fp32
-// 1.9 to 3.3e-7), and the loop is shorter by 1 iteration of 7 at eps = 1, 2 of 15 at 0.3, 3 of 32 at 0.1, the longest of a
-// batch of 64 or 128 images at eps = 1 by 6 of 15 and 7 of 18: 1 x 400 48.3 -> 45.6 us, 32 x 256 65.4 -> 61.7, 64 x 400 105.5
-// -> 103.9, 128 of 456-1156 433 -> 424, 64 of them at eps = 0.1 590 -> 576.
+// dustbin's among them.  Settled: they lie within 2^-22 of each other, so that every column is within 2^-23 of its value (one to
+// two units in the last place, by its mantissa) of a common factor: what single duals that each move by 2^-23 at most, up or down,
+// can spread over.  One column alone may move by two or three units; one that drifts by more against the others keeps the loop
+// going.  Measured against 64 bits on the device: the weights' rms error is that of the rule for single
+// duals and of all 100 iterations within 1 % (bf16 storage 1.0e-6 at eps = 1, 1.6e-6 at 0.3, 2.2e-6 at 0.1, 3.6 to 4.2e-6 at 0.05; fp32
+// 1.6 to 1.9e-6 at 0.05 to 0.07; 64 to 1156 tokens), and images leave after 6.4 iterations instead of 7.5 on average at eps = 1 (the
+// longest of 64 after 8 instead of 12), 12.4 instead of 14.9 at 0.3, 25 instead of 28 at 0.1, 34 to 82 instead of 37 to 83 at 0.05.
 constexpr float kPlanSpread = 2.38418579e-7f;      // 2 * 2^-23
 // (Where a column is not a number, lo and hi are none either: the rule for single duals decides.)
 __host__ __device__ inline bool plan_settled(float lo, float hi) { return hi - lo <= kPlanSpread; }

@@ -1,5 +1,6 @@
 """The rule by which an iteration of the scaling form counts as settled up to a common factor (csrc/settled.h), compiled for
-the host: a factor that all columns share ends the loop, a column that moves against the others does not, however slowly."""
+the host: a factor that all columns share ends the loop, a column that moves against the others by more than 2^-22 of its value
+(two or three units in the last place, by its mantissa) does not."""
 import ctypes
 import os
 import subprocess
@@ -50,3 +51,13 @@ def test_a_common_factor_settles_and_a_column_that_drifts_does_not(settled, colu
             far = last.copy()
             far[0] = last[0] * (1 + sign * steps * unit)
             assert not settled(far, last), (sign, steps)
+
+
+@pytest.mark.parametrize("mantissa,most", [(1.0, 2), (1.25, 2), (1.5, 3), (1.99999, 3)])
+def test_how_far_one_column_may_move_alone(settled, mantissa, most):
+    for scale in (2.0 ** -30, 1.0, 2.0 ** 40):
+        last = np.array([1.0, mantissa * scale, 3.0], np.float32)
+        for ulps in range(1, 6):
+            now = last.copy()
+            now.view(np.int32)[1] += ulps
+            assert settled(now, last) == (ulps <= most), (scale, ulps)
