@@ -17,7 +17,7 @@
 // fifths of a long one), own rows by another path instead of as UMMA operands against an identity tile.
 // Against token tiles with own rows through the tensor cores (event times): 1024 x 400 at r = 0.25 426 -> 344 us,
 // 128 images of 456-1156 tokens 141 -> 113, 16 x 2137 133 -> 71, 8 x 4512 223 -> 111, 64 x 400 39 -> 37; 1014 images of 69
-// tokens 90 -> 102 (half-empty tiles: too few own rows in flight).
+// tokens 91 -> 89 at r = 0.25, 89 -> 95 at a dynamic ratio (99 and 103 while a unit of up to 64 rows took two tiles of own rows).
 // The kernel is persistent: CTA c takes units c, c + gridDim.x, ...  When the Sinkhorn kernel ahead
 // publishes a list of finished images, the units follow that list (its s-th entry takes the place of
 // image s), the CTAs draw them from a counter, and the scheduler waits, bounded, for the entry it
